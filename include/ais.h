@@ -358,7 +358,7 @@ int ais_scatter_words(const void* src, const int32_t* row_index, int64_t n, void
  * the library is loaded holds it until the process exits.  The call allocates and frees nothing.
  *   - T must not exceed AIS_STATIC_MAX_ROWS; a larger T returns AIS_ERR_LIMIT and enqueues nothing.
  *   - shape->d must be a multiple of 64 and V of 8; P, G and fp8_block are not read.  The vocabulary
- *     is always streamed in 4 ranges.
+ *     is streamed in 4 ranges at the row limit, in as many as keep the GPU busy for fewer rows.
  *   - The first call on each device resolves the array's device address and prepares the kernels; that is
  *     also the moment at which the CUDA runtime may load this part of the library onto the device, and the
  *     1.5 MiB array comes with it.  So the device does take that memory once, at the first call, not at a

@@ -78,6 +78,29 @@ bool make_tmap(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, ui
     return r == CUDA_SUCCESS;
 }
 
+// The units of a pass are (row tile, vocabulary range) pairs handed round robin to one persistent CTA per SM, so its time
+// is waves x tiles of the longest range.  Four ranges for everybody left a response of 613 rows (5 row tiles) on 20 of 148
+// SMs (3.2 ms per pass at d = 4096, V = 151936) and ran 79 row tiles as three waves where 2.1 were full.  The number of
+// ranges with the least waves x tiles wins, with a slight handicap for many ranges: the fewer row tiles are in flight, the
+// more often W is read.  From below it is bounded by L2: the hidden rows of the row tiles in flight are read again for
+// every column tile and should take no more than 40 MB of it.
+int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most) {
+    if (row_tiles < 1) row_tiles = 1;
+    if (most > col_tiles) most = col_tiles;
+    if (most < 1) most = 1;
+    int best = 1;
+    double best_cost = 0.0;
+    for (int s = 1; s <= most; ++s) {
+        int64_t in_flight = kSms / s > 0 ? kSms / s : 1;
+        if (in_flight > row_tiles) in_flight = row_tiles;
+        if (in_flight * kBM * d * 2 > (int64_t(40) << 20) && s < most) continue;
+        const int64_t waves = (row_tiles * s + kSms - 1) / kSms;
+        const double cost = static_cast<double>(waves) * ((col_tiles + s - 1) / s) * (1.0 + s / 400.0);
+        if (best_cost == 0.0 || cost < best_cost) { best = s; best_cost = cost; }
+    }
+    return best;
+}
+
 }  // namespace ais
 
 namespace {
@@ -122,14 +145,35 @@ int check_params(const ais_params* p) {
     return AIS_OK;
 }
 
-int pick_nsplit(const ais_shape* s, const ais_params* p) {
+// vocab_chunk asks for its own ranges (at most 64); otherwise the pass gets what plan_ranges finds best.
+int pick_nsplit(const ais_shape* s, const ais_params* p, int64_t row_tiles) {
     const int n_col_tiles = (s->V + kBN - 1) / kBN;
-    int nsplit = 4;
-    if (p->vocab_chunk > 0) nsplit = (s->V + p->vocab_chunk - 1) / p->vocab_chunk;
+    if (p->vocab_chunk <= 0) return plan_ranges(row_tiles, n_col_tiles, s->d, kMaxRanges);
+    int nsplit = (s->V + p->vocab_chunk - 1) / p->vocab_chunk;
     if (nsplit > 64) nsplit = 64;
     if (nsplit > n_col_tiles) nsplit = n_col_tiles;
-    if (nsplit < 1) nsplit = 1;
-    return nsplit;
+    return nsplit < 1 ? 1 : nsplit;
+}
+
+// dH: the last, partial wave of 256 x 256 output tiles would leave most SMs idle for the length of a whole contraction
+// over the vocabulary (16 tiles of 148 SMs for one row pair at d = 4096, 60 of the 800 = 5.4 waves for 10,003 rows at
+// d = 5120).  Its tiles are split into ranges of the contraction whose fp32 partial tiles are added afterwards.
+// split_cost: microseconds of the tail for ks ranges, from the 0.83 us of a stage fill at 1.5 PFLOP/s and 256 KB written
+// and read per partial tile at 6 TB/s plus the extra launch.  A range keeps at least four stage fills (the depth of the
+// ring plus one), and the partial tiles number at most kSplitSlots (116 MB).
+constexpr int kSplitSlots = 3 * kSms;
+double split_cost(int tiles, int ks, int ksteps) {
+    const double waves = (static_cast<int64_t>(tiles) * ks + kSms - 1) / kSms;
+    return waves * ((ksteps + ks - 1) / ks) * 0.83 + (ks > 1 ? 6.0 + tiles * ks * 0.087 : 0.0);
+}
+int pick_ksplit(int tiles, int ksteps, int slots) {
+    int best = 1;
+    double best_cost = split_cost(tiles, 1, ksteps);
+    for (int ks = 2; ks <= 64 && ks * tiles <= slots && ks * 4 <= ksteps; ++ks) {
+        const double c = split_cost(tiles, ks, ksteps);
+        if (c < 0.97 * best_cost) { best = ks; best_cost = c; }
+    }
+    return best;
 }
 
 struct Layout {
@@ -141,6 +185,8 @@ struct Layout {
     size_t off_pace;                              // ring of counters that keeps the CTAs of a tensor-core launch in step
     size_t off_coef, off_nseq;                    // backward: c_t, valid rows per sequence
     size_t off_seqw;                              // sequence-level variant: log weight per sequence
+    size_t off_split;                             // dH: partial tiles of the split units
+    int split_slots, ksplit;                      // how many there is room for; ksplit > 0: ranges fixed by the shape alone
     size_t off_u;                                 // backward scratch
     int64_t ldU;
     size_t fixed_bytes;                           // everything but the scratch rows
@@ -150,7 +196,7 @@ struct Layout {
 Layout make_layout(const ais_shape* s, const ais_params* p) {
     Layout L;
     L.t_ld = static_cast<int64_t>(align_up(static_cast<size_t>(s->T > 0 ? s->T : 1), 64));
-    L.nsplit = pick_nsplit(s, p);
+    L.nsplit = pick_nsplit(s, p, (s->T + kBM - 1) / kBM);
     L.nparts = L.nsplit * 2;
     size_t off = 0;
     const size_t part_bytes = align_up(static_cast<size_t>(L.nparts) * L.t_ld * sizeof(float), 256);
@@ -163,6 +209,19 @@ Layout make_layout(const ais_shape* s, const ais_params* p) {
     L.off_coef = off;   off += align_up(static_cast<size_t>(L.t_ld) * sizeof(float), 256);
     L.off_nseq = off;   off += align_up(static_cast<size_t>(s->P) * s->G * sizeof(int32_t), 256);
     L.off_seqw = off;   off += align_up(static_cast<size_t>(s->P) * s->G * sizeof(float), 256);
+    {
+        // a batch whose dH tiles do not fill one wave gets its ranges from its size alone, so that the split (and with it
+        // every bit of dH) is the same whatever the workspace lets a pass hold
+        const int64_t tiles = ((s->T + kDhRows - 1) / kDhRows) * ((s->d + kBN - 1) / kBN);
+        const int ksteps = (s->V + 63) / 64;
+        L.ksplit = 0;
+        L.split_slots = kSplitSlots;
+        if (tiles < kSms) {
+            L.ksplit = tiles > 0 ? pick_ksplit(static_cast<int>(tiles), ksteps, kSplitSlots) : 1;
+            L.split_slots = L.ksplit > 1 ? static_cast<int>(tiles) * L.ksplit : 0;
+        }
+    }
+    L.off_split = off;  off += static_cast<size_t>(L.split_slots) * kPartTileFloats * sizeof(float);
     L.off_u = off;
     L.ldU = static_cast<int64_t>(align_up(static_cast<size_t>(s->V), 64));
     L.fixed_bytes = off;
@@ -170,7 +229,7 @@ Layout make_layout(const ais_shape* s, const ais_params* p) {
     return L;
 }
 
-constexpr int64_t kBwdRowsRecommended = 2 * 148 * kBM;
+constexpr int64_t kBwdRowsRecommended = 2 * kSms * kBM;
 
 // Zeroes the pacing ring and points the launch at it.  tiles_per_unit = the largest number of column tiles a unit of
 // the launch walks; a launch of a single wave has nobody to keep in step with over time and runs without pacing only
@@ -450,7 +509,7 @@ int ais_diagnostics(const ais_shape* shape, const ais_params* params, const floa
     if (!aligned(diag, 8)) return AIS_ERR_ALIGN;
     const Layout L = make_layout(shape, params);
     const bool seq_level = params->seq_level_weights != 0;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < (seq_level ? L.off_u : L.off_coef)) return AIS_ERR_WORKSPACE;
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < (seq_level ? L.off_split : L.off_coef)) return AIS_ERR_WORKSPACE;
     st = device_setup(nullptr);
     if (st != AIS_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -591,7 +650,7 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
         // recompute softmax - onehot into the scratch
         a.ncols = shape->V;
         a.n_col_tiles = (shape->V + kBN - 1) / kBN;
-        a.nsplit = L.nsplit;
+        a.nsplit = pick_nsplit(shape, params, a.n_row_tiles);
         a.ksteps = shape->d / 64;
         int units = a.n_row_tiles * a.nsplit;
         if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, units < num_sms ? units : num_sms, s) != cudaSuccess)
@@ -605,9 +664,23 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
         a.nsplit = 1;
         a.ksteps = (shape->V + 63) / 64;
         units = a.n_row_tiles * a.n_col_tiles;
+        const int tail = units % kSms;
+        a.split_from = units;
+        a.ksplit = 1;
+        if (tail > 0) {
+            int ks = L.ksplit > 0 ? L.ksplit : pick_ksplit(tail, a.ksteps, L.split_slots);
+            if (ks > 1 && ks * tail > L.split_slots) ks = L.split_slots / tail;
+            if (ks > 1) {
+                a.split_from = units - tail;
+                a.ksplit = ks;
+                a.part_acc = reinterpret_cast<float*>(ws + L.off_split);
+                units = a.split_from + tail * ks;
+            }
+        }
         if (arm_pace(a, ws, L, 1, units < num_sms ? units : num_sms, s) != cudaSuccess) return AIS_ERR_DEVICE;
         if (launch_lmhead(dv ? kBwdDhDv : kBwdDh, tmU, tmW_n, tmU, tmW_n, a, units < num_sms ? units : num_sms, s) != cudaSuccess)
             return AIS_ERR_DEVICE;
+        if (a.ksplit > 1 && launch_dh_reduce(a, s) != cudaSuccess) return AIS_ERR_DEVICE;
         if (dW) {
             // dW (+)= U^T H over the rows of this pass: both operands are read with the rows as contraction axis;
             // the maps end at `rows`, so rows the scratch still holds from an earlier pass read as zeros

@@ -14,6 +14,10 @@ int device_setup(int* num_sms);
 bool make_tmap(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, uint64_t dim0, uint64_t dim1,
                uint64_t stride1_bytes, uint32_t box0, uint32_t box1, CUtensorMapSwizzle swz);
 
+// How many vocabulary ranges a forward or recompute pass over `row_tiles` x `col_tiles` tiles splits each row tile into,
+// at most `most`; `d` is the hidden size.
+int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most);
+
 // Bound of the kernels' device-side waits in clock ticks as set by ais_set_wait_cycles (0 = the kernels' default).
 int64_t wait_cycles();
 

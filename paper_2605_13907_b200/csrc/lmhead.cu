@@ -55,7 +55,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     constexpr int kScaleWarp0 = 12;                                             // MX: first of the four scale warps
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int num_units = TWO_ACC ? a.n_row_tiles * a.n_col_tiles : a.n_row_tiles * a.nsplit;
+    const int num_units = count_units<BASE>(a);
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); mbar_init(&sfull[i], 4); }
@@ -95,7 +95,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                 }
                 int fills = 0;                                  // stage fills of this unit so far
                 for (int t = w.t0; t < w.t1 && ok; ++t) {
-                    for (int ks = 0; ks < a.ksteps; ++ks, ++fills) {
+                    for (int ks = w.k0; ks < w.k1; ++ks, ++fills) {
                         if (pacer.ring && fills % kPaceFills == 0) pacer.announce(n, fills / kPaceFills);
                         if (pacer.ring && fills % kPaceFills == kPaceSettle) pacer.settle();
                         if (!mbar_wait(&empty[st.idx], st.phase ^ 1u, abort_flag, a.wait_cycles)) { ok = false; break; }
@@ -163,7 +163,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                 for (int t = w.t0; t < w.t1 && ok; ++t) {
                     if (!mbar_wait(&tempty[tb.idx], tb.phase ^ 1u, abort_flag, a.wait_cycles)) { ok = false; break; }
                     tc_fence_after();
-                    for (int ks = 0; ks < a.ksteps; ++ks) {
+                    for (int ks = w.k0; ks < w.k1; ++ks) {
                         if (!mbar_wait(&full[st.idx], st.phase, abort_flag, a.wait_cycles)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t sA = smem_u32(stage_base + st.idx * STG_BYTES);
@@ -174,7 +174,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                             for (int j = 0; j < 4; ++j) {
                                 const uint64_t bdesc = B_MN ? smem_desc_sw128(sB + j * 2048, kBStageBytes / 4, 1024)
                                                             : smem_desc_sw128(sB + j * 32, 16, 1024);
-                                const uint32_t accum = (ks > 0 || j > 0) ? 1u : 0u;
+                                const uint32_t accum = (ks > w.k0 || j > 0) ? 1u : 0u;
                                 mma_f16(tmem_base, smem_desc_sw128(sA + j * 32, 16, 1024), bdesc, idesc, accum);
                                 mma_f16(tmem_base + kBN, smem_desc_sw128(sA + kAStageBytes + j * 32, 16, 1024), bdesc, idesc, accum);
                             }
@@ -184,7 +184,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
                                 const uint64_t bdesc = smem_desc_sw128(sB + j * 2048, kBStageBytes / 4, 1024);
-                                const uint32_t accum = (ks > 0 || j > 0) ? 1u : 0u;
+                                const uint32_t accum = (ks > w.k0 || j > 0) ? 1u : 0u;
                                 mma_f16(tmem_base, smem_desc_sw128(sA + j * 2048, kAStageBytes / 2, 1024), bdesc, idesc, accum);
                                 mma_f16(tmem_base + kBN, smem_desc_sw128(sA + kAStageBytes + j * 2048, kAStageBytes / 2, 1024), bdesc,
                                         idesc, accum);
@@ -201,7 +201,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                             for (int j = 0; j < 4; ++j) {
                                 const uint64_t adesc = smem_desc_sw128(sA + j * 32, 16, 1024);
                                 const uint64_t bdesc = smem_desc_sw128(sB + j * 32, 16, 1024);
-                                const uint32_t accum = (ks > 0 || j > 0) ? 1u : 0u;
+                                const uint32_t accum = (ks > w.k0 || j > 0) ? 1u : 0u;
                                 if (FP4) {
                                     // instruction j covers scale blocks 2j, 2j+1: chunk j / 2, bytes 2 (j % 2) and the next
                                     const uint32_t id = 2u * (j & 1), sel = id << 30;
@@ -219,8 +219,8 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                                 const uint64_t adesc = smem_desc_sw128(sA + j * 32, 16, 1024);
                                 const uint64_t bdesc = B_MN ? smem_desc_sw128(sB + j * 2048, kBStageBytes / 4, 1024)
                                                             : smem_desc_sw128(sB + j * 32, 16, 1024);
-                                if (MODE == kFwdFp8T) mma_f8(dcol, adesc, bdesc, idesc, (ks > 0 || j > 0) ? 1u : 0u);
-                                else mma_f16(dcol, adesc, bdesc, idesc, (ks > 0 || j > 0) ? 1u : 0u);
+                                if (MODE == kFwdFp8T) mma_f8(dcol, adesc, bdesc, idesc, (ks > w.k0 || j > 0) ? 1u : 0u);
+                                else mma_f16(dcol, adesc, bdesc, idesc, (ks > w.k0 || j > 0) ? 1u : 0u);
                             }
                         }
                         tc_commit(&empty[st.idx]);
@@ -254,7 +254,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             const Unit w = decode_unit<BASE>(a, u);
             if (!unit_active<BASE>(a, w)) continue;
             for (int t = w.t0; t < w.t1 && ok; ++t) {
-                for (int ks = 0; ks < a.ksteps; ++ks) {
+                for (int ks = w.k0; ks < w.k1; ++ks) {
                     if (!mbar_wait_warp(&full[st.idx], st.phase, abort_flag, a.wait_cycles)) { ok = false; break; }
                     const uint4* src = reinterpret_cast<const uint4*>(mx_scale_base + st.idx * kMxStageScaleBytes) + lane;
                     const uint32_t tsf = tmem_base + lane_addr + kMxScaleCol + st.idx * kMxSetCols;
@@ -282,7 +282,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             const Unit w = decode_unit<BASE>(a, u);
             if (!unit_active<BASE>(a, w)) {
                 // nothing was loaded or multiplied for this unit: write the neutral output where later passes read it
-                if (BASE == kBwdDh) {
+                if (BASE == kBwdDh && w.slot < 0) {
 #pragma unroll
                     for (int sub = 0; sub < 2; ++sub) {
                         const int64_t lr = static_cast<int64_t>(w.rt) * kDhRows + sub * kBM + r_in_tile;
@@ -322,7 +322,16 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                         uint32_t v[32];
                         tmem_ld32(taddr2 + c * 32, v);
                         tmem_ld_wait(v);
-                        if (in && col0 < a.ncols) {
+                        if (w.slot >= 0) {
+                            // one of several ranges of the contraction: the fp32 sums go to the unit's partial tile, 16 bytes
+                            // per lane on consecutive addresses
+                            float4* dst = reinterpret_cast<float4*>(a.part_acc + static_cast<int64_t>(w.slot) * kPartTileFloats) +
+                                          (sub * (kBN / 4) + half * 32 + c * 8) * kBM + r_in_tile;
+#pragma unroll
+                            for (int j = 0; j < 8; ++j)
+                                dst[j * kBM] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                                                           __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+                        } else if (in && col0 < a.ncols) {
                             uint32_t pk[16];
 #pragma unroll
                             for (int i = 0; i < 32; i += 2) {
@@ -507,7 +516,49 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     }
 }
 
+// dH rows of the units whose contraction was split: the partial tiles are added in the order of their ranges and rounded
+// to bf16 once.  A thread owns one row and 16 columns (32 bytes of dH); the partial tiles are read 16 bytes per lane on
+// consecutive addresses.  The pass is a plain sweep of ksplit x 256 KB per tile, mostly still in L2 (64 tiles x 9 ranges:
+// 151 MB).  Tiles without work have no partial sums and become zeros.
+__global__ void __launch_bounds__(256) dh_reduce_kernel(const LmheadArgs a) {
+    const int tail = a.n_row_tiles * a.n_col_tiles - a.split_from;
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    const int row = i & (kBM - 1), cg = (i >> 7) & 15, sub = (i >> 11) & 1, tile = i >> 12;
+    Unit w;
+    w.rt = (a.split_from + tile) / a.n_col_tiles;
+    const int col0 = ((a.split_from + tile) % a.n_col_tiles) * kBN + cg * 16;
+    const int64_t lr = static_cast<int64_t>(w.rt) * kDhRows + sub * kBM + row;
+    if (lr >= a.rows || col0 >= a.ncols) return;
+    float4 acc[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (unit_active<kBwdDh>(a, w)) {
+        const float4* src = reinterpret_cast<const float4*>(a.part_acc + static_cast<int64_t>(tile) * kPartTileFloats) +
+                            (sub * (kBN / 4) + cg * 4) * kBM + row;
+        const int64_t step = static_cast<int64_t>(tail) * (kPartTileFloats / 4);
+#pragma unroll 2
+        for (int k = 0; k < a.ksplit; ++k) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float4 v = __ldcs(src + k * step + j * kBM);
+                acc[j].x += v.x; acc[j].y += v.y; acc[j].z += v.z; acc[j].w += v.w;
+            }
+        }
+    }
+    uint4* dst = reinterpret_cast<uint4*>(a.dH + (a.row0 + lr) * a.lddh + col0);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+        dst[j] = make_uint4(pack_bf16(acc[2 * j].x, acc[2 * j].y), pack_bf16(acc[2 * j].z, acc[2 * j].w),
+                            pack_bf16(acc[2 * j + 1].x, acc[2 * j + 1].y), pack_bf16(acc[2 * j + 1].z, acc[2 * j + 1].w));
+}
+
 }  // namespace
+
+cudaError_t launch_dh_reduce(const LmheadArgs& args, cudaStream_t stream) {
+    const int tail = args.n_row_tiles * args.n_col_tiles - args.split_from;
+    dh_reduce_kernel<<<tail * 16, 256, 0, stream>>>(args);
+    return cudaGetLastError();
+}
 
 template <int MODE>
 static cudaError_t launch_mode(const CUtensorMap& tmA, const CUtensorMap& tmB, const LmheadArgs& args, int num_ctas,

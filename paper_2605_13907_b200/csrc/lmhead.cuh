@@ -33,6 +33,8 @@ __host__ __device__ constexpr bool b_mn_major(int mode) {
     return mode == kBwdDh || mode == kBwdDw || mode == kFwdBf16Dv || mode == kBwdPDv;
 }
 
+constexpr int kSms = 148;                // SMs of the part; the work splits below are planned for it
+constexpr int kMaxRanges = kSms;         // most vocabulary ranges of a row tile
 constexpr int kBM = 128;                 // rows per tile (TMEM lanes)
 constexpr int kBN = 256;                 // columns per tile (TMEM columns of one accumulator)
 constexpr int kStageKBytes = 128;        // bytes of K per shared-memory stage row (one swizzle span)
@@ -54,6 +56,10 @@ constexpr int kThreads = 384;            // warp 0 TMA, warp 1 MMA, warps 2..3 i
 constexpr int kEpiWarps = 8;
 constexpr int kMxThreads = 512;          // microscaling passes: warps 12..15 move the block scales into tensor memory
 constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kStages * kMxStageScaleBytes + kNumBarriers * 8 + 64;
+
+// dH: one partial tile of a split unit, 256 x 256 fp32, ordered for 16-byte accesses with the rows across the lanes:
+// [row half][group of 4 columns][128 rows][4 columns]
+constexpr int kPartTileFloats = kDhRows * kBN;
 
 // Pacing of the CTAs of a launch (lmhead_common.cuh): stage fills per announcement, counters in the ring.
 constexpr int kPaceFills = 16;
@@ -92,6 +98,9 @@ struct LmheadArgs {
     int64_t lddh;
     uint32_t* status;
     int64_t wait_cycles;   // bound of every device-side wait in clock ticks; 0 = the default (about two seconds)
+    int32_t split_from;    // dH: units from here on are split along the contraction (the last, partial wave); others whole
+    int32_t ksplit;        // dH: ranges of the contraction per split unit (1 = nothing is split)
+    float* part_acc;       // dH: fp32 partial tiles of the split units, [slot][kPartTileFloats] (see dh_reduce_kernel)
     uint32_t* pace;        // ring of kPaceRing zeroed counters that keeps the CTAs of the launch in step; NULL = no pacing
     int32_t pace_per_unit; // announcements per unit = ceil(largest number of stage fills of a unit / fills per announcement)
 };
@@ -99,6 +108,8 @@ struct LmheadArgs {
 // Launches one pass.  tmSA / tmSB are only read in kFwdFp8 mode.
 cudaError_t launch_lmhead(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,
                           const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream);
+// Sums the partial tiles of a dH launch's split units (args as that launch got them) and writes their part of dH.
+cudaError_t launch_dh_reduce(const LmheadArgs& args, cudaStream_t stream);
 cudaError_t lmhead_prepare();   // sets the dynamic shared-memory attribute of every instantiation
 
 // The rollout pass with per-block scales (mode kFwdFp8; args.sgroups = 128 / block = 1, 2 or 4).  tmSA / tmSB map the

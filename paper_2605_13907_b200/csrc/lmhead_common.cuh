@@ -104,14 +104,33 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// Which row tile and which column tiles a work unit covers.
+// Which row tile and which column tiles a work unit covers, which K steps, and (split dH units) the partial tile it fills.
 struct Unit {
     int rt, t0, t1, part;
+    int k0, k1;            // K steps (stage fills per column tile)
+    int slot;              // partial tile of a split unit; -1: the unit's result is final
 };
+template <int MODE>
+__device__ __forceinline__ int count_units(const LmheadArgs& a) {
+    if (MODE == kBwdDh) return a.split_from + (a.n_row_tiles * a.n_col_tiles - a.split_from) * a.ksplit;
+    return MODE == kBwdDw ? a.n_row_tiles * a.n_col_tiles : a.n_row_tiles * a.nsplit;
+}
 template <int MODE>
 __device__ __forceinline__ Unit decode_unit(const LmheadArgs& a, int u) {
     Unit w;
+    w.k0 = 0;
+    w.k1 = a.ksteps;
+    w.slot = -1;
     if (MODE == kBwdDh || MODE == kBwdDw) {
+        if (MODE == kBwdDh && u >= a.split_from && a.ksplit > 1) {
+            // consecutive units share a range of the contraction, so the CTAs that run together share their operand slices
+            const int tail = a.n_row_tiles * a.n_col_tiles - a.split_from;
+            w.slot = u - a.split_from;
+            const int kr = w.slot / tail;
+            w.k0 = static_cast<int>((static_cast<int64_t>(kr) * a.ksteps) / a.ksplit);
+            w.k1 = static_cast<int>((static_cast<int64_t>(kr + 1) * a.ksteps) / a.ksplit);
+            u = a.split_from + w.slot % tail;
+        }
         w.rt = u / a.n_col_tiles;
         w.t0 = u % a.n_col_tiles;
         w.t1 = w.t0 + 1;

@@ -16,12 +16,10 @@ namespace {
 
 using namespace ais;
 
-constexpr int kStaticNsplit = 4;                                   // vocabulary ranges per row tile
-constexpr int kStaticParts = 2 * kStaticNsplit;                    // two column halves per range
-constexpr int64_t kStaticLd = AIS_STATIC_MAX_ROWS;                 // rows per partial plane
-constexpr size_t kStaticFloats = static_cast<size_t>(3) * kStaticParts * kStaticLd;
+constexpr size_t kStaticPlane = static_cast<size_t>(8) * AIS_STATIC_MAX_ROWS;   // floats per plane: 4 ranges x 2 column halves
+constexpr size_t kStaticFloats = 3 * kStaticPlane;                               // of the largest batch, more ranges of smaller ones
 
-// 3 planes (running max, sum of exponentials, target logit) x 8 parts x 16384 rows of float = 1.5 MiB.
+// 3 planes (running max, sum of exponentials, target logit) x 131,072 floats (8 parts x 16384 rows at most) = 1.5 MiB.
 // Every GPU on which the library is loaded holds this array until the process exits.
 static __device__ __align__(256) float g_static_partials[kStaticFloats];
 
@@ -65,7 +63,9 @@ extern "C" int ais_logprob_train_static(const ais_shape* shape, const void* H, c
     if (shape->T == 0) return AIS_OK;
 
     const int n_col_tiles = (shape->V + kBN - 1) / kBN;
-    const int nsplit = n_col_tiles < kStaticNsplit ? n_col_tiles : kStaticNsplit;
+    const int64_t ld = (shape->T + 63) / 64 * 64;                  // rows of one part
+    const int64_t room = static_cast<int64_t>(kStaticPlane) / (2 * ld);
+    const int nsplit = plan_ranges((shape->T + kBM - 1) / kBM, n_col_tiles, shape->d, room < kMaxRanges ? static_cast<int>(room) : kMaxRanges);
     LmheadArgs a;
     memset(&a, 0, sizeof(a));
     a.wait_cycles = wait_cycles();
@@ -80,9 +80,9 @@ extern "C" int ais_logprob_train_static(const ais_shape* shape, const void* H, c
     a.tokens = tokens;
     a.mask = mask;
     a.part_m = partials;
-    a.part_s = partials + static_cast<size_t>(kStaticParts) * kStaticLd;
-    a.part_z = partials + static_cast<size_t>(2 * kStaticParts) * kStaticLd;
-    a.part_ld = kStaticLd;
+    a.part_s = partials + kStaticPlane;
+    a.part_z = partials + 2 * kStaticPlane;
+    a.part_ld = ld;
     a.status = dev_status;
     CUtensorMap tmA, tmB;
     if (!make_tmap(&tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, H, static_cast<uint64_t>(shape->d), static_cast<uint64_t>(shape->T),
@@ -96,7 +96,7 @@ extern "C" int ais_logprob_train_static(const ais_shape* shape, const void* H, c
     // pass just before it, so nothing left over from an earlier call is ever read and nothing needs zeroing.
     if (launch_lmhead(kFwdBf16, tmA, tmB, tmA, tmB, a, units < num_sms ? units : num_sms, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
-    if (launch_combine(a.part_m, a.part_s, a.part_z, nsplit * 2, kStaticLd, mask, shape->T, lp_train, lse_train, dev_status, s) !=
+    if (launch_combine(a.part_m, a.part_s, a.part_z, nsplit * 2, ld, mask, shape->T, lp_train, lse_train, dev_status, s) !=
         cudaSuccess)
         return AIS_ERR_DEVICE;
     return AIS_OK;

@@ -383,40 +383,58 @@ __global__ void __launch_bounds__(256) tensor_quantize_kernel(const __nv_bfloat1
 // ------------------------------------------------------------------------------------------------
 // Merge of the per-split (max, sum-exp, target-logit) triples into lp and lse.
 // ------------------------------------------------------------------------------------------------
-__global__ void combine_kernel(const float* __restrict__ part_m, const float* __restrict__ part_s,
-                               const float* __restrict__ part_z, int nparts, int64_t part_ld,
-                               const uint8_t* __restrict__ mask, int64_t T, float* __restrict__ lp,
-                               float* __restrict__ lse, uint32_t* status) {
-    uint32_t flags = 0;
-    for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < T;
-         t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        float out_lp = 0.f, out_lse = 0.f;
-        if (mask[t]) {
-            float M = -INFINITY, zy = -INFINITY;
-            for (int j = 0; j < nparts; ++j) {
-                M = fmaxf(M, part_m[j * part_ld + t]);
-                zy = fmaxf(zy, part_z[j * part_ld + t]);
-            }
-            float S = 0.f;
-            for (int j = 0; j < nparts; ++j) S += part_s[j * part_ld + t] * expf(part_m[j * part_ld + t] - M);
-            out_lse = M + logf(S);
-            if (zy == -INFINITY) {
-                out_lp = 0.f;                       // token id out of range: flagged by the producer kernel
-            } else {
-                out_lp = zy - out_lse;
-            }
-            if (!isfinite(out_lse) || !isfinite(out_lp)) {
-                // a non-finite hidden state or weight reached this row: flag it, give it the neutral log-prob, and mark
-                // its log-sum-exp so that the backward pass leaves the row out (gradient factor 0)
-                flags |= AIS_FLAG_NONFINITE;
-                out_lp = 0.f;
-                out_lse = __int_as_float(0x7fc00000);
-            }
+// A block merges 32 rows: lane = row (coalesced), the parts are dealt out to the eight warps and each warp's running
+// (max, sum) goes through shared memory to warp 0, in warp order.  With one thread per row the up to 296 parts of a small
+// batch were a chain of dependent loads.
+constexpr int kCombWarps = 8;
+__global__ void __launch_bounds__(32 * kCombWarps) combine_kernel(const float* __restrict__ part_m, const float* __restrict__ part_s,
+                                                                  const float* __restrict__ part_z, int nparts, int64_t part_ld,
+                                                                  const uint8_t* __restrict__ mask, int64_t T,
+                                                                  float* __restrict__ lp, float* __restrict__ lse,
+                                                                  uint32_t* status) {
+    __shared__ float sm[kCombWarps][32], ss[kCombWarps][32], sz[kCombWarps][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t t = static_cast<int64_t>(blockIdx.x) * 32 + lane;
+    const bool live = t < T && mask[t] != 0;
+    float M = -INFINITY, S = 0.f, Z = -INFINITY;
+    if (live) {
+#pragma unroll 4
+        for (int j = warp; j < nparts; j += kCombWarps) {
+            const float m = part_m[j * part_ld + t], s = part_s[j * part_ld + t];
+            Z = fmaxf(Z, part_z[j * part_ld + t]);
+            const float n = fmaxf(M, m);
+            S = S * expf(M - n) + s * expf(m - n);
+            M = n;
         }
-        lp[t] = out_lp;
-        if (lse) lse[t] = out_lse;
     }
-    if (flags && status) atomicOr(status, flags);
+    sm[warp][lane] = M;
+    ss[warp][lane] = S;
+    sz[warp][lane] = Z;
+    __syncthreads();
+    if (warp != 0 || t >= T) return;
+    float out_lp = 0.f, out_lse = 0.f;
+    if (live) {
+#pragma unroll
+        for (int w = 1; w < kCombWarps; ++w) {
+            M = fmaxf(M, sm[w][lane]);
+            Z = fmaxf(Z, sz[w][lane]);
+        }
+        S = 0.f;
+#pragma unroll
+        for (int w = 0; w < kCombWarps; ++w)
+            if (w < nparts) S += ss[w][lane] * expf(sm[w][lane] - M);
+        out_lse = M + logf(S);
+        out_lp = Z == -INFINITY ? 0.f : Z - out_lse;    // no target logit: token id out of range, flagged by the producer kernel
+        if (!isfinite(out_lse) || !isfinite(out_lp)) {
+            // a non-finite hidden state or weight reached this row: flag it, give it the neutral log-prob, and mark its
+            // log-sum-exp so that the backward pass leaves the row out (gradient factor 0)
+            if (status) atomicOr(status, AIS_FLAG_NONFINITE);
+            out_lp = 0.f;
+            out_lse = __int_as_float(0x7fc00000);
+        }
+    }
+    lp[t] = out_lp;
+    if (lse) lse[t] = out_lse;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1382,8 +1400,7 @@ cudaError_t launch_quantize_tensor(const void* x, int64_t rows, int64_t cols, in
 cudaError_t launch_combine(const float* part_m, const float* part_s, const float* part_z, int nparts, int64_t part_ld,
                            const uint8_t* mask, int64_t T, float* lp, float* lse, uint32_t* status, cudaStream_t stream) {
     if (T == 0) return cudaSuccess;
-    const int blocks = static_cast<int>(((T + 255) / 256) < 1184 ? ((T + 255) / 256) : 1184);
-    combine_kernel<<<blocks, 256, 0, stream>>>(part_m, part_s, part_z, nparts, part_ld, mask, T, lp, lse, status);
+    combine_kernel<<<static_cast<unsigned>((T + 31) / 32), 32 * kCombWarps, 0, stream>>>(part_m, part_s, part_z, nparts, part_ld, mask, T, lp, lse, status);
     return cudaGetLastError();
 }
 
