@@ -146,8 +146,7 @@ int check_params(const ais_params* p) {
 }
 
 // vocab_chunk asks for its own ranges (at most 64); otherwise the pass gets what plan_ranges finds best.
-int pick_nsplit(const ais_shape* s, const ais_params* p, int64_t row_tiles) {
-    const int n_col_tiles = (s->V + kBN - 1) / kBN;
+int pick_nsplit(const ais_shape* s, const ais_params* p, int64_t row_tiles, int n_col_tiles) {
     if (p->vocab_chunk <= 0) return plan_ranges(row_tiles, n_col_tiles, s->d, kMaxRanges);
     int nsplit = (s->V + p->vocab_chunk - 1) / p->vocab_chunk;
     if (nsplit > 64) nsplit = 64;
@@ -178,7 +177,8 @@ int pick_ksplit(int tiles, int ksteps, int slots) {
 
 struct Layout {
     int64_t t_ld;          // padded length of per-row vectors
-    int nsplit, nparts;
+    int nsplit, nsplit_pair;   // vocabulary ranges: one-row-tile passes, two-row-tile FP8 pass
+    int nparts;
     size_t off_part_m, off_part_s, off_part_z;   // forward partials
     size_t off_diag;                              // reduction partials (doubles)
     size_t off_flags;                             // one byte per 128-row tile: anything to compute there?
@@ -196,8 +196,9 @@ struct Layout {
 Layout make_layout(const ais_shape* s, const ais_params* p) {
     Layout L;
     L.t_ld = static_cast<int64_t>(align_up(static_cast<size_t>(s->T > 0 ? s->T : 1), 64));
-    L.nsplit = pick_nsplit(s, p, (s->T + kBM - 1) / kBM);
-    L.nparts = L.nsplit * 2;
+    L.nsplit = pick_nsplit(s, p, (s->T + kBM - 1) / kBM, (s->V + kBN - 1) / kBN);
+    L.nsplit_pair = pick_nsplit(s, p, (s->T + kPairRows - 1) / kPairRows, (s->V + kPairCols - 1) / kPairCols);
+    L.nparts = 2 * L.nsplit > kPairParts * L.nsplit_pair ? 2 * L.nsplit : kPairParts * L.nsplit_pair;
     size_t off = 0;
     const size_t part_bytes = align_up(static_cast<size_t>(L.nparts) * L.t_ld * sizeof(float), 256);
     L.off_part_m = off; off += part_bytes;
@@ -446,7 +447,7 @@ int ais_logprob_fwd(const ais_shape* shape, const ais_params* params, const void
         a.ksteps = shape->d / 64;
         if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
         if (launch_lmhead(dv ? kFwdBf16Dv : kFwdBf16, tmA, tmB, tmA, tmB, a, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_combine(a.part_m, a.part_s, a.part_z, L.nparts, L.t_ld, mask, shape->T, lp_train, lse_train, dev_status, s) !=
+        if (launch_combine(a.part_m, a.part_s, a.part_z, 2 * L.nsplit, L.t_ld, mask, shape->T, lp_train, lse_train, dev_status, s) !=
             cudaSuccess)
             return AIS_ERR_DEVICE;
     }
@@ -465,7 +466,7 @@ int ais_logprob_fwd(const ais_shape* shape, const ais_params* params, const void
         a.nk4 = shape->d / 128;
         if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
         if (launch_lmhead(fp4 ? kFwdMx4 : kFwdMx, tmA, tmB, tmA, tmB, a, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_combine(a.part_m, a.part_s, a.part_z, L.nparts, L.t_ld, mask, shape->T, lp_roll, lse_roll, dev_status, s) !=
+        if (launch_combine(a.part_m, a.part_s, a.part_z, 2 * L.nsplit, L.t_ld, mask, shape->T, lp_roll, lse_roll, dev_status, s) !=
             cudaSuccess)
             return AIS_ERR_DEVICE;
     } else if (do_roll && per_tensor) {
@@ -478,20 +479,25 @@ int ais_logprob_fwd(const ais_shape* shape, const ais_params* params, const void
         a.scale_b = sW;
         if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
         if (launch_lmhead(kFwdFp8T, tmA, tmB, tmA, tmB, a, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_combine(a.part_m, a.part_s, a.part_z, L.nparts, L.t_ld, mask, shape->T, lp_roll, lse_roll, dev_status, s) !=
+        if (launch_combine(a.part_m, a.part_s, a.part_z, 2 * L.nsplit, L.t_ld, mask, shape->T, lp_roll, lse_roll, dev_status, s) !=
             cudaSuccess)
             return AIS_ERR_DEVICE;
     } else if (do_roll) {
+        // tiles of 256 rows x 128 columns
         const uint64_t nkb = d / shape->fp8_block;
-        if (!make_tmap(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, d, T, shape->ldh, 128, kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !make_tmap(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, qW, d, V, dv ? d : shape->ldw, 128, kBN, CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !make_tmap(&tmSA, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sH, T, nkb, ldsH * 4, kBM, a.sgroups, CU_TENSOR_MAP_SWIZZLE_NONE) ||
-            !make_tmap(&tmSB, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sW, V, nkb, ldsW * 4, kBN, a.sgroups, CU_TENSOR_MAP_SWIZZLE_NONE))
+        if (!make_tmap(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, d, T, shape->ldh, 128, kPairRows, CU_TENSOR_MAP_SWIZZLE_128B) ||
+            !make_tmap(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, qW, d, V, dv ? d : shape->ldw, 128, kPairCols, CU_TENSOR_MAP_SWIZZLE_128B) ||
+            !make_tmap(&tmSA, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sH, T, nkb, ldsH * 4, kPairRows, a.sgroups, CU_TENSOR_MAP_SWIZZLE_NONE) ||
+            !make_tmap(&tmSB, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sW, V, nkb, ldsW * 4, kPairCols, a.sgroups, CU_TENSOR_MAP_SWIZZLE_NONE))
             return AIS_ERR_DEVICE;
         a.ksteps = shape->d / 128;
-        if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_lmhead(kFwdFp8, tmA, tmB, tmSA, tmSB, a, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_combine(a.part_m, a.part_s, a.part_z, L.nparts, L.t_ld, mask, shape->T, lp_roll, lse_roll, dev_status, s) !=
+        a.n_row_tiles = static_cast<int32_t>((shape->T + kPairRows - 1) / kPairRows);
+        a.n_col_tiles = (shape->V + kPairCols - 1) / kPairCols;
+        a.nsplit = L.nsplit_pair;
+        const int pair_units = a.n_row_tiles * a.nsplit, pair_ctas = pair_units < num_sms ? pair_units : num_sms;
+        if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, pair_ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
+        if (launch_lmhead(kFwdFp8, tmA, tmB, tmSA, tmSB, a, pair_ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
+        if (launch_combine(a.part_m, a.part_s, a.part_z, kPairParts * a.nsplit, L.t_ld, mask, shape->T, lp_roll, lse_roll, dev_status, s) !=
             cudaSuccess)
             return AIS_ERR_DEVICE;
     }
@@ -650,7 +656,7 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
         // recompute softmax - onehot into the scratch
         a.ncols = shape->V;
         a.n_col_tiles = (shape->V + kBN - 1) / kBN;
-        a.nsplit = pick_nsplit(shape, params, a.n_row_tiles);
+        a.nsplit = pick_nsplit(shape, params, a.n_row_tiles, a.n_col_tiles);
         a.ksteps = shape->d / 64;
         int units = a.n_row_tiles * a.nsplit;
         if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, units < num_sms ? units : num_sms, s) != cudaSuccess)

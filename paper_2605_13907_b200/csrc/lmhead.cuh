@@ -46,6 +46,11 @@ constexpr int kStages = 4;
 constexpr int kDhRows = 2 * kBM;
 constexpr int kDhStageBytes = 2 * kAStageBytes + kBStageBytes;
 constexpr int kDhStages = 3;
+// rollout pass with fp32 block scales: a tile is two row tiles (256 rows) x 128 columns, so that a column scale read from
+// shared memory serves two rows of a thread
+constexpr int kPairRows = 2 * kBM;
+constexpr int kPairCols = 128;
+constexpr int kPairParts = 2;            // partial triples per row and vocabulary range: one per column group of the promotion warps
 static_assert(kDhStages * kDhStageBytes <= kStages * kStageBytes, "the dH stage ring must fit the same shared memory");
 constexpr int kNumBarriers = 3 * kStages + 4 + 1;
 // microscaling passes: per 128-byte K stage one 512-byte scale chunk for the 128 rows of A and two for the 256 rows of B

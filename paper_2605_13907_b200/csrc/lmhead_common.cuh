@@ -152,12 +152,18 @@ template <int MODE>
 __device__ __forceinline__ bool unit_active(const LmheadArgs& a, const Unit& w) {
     if (MODE == kBwdDw || a.tile_active == nullptr) return true;
     const int64_t g = a.row0 / kBM;
-    if (MODE == kBwdDh) {
+    if (MODE == kBwdDh || MODE == kFwdFp8) {                  // units of two row tiles
         const int64_t t0 = g + 2 * static_cast<int64_t>(w.rt);
         const bool second = (2 * static_cast<int64_t>(w.rt) + 1) * kBM < a.rows;
         return a.tile_active[t0] != 0 || (second && a.tile_active[t0 + 1] != 0);
     }
     return a.tile_active[g + w.rt] != 0;
+}
+
+// Units of two row tiles: does the second one hold rows to compute?
+__device__ __forceinline__ bool second_tile_active(const LmheadArgs& a, const Unit& w) {
+    const int64_t second = 2 * static_cast<int64_t>(w.rt) + 1;
+    return second * kBM < a.rows && (a.tile_active == nullptr || a.tile_active[a.row0 / kBM + second] != 0);
 }
 
 // After every role has left its loops: if the CTA gave up on a wait, the tile copies that the producer issued last

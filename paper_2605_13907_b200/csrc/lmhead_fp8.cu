@@ -3,25 +3,26 @@
 // The scales are arbitrary fp32 numbers, so the hardware's block-scaled MMA kinds (power-of-two scales) do not
 // apply: every scale block's partial sum is accumulated alone in tensor memory, read back and promoted on the
 // CUDA cores as acc += (partial * sH[row]) * sW[col], two columns per instruction (packed fp32).  One persistent CTA per SM:
-//   warp 0      TMA producer: one stage = 128 K-bytes of A (128 rows) and B (256 rows) plus the stage's scale
+//   warp 0      TMA producer: one stage = 128 K-bytes of A (256 rows) and B (128 rows) plus the stage's scale
 //               vectors, all completing on the stage's barrier
-//   warps 1, 2  MMA issuers: SG blocks per stage, PER = 4 / SG instructions per block, one commit per block; two
+//   warps 1, 2  MMA issuers: SG blocks per stage, PER = 4 / SG instructions per block and row tile, one commit per block; two
 //               256-column tensor-memory buffers alternate between blocks, issuer i owning buffer i
-//   warps 4-11  promotion + streaming log-sum-exp: warp w reads lane quarter w % 4, column half (w - 4) / 4 with
-//               32x32b loads (a thread owns one row x 128 columns: its row scale is one register, the column
-//               scales come as broadcast 16-byte shared-memory loads).  The four 32-register pieces of a partial
-//               tile are software-pipelined: the load of piece p + 1 is in flight during the arithmetic of piece
-//               p, and the buffer goes back to its MMA issuer as soon as the last piece has landed.
+//   warps 4-11  promotion + streaming log-sum-exp.  A tile is two row tiles x 128 columns (partial sums of the second
+//               row tile 128 tensor-memory columns further on): warp w reads lane quarter w % 4, column half (w - 4) / 4
+//               of both, so a thread owns two rows x 64 columns (128 fp32 sums).  The row scales are two registers; the
+//               column scales come as broadcast 16-byte shared-memory loads, each used for both rows.  Pieces of
+//               2 x 16 columns are software-pipelined: the load of piece p + 1 is in flight during the arithmetic of
+//               piece p, and the buffer goes back to its MMA issuer as soon as the last piece has landed.
 // The epilogue never waits for the scales separately: an MMA issuer saw the stage barrier complete before it
 // issued the block whose completion the epilogue waits for.  The first warpgroup hands registers to the other
 // two (384 threads x 168 registers at launch = 128 x 40 + 256 x 232).
-// Measured per 128 x 256 x 128 block on the busiest SM: about 1,280 clocks against 542 of tensor-core time.  No single
-// unit is the bound (timing-only variants: 790 clocks with an epilogue that only hands the buffers back, 660 without
-// the operand copies as well; the tensor-memory loads need about 280 clocks at the 32x32b shape and twice that at
-// the 16x256b fragment shape, the packed arithmetic about 350, the column-scale loads about 225): the block goes
-// round MMA -> commit -> wait -> load -> release -> wait -> MMA through two buffers, every hand-over costing
-// 200-300 clocks, which is why the MMA side is spread over two threads, the arithmetic is packed, and the promotion
-// warps poll their barrier without blocking (the blocking form cost 70 clocks per block).
+// What bounds it: the promotion warps.  Running free (no barriers, no MMAs; timing-only copy) they take 820 clocks per
+// 128 x 256 x 128 of work: arithmetic 570, broadcast loads +110 to +200, tensor-memory loads +110, which add up instead of
+// overlapping; with one row tile x 256 columns per tile (each column scale used once) the broadcast loads cost twice that
+// and the pass took 1,430 clocks against 1,290 now (9,216 rows, d = 4096, 65,536 columns, same box), with block 32 1,210
+// against 1,000 clocks per scale block.  Passing a barrier that completed long ago costs a warp about 250 clocks, which is
+// why the next block's barrier is tested before the last arithmetic of this one (block 32: 1,090 -> 1,000).  Sixteen and
+// twelve promotion warps (32 columns each) and scale loads hoisted above the waits measured slower or the same.
 #include <type_traits>
 
 #include "lmhead_common.cuh"
@@ -31,11 +32,14 @@ namespace ais {
 
 namespace {
 
+constexpr int kHalfCols = kPairCols / 2;                              // columns of a promotion warp
+constexpr int kPairABytes = kPairRows * kStageKBytes;               // A part of a stage (two row tiles), then B
+
 template <int SG>
 struct Fp8Cfg {
     static constexpr int kSlots = (SG == 4) ? 5 : 8;                  // scale slots: more than stages + buffers in flight
-    static constexpr int kSlotBytes = SG * (kBM + kBN) * 4;
-    static constexpr int kSlotBOffset = SG * kBM * 4;
+    static constexpr int kSlotBytes = SG * (kPairRows + kPairCols) * 4;
+    static constexpr int kSlotBOffset = SG * kPairRows * 4;
     static constexpr int kBarriers = 2 * kStages + 4 + kSlots + 1;
     static constexpr int kSmem = 1024 + kStages * kStageBytes + kSlots * kSlotBytes + kBarriers * 8 + 64;
 };
@@ -117,10 +121,10 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                             uint8_t* sA = stage_base + st.idx * kStageBytes;
                             uint8_t* sS = scale_base + sc.idx * C::kSlotBytes;
                             mbar_expect_tx(&full[st.idx], kStageBytes + C::kSlotBytes);
-                            tma_load_2d(sS, &tmSA, &full[st.idx], w.rt * kBM, ks * SG);
-                            tma_load_2d(sS + C::kSlotBOffset, &tmSB, &full[st.idx], t * kBN, ks * SG);
-                            tma_load_2d(sA, &tmA, &full[st.idx], ks * 128, w.rt * kBM);
-                            tma_load_2d(sA + kAStageBytes, &tmB, &full[st.idx], ks * 128, t * kBN);
+                            tma_load_2d(sS, &tmSA, &full[st.idx], w.rt * kPairRows, ks * SG);
+                            tma_load_2d(sS + C::kSlotBOffset, &tmSB, &full[st.idx], t * kPairCols, ks * SG);
+                            tma_load_2d(sA, &tmA, &full[st.idx], ks * 128, w.rt * kPairRows);
+                            tma_load_2d(sA + kPairABytes, &tmB, &full[st.idx], ks * 128, t * kPairCols);
                             ++issued;
                             st.advance();
                             sc.advance();
@@ -140,9 +144,9 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             // 542 the tensor core needs.  The two threads are independent: different buffers, different barriers.
             if (lane == 0) {
                 const uint32_t me = warp - 1;
-                constexpr uint32_t idesc = make_idesc(kFmtE4M3, kFmtE4M3, kBM, kBN, 0, 0);
+                constexpr uint32_t idesc = make_idesc(kFmtE4M3, kFmtE4M3, kBM, kPairCols, 0, 0);
                 const uint64_t desc0 = smem_desc_sw128(0, 16, 1024);           // descriptor of address 0: add (address >> 4)
-                const uint32_t dcol = tmem_base + me * kBN;
+                const uint32_t dcol = tmem_base + me * (2 * kPairCols);
                 Pipe st(kStages);
                 uint32_t tphase = 0;                                            // phase of this issuer's buffer barriers
                 uint32_t nstage = 0;                                            // stages seen so far (SG == 1: parity picks the owner)
@@ -151,6 +155,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     const Unit w = decode_unit<MODE>(a, u);
                     if (!unit_active<MODE>(a, w)) continue;
                     const int nst = (w.t1 - w.t0) * a.ksteps;
+                    const bool two = second_tile_active(a, w);
                     for (int i = 0; i < nst && ok; ++i, ++nstage) {
                         if (SG > 1 || (nstage & 1u) == me) {
                             if (!mbar_wait(&full[st.idx], st.phase, abort_flag, a.wait_cycles)) { ok = false; break; }
@@ -163,7 +168,9 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 #pragma unroll
                                 for (int j = 0; j < PER; ++j) {
                                     const uint64_t ad = adesc + 2 * (g * PER + j);       // 32 bytes of K further on
-                                    mma_f8(dcol, ad, ad + (kAStageBytes >> 4), idesc, j > 0 ? 1u : 0u);
+                                    const uint64_t bd = ad + (kPairABytes >> 4);
+                                    mma_f8(dcol, ad, bd, idesc, j > 0 ? 1u : 0u);
+                                    if (two) mma_f8(dcol + kPairCols, ad + (kAStageBytes >> 4), bd, idesc, j > 0 ? 1u : 0u);
                                 }
                                 tc_commit(&tfull[me]);
                                 tphase ^= 1u;
@@ -188,46 +195,59 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         bool ok = true;
         uint32_t flags = 0;
         uint32_t va[32], vb[32];
+        bool ready = false;                           // the next block was seen complete before its turn
+        // piece p: 16 columns of both row tiles
         auto ld_piece = [&](uint32_t buf, int p, uint32_t (&v)[32]) {
-            tmem_ld32(tmem_base + lane_base + buf * kBN + half * 128 + p * 32, v);
+            const uint32_t at = tmem_base + lane_base + buf * (2 * kPairCols) + half * kHalfCols + p * 16;
+            tmem_ld16(at, v, 0);
+            tmem_ld16(at + kPairCols, v, 16);
         };
         for (int u = blockIdx.x; u < num_units && ok; u += gridDim.x) {
             const Unit w = decode_unit<MODE>(a, u);
             if (!unit_active<MODE>(a, w)) continue;     // every row masked: the merge kernel never reads these partials
-            const int64_t lr = static_cast<int64_t>(w.rt) * kBM + q * 32 + lane;
-            const bool rok = lr < a.rows;
-            const int64_t grow = a.row0 + lr;
-            int y = -1;
-            if (rok) {
-                y = a.tokens[grow];
-                if (a.mask[grow] != 0 && (y < 0 || y >= a.ncols)) { flags |= AIS_FLAG_TOKEN_RANGE; y = -1; }
-            }
-            float m_run = kNegBig, s_run = 0.f, zy = -INFINITY;
-            for (int t = w.t0; t < w.t1 && ok; ++t) {
-                F2 acc[64];                                // columns 2 n, 2 n + 1 of this thread's 128
+            int64_t grow[2];
+            bool rok[2];
+            int y[2];
 #pragma unroll
-                for (int n = 0; n < 64; ++n) acc[n] = F2{0.f, 0.f};
+            for (int i = 0; i < 2; ++i) {
+                const int64_t lr = static_cast<int64_t>(w.rt) * kPairRows + i * kBM + q * 32 + lane;
+                rok[i] = lr < a.rows;
+                grow[i] = a.row0 + lr;
+                y[i] = -1;
+                if (rok[i]) {
+                    y[i] = a.tokens[grow[i]];
+                    if (a.mask[grow[i]] != 0 && (y[i] < 0 || y[i] >= a.ncols)) { flags |= AIS_FLAG_TOKEN_RANGE; y[i] = -1; }
+                }
+            }
+            float m_run[2] = {kNegBig, kNegBig}, s_run[2] = {0.f, 0.f}, zy[2] = {-INFINITY, -INFINITY};
+            for (int t = w.t0; t < w.t1 && ok; ++t) {
+                F2 acc[2][kHalfCols / 2];                  // columns 2 n, 2 n + 1 of this thread's half, rows of both tiles
+#pragma unroll
+                for (int n = 0; n < kHalfCols / 2; ++n) acc[0][n] = acc[1][n] = F2{0.f, 0.f};
                 for (int ks = 0; ks < a.ksteps && ok; ++ks) {
                     const float* sS = reinterpret_cast<const float*>(scale_base + sc.idx * C::kSlotBytes);
 #pragma unroll 1
                     for (int g = 0; g < SG; ++g) {
-                        if (!mbar_wait_warp_spin(&tfull[tb.idx], tb.phase, abort_flag, a.wait_cycles)) { ok = false; break; }
+                        if (!ready && !mbar_wait_warp_spin(&tfull[tb.idx], tb.phase, abort_flag, a.wait_cycles)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t buf = tb.idx;
                         ld_piece(buf, 0, va);
-                        const float shx = sS[g * kBM + q * 32 + lane];
-                        const F2 sh = {shx, shx};
-                        // every lane reads the same column scales: broadcast 16-byte loads
-                        const float4* sw4 = reinterpret_cast<const float4*>(sS + (C::kSlotBOffset / 4) + g * kBN + half * 128);
+                        const float sh0 = sS[g * kPairRows + q * 32 + lane], sh1 = sS[g * kPairRows + kBM + q * 32 + lane];
+                        const F2 r0 = {sh0, sh0}, r1 = {sh1, sh1};
+                        // every lane reads the same column scales: broadcast 16-byte loads, each used for two rows
+                        const float4* sw4 = reinterpret_cast<const float4*>(sS + (C::kSlotBOffset / 4) + g * kPairCols + half * kHalfCols);
                         auto promote = [&](auto PP, uint32_t (&v)[32]) {
                             constexpr int pp = decltype(PP)::value;
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const float4 swf = sw4[pp * 8 + j];
-                                const F2 x0 = {__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1])};
-                                const F2 x1 = {__uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])};
-                                acc[pp * 16 + 2 * j] = fma2(mul2(x0, sh), F2{swf.x, swf.y}, acc[pp * 16 + 2 * j]);
-                                acc[pp * 16 + 2 * j + 1] = fma2(mul2(x1, sh), F2{swf.z, swf.w}, acc[pp * 16 + 2 * j + 1]);
+                            for (int j = 0; j < 4; ++j) {
+                                const float4 swf = sw4[pp * 4 + j];
+                                const F2 c0 = {swf.x, swf.y}, c1 = {swf.z, swf.w};
+                                F2* p0 = &acc[0][pp * 8 + 2 * j];
+                                F2* p1 = &acc[1][pp * 8 + 2 * j];
+                                p0[0] = fma2(mul2(F2{__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1])}, r0), c0, p0[0]);
+                                p0[1] = fma2(mul2(F2{__uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])}, r0), c1, p0[1]);
+                                p1[0] = fma2(mul2(F2{__uint_as_float(v[16 + 4 * j]), __uint_as_float(v[17 + 4 * j])}, r1), c0, p1[0]);
+                                p1[1] = fma2(mul2(F2{__uint_as_float(v[18 + 4 * j]), __uint_as_float(v[19 + 4 * j])}, r1), c1, p1[1]);
                             }
                         };
                         using I0 = std::integral_constant<int, 0>;
@@ -249,7 +269,10 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&tempty[buf]);
                         tb.advance();
+                        // ask for the next block's barrier now: the answer comes back behind the last arithmetic
+                        const bool seen = mbar_test_wait(&tfull[tb.idx], tb.phase);
                         promote(I3{}, vb);
+                        ready = __all_sync(0xffffffffu, seen);
                     }
                     if (!ok) break;
                     __syncwarp();
@@ -257,42 +280,47 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     sc.advance();
                 }
                 if (!ok) break;
-                // streaming log-sum-exp over this thread's 128 columns of its row
-                const int cbase = t * kBN + half * 128;                    // column of acc[0].x
-                const int yy = y - cbase;
-                if (yy >= 0 && yy < 128) {
-                    // written as a running maximum on purpose: a chain of "if (k == n) z = acc[n]" is folded by
-                    // the compiler into acc[k], and a dynamically indexed array leaves the register file
+                // streaming log-sum-exp over this thread's columns of its two rows
+                const int cbase = t * kPairCols + half * kHalfCols;        // column of acc[.][0].x
 #pragma unroll
-                    for (int n = 0; n < 64; ++n) {
-                        zy = fmaxf(zy, (yy == 2 * n) ? acc[n].x : -INFINITY);
-                        zy = fmaxf(zy, (yy == 2 * n + 1) ? acc[n].y : -INFINITY);
+                for (int i = 0; i < 2; ++i) {
+                    const int yy = y[i] - cbase;
+                    if (yy >= 0 && yy < kHalfCols) {
+                        // written as a running maximum on purpose: a chain of "if (k == n) z = acc[n]" is folded by
+                        // the compiler into acc[k], and a dynamically indexed array leaves the register file
+#pragma unroll
+                        for (int n = 0; n < kHalfCols / 2; ++n) {
+                            zy[i] = fmaxf(zy[i], (yy == 2 * n) ? acc[i][n].x : -INFINITY);
+                            zy[i] = fmaxf(zy[i], (yy == 2 * n + 1) ? acc[i][n].y : -INFINITY);
+                        }
                     }
-                }
-                if (t * kBN + kBN > a.ncols) {
+                    if (t * kPairCols + kPairCols > a.ncols) {
 #pragma unroll
-                    for (int n = 0; n < 64; ++n) {
-                        if (cbase + 2 * n >= a.ncols) acc[n].x = -INFINITY;
-                        if (cbase + 2 * n + 1 >= a.ncols) acc[n].y = -INFINITY;
+                        for (int n = 0; n < kHalfCols / 2; ++n) {
+                            if (cbase + 2 * n >= a.ncols) acc[i][n].x = -INFINITY;
+                            if (cbase + 2 * n + 1 >= a.ncols) acc[i][n].y = -INFINITY;
+                        }
                     }
+                    float cm = acc[i][0].x;
+#pragma unroll
+                    for (int n = 0; n < kHalfCols / 2; ++n) cm = fmaxf(cm, fmaxf(acc[i][n].x, acc[i][n].y));
+                    const float m_new = fmaxf(m_run[i], cm * kLog2e);
+                    float add = 0.f;
+#pragma unroll
+                    for (int n = 0; n < kHalfCols / 2; ++n)
+                        add += ex2(fmaf(acc[i][n].x, kLog2e, -m_new)) + ex2(fmaf(acc[i][n].y, kLog2e, -m_new));
+                    s_run[i] = fmaf(s_run[i], ex2(m_run[i] - m_new), add);
+                    m_run[i] = m_new;
                 }
-                float cm = acc[0].x;
-#pragma unroll
-                for (int n = 0; n < 64; ++n) cm = fmaxf(cm, fmaxf(acc[n].x, acc[n].y));
-                const float m_new = fmaxf(m_run, cm * kLog2e);
-                float add = 0.f;
-#pragma unroll
-                for (int n = 0; n < 64; ++n)
-                    add += ex2(fmaf(acc[n].x, kLog2e, -m_new)) + ex2(fmaf(acc[n].y, kLog2e, -m_new));
-                s_run = fmaf(s_run, ex2(m_run - m_new), add);
-                m_run = m_new;
             }
-            if (ok && rok) {
-                const int64_t o = static_cast<int64_t>(w.part * 2 + half) * a.part_ld + grow;
-                a.part_m[o] = m_run * kLn2;
-                a.part_s[o] = s_run;
-                a.part_z[o] = zy;
-            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (ok && rok[i]) {
+                    const int64_t o = static_cast<int64_t>(w.part * 2 + half) * a.part_ld + grow[i];
+                    a.part_m[o] = m_run[i] * kLn2;
+                    a.part_s[o] = s_run[i];
+                    a.part_z[o] = zy[i];
+                }
         }
         if (flags && a.status) atomicOr(a.status, flags);
     }

@@ -219,6 +219,17 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "r"(taddr)
         : "memory");
 }
+// 32 lanes x 16 consecutive columns into r[at .. at + 15].
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[32], int at) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[at]), "=r"(r[at + 1]), "=r"(r[at + 2]), "=r"(r[at + 3]), "=r"(r[at + 4]), "=r"(r[at + 5]), "=r"(r[at + 6]),
+          "=r"(r[at + 7]), "=r"(r[at + 8]), "=r"(r[at + 9]), "=r"(r[at + 10]), "=r"(r[at + 11]), "=r"(r[at + 12]),
+          "=r"(r[at + 13]), "=r"(r[at + 14]), "=r"(r[at + 15])
+        : "r"(taddr)
+        : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
