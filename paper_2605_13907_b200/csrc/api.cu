@@ -175,14 +175,17 @@ int pick_ksplit(int tiles, int ksteps, int slots) {
     return best;
 }
 
+constexpr size_t kPaceRingBytes = kPaceRing * sizeof(uint32_t);
+
 struct Layout {
     int64_t t_ld;          // padded length of per-row vectors
     int nsplit, nsplit_pair;   // vocabulary ranges: one-row-tile passes, two-row-tile FP8 pass
     int nparts;
-    size_t off_part_m, off_part_s, off_part_z;   // forward partials
+    size_t off_part[2], part_bytes;               // forward partials of the trainer and the rollout pass: max, sum, target planes
     size_t off_diag;                              // reduction partials (doubles)
     size_t off_flags;                             // one byte per 128-row tile: anything to compute there?
-    size_t off_pace;                              // ring of counters that keeps the CTAs of a tensor-core launch in step
+    size_t off_pace;                              // two rings of counters that keep the CTAs of a tensor-core launch in step
+    size_t off_ticket;                            // block counter of the batch reductions
     size_t off_coef, off_nseq;                    // backward: c_t, valid rows per sequence
     size_t off_seqw;                              // sequence-level variant: log weight per sequence
     size_t off_split;                             // dH: partial tiles of the split units
@@ -200,12 +203,11 @@ Layout make_layout(const ais_shape* s, const ais_params* p) {
     L.nsplit_pair = pick_nsplit(s, p, (s->T + kPairRows - 1) / kPairRows, (s->V + kPairCols - 1) / kPairCols);
     L.nparts = 2 * L.nsplit > kPairParts * L.nsplit_pair ? 2 * L.nsplit : kPairParts * L.nsplit_pair;
     size_t off = 0;
-    const size_t part_bytes = align_up(static_cast<size_t>(L.nparts) * L.t_ld * sizeof(float), 256);
-    L.off_part_m = off; off += part_bytes;
-    L.off_part_s = off; off += part_bytes;
-    L.off_part_z = off; off += part_bytes;
+    L.part_bytes = align_up(static_cast<size_t>(L.nparts) * L.t_ld * sizeof(float), 256);
+    for (int i = 0; i < 2; ++i) { L.off_part[i] = off; off += 3 * L.part_bytes; }
     L.off_flags = off;  off += align_up(static_cast<size_t>(L.t_ld / kBM + 2), 256);
-    L.off_pace = off;   off += align_up(static_cast<size_t>(kPaceRing) * sizeof(uint32_t), 256);
+    L.off_pace = off;   off += 2 * kPaceRingBytes;
+    L.off_ticket = off; off += 256;
     L.off_diag = off;   off += align_up(static_cast<size_t>(kDiagBlocks) * kNumMoments * sizeof(double), 256);
     L.off_coef = off;   off += align_up(static_cast<size_t>(L.t_ld) * sizeof(float), 256);
     L.off_nseq = off;   off += align_up(static_cast<size_t>(s->P) * s->G * sizeof(int32_t), 256);
@@ -232,17 +234,18 @@ Layout make_layout(const ais_shape* s, const ais_params* p) {
 
 constexpr int64_t kBwdRowsRecommended = 2 * kSms * kBM;
 
-// Zeroes the pacing ring and points the launch at it.  tiles_per_unit = the largest number of column tiles a unit of
-// the launch walks; a launch of a single wave has nobody to keep in step with over time and runs without pacing only
-// when it has a single CTA.
-cudaError_t arm_pace(LmheadArgs& a, uint8_t* ws, const Layout& L, int tiles_per_unit, int ctas, cudaStream_t s) {
-    a.pace = nullptr;
-    a.pace_per_unit = 0;
-    if (ctas < 2) return cudaSuccess;
+// Points a pass at its pacing ring.  The passes of a call alternate between two rings: the kernel before the first pass
+// clears both (ring_bytes of them), every later pass finds its own cleared by the one before it (`clears_next`).
+// tiles_per_unit = the largest number of column tiles a unit of the launch walks.  A CTA with only a few announcements to
+// make cannot drift far enough to matter and runs without pacing, so small batches have no rings to clear either.
+constexpr int64_t kPaceMinFills = 256;
+bool arm_pace(LmheadArgs& a, uint8_t* ws, const Layout& L, int tiles_per_unit, int units, int ctas, int pass, bool clears_next) {
     const int64_t fills = static_cast<int64_t>(tiles_per_unit) * a.ksteps;
-    a.pace = reinterpret_cast<uint32_t*>(ws + L.off_pace);
+    const int64_t waves = (units + ctas - 1) / ctas;
+    a.pace_clear = clears_next ? reinterpret_cast<uint32_t*>(ws + L.off_pace + ((pass + 1) & 1) * kPaceRingBytes) : nullptr;
+    a.pace = ctas < 2 || fills * waves < kPaceMinFills ? nullptr : reinterpret_cast<uint32_t*>(ws + L.off_pace + (pass & 1) * kPaceRingBytes);
     a.pace_per_unit = static_cast<int32_t>((fills + kPaceFills - 1) / kPaceFills);
-    return cudaMemsetAsync(a.pace, 0, static_cast<size_t>(kPaceRing) * sizeof(uint32_t), s);
+    return a.pace != nullptr;
 }
 
 }  // namespace
@@ -403,7 +406,7 @@ int ais_logprob_fwd(const ais_shape* shape, const ais_params* params, const void
         }
     }
     const Layout L = make_layout(shape, params);
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < L.off_diag) return AIS_ERR_WORKSPACE;
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < L.off_ticket) return AIS_ERR_WORKSPACE;
     int num_sms = 0;
     st = device_setup(&num_sms);
     if (st != AIS_OK) return st;
@@ -411,96 +414,90 @@ int ais_logprob_fwd(const ais_shape* shape, const ais_params* params, const void
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    LmheadArgs a;
-    memset(&a, 0, sizeof(a));
-    a.wait_cycles = wait_cycles();
-    a.rows = shape->T;
-    a.row0 = 0;
-    a.n_row_tiles = static_cast<int32_t>((shape->T + kBM - 1) / kBM);
-    a.ncols = shape->V;
-    a.n_col_tiles = (shape->V + kBN - 1) / kBN;
-    a.nsplit = L.nsplit;
-    a.sgroups = (per_tensor || mx) ? 1 : 128 / shape->fp8_block;
-    a.tokens = tokens;
-    a.mask = mask;
-    a.part_m = reinterpret_cast<float*>(ws + L.off_part_m);
-    a.part_s = reinterpret_cast<float*>(ws + L.off_part_s);
-    a.part_z = reinterpret_cast<float*>(ws + L.off_part_z);
-    a.part_ld = L.t_ld;
-    a.status = dev_status;
-    // row tiles without a single valid row are skipped by the tensor-core passes
-    a.tile_active = ws + L.off_flags;
-    if (launch_tile_flags_mask(mask, shape->T, ws + L.off_flags, s) != cudaSuccess) return AIS_ERR_DEVICE;
-    const int units = a.n_row_tiles * a.nsplit;
-    const int ctas = units < num_sms ? units : num_sms;
-    const uint64_t T = static_cast<uint64_t>(shape->T), V = static_cast<uint64_t>(shape->V), d = static_cast<uint64_t>(shape->d);
-
-    CUtensorMap tmA, tmB, tmSA, tmSB;
+    LmheadArgs base;
+    memset(&base, 0, sizeof(base));
+    base.wait_cycles = wait_cycles();
+    base.rows = shape->T;
+    base.tokens = tokens;
+    base.mask = mask;
+    base.ncols = shape->V;
+    base.part_ld = L.t_ld;
+    base.status = dev_status;
+    base.tile_active = ws + L.off_flags;         // row tiles without a single valid row are skipped by the tensor-core passes
+    const int64_t T = shape->T, V = shape->V, d = shape->d;
     const bool dv = shape->w_layout == AIS_W_DV;
+
+    // One pass: its arguments, its tensor maps, its share of the merge.
+    struct Pass {
+        LmheadArgs a;
+        CUtensorMap tmA, tmB, tmSA, tmSB;
+        int mode, units, ctas;
+    } pass[2];
+    CombineJob jobs[2];
+    int n = 0;
+    bool paced = false;
+    auto add = [&](int mode, int64_t rows_per_tile, int cols_per_tile, int nsplit, int ksteps, float* lp, float* lse) -> Pass& {
+        Pass& p = pass[n];
+        p.mode = mode;
+        p.a = base;
+        p.a.n_row_tiles = static_cast<int32_t>((T + rows_per_tile - 1) / rows_per_tile);
+        p.a.n_col_tiles = static_cast<int32_t>((V + cols_per_tile - 1) / cols_per_tile);
+        p.a.nsplit = nsplit;
+        p.a.ksteps = ksteps;
+        p.a.sgroups = 1;
+        float* parts = reinterpret_cast<float*>(ws + L.off_part[n]);
+        p.a.part_m = parts;
+        p.a.part_s = parts + L.part_bytes / sizeof(float);
+        p.a.part_z = parts + 2 * (L.part_bytes / sizeof(float));
+        p.units = p.a.n_row_tiles * nsplit;
+        p.ctas = p.units < num_sms ? p.units : num_sms;
+        paced |= arm_pace(p.a, ws, L, (p.a.n_col_tiles + nsplit - 1) / nsplit, p.units, p.ctas, n, false);
+        // the rollout pass needs nothing from the trainer pass: it fills the SMs that the other one leaves or never had
+        p.a.overlap = n > 0 ? 1 : 0;
+        jobs[n] = {p.a.part_m, p.a.part_s, p.a.part_z, (mode == kFwdFp8 ? kPairParts : 2) * nsplit, lp, lse};
+        ++n;
+        return p;
+    };
+    bool maps = true;
     if (do_train) {
         // W [V, d]: K-major boxes of 64 hidden units x 256 vocabulary rows.  W [d, V]: the vocabulary is the contiguous
         // axis, boxes of 64 vocabulary columns x 64 hidden units (four of them per stage)
-        if (!make_tmap(&tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, H, d, T, shape->ldh * 2, 64, kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !(dv ? make_tmap(&tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, V, d, shape->ldw * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
-                 : make_tmap(&tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, d, V, shape->ldw * 2, 64, kBN, CU_TENSOR_MAP_SWIZZLE_128B)))
-            return AIS_ERR_DEVICE;
-        a.ksteps = shape->d / 64;
-        if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_lmhead(dv ? kFwdBf16Dv : kFwdBf16, tmA, tmB, tmA, tmB, a, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_combine(a.part_m, a.part_s, a.part_z, 2 * L.nsplit, L.t_ld, mask, shape->T, lp_train, lse_train, dev_status, s) !=
-            cudaSuccess)
-            return AIS_ERR_DEVICE;
+        Pass& p = add(dv ? kFwdBf16Dv : kFwdBf16, kBM, kBN, L.nsplit, shape->d / 64, lp_train, lse_train);
+        maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, H, d, T, shape->ldh * 2, 64, kBM, CU_TENSOR_MAP_SWIZZLE_128B) &&
+                (dv ? make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, V, d, shape->ldw * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
+                    : make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, d, V, shape->ldw * 2, 64, kBN, CU_TENSOR_MAP_SWIZZLE_128B));
     }
-    if (do_roll && mx) {
-        // power-of-two scales per 32 elements: the block-scaled MMA applies them, the contraction stays in tensor memory
-        // FP4 codes are two per byte: the maps see d / 2 bytes per row with half the row stride
-        const uint64_t kb = fp4 ? d / 2 : d;
-        if (!make_tmap(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, kb, T, fp4 ? shape->ldh / 2 : shape->ldh, 128, kBM,
-                       CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !make_tmap(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, qW, kb, V, fp4 ? shape->ldw / 2 : shape->ldw, 128, kBN,
-                       CU_TENSOR_MAP_SWIZZLE_128B))
-            return AIS_ERR_DEVICE;
-        a.ksteps = static_cast<int32_t>(kb / 128);
-        a.sf_a = static_cast<const uint8_t*>(sH_);
-        a.sf_b = static_cast<const uint8_t*>(sW_);
-        a.nk4 = shape->d / 128;
-        if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_lmhead(fp4 ? kFwdMx4 : kFwdMx, tmA, tmB, tmA, tmB, a, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_combine(a.part_m, a.part_s, a.part_z, 2 * L.nsplit, L.t_ld, mask, shape->T, lp_roll, lse_roll, dev_status, s) !=
-            cudaSuccess)
-            return AIS_ERR_DEVICE;
-    } else if (do_roll && per_tensor) {
-        // one scale per tensor: the whole contraction accumulates in tensor memory, the scales meet in the epilogue
-        if (!make_tmap(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, d, T, shape->ldh, 128, kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !make_tmap(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, qW, d, V, shape->ldw, 128, kBN, CU_TENSOR_MAP_SWIZZLE_128B))
-            return AIS_ERR_DEVICE;
-        a.ksteps = shape->d / 128;
-        a.scale_a = sH;
-        a.scale_b = sW;
-        if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_lmhead(kFwdFp8T, tmA, tmB, tmA, tmB, a, ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_combine(a.part_m, a.part_s, a.part_z, 2 * L.nsplit, L.t_ld, mask, shape->T, lp_roll, lse_roll, dev_status, s) !=
-            cudaSuccess)
-            return AIS_ERR_DEVICE;
+    if (do_roll && (mx || per_tensor)) {
+        // Power-of-two scales per 32 elements: the block-scaled MMA applies them.  One scale per tensor: the two meet in the
+        // epilogue.  Either way the whole contraction stays in tensor memory.  FP4 codes are two per byte: the maps see
+        // d / 2 bytes per row with half the row stride.
+        const int64_t kb = fp4 ? d / 2 : d;
+        Pass& p = add(per_tensor ? kFwdFp8T : fp4 ? kFwdMx4 : kFwdMx, kBM, kBN, L.nsplit, static_cast<int>(kb / 128), lp_roll, lse_roll);
+        p.a.sf_a = static_cast<const uint8_t*>(sH_);
+        p.a.sf_b = static_cast<const uint8_t*>(sW_);
+        p.a.nk4 = shape->d / 128;
+        p.a.scale_a = sH;
+        p.a.scale_b = sW;
+        maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, kb, T, fp4 ? shape->ldh / 2 : shape->ldh, 128, kBM, CU_TENSOR_MAP_SWIZZLE_128B) &&
+                make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, qW, kb, V, fp4 ? shape->ldw / 2 : shape->ldw, 128, kBN, CU_TENSOR_MAP_SWIZZLE_128B);
     } else if (do_roll) {
         // tiles of 256 rows x 128 columns
-        const uint64_t nkb = d / shape->fp8_block;
-        if (!make_tmap(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, d, T, shape->ldh, 128, kPairRows, CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !make_tmap(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, qW, d, V, dv ? d : shape->ldw, 128, kPairCols, CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !make_tmap(&tmSA, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sH, T, nkb, ldsH * 4, kPairRows, a.sgroups, CU_TENSOR_MAP_SWIZZLE_NONE) ||
-            !make_tmap(&tmSB, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sW, V, nkb, ldsW * 4, kPairCols, a.sgroups, CU_TENSOR_MAP_SWIZZLE_NONE))
-            return AIS_ERR_DEVICE;
-        a.ksteps = shape->d / 128;
-        a.n_row_tiles = static_cast<int32_t>((shape->T + kPairRows - 1) / kPairRows);
-        a.n_col_tiles = (shape->V + kPairCols - 1) / kPairCols;
-        a.nsplit = L.nsplit_pair;
-        const int pair_units = a.n_row_tiles * a.nsplit, pair_ctas = pair_units < num_sms ? pair_units : num_sms;
-        if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, pair_ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_lmhead(kFwdFp8, tmA, tmB, tmSA, tmSB, a, pair_ctas, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_combine(a.part_m, a.part_s, a.part_z, kPairParts * a.nsplit, L.t_ld, mask, shape->T, lp_roll, lse_roll, dev_status, s) !=
-            cudaSuccess)
-            return AIS_ERR_DEVICE;
+        const int64_t nkb = d / shape->fp8_block;
+        const int sg = 128 / shape->fp8_block;
+        Pass& p = add(kFwdFp8, kPairRows, kPairCols, L.nsplit_pair, shape->d / 128, lp_roll, lse_roll);
+        p.a.sgroups = sg;
+        maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, d, T, shape->ldh, 128, kPairRows, CU_TENSOR_MAP_SWIZZLE_128B) &&
+                make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, qW, d, V, dv ? d : shape->ldw, 128, kPairCols, CU_TENSOR_MAP_SWIZZLE_128B) &&
+                make_tmap(&p.tmSA, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sH, T, nkb, ldsH * 4, kPairRows, sg, CU_TENSOR_MAP_SWIZZLE_NONE) &&
+                make_tmap(&p.tmSB, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sW, V, nkb, ldsW * 4, kPairCols, sg, CU_TENSOR_MAP_SWIZZLE_NONE);
     }
+    if (!maps) return AIS_ERR_DEVICE;
+    if (launch_tile_flags_mask(mask, T, ws + L.off_flags, paced ? ws + L.off_pace : nullptr, 2 * kPaceRingBytes, s) != cudaSuccess)
+        return AIS_ERR_DEVICE;
+    for (int i = 0; i < n; ++i)
+        if (launch_lmhead(pass[i].mode, pass[i].tmA, pass[i].tmB, pass[i].tmSA, pass[i].tmSB, pass[i].a, pass[i].ctas, s) != cudaSuccess)
+            return AIS_ERR_DEVICE;
+    if (launch_combine(jobs, n, L.t_ld, mask, T, dev_status, s) != cudaSuccess) return AIS_ERR_DEVICE;
     return AIS_OK;
 }
 
@@ -521,10 +518,10 @@ int ais_diagnostics(const ais_shape* shape, const ais_params* params, const floa
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int S = shape->P * shape->G;
-    if (launch_advantages(rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, s) != cudaSuccess)
+    if (launch_advantages(rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, reinterpret_cast<uint32_t*>(ws + L.off_ticket), s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     if (launch_diag(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag),
-                    n_valid_seq, seq_level ? reinterpret_cast<float*>(ws + L.off_seqw) : nullptr, rho, w_tilde, diag, s) !=
+                    reinterpret_cast<uint32_t*>(ws + L.off_ticket), n_valid_seq, seq_level ? reinterpret_cast<float*>(ws + L.off_seqw) : nullptr, rho, w_tilde, diag, s) !=
         cudaSuccess)
         return AIS_ERR_DEVICE;
     return AIS_OK;
@@ -547,10 +544,10 @@ int ais_diag_moments(const ais_shape* shape, const ais_params* params, const flo
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int S = shape->P * shape->G;
-    if (launch_advantages(rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, s) != cudaSuccess)
+    if (launch_advantages(rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, reinterpret_cast<uint32_t*>(ws + L.off_ticket), s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     if (launch_moments(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag),
-                       n_valid_seq, params->seq_level_weights != 0 ? seq_logw : nullptr, moments, s) != cudaSuccess)
+                       reinterpret_cast<uint32_t*>(ws + L.off_ticket), n_valid_seq, params->seq_level_weights != 0 ? seq_logw : nullptr, moments, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     return AIS_OK;
 }
@@ -599,14 +596,15 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
     const int S = shape->P * shape->G;
     float* coef = reinterpret_cast<float*>(ws + L.off_coef);
     int32_t* nseq = reinterpret_cast<int32_t*>(ws + L.off_nseq);
-    if (launch_seq_counts(mask, seq_offsets, S, nseq, s) != cudaSuccess) return AIS_ERR_DEVICE;
+    uint32_t* ticket = reinterpret_cast<uint32_t*>(ws + L.off_ticket);
+    if (launch_seq_counts(mask, seq_offsets, S, nseq, ticket, s) != cudaSuccess) return AIS_ERR_DEVICE;
     const int P_norm = shape->P_total > 0 ? shape->P_total : shape->P;
-    if (launch_loss_coef(lp_train, lp_old, lp_ref, params->beta_kl, mask, seq_offsets, adv, w_tilde, nseq, shape->T, S, P_norm * shape->G, params->clip_eps,
-                         reinterpret_cast<double*>(ws + L.off_diag), coef, loss, diag, lse_train, s) != cudaSuccess)
+    // row tiles whose gradient factors are all zero (masked rows, zero advantage) are skipped by the recompute and dH passes
+    if (launch_loss_coef(lp_train, lp_old, lp_ref, params->beta_kl, mask, seq_offsets, adv, w_tilde, nseq, shape->T, S, P_norm * shape->G,
+                         params->clip_eps, reinterpret_cast<double*>(ws + L.off_diag), ticket, coef, ws + L.off_flags, ws + L.off_pace,
+                         2 * kPaceRingBytes, loss, diag, lse_train, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     if (shape->T == 0) return AIS_OK;
-    // row tiles whose gradient factors are all zero (masked rows, zero advantage) are skipped by the recompute and dH passes
-    if (launch_tile_flags_coef(coef, shape->T, ws + L.off_flags, s) != cudaSuccess) return AIS_ERR_DEVICE;
 
     // rows of scratch the workspace can hold (whole row tiles)
     int64_t blk_rows = static_cast<int64_t>((workspace_bytes - L.fixed_bytes) / L.u_row_bytes) / kBM * kBM;
@@ -629,6 +627,7 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
                    CU_TENSOR_MAP_SWIZZLE_128B))
         return AIS_ERR_DEVICE;
 
+    int pass = 0;                                           // tensor-core launches so far
     for (int64_t r0 = 0; r0 < shape->T; r0 += blk_rows) {
         const int64_t rows = (shape->T - r0) < blk_rows ? (shape->T - r0) : blk_rows;
         CUtensorMap tmH;
@@ -659,9 +658,10 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
         a.nsplit = pick_nsplit(shape, params, a.n_row_tiles, a.n_col_tiles);
         a.ksteps = shape->d / 64;
         int units = a.n_row_tiles * a.nsplit;
-        if (arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, units < num_sms ? units : num_sms, s) != cudaSuccess)
-            return AIS_ERR_DEVICE;
-        if (launch_lmhead(dv ? kBwdPDv : kBwdP, tmH, tmW_k, tmH, tmW_k, a, units < num_sms ? units : num_sms, s) != cudaSuccess)
+        int ctas = units < num_sms ? units : num_sms;
+        arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, units, ctas, pass, pass > 0);
+        ++pass;
+        if (launch_lmhead(dv ? kBwdPDv : kBwdP, tmH, tmW_k, tmH, tmW_k, a, ctas, s) != cudaSuccess)
             return AIS_ERR_DEVICE;
         // dH = c (.) (U W)
         a.ncols = shape->d;
@@ -683,8 +683,10 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
                 units = a.split_from + tail * ks;
             }
         }
-        if (arm_pace(a, ws, L, 1, units < num_sms ? units : num_sms, s) != cudaSuccess) return AIS_ERR_DEVICE;
-        if (launch_lmhead(dv ? kBwdDhDv : kBwdDh, tmU, tmW_n, tmU, tmW_n, a, units < num_sms ? units : num_sms, s) != cudaSuccess)
+        ctas = units < num_sms ? units : num_sms;
+        arm_pace(a, ws, L, 1, units, ctas, pass, true);
+        ++pass;
+        if (launch_lmhead(dv ? kBwdDhDv : kBwdDh, tmU, tmW_n, tmU, tmW_n, a, ctas, s) != cudaSuccess)
             return AIS_ERR_DEVICE;
         if (a.ksplit > 1 && launch_dh_reduce(a, s) != cudaSuccess) return AIS_ERR_DEVICE;
         if (dW) {
@@ -711,8 +713,10 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
             units = w.n_row_tiles * w.n_col_tiles;
             const CUtensorMap& tmRow = dv ? tmH_t : tmU_t;
             const CUtensorMap& tmCol = dv ? tmU_t : tmH_t;
-            if (arm_pace(w, ws, L, 1, units < num_sms ? units : num_sms, s) != cudaSuccess) return AIS_ERR_DEVICE;
-            if (launch_lmhead(kBwdDw, tmRow, tmCol, tmRow, tmCol, w, units < num_sms ? units : num_sms, s) != cudaSuccess)
+            ctas = units < num_sms ? units : num_sms;
+            arm_pace(w, ws, L, 1, units, ctas, pass, true);
+            ++pass;
+            if (launch_lmhead(kBwdDw, tmRow, tmCol, tmRow, tmCol, w, ctas, s) != cudaSuccess)
                 return AIS_ERR_DEVICE;
         }
     }

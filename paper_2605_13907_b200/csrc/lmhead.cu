@@ -71,6 +71,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
+    enter_pass(a);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -514,6 +515,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         drain_stage_copies(full, *issued_slot, STG);
         if (a.status) atomicOr(a.status, AIS_FLAG_TIMEOUT);
     }
+    leave_pass(a);
 }
 
 // dH rows of the units whose contraction was split: the partial tiles are added in the order of their ranges and rounded
@@ -521,6 +523,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 // consecutive addresses.  The pass is a plain sweep of ksplit x 256 KB per tile, mostly still in L2 (64 tiles x 9 ranges:
 // 151 MB).  Tiles without work have no partial sums and become zeros.
 __global__ void __launch_bounds__(256) dh_reduce_kernel(const LmheadArgs a) {
+    pdl_enter();
     const int tail = a.n_row_tiles * a.n_col_tiles - a.split_from;
     const int i = blockIdx.x * 256 + threadIdx.x;
     const int row = i & (kBM - 1), cg = (i >> 7) & 15, sub = (i >> 11) & 1, tile = i >> 12;
@@ -556,15 +559,13 @@ __global__ void __launch_bounds__(256) dh_reduce_kernel(const LmheadArgs a) {
 
 cudaError_t launch_dh_reduce(const LmheadArgs& args, cudaStream_t stream) {
     const int tail = args.n_row_tiles * args.n_col_tiles - args.split_from;
-    dh_reduce_kernel<<<tail * 16, 256, 0, stream>>>(args);
-    return cudaGetLastError();
+    return launch_pdl(dh_reduce_kernel, tail * 16, 256, 0, stream, args);
 }
 
 template <int MODE>
 static cudaError_t launch_mode(const CUtensorMap& tmA, const CUtensorMap& tmB, const LmheadArgs& args, int num_ctas,
                                cudaStream_t stream) {
-    lmhead_kernel<MODE><<<num_ctas, threads_of(MODE), kSmemBytes, stream>>>(tmA, tmB, args);
-    return cudaGetLastError();
+    return launch_pdl(lmhead_kernel<MODE>, num_ctas, threads_of(MODE), kSmemBytes, stream, tmA, tmB, args);
 }
 
 cudaError_t launch_lmhead(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,

@@ -107,6 +107,9 @@ struct LmheadArgs {
     int32_t ksplit;        // dH: ranges of the contraction per split unit (1 = nothing is split)
     float* part_acc;       // dH: fp32 partial tiles of the split units, [slot][kPartTileFloats] (see dh_reduce_kernel)
     uint32_t* pace;        // ring of kPaceRing zeroed counters that keeps the CTAs of the launch in step; NULL = no pacing
+    uint32_t* pace_clear;  // ring of the next pass of the same call, cleared by this one; NULL = nothing to clear
+    int32_t overlap;       // the pass needs nothing from the kernel before it (the other pass of the same call): it starts
+                           // while that one drains and waits for it only at its own end
     int32_t pace_per_unit; // announcements per unit = ceil(largest number of stage fills of a unit / fills per announcement)
 };
 

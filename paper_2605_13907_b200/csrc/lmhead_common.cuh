@@ -2,6 +2,7 @@
 // register re-splitting, work-unit decoding and the test for row tiles without work.
 #pragma once
 
+#include "launch.cuh"
 #include "lmhead.cuh"
 #include "ptx.cuh"
 
@@ -164,6 +165,20 @@ __device__ __forceinline__ bool unit_active(const LmheadArgs& a, const Unit& w) 
 __device__ __forceinline__ bool second_tile_active(const LmheadArgs& a, const Unit& w) {
     const int64_t second = 2 * static_cast<int64_t>(w.rt) + 1;
     return second * kBM < a.rows && (a.tile_active == nullptr || a.tile_active[a.row0 / kBM + second] != 0);
+}
+
+// Opening of a pass, by every thread, after the set-up that touches no global memory.  The trigger comes after the wait,
+// so whatever a dependent that does not wait (args.overlap) reads was complete before that dependent could start.
+__device__ __forceinline__ void enter_pass(const LmheadArgs& a) {
+    if (!a.overlap) pdl_wait();
+    pdl_trigger();
+    if (a.pace_clear != nullptr)
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kPaceRing / 4; i += gridDim.x * blockDim.x)
+            reinterpret_cast<uint4*>(a.pace_clear)[i] = make_uint4(0, 0, 0, 0);
+}
+// Its end, by every thread: a pass that did not wait at the start completes only after the kernel before it has.
+__device__ __forceinline__ void leave_pass(const LmheadArgs& a) {
+    if (a.overlap) pdl_wait();
 }
 
 // After every role has left its loops: if the CTA gave up on a wait, the tile copies that the producer issued last

@@ -90,6 +90,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
+    enter_pass(a);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -339,6 +340,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         drain_stage_copies(full, *issued_slot, kStages);
         if (a.status) atomicOr(a.status, AIS_FLAG_TIMEOUT);
     }
+    leave_pass(a);
 }
 
 }  // namespace
@@ -346,12 +348,11 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 cudaError_t launch_lmhead_fp8_block(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,
                                     const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream) {
     switch (args.sgroups) {
-        case 1: lmhead_fp8_block_kernel<1><<<num_ctas, kThreads, Fp8Cfg<1>::kSmem, stream>>>(tmA, tmB, tmSA, tmSB, args); break;
-        case 2: lmhead_fp8_block_kernel<2><<<num_ctas, kThreads, Fp8Cfg<2>::kSmem, stream>>>(tmA, tmB, tmSA, tmSB, args); break;
-        case 4: lmhead_fp8_block_kernel<4><<<num_ctas, kThreads, Fp8Cfg<4>::kSmem, stream>>>(tmA, tmB, tmSA, tmSB, args); break;
+        case 1: return launch_pdl(lmhead_fp8_block_kernel<1>, num_ctas, kThreads, Fp8Cfg<1>::kSmem, stream, tmA, tmB, tmSA, tmSB, args);
+        case 2: return launch_pdl(lmhead_fp8_block_kernel<2>, num_ctas, kThreads, Fp8Cfg<2>::kSmem, stream, tmA, tmB, tmSA, tmSB, args);
+        case 4: return launch_pdl(lmhead_fp8_block_kernel<4>, num_ctas, kThreads, Fp8Cfg<4>::kSmem, stream, tmA, tmB, tmSA, tmSB, args);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t lmhead_fp8_block_prepare() {

@@ -96,8 +96,7 @@ extern "C" int ais_logprob_train_static(const ais_shape* shape, const void* H, c
     // pass just before it, so nothing left over from an earlier call is ever read and nothing needs zeroing.
     if (launch_lmhead(kFwdBf16, tmA, tmB, tmA, tmB, a, units < num_sms ? units : num_sms, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
-    if (launch_combine(a.part_m, a.part_s, a.part_z, nsplit * 2, ld, mask, shape->T, lp_train, lse_train, dev_status, s) !=
-        cudaSuccess)
-        return AIS_ERR_DEVICE;
+    const CombineJob job = {a.part_m, a.part_s, a.part_z, nsplit * 2, lp_train, lse_train};
+    if (launch_combine(&job, 1, ld, mask, shape->T, dev_status, s) != cudaSuccess) return AIS_ERR_DEVICE;
     return AIS_OK;
 }

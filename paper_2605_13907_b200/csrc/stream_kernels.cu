@@ -2,6 +2,7 @@
 #include <type_traits>
 
 #include "stream_kernels.cuh"
+#include "launch.cuh"
 #include "ptx.cuh"
 
 #include <cuda_bf16.h>
@@ -90,6 +91,7 @@ template <int BLOCK>
 __global__ void __launch_bounds__(kQThreads) quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
                                                              int64_t ld, uint8_t* __restrict__ codes, int64_t ldq,
                                                              float* __restrict__ scales, int64_t lds) {
+    pdl_enter();
     constexpr int kLanesPerBlock = BLOCK / 8;
     constexpr int kBlocksPerTile = kQCols / BLOCK;
     __shared__ float sc[kBlocksPerTile][kQRows + 1];
@@ -163,6 +165,7 @@ template <int BLOCK>
 __global__ void __launch_bounds__(256) quantize_cols_kernel(const __nv_bfloat16* __restrict__ x, int64_t K, int64_t N, int64_t ld,
                                                             uint8_t* __restrict__ codes, int64_t ldq,
                                                             float* __restrict__ scales, int64_t lds) {
+    pdl_enter();
     __shared__ __align__(16) uint16_t tile[kQcTile][kQcPitch];
     __shared__ uint32_t half_max[2][kQcTile];
     const int tid = threadIdx.x;
@@ -233,6 +236,7 @@ __global__ void __launch_bounds__(256) quantize_cols_kernel(const __nv_bfloat16*
 __global__ void __launch_bounds__(kQThreads) quantize_mx_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
                                                                 int64_t ld, uint8_t* __restrict__ codes, int64_t ldq,
                                                                 uint8_t* __restrict__ scales) {
+    pdl_enter();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t row0 = static_cast<int64_t>(blockIdx.y) * kQRows;
     const int64_t col0 = static_cast<int64_t>(blockIdx.x) * kQCols;
@@ -287,6 +291,7 @@ __device__ __forceinline__ uint32_t cvt_e2m1x2(float hi, float lo) {
 __global__ void __launch_bounds__(kQThreads) quantize_mxfp4_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
                                                                    int64_t ld, uint8_t* __restrict__ codes, int64_t ldq,
                                                                    uint8_t* __restrict__ scales) {
+    pdl_enter();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t row0 = static_cast<int64_t>(blockIdx.y) * kQRows;
     const int64_t col0 = static_cast<int64_t>(blockIdx.x) * kQCols;
@@ -332,6 +337,7 @@ __global__ void __launch_bounds__(kQThreads) quantize_mxfp4_kernel(const __nv_bf
 // ------------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) tensor_amax_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
                                                            uint32_t* __restrict__ amax_bits) {
+    pdl_enter();
     const int64_t vec_per_row = cols / 8;
     const int64_t total = rows * vec_per_row;
     uint32_t m = 0;
@@ -348,6 +354,7 @@ __global__ void __launch_bounds__(256) tensor_amax_kernel(const __nv_bfloat16* _
 }
 
 __global__ void tensor_scale_kernel(uint32_t* scale_word) {
+    pdl_enter();
     const uint32_t m = *scale_word;                        // bf16 pattern of max|x|
     const float s = (m == 0u) ? 1.0f : __fdiv_rn(__uint_as_float(m << 16), 448.0f);
     *reinterpret_cast<float*>(scale_word) = s;
@@ -356,6 +363,7 @@ __global__ void tensor_scale_kernel(uint32_t* scale_word) {
 __global__ void __launch_bounds__(256) tensor_quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
                                                                int64_t ld, uint8_t* __restrict__ codes, int64_t ldq,
                                                                const float* __restrict__ scale) {
+    pdl_enter();
     const float s = *scale;
     const bool fast = s > 0x1p-100f && s < 0x1p100f;
     const float y = fast ? __frcp_rn(s) : 0.f;
@@ -387,11 +395,13 @@ __global__ void __launch_bounds__(256) tensor_quantize_kernel(const __nv_bfloat1
 // (max, sum) goes through shared memory to warp 0, in warp order.  With one thread per row the up to 296 parts of a small
 // batch were a chain of dependent loads.
 constexpr int kCombWarps = 8;
-__global__ void __launch_bounds__(32 * kCombWarps) combine_kernel(const float* __restrict__ part_m, const float* __restrict__ part_s,
-                                                                  const float* __restrict__ part_z, int nparts, int64_t part_ld,
-                                                                  const uint8_t* __restrict__ mask, int64_t T,
-                                                                  float* __restrict__ lp, float* __restrict__ lse,
-                                                                  uint32_t* status) {
+__global__ void __launch_bounds__(32 * kCombWarps) combine_kernel(const CombineJob j0, const CombineJob j1, int64_t part_ld,
+                                                                  const uint8_t* __restrict__ mask, int64_t T, uint32_t* status) {
+    pdl_enter();
+    const CombineJob job = blockIdx.y == 0 ? j0 : j1;
+    const float *part_m = job.part_m, *part_s = job.part_s, *part_z = job.part_z;
+    const int nparts = job.nparts;
+    float *lp = job.lp, *lse = job.lse;
     __shared__ float sm[kCombWarps][32], ss[kCombWarps][32], sz[kCombWarps][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t t = static_cast<int64_t>(blockIdx.x) * 32 + lane;
@@ -463,14 +473,14 @@ __device__ double block_sum(double v, double* scratch /*[32]*/) {
 
 // Sum of partials[b * stride + offset] over b < nblocks by one warp, in a fixed order: lane l takes blocks l, l + 32, ...
 // (loaded sixteen at a time so that the loads overlap), then the shuffle tree of warp_sum.
-__device__ __forceinline__ double warp_ordered_sum(const double* __restrict__ partials, int nblocks, int stride, int offset, int lane) {
+__device__ __forceinline__ double warp_ordered_sum(const double* partials, int nblocks, int stride, int offset, int lane) {
     double acc = 0.0;
     for (int base = lane; base < nblocks; base += 32 * 16) {
         double v[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
             const int b = base + 32 * j;
-            v[j] = b < nblocks ? partials[b * stride + offset] : 0.0;
+            v[j] = b < nblocks ? __ldcg(partials + b * stride + offset) : 0.0;      // written by other blocks, possibly of this launch
         }
 #pragma unroll
         for (int j = 0; j < 16; ++j) acc += v[j];
@@ -478,9 +488,43 @@ __device__ __forceinline__ double warp_ordered_sum(const double* __restrict__ pa
     return warp_sum(acc);
 }
 
+// The same sums for N values at once (same order each): two barriers for all of them instead of two for each; results in
+// out[0 .. N-1], valid for every thread after the call.
+template <int N>
+__device__ __forceinline__ void block_sums(double (&v)[N], double (*scratch)[32] /*[N][32]*/, double* out) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        v[i] = warp_sum(v[i]);
+        if (lane == 0) scratch[i][warp] = v[i];
+    }
+    __syncthreads();
+    if (threadIdx.x < N) {
+        double tot = 0.0;
+        const int nw = (blockDim.x + 31) >> 5;
+        for (int i = 0; i < nw; ++i) tot += scratch[threadIdx.x][i];
+        out[threadIdx.x] = tot;
+    }
+    __syncthreads();
+}
+
+// True in every thread of the block that arrives last at `ticket` (zeroed before the launch): that block sees what all
+// blocks wrote before their arrival.
+__device__ __forceinline__ bool last_block(uint32_t* ticket) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    __threadfence();
+    return last;
+}
+
 // Valid rows of each sequence: one warp per sequence, 4 mask bytes per lane and load where the row range allows it.
 __global__ void __launch_bounds__(256) seq_count_kernel(const uint8_t* __restrict__ mask, const int32_t* __restrict__ seq_offsets,
-                                                         int S, int32_t* __restrict__ n_valid_seq) {
+                                                         int S, int32_t* __restrict__ n_valid_seq, uint32_t* __restrict__ ticket) {
+    pdl_enter();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
     const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= S) return;
     const int lane = threadIdx.x & 31;
@@ -503,7 +547,9 @@ __global__ void __launch_bounds__(256) seq_count_kernel(const uint8_t* __restric
 // Group-relative advantages (Eq. grpo_adv): one thread per sequence.  With `zero_counts` the per-sequence row
 // counts are cleared for the moments kernel, which adds them up.
 __global__ void adv_kernel(const float* __restrict__ rewards, int S, int G, int adv_std_norm, float eps, float* __restrict__ adv,
-                           int32_t* __restrict__ zero_counts) {
+                           int32_t* __restrict__ zero_counts, uint32_t* __restrict__ ticket) {
+    pdl_enter();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= S) return;
     if (zero_counts) zero_counts[s] = 0;
@@ -529,6 +575,7 @@ __global__ void adv_kernel(const float* __restrict__ rewards, int S, int G, int 
 __global__ void __launch_bounds__(256) seq_logw_kernel(const float* __restrict__ lp_train, const float* __restrict__ lp_roll,
                                                         const uint8_t* __restrict__ mask, const int32_t* __restrict__ seq_offsets,
                                                         int S, float* __restrict__ seq_logw) {
+    pdl_enter();
     const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= S) return;
     const int lane = threadIdx.x & 31;
@@ -539,13 +586,18 @@ __global__ void __launch_bounds__(256) seq_logw_kernel(const float* __restrict__
     if (lane == 0) seq_logw[s] = static_cast<float>(acc);
 }
 
-// One byte per 128-row tile: does any row of the tile need computing?  (mask != 0 / gradient factor != 0)
+// One byte per 128-row tile: does any row of the tile need computing?  (mask != 0 / gradient factor != 0)  The same launch
+// clears the pacing rings of the passes that follow (`clear`: uint4 words, may be NULL).
 template <typename T>
-__global__ void tile_flags_kernel(const T* __restrict__ pred, int64_t n, uint8_t* __restrict__ flags) {
+__global__ void tile_flags_kernel(const T* __restrict__ pred, int64_t n, uint8_t* __restrict__ flags, uint4* __restrict__ clear,
+                                  int nclear) {
+    pdl_enter();
     const int64_t tile = blockIdx.x;
     const int64_t i = tile * 128 + threadIdx.x;
     const int any = __syncthreads_or(i < n && pred[i] != T(0));
     if (threadIdx.x == 0) flags[tile] = any ? 1 : 0;
+    if (clear)
+        for (int64_t k = i; k < nclear; k += static_cast<int64_t>(gridDim.x) * 128) clear[k] = make_uint4(0, 0, 0, 0);
 }
 
 __device__ __forceinline__ int seq_of_row(const int32_t* __restrict__ seq_offsets, int S, int64_t t) {
@@ -555,6 +607,52 @@ __device__ __forceinline__ int seq_of_row(const int32_t* __restrict__ seq_offset
         if (static_cast<int64_t>(seq_offsets[mid]) <= t) lo = mid; else hi = mid;
     }
     return lo;
+}
+
+// The diagnostics and alpha from the ten sums over the batch.
+__device__ __noinline__ void derive_diag(const double* m, const ais_params& p, ais_diag* __restrict__ diag) {
+    ais_diag d;
+    d.status_flags = 0;
+    d.reserved = 0;
+    d.loss = 0.0;
+    d.kl_ref = 0.0;
+    const double N = m[0];
+    d.n_valid = N;
+    if (N <= 0.0) {
+        d.mean_w = 1.0; d.cv2 = 0.0; d.ess = 0.0; d.ess_ratio = 1.0; d.alpha_ess = 1.0; d.d_bar = 0.0;
+        d.alpha_mis = 0.0; d.std_A = 0.0; d.std_Aw = 0.0; d.delta_sigma = 0.0; d.alpha_var = 0.0;
+        d.alpha_adaptive = 0.0; d.kl_k1 = 0.0; d.mean_abs_dp = 0.0;
+        d.status_flags |= AIS_FLAG_EMPTY;
+    } else {
+        // Population variance E[x^2] - E[x]^2 in fp64.  The sums reach this point with fp64 accuracy relative to the
+        // spread of the data (add_run), so what is left is the rounding of the fp64 additions themselves: a result
+        // below 2^-44 of the mean square (a few hundred ulps of it; a standard deviation below 2.4e-7 of the rms
+        // value) is that rounding and is reported as exactly zero.
+        auto variance = [&](double sum, double sumsq) {
+            const double mean = sum / N, ms = sumsq / N;
+            const double v = ms - mean * mean;
+            return v > ms * 0x1p-44 ? v : 0.0;
+        };
+        const double mu = m[1] / N;
+        const double var = variance(m[1], m[2]);
+        d.mean_w = mu;
+        d.cv2 = var / (mu * mu);
+        d.ess = m[1] * m[1] / m[2];
+        d.ess_ratio = d.ess / N;
+        d.alpha_ess = 1.0 / sqrt(1.0 + d.cv2);
+        d.d_bar = m[3] / N;
+        d.alpha_mis = fmin(1.0, d.d_bar / static_cast<double>(p.delta));
+        d.std_A = sqrt(variance(m[4], m[5]));
+        d.std_Aw = sqrt(variance(m[6], m[7]));
+        d.delta_sigma = d.std_Aw / (d.std_A + static_cast<double>(p.eps));
+        d.alpha_var = fmax(0.0, (d.delta_sigma - static_cast<double>(p.gamma)) / static_cast<double>(p.gamma));
+        d.alpha_adaptive = fmin(1.0, fmax(0.0, d.alpha_ess - static_cast<double>(p.beta_var) * d.alpha_var)) * d.alpha_mis;
+        d.kl_k1 = m[8] / N;
+        d.mean_abs_dp = m[9] / N;
+    }
+    if (isnan(N)) d.status_flags |= AIS_FLAG_TIMEOUT;       // a block of the moments kernel gave up on a bounded wait
+    d.alpha = isnan(p.alpha_override) ? d.alpha_adaptive : static_cast<double>(p.alpha_override);
+    *diag = d;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -642,6 +740,7 @@ __global__ void __launch_bounds__(kDiagThreads) moments_kernel(const float* __re
                                                                 const float* __restrict__ adv, int64_t T, int S, float C,
                                                                 double* __restrict__ partials, int32_t* __restrict__ n_valid_seq,
                                                                 const float* __restrict__ seq_logw) {
+    pdl_enter();
     __shared__ double scratch[32];
     double acc[kNumMoments];
 #pragma unroll
@@ -798,21 +897,30 @@ __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, int*
     return mbar_wait(bar, parity, abort_flag);
 }
 
-// SEQ: every row carries its sequence's truncated weight instead of its own.  EXACT: the second of two launches (see
-// add_rows below): a block returns at once unless the first launch found all of its log-probability gaps tiny.
-template <bool SEQ, bool EXACT>
+// What the last block of the moments kernel leaves behind.
+struct DiagFinish {
+    ais_params params;
+    ais_diag* diag;        // diagnostics and alpha (may be NULL)
+    double* moments;       // the sums themselves (may be NULL)
+    uint32_t* ticket;      // arrivals of the blocks, zeroed before the launch
+};
+
+// SEQ: every row carries its sequence's truncated weight instead of its own.  The block that finishes last adds up the
+// blocks' partial sums in their order and writes the diagnostics (fin.diag) or the sums themselves (fin.moments), so that
+// the batch step needs no launch of its own for that.
+template <bool SEQ>
 __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const float* __restrict__ lp_train,
                                                                          const float* __restrict__ lp_roll,
                                                                          const uint8_t* __restrict__ mask,
                                                                          const int32_t* __restrict__ seq_offsets,
                                                                          const float* __restrict__ adv, int T, int S, float C,
-                                                                         double* __restrict__ partials,
-                                                                         int32_t* __restrict__ n_valid_seq,
-                                                                         const float* __restrict__ seq_logw) {
+                                                                         double* partials, int32_t* __restrict__ n_valid_seq,
+                                                                         const float* __restrict__ seq_logw, const DiagFinish fin) {
     static_assert(kDiagThreads * 8 == kMomRows, "one 8-row group per thread and tile");
     extern __shared__ __align__(128) uint8_t stages[];          // kMomStages stages, then the barriers
     uint64_t* full = reinterpret_cast<uint64_t*>(stages + kMomStages * kMomStageBytes);
-    __shared__ double scratch[32];
+    __shared__ double scratch[10][32];
+    __shared__ double totals[kNumMoments];
     __shared__ int abort_flag;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
@@ -820,18 +928,12 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
     const int per = (ntiles + gridDim.x - 1) / gridDim.x;
     const int tile0 = blockIdx.x * per < ntiles ? blockIdx.x * per : ntiles;
     const int tile1 = tile0 + per < ntiles ? tile0 + per : ntiles;
-    if (EXACT) {
-        // slots 10 and 11 of the block's partial sums: its groups with a gap above 2^-6 and its groups of valid rows without,
-        // as counted by the first launch; slot 0 is NaN when that launch gave up on a wait
-        const double big = partials[blockIdx.x * kNumMoments + 10], small = partials[blockIdx.x * kNumMoments + 11];
-        const double n0 = partials[blockIdx.x * kNumMoments];
-        if (big != 0.0 || small == 0.0 || n0 != n0) return;
-    }
     if (tid == 0) {
         for (int i = 0; i < kMomStages; ++i) mbar_init(&full[i], 1);
         abort_flag = 0;
         fence_barrier_init();
     }
+    pdl_enter();
     __syncthreads();
     auto issue = [&](int tile, int st) {               // thread 0: the three copies of one tile onto the stage's barrier
         uint8_t* dst = stages + st * kMomStageBytes;
@@ -893,12 +995,12 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
     // `cur`; returns how many they are.  Rows go two at a time through the packed fp32 instructions.  The weight pivot
     // is w - 1 of the first valid row this thread meets and stays: any value of the data serves.
     // rho - 1 comes from the fast exponential, which is good to 1e-7 ABSOLUTE: enough unless the gaps D themselves are
-    // tiny, when it is only a thousandth of a weight that differs from 1 by 1e-4.  The EXACT form of this kernel uses a
-    // short series for groups whose |D| are all at most 2^-6 (their sum is), which gives e^D - 1 to fp32 accuracy
-    // relative to itself.  It is slower (the second path costs registers and scheduling freedom: a fifth of the
-    // bandwidth), so the fast form runs first and counts each block's groups above 2^-6, and the exact form is launched
-    // after it: there only the blocks that met no such group walk their tiles again and replace their partial sums.
-    auto add_rows = [&](const float (&lt)[8], const float (&lr)[8], uint32_t m0, uint32_t m1) -> int {
+    // tiny, when it is only a thousandth of a weight that differs from 1 by 1e-4.  The exact walk uses a short series for
+    // groups whose |D| are all at most 2^-6 (their sum is), which gives e^D - 1 to fp32 accuracy relative to itself.  Both
+    // in one walk cost registers and scheduling freedom (a fifth of the bandwidth), so the fast walk comes first and counts
+    // the block's groups above 2^-6; a block that met none walks its tiles a second time, exactly.
+    auto add_rows = [&](auto exact, const float (&lt)[8], const float (&lr)[8], uint32_t m0, uint32_t m1) -> int {
+        constexpr bool EXACT = decltype(exact)::value;
         const uint32_t v0 = __vcmpne4(m0, 0u), v1 = __vcmpne4(m1, 0u);     // 0xFF in the byte of every valid row
         const int n = (__popc(v0) + __popc(v1)) >> 3;
         bool on[8];
@@ -978,11 +1080,11 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
         return n;
     };
 
-    // The walk over the block's tiles; the first launch also adds up the valid rows per sequence on the way.
-    constexpr bool count = !EXACT;
+    // One walk over the block's tiles, the `base`-th tile of the stage ring first; the fast one also adds up the valid rows
+    // per sequence on the way.
     bool failed = false;
-    {
-        constexpr int base = 0;
+    auto walk = [&](auto exact, int base) {
+        constexpr bool count = !decltype(exact)::value;
         int issued = tile0;                             // first tile not yet requested (thread 0)
         if (tid == 0)
             for (; issued < tile1 && issued < tile0 + kMomStages; ++issued) issue(issued, (base + issued - tile0) % kMomStages);
@@ -1007,7 +1109,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
                 const float lt[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
                 const float lr[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
                 if (single) {
-                    if ((mk.x | mk.y) != 0u) n = add_rows(lt, lr, mk.x, mk.y);
+                    if ((mk.x | mk.y) != 0u) n = add_rows(exact, lt, lr, mk.x, mk.y);
                 } else if ((mk.x | mk.y) != 0u) {
                     const uint64_t m64 = (static_cast<uint64_t>(mk.y) << 32) | mk.x;
                     int j = 0;
@@ -1017,7 +1119,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
                         const int j1 = left < 8 - j ? j + left : 8;
                         enter();
                         const uint64_t run = (j1 == 8 ? ~uint64_t(0) : (uint64_t(1) << (8 * j1)) - 1u) & ~((uint64_t(1) << (8 * j)) - 1u);
-                        const int nr = add_rows(lt, lr, static_cast<uint32_t>(m64 & run), static_cast<uint32_t>((m64 & run) >> 32));
+                        const int nr = add_rows(exact, lt, lr, static_cast<uint32_t>(m64 & run), static_cast<uint32_t>((m64 & run) >> 32));
                         if (count && n_valid_seq && nr > 0) atomicAdd(&n_valid_seq[sq], nr);
                         j = j1;
                     }
@@ -1053,8 +1155,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
                     mbar_wait_drain(&full[q % kMomStages], (q / kMomStages) & 1u);
                 }
         }
-    }
-    if (count && n_valid_seq && lane == 0 && wsq >= 0 && wcnt > 0) atomicAdd(&n_valid_seq[wsq], wcnt);
+        if (count && n_valid_seq && lane == 0 && wsq >= 0 && wcnt > 0) atomicAdd(&n_valid_seq[wsq], wcnt);
     // rows after the last whole tile: the first threads of the grid, one row each
     for (int t = ntiles * kMomRows + static_cast<int>(blockIdx.x * blockDim.x) + tid; t < T; t += gridDim.x * blockDim.x) {
         if (!mask[t]) continue;
@@ -1062,10 +1163,19 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
         seek(t);
         enter();
         const float lt[8] = {lp_train[t], 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, lr[8] = {lp_roll[t], 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        add_rows(lt, lr, 1u, 0u);
+        add_rows(exact, lt, lr, 1u, 0u);
         if (count && n_valid_seq) atomicAdd(&n_valid_seq[sq], 1);
     }
-    double acc[10];
+    };
+    walk(std::false_type{}, 0);
+    const bool any_big = __syncthreads_or(nbig) != 0;
+    const bool any_small = __syncthreads_or(nsmall) != 0;
+    if (!any_big && any_small && !__syncthreads_or(failed ? 1 : 0)) {
+        reset();
+        walk(std::true_type{}, tile1 - tile0);
+    }
+    constexpr int kSums = 10;                            // slots 10 and 11 are no moments
+    double acc[kSums];
     {
         // from the shifted sums to the sums of w, w^2, A, A^2, A w, (A w)^2 in fp64, once per thread:
         // w = P + v with P = 1 + pivot;  A = Ap + dA;  A w = K + x with K = Ap P
@@ -1084,75 +1194,36 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
         acc[9] = static_cast<double>(f9);
     }
     if (failed) acc[0] = __longlong_as_double(0x7ff8000000000000LL);     // a NaN count marks the batch as not reduced
-    // slots 10 and 11: what the second launch looks at (no moments; the reductions over the blocks leave them out)
-    const double big = EXACT ? 0.0 : block_sum(static_cast<double>(nbig), scratch);
-    const double small = EXACT ? 0.0 : block_sum(static_cast<double>(nsmall), scratch);
-#pragma unroll
-    for (int i = 0; i < kNumMoments; ++i) {
-        const double tot = i < 10 ? block_sum(acc[i < 10 ? i : 0], scratch) : 0.0;
-        if (tid == 0) partials[blockIdx.x * kNumMoments + i] = i == 10 ? big : i == 11 ? small : tot;
+    block_sums(acc, scratch, totals);
+    if (tid < kSums) partials[blockIdx.x * kNumMoments + tid] = totals[tid];
+    if (!last_block(fin.ticket)) return;
+    for (int i = tid >> 5; i < kNumMoments; i += kDiagThreads / 32) {
+        const double m = i < kSums ? warp_ordered_sum(partials, gridDim.x, kNumMoments, i, lane) : 0.0;
+        if (lane == 0) totals[i] = m;
     }
+    __syncthreads();
+    if (fin.moments != nullptr && tid < kNumMoments) fin.moments[tid] = totals[tid];
+    if (fin.diag != nullptr && tid == 0) derive_diag(totals, fin.params, fin.diag);
 }
 
-__global__ void diag_finalize_kernel(const double* __restrict__ partials, int nblocks, ais_params p, ais_diag* __restrict__ diag) {
-    // one warp per moment sums the partials in a fixed order;
-    // thread 0 then derives the diagnostics
+__global__ void __launch_bounds__(32 * kNumMoments) diag_finalize_kernel(const double* __restrict__ partials, int nblocks, ais_params p,
+                                                                       ais_diag* __restrict__ diag) {
+    // one warp per moment sums the partials in a fixed order; thread 0 then derives the diagnostics
     __shared__ double m[kNumMoments];
-    if (blockIdx.x != 0) return;
+    pdl_enter();
     {
         const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
         const double acc = warp_ordered_sum(partials, nblocks, kNumMoments, i, lane);
         if (lane == 0) m[i] = acc;
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    ais_diag d;
-    d.status_flags = 0;
-    d.reserved = 0;
-    d.loss = 0.0;
-    d.kl_ref = 0.0;
-    const double N = m[0];
-    d.n_valid = N;
-    if (N <= 0.0) {
-        d.mean_w = 1.0; d.cv2 = 0.0; d.ess = 0.0; d.ess_ratio = 1.0; d.alpha_ess = 1.0; d.d_bar = 0.0;
-        d.alpha_mis = 0.0; d.std_A = 0.0; d.std_Aw = 0.0; d.delta_sigma = 0.0; d.alpha_var = 0.0;
-        d.alpha_adaptive = 0.0; d.kl_k1 = 0.0; d.mean_abs_dp = 0.0;
-        d.status_flags |= AIS_FLAG_EMPTY;
-    } else {
-        // Population variance E[x^2] - E[x]^2 in fp64.  The sums reach this point with fp64 accuracy relative to the
-        // spread of the data (add_run), so what is left is the rounding of the fp64 additions themselves: a result
-        // below 2^-44 of the mean square (a few hundred ulps of it; a standard deviation below 2.4e-7 of the rms
-        // value) is that rounding and is reported as exactly zero.
-        auto variance = [&](double sum, double sumsq) {
-            const double mean = sum / N, ms = sumsq / N;
-            const double v = ms - mean * mean;
-            return v > ms * 0x1p-44 ? v : 0.0;
-        };
-        const double mu = m[1] / N;
-        const double var = variance(m[1], m[2]);
-        d.mean_w = mu;
-        d.cv2 = var / (mu * mu);
-        d.ess = m[1] * m[1] / m[2];
-        d.ess_ratio = d.ess / N;
-        d.alpha_ess = 1.0 / sqrt(1.0 + d.cv2);
-        d.d_bar = m[3] / N;
-        d.alpha_mis = fmin(1.0, d.d_bar / static_cast<double>(p.delta));
-        d.std_A = sqrt(variance(m[4], m[5]));
-        d.std_Aw = sqrt(variance(m[6], m[7]));
-        d.delta_sigma = d.std_Aw / (d.std_A + static_cast<double>(p.eps));
-        d.alpha_var = fmax(0.0, (d.delta_sigma - static_cast<double>(p.gamma)) / static_cast<double>(p.gamma));
-        d.alpha_adaptive = fmin(1.0, fmax(0.0, d.alpha_ess - static_cast<double>(p.beta_var) * d.alpha_var)) * d.alpha_mis;
-        d.kl_k1 = m[8] / N;
-        d.mean_abs_dp = m[9] / N;
-    }
-    if (isnan(N)) d.status_flags |= AIS_FLAG_TIMEOUT;       // a block of the moments kernel gave up on a bounded wait
-    d.alpha = isnan(p.alpha_override) ? d.alpha_adaptive : static_cast<double>(p.alpha_override);
-    *diag = d;
+    if (threadIdx.x == 0) derive_diag(m, p, diag);
 }
 
 // Sums the per-block partial moments in block order into one vector of kNumMoments doubles.
 // One warp per moment, fixed order.
 __global__ void moments_reduce_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ moments) {
+    pdl_enter();
     if (blockIdx.x != 0) return;
     const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const double m = i < 10 ? warp_ordered_sum(partials, nblocks, kNumMoments, i, lane) : 0.0;   // 10, 11 are no moments
@@ -1165,6 +1236,14 @@ __global__ void __launch_bounds__(256) rectify_kernel(const float* __restrict__ 
                                                       const ais_diag* __restrict__ diag, float* __restrict__ rho,
                                                       float* __restrict__ w_tilde, const int32_t* __restrict__ seq_offsets,
                                                       int S, const float* __restrict__ seq_logw) {
+    // the log-probs and the mask were there before the kernel this one follows: the first group is loaded while that one
+    // still runs, the wait is for alpha
+    const int64_t ngroups = T / VEC;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    const int64_t g0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    RowGroup<VEC> in;
+    if (g0 < ngroups) in = load_group<VEC>(lp_train, lp_roll, mask, g0);
+    pdl_enter();
     const float alpha = static_cast<float>(diag->alpha);
     auto one = [&](float lt, float lr, uint8_t mk, float& r, float& wt, int64_t t) {
         r = 1.0f;
@@ -1176,10 +1255,8 @@ __global__ void __launch_bounds__(256) rectify_kernel(const float* __restrict__ 
             wt = fmaf(alpha, fminf(w, C) - 1.0f, 1.0f);
         }
     };
-    const int64_t ngroups = T / VEC;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t g = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; g < ngroups; g += stride) {
-        const RowGroup<VEC> in = load_group<VEC>(lp_train, lp_roll, mask, g);
+    for (int64_t g = g0; g < ngroups; g += stride) {
+        if (g != g0) in = load_group<VEC>(lp_train, lp_roll, mask, g);
         float r[VEC], wt[VEC];
 #pragma unroll
         for (int j = 0; j < VEC; ++j) one(in.lt[j], in.lr[j], in.mk[j], r[j], wt[j], g * VEC + j);
@@ -1202,90 +1279,99 @@ __global__ void __launch_bounds__(256) rectify_kernel(const float* __restrict__ 
 // ------------------------------------------------------------------------------------------------
 // Per-token gradient factor c_t and the surrogate loss (Eq. ais-grpo without the KL term).
 // ------------------------------------------------------------------------------------------------
-template <int VEC>
-__global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const float* __restrict__ lp_train, const float* __restrict__ lp_old,
-                                                                  const float* __restrict__ lp_ref, double beta_kl,
-                                                                  const uint8_t* __restrict__ mask,
-                                                                  const int32_t* __restrict__ seq_offsets,
-                                                                  const float* __restrict__ adv, const float* __restrict__ w_tilde,
-                                                                  const int32_t* __restrict__ n_valid_seq, int64_t T, int S,
-                                                                  int S_norm, double clip_eps, double* __restrict__ partials,
-                                                                  float* __restrict__ coef, const float* __restrict__ lse) {
-    __shared__ double scratch[32];
+// One thread per group of four rows, one warp per 128-row tile, so that the kernel also says which tiles have a gradient
+// (tile_flags) -- and, as its last block, adds up the loss.  VEC: the vectors allow 16-byte accesses.
+struct LossArgs {
+    const float *lp_train, *lp_old, *lp_ref, *lse, *adv, *w_tilde;
+    const uint8_t* mask;
+    const int32_t *seq_offsets, *n_valid_seq;
+    int64_t T;
+    int32_t S, S_norm;
+    double beta_kl, clip_eps;
+    double* partials;
+    float* coef;
+    uint8_t* tile_flags;
+    uint4* clear;          // pacing rings of the passes that follow
+    int32_t nclear;
+    uint32_t* ticket;
+    float* loss;
+    ais_diag* diag;
+};
+
+template <bool VEC>
+__global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const LossArgs a) {
+    __shared__ double scratch[2][32];
+    __shared__ double totals[2];
+    pdl_enter();
+    const int lane = threadIdx.x & 31;
     double J = 0.0, KL = 0.0;
     // one valid row of sequence sq: its share of the objective, of the KL estimate, and its gradient factor
     auto one = [&](int64_t t, int sq, float wtf) -> float {
-        if (!isfinite(lse[t])) return 0.f;       // the forward pass marked this row (non-finite logits): it takes no part
-        const double A = adv[sq];
-        const int n = n_valid_seq[sq] > 0 ? n_valid_seq[sq] : 1;
-        const double norm = 1.0 / (static_cast<double>(S_norm) * static_cast<double>(n));
-        const double rho_on = lp_old ? exp(static_cast<double>(lp_train[t]) - static_cast<double>(lp_old[t])) : 1.0;
+        if (!isfinite(a.lse[t])) return 0.f;     // the forward pass marked this row (non-finite logits): it takes no part
+        const double A = a.adv[sq];
+        const int n = a.n_valid_seq[sq] > 0 ? a.n_valid_seq[sq] : 1;
+        const double norm = 1.0 / (static_cast<double>(a.S_norm) * static_cast<double>(n));
+        const double rho_on = a.lp_old ? exp(static_cast<double>(a.lp_train[t]) - static_cast<double>(a.lp_old[t])) : 1.0;
         const double un = rho_on * A;
-        const double cl = fmin(fmax(rho_on, 1.0 - clip_eps), 1.0 + clip_eps) * A;
+        const double cl = fmin(fmax(rho_on, 1.0 - a.clip_eps), 1.0 + a.clip_eps) * A;
         const double wt = wtf;
         double c = 0.0;
         J += wt * fmin(un, cl) * norm;
         if (un <= cl) c = wt * A * rho_on * norm;
-        if (lp_ref) {
+        if (a.lp_ref) {
             // KL(pi_theta || pi_ref) estimate r - log r - 1, r = pi_ref / pi_theta; its slope in lp_theta is 1 - r
-            const double log_r = static_cast<double>(lp_ref[t]) - static_cast<double>(lp_train[t]);
+            const double log_r = static_cast<double>(a.lp_ref[t]) - static_cast<double>(a.lp_train[t]);
             const double r = exp(log_r);
             KL += (r - log_r - 1.0) * norm;
-            c -= beta_kl * (1.0 - r) * norm;
+            c -= a.beta_kl * (1.0 - r) * norm;
         }
         return static_cast<float>(c);
     };
-    const int64_t ngroups = T / VEC;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t g = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; g < ngroups; g += stride) {
-        float c[VEC], wt[VEC];
-        uint8_t mk[VEC];
-        bool any = false;
-        if (VEC == 4) {
-            const uchar4 m = reinterpret_cast<const uchar4*>(mask)[g];
-            const float4 w4 = reinterpret_cast<const float4*>(w_tilde)[g];
-            mk[0] = m.x; mk[1 % VEC] = m.y; mk[2 % VEC] = m.z; mk[3 % VEC] = m.w;
-            wt[0] = w4.x; wt[1 % VEC] = w4.y; wt[2 % VEC] = w4.z; wt[3 % VEC] = w4.w;
+    const int64_t tiles = (a.T + 127) / 128;
+    const int64_t nwarps = static_cast<int64_t>(gridDim.x) * (kDiagThreads / 32);
+    for (int64_t tile = static_cast<int64_t>(blockIdx.x) * (kDiagThreads / 32) + (threadIdx.x >> 5); tile < tiles; tile += nwarps) {
+        const int64_t t0 = tile * 128 + 4 * lane;
+        const int rows = t0 + 4 <= a.T ? 4 : t0 < a.T ? static_cast<int>(a.T - t0) : 0;
+        float c[4] = {0.f, 0.f, 0.f, 0.f}, wt[4] = {0.f, 0.f, 0.f, 0.f};
+        uint32_t mk = 0;                                          // mask bytes of the four rows
+        if (VEC && rows == 4) {
+            mk = *reinterpret_cast<const uint32_t*>(a.mask + t0);
+            const float4 w4 = *reinterpret_cast<const float4*>(a.w_tilde + t0);
+            wt[0] = w4.x; wt[1] = w4.y; wt[2] = w4.z; wt[3] = w4.w;
         } else {
-            mk[0] = mask[g];
-            wt[0] = w_tilde[g];
-        }
-#pragma unroll
-        for (int j = 0; j < VEC; ++j) { c[j] = 0.f; any |= (mk[j] != 0); }
-        if (any) {
-            const int64_t t0 = g * VEC;
-            int sq = seq_of_row(seq_offsets, S, t0);
-#pragma unroll
-            for (int j = 0; j < VEC; ++j) {
-                while (sq + 1 < S && static_cast<int64_t>(seq_offsets[sq + 1]) <= t0 + j) ++sq;
-                if (mk[j]) c[j] = one(t0 + j, sq, wt[j]);
+            for (int j = 0; j < rows; ++j) {
+                mk |= static_cast<uint32_t>(a.mask[t0 + j]) << (8 * j);
+                wt[j] = a.w_tilde[t0 + j];
             }
         }
-        if (VEC == 4) reinterpret_cast<float4*>(coef)[g] = make_float4(c[0], c[1 % VEC], c[2 % VEC], c[3 % VEC]);
-        else coef[g] = c[0];
+        if (mk != 0u) {
+            int sq = seq_of_row(a.seq_offsets, a.S, t0);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                while (sq + 1 < a.S && static_cast<int64_t>(a.seq_offsets[sq + 1]) <= t0 + j) ++sq;
+                if ((mk >> (8 * j)) & 0xFFu) c[j] = one(t0 + j, sq, wt[j]);
+            }
+        }
+        if (rows == 4) *reinterpret_cast<float4*>(a.coef + t0) = make_float4(c[0], c[1], c[2], c[3]);     // workspace: aligned
+        else
+            for (int j = 0; j < rows; ++j) a.coef[t0 + j] = c[j];
+        const bool any = __any_sync(0xffffffffu, c[0] != 0.f || c[1] != 0.f || c[2] != 0.f || c[3] != 0.f);
+        if (lane == 0) a.tile_flags[tile] = any ? 1 : 0;
     }
-    for (int64_t t = ngroups * VEC + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < T; t += stride)
-        coef[t] = mask[t] ? one(t, seq_of_row(seq_offsets, S, t), w_tilde[t]) : 0.f;
-    const double tot = block_sum(J, scratch);
-    const double tot_kl = block_sum(KL, scratch);
-    if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = tot;
-        partials[2 * blockIdx.x + 1] = tot_kl;
-    }
-}
-
-__global__ void loss_finalize_kernel(const double* __restrict__ partials, int nblocks, double beta_kl, float* loss,
-                                     ais_diag* diag) {
-    // one warp, fixed order
-    if (threadIdx.x >= 32 || blockIdx.x != 0) return;
-    const double J = warp_ordered_sum(partials, nblocks, 2, 0, threadIdx.x);
-    const double KL = warp_ordered_sum(partials, nblocks, 2, 1, threadIdx.x);
-    if (threadIdx.x != 0) return;
-    const double total = -J + beta_kl * KL;
-    if (loss) *loss = static_cast<float>(total);
-    if (diag) {
-        diag->loss = total;
-        diag->kl_ref = KL;
+    if (a.clear)
+        for (int i = blockIdx.x * kDiagThreads + threadIdx.x; i < a.nclear; i += gridDim.x * kDiagThreads) a.clear[i] = make_uint4(0, 0, 0, 0);
+    double sums[2] = {J, KL};
+    block_sums(sums, scratch, totals);
+    if (threadIdx.x < 2) a.partials[2 * blockIdx.x + threadIdx.x] = totals[threadIdx.x];
+    if (!last_block(a.ticket) || threadIdx.x >= 32) return;
+    const double Jall = warp_ordered_sum(a.partials, gridDim.x, 2, 0, lane);
+    const double KLall = warp_ordered_sum(a.partials, gridDim.x, 2, 1, lane);
+    if (lane != 0) return;
+    const double total = -Jall + a.beta_kl * KLall;
+    if (a.loss) *a.loss = static_cast<float>(total);
+    if (a.diag) {
+        a.diag->loss = total;
+        a.diag->kl_ref = KLall;
     }
 }
 
@@ -1296,49 +1382,52 @@ inline bool vec4_ok(const void* a, const void* b, const void* c, const void* d, 
     return (f % 16 == 0) && (reinterpret_cast<uintptr_t>(m) % 4 == 0);
 }
 
-void launch_moments_kernel(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
-                           const float* adv, int64_t T, int S, float C, double* partials, int32_t* n_valid_seq,
-                           float* seq_logw, cudaStream_t stream) {
-    if (seq_logw && S > 0) seq_logw_kernel<<<(S + 7) / 8, 256, 0, stream>>>(lp_train, lp_roll, mask, seq_offsets, S, seq_logw);
-    if (vec4_ok(lp_train, lp_roll, nullptr, nullptr, mask) && reinterpret_cast<uintptr_t>(mask) % 16 == 0 && T < (int64_t(1) << 31) - 2 * kMomRows) {      // 32-bit row indices inside
-        // the fast form, then the exact form for the blocks whose gaps were all tiny (usually none: those blocks return at once)
-        const int Ti = static_cast<int>(T);
-        if (seq_logw) {
-            moments_staged_kernel<true, false><<<kDiagBlocks, kDiagThreads, kMomSmemBytes, stream>>>(lp_train, lp_roll, mask, seq_offsets, adv, Ti, S, C, partials, n_valid_seq, seq_logw);
-            moments_staged_kernel<true, true><<<kDiagBlocks, kDiagThreads, kMomSmemBytes, stream>>>(lp_train, lp_roll, mask, seq_offsets, adv, Ti, S, C, partials, n_valid_seq, seq_logw);
-        } else {
-            moments_staged_kernel<false, false><<<kDiagBlocks, kDiagThreads, kMomSmemBytes, stream>>>(lp_train, lp_roll, mask, seq_offsets, adv, Ti, S, C, partials, n_valid_seq, seq_logw);
-            moments_staged_kernel<false, true><<<kDiagBlocks, kDiagThreads, kMomSmemBytes, stream>>>(lp_train, lp_roll, mask, seq_offsets, adv, Ti, S, C, partials, n_valid_seq, seq_logw);
-        }
-    } else if (vec4_ok(lp_train, lp_roll, nullptr, nullptr, mask))
-        moments_kernel<4><<<kDiagBlocks, kDiagThreads, 0, stream>>>(lp_train, lp_roll, mask, seq_offsets, adv, T, S, C, partials,
-                                                                      n_valid_seq, seq_logw);
-    else
-        moments_kernel<1><<<kDiagBlocks, kDiagThreads, 0, stream>>>(lp_train, lp_roll, mask, seq_offsets, adv, T, S, C, partials,
-                                                                      n_valid_seq, seq_logw);
+// Blocks of a batch reduction: one per `rows` rows up to the fixed maximum, a function of the batch size alone so that the
+// summation order is.
+inline int reduce_blocks(int64_t T, int rows) {
+    const int64_t b = (T + rows - 1) / rows;
+    return static_cast<int>(b < 1 ? 1 : b > kDiagBlocks ? kDiagBlocks : b);
 }
 
-void launch_rectify_kernel(const float* lp_train, const float* lp_roll, const uint8_t* mask, int64_t T, float C,
+// The masked sums of the batch into fin.diag and / or fin.moments.
+cudaError_t launch_moments_kernel(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
+                                  const float* adv, int64_t T, int S, float C, double* partials, int32_t* n_valid_seq,
+                                  float* seq_logw, const DiagFinish& fin, cudaStream_t stream) {
+    cudaError_t e;
+    if (seq_logw && S > 0) {
+        e = launch_pdl(seq_logw_kernel, (S + 7) / 8, 256, 0, stream, lp_train, lp_roll, mask, seq_offsets, S, seq_logw);
+        if (e != cudaSuccess) return e;
+    }
+    if (vec4_ok(lp_train, lp_roll, nullptr, nullptr, mask) && reinterpret_cast<uintptr_t>(mask) % 16 == 0 && T < (int64_t(1) << 31) - 2 * kMomRows) {      // 32-bit row indices inside
+        const int blocks = reduce_blocks(T, kMomRows);
+        const int Ti = static_cast<int>(T);
+        return launch_pdl(seq_logw ? moments_staged_kernel<true> : moments_staged_kernel<false>, blocks, kDiagThreads, kMomSmemBytes, stream,
+                          lp_train, lp_roll, mask, seq_offsets, adv, Ti, S, C, partials, n_valid_seq, seq_logw, fin);
+    }
+    e = launch_pdl(vec4_ok(lp_train, lp_roll, nullptr, nullptr, mask) ? moments_kernel<4> : moments_kernel<1>, kDiagBlocks, kDiagThreads, 0, stream,
+                   lp_train, lp_roll, mask, seq_offsets, adv, T, S, C, partials, n_valid_seq, seq_logw);
+    if (e != cudaSuccess) return e;
+    if (fin.moments) e = launch_pdl(moments_reduce_kernel, 1, 32 * kNumMoments, 0, stream, partials, kDiagBlocks, fin.moments);
+    if (e == cudaSuccess && fin.diag)
+        e = launch_pdl(diag_finalize_kernel, 1, 32 * kNumMoments, 0, stream, partials, kDiagBlocks, fin.params, fin.diag);
+    return e;
+}
+
+cudaError_t launch_rectify_kernel(const float* lp_train, const float* lp_roll, const uint8_t* mask, int64_t T, float C,
                            const ais_diag* diag, float* rho, float* w_tilde, const int32_t* seq_offsets, int S,
                            const float* seq_logw, cudaStream_t stream) {
     const int64_t groups = (T + 3) / 4;
     const int blocks = static_cast<int>(((groups + 255) / 256) < 2368 ? ((groups + 255) / 256) : 2368);
-    if (vec4_ok(lp_train, lp_roll, rho, w_tilde, mask))
-        rectify_kernel<4><<<blocks, 256, 0, stream>>>(lp_train, lp_roll, mask, T, C, diag, rho, w_tilde, seq_offsets, S, seq_logw);
-    else
-        rectify_kernel<1><<<blocks, 256, 0, stream>>>(lp_train, lp_roll, mask, T, C, diag, rho, w_tilde, seq_offsets, S, seq_logw);
+    return launch_pdl(vec4_ok(lp_train, lp_roll, rho, w_tilde, mask) ? rectify_kernel<4> : rectify_kernel<1>, blocks, 256, 0, stream,
+                      lp_train, lp_roll, mask, T, C, diag, rho, w_tilde, seq_offsets, S, seq_logw);
 }
 
 }  // namespace
 
 cudaError_t stream_prepare() {
-    cudaError_t e = cudaFuncSetAttribute(moments_staged_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(moments_staged_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(moments_staged_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(moments_staged_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(moments_staged_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
+    return cudaFuncSetAttribute(moments_staged_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
 }
 
 // ------------------------------------------------------------------------------------------------ launchers
@@ -1348,12 +1437,11 @@ cudaError_t launch_quantize(const void* x, int64_t rows, int64_t cols, int64_t l
     dim3 grid(static_cast<unsigned>((cols + kQCols - 1) / kQCols), static_cast<unsigned>((rows + kQRows - 1) / kQRows));
     const __nv_bfloat16* xp = static_cast<const __nv_bfloat16*>(x);
     switch (block) {
-        case 32:  quantize_kernel<32><<<grid, kQThreads, 0, stream>>>(xp, rows, cols, ld, codes, ldq, scales, lds); break;
-        case 64:  quantize_kernel<64><<<grid, kQThreads, 0, stream>>>(xp, rows, cols, ld, codes, ldq, scales, lds); break;
-        case 128: quantize_kernel<128><<<grid, kQThreads, 0, stream>>>(xp, rows, cols, ld, codes, ldq, scales, lds); break;
+        case 32:  return launch_pdl(quantize_kernel<32>, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scales, lds);
+        case 64:  return launch_pdl(quantize_kernel<64>, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scales, lds);
+        case 128: return launch_pdl(quantize_kernel<128>, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scales, lds);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_quantize_cols(const void* x, int64_t K, int64_t N, int64_t ld, int block, uint8_t* codes, int64_t ldq,
@@ -1362,12 +1450,11 @@ cudaError_t launch_quantize_cols(const void* x, int64_t K, int64_t N, int64_t ld
     dim3 grid(static_cast<unsigned>((N + kQcTile - 1) / kQcTile), static_cast<unsigned>((K + kQcTile - 1) / kQcTile));
     const __nv_bfloat16* xp = static_cast<const __nv_bfloat16*>(x);
     switch (block) {
-        case 32:  quantize_cols_kernel<32><<<grid, 256, 0, stream>>>(xp, K, N, ld, codes, ldq, scales, lds); break;
-        case 64:  quantize_cols_kernel<64><<<grid, 256, 0, stream>>>(xp, K, N, ld, codes, ldq, scales, lds); break;
-        case 128: quantize_cols_kernel<128><<<grid, 256, 0, stream>>>(xp, K, N, ld, codes, ldq, scales, lds); break;
+        case 32:  return launch_pdl(quantize_cols_kernel<32>, grid, 256, 0, stream, xp, K, N, ld, codes, ldq, scales, lds);
+        case 64:  return launch_pdl(quantize_cols_kernel<64>, grid, 256, 0, stream, xp, K, N, ld, codes, ldq, scales, lds);
+        case 128: return launch_pdl(quantize_cols_kernel<128>, grid, 256, 0, stream, xp, K, N, ld, codes, ldq, scales, lds);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_quantize_mx(const void* x, int64_t rows, int64_t cols, int64_t ld, uint8_t* codes, int64_t ldq,
@@ -1377,11 +1464,8 @@ cudaError_t launch_quantize_mx(const void* x, int64_t rows, int64_t cols, int64_
     if (e != cudaSuccess) return e;
     if (rows == 0 || cols == 0) return cudaSuccess;
     dim3 grid(static_cast<unsigned>((cols + kQCols - 1) / kQCols), static_cast<unsigned>((rows + kQRows - 1) / kQRows));
-    if (fp4)
-        quantize_mxfp4_kernel<<<grid, kQThreads, 0, stream>>>(static_cast<const __nv_bfloat16*>(x), rows, cols, ld, codes, ldq, scales);
-    else
-        quantize_mx_kernel<<<grid, kQThreads, 0, stream>>>(static_cast<const __nv_bfloat16*>(x), rows, cols, ld, codes, ldq, scales);
-    return cudaGetLastError();
+    return launch_pdl(fp4 ? quantize_mxfp4_kernel : quantize_mx_kernel, grid, kQThreads, 0, stream, static_cast<const __nv_bfloat16*>(x), rows,
+                      cols, ld, codes, ldq, scales);
 }
 
 cudaError_t launch_quantize_tensor(const void* x, int64_t rows, int64_t cols, int64_t ld, uint8_t* codes, int64_t ldq,
@@ -1391,86 +1475,90 @@ cudaError_t launch_quantize_tensor(const void* x, int64_t rows, int64_t cols, in
     const __nv_bfloat16* xp = static_cast<const __nv_bfloat16*>(x);
     const int64_t total = rows * (cols / 8);
     const int blocks = static_cast<int>(total <= 0 ? 1 : ((total + 255) / 256 < 148 * 16 ? (total + 255) / 256 : 148 * 16));
-    if (total > 0) tensor_amax_kernel<<<blocks, 256, 0, stream>>>(xp, rows, cols, ld, reinterpret_cast<uint32_t*>(scale));
-    tensor_scale_kernel<<<1, 1, 0, stream>>>(reinterpret_cast<uint32_t*>(scale));
-    if (total > 0) tensor_quantize_kernel<<<blocks, 256, 0, stream>>>(xp, rows, cols, ld, codes, ldq, scale);
-    return cudaGetLastError();
+    if (total > 0) {
+        e = launch_pdl(tensor_amax_kernel, blocks, 256, 0, stream, xp, rows, cols, ld, reinterpret_cast<uint32_t*>(scale));
+        if (e != cudaSuccess) return e;
+    }
+    e = launch_pdl(tensor_scale_kernel, 1, 1, 0, stream, reinterpret_cast<uint32_t*>(scale));
+    if (e != cudaSuccess || total <= 0) return e;
+    return launch_pdl(tensor_quantize_kernel, blocks, 256, 0, stream, xp, rows, cols, ld, codes, ldq, scale);
 }
 
-cudaError_t launch_combine(const float* part_m, const float* part_s, const float* part_z, int nparts, int64_t part_ld,
-                           const uint8_t* mask, int64_t T, float* lp, float* lse, uint32_t* status, cudaStream_t stream) {
+cudaError_t launch_combine(const CombineJob* jobs, int njobs, int64_t part_ld, const uint8_t* mask, int64_t T, uint32_t* status,
+                           cudaStream_t stream) {
     if (T == 0) return cudaSuccess;
-    combine_kernel<<<static_cast<unsigned>((T + 31) / 32), 32 * kCombWarps, 0, stream>>>(part_m, part_s, part_z, nparts, part_ld, mask, T, lp, lse, status);
-    return cudaGetLastError();
+    return launch_pdl(combine_kernel, dim3(static_cast<unsigned>((T + 31) / 32), static_cast<unsigned>(njobs)), 32 * kCombWarps, 0, stream, jobs[0],
+                      jobs[njobs - 1], part_ld, mask, T, status);
 }
 
-cudaError_t launch_tile_flags_mask(const uint8_t* mask, int64_t T, uint8_t* flags, cudaStream_t stream) {
+cudaError_t launch_tile_flags_mask(const uint8_t* mask, int64_t T, uint8_t* flags, void* clear, size_t clear_bytes, cudaStream_t stream) {
     if (T <= 0) return cudaSuccess;
-    tile_flags_kernel<uint8_t><<<static_cast<unsigned>((T + 127) / 128), 128, 0, stream>>>(mask, T, flags);
-    return cudaGetLastError();
+    return launch_pdl(tile_flags_kernel<uint8_t>, static_cast<unsigned>((T + 127) / 128), 128, 0, stream, mask, T, flags,
+                      static_cast<uint4*>(clear), static_cast<int>(clear_bytes / 16));
 }
 
-cudaError_t launch_tile_flags_coef(const float* coef, int64_t T, uint8_t* flags, cudaStream_t stream) {
-    if (T <= 0) return cudaSuccess;
-    tile_flags_kernel<float><<<static_cast<unsigned>((T + 127) / 128), 128, 0, stream>>>(coef, T, flags);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_seq_counts(const uint8_t* mask, const int32_t* seq_offsets, int S, int32_t* n_valid_seq, cudaStream_t stream) {
-    if (S == 0) return cudaSuccess;
-    seq_count_kernel<<<(S + 7) / 8, 256, 0, stream>>>(mask, seq_offsets, S, n_valid_seq);
-    return cudaGetLastError();
+cudaError_t launch_seq_counts(const uint8_t* mask, const int32_t* seq_offsets, int S, int32_t* n_valid_seq, uint32_t* ticket, cudaStream_t stream) {
+    return launch_pdl(seq_count_kernel, (S + 7) / 8, 256, 0, stream, mask, seq_offsets, S, n_valid_seq, ticket);
 }
 
 cudaError_t launch_advantages(const float* rewards, int S, int G, int adv_std_norm, float eps, float* adv, int32_t* zero_counts,
-                              cudaStream_t stream) {
-    if (S == 0) return cudaSuccess;
-    adv_kernel<<<(S + 255) / 256, 256, 0, stream>>>(rewards, S, G, adv_std_norm, eps, adv, zero_counts);
-    return cudaGetLastError();
+                              uint32_t* ticket, cudaStream_t stream) {
+    return launch_pdl(adv_kernel, (S + 255) / 256, 256, 0, stream, rewards, S, G, adv_std_norm, eps, adv, zero_counts, ticket);
 }
 
 cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
-                        const float* adv, int64_t T, int S, const ais_params& p, double* partials, int32_t* n_valid_seq,
-                        float* seq_logw, float* rho, float* w_tilde, ais_diag* diag, cudaStream_t stream) {
-    const float C = p.C;
-    launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, C, partials, n_valid_seq, seq_logw, stream);
-    diag_finalize_kernel<<<1, 32 * kNumMoments, 0, stream>>>(partials, kDiagBlocks, p, diag);
-    if (T > 0) launch_rectify_kernel(lp_train, lp_roll, mask, T, C, diag, rho, w_tilde, seq_offsets, S, seq_logw, stream);
-    return cudaGetLastError();
+                        const float* adv, int64_t T, int S, const ais_params& p, double* partials, uint32_t* ticket,
+                        int32_t* n_valid_seq, float* seq_logw, float* rho, float* w_tilde, ais_diag* diag, cudaStream_t stream) {
+    const DiagFinish fin = {p, diag, nullptr, ticket};
+    const cudaError_t e = launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, fin, stream);
+    if (e != cudaSuccess || T == 0) return e;
+    return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, diag, rho, w_tilde, seq_offsets, S, seq_logw, stream);
 }
 
 cudaError_t launch_moments(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
-                           const float* adv, int64_t T, int S, const ais_params& p, double* partials, int32_t* n_valid_seq,
-                           float* seq_logw, double* moments, cudaStream_t stream) {
-    launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, stream);
-    moments_reduce_kernel<<<1, 32 * kNumMoments, 0, stream>>>(partials, kDiagBlocks, moments);
-    return cudaGetLastError();
+                           const float* adv, int64_t T, int S, const ais_params& p, double* partials, uint32_t* ticket,
+                           int32_t* n_valid_seq, float* seq_logw, double* moments, cudaStream_t stream) {
+    const DiagFinish fin = {p, nullptr, moments, ticket};
+    return launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, fin, stream);
 }
 
 cudaError_t launch_finalize(const double* moments, const float* lp_train, const float* lp_roll, const uint8_t* mask, int64_t T,
                             const ais_params& p, float* rho, float* w_tilde, ais_diag* diag, const int32_t* seq_offsets, int S,
                             const float* seq_logw, cudaStream_t stream) {
-    diag_finalize_kernel<<<1, 32 * kNumMoments, 0, stream>>>(moments, 1, p, diag);
-    if (T > 0) launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, diag, rho, w_tilde, seq_offsets, S, seq_logw, stream);
-    return cudaGetLastError();
+    const cudaError_t e = launch_pdl(diag_finalize_kernel, 1, 32 * kNumMoments, 0, stream, moments, 1, p, diag);
+    if (e != cudaSuccess || T == 0) return e;
+    return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, diag, rho, w_tilde, seq_offsets, S, seq_logw, stream);
 }
 
 cudaError_t launch_loss_coef(const float* lp_train, const float* lp_old, const float* lp_ref, float beta_kl, const uint8_t* mask,
-                             const int32_t* seq_offsets,
-                             const float* adv, const float* w_tilde, const int32_t* n_valid_seq, int64_t T, int S, int S_norm,
-                             float clip_eps, double* partials, float* coef, float* loss, ais_diag* diag, const float* lse,
-                             cudaStream_t stream) {
-    const float* ref = (beta_kl != 0.f) ? lp_ref : nullptr;
-    if (vec4_ok(w_tilde, coef, nullptr, nullptr, mask))
-        loss_coef_kernel<4><<<kDiagBlocks, kDiagThreads, 0, stream>>>(lp_train, lp_old, ref, static_cast<double>(beta_kl), mask,
-                                                                        seq_offsets, adv, w_tilde, n_valid_seq, T, S, S_norm,
-                                                                        static_cast<double>(clip_eps), partials, coef, lse);
-    else
-        loss_coef_kernel<1><<<kDiagBlocks, kDiagThreads, 0, stream>>>(lp_train, lp_old, ref, static_cast<double>(beta_kl), mask,
-                                                                        seq_offsets, adv, w_tilde, n_valid_seq, T, S, S_norm,
-                                                                        static_cast<double>(clip_eps), partials, coef, lse);
-    loss_finalize_kernel<<<1, 32, 0, stream>>>(partials, kDiagBlocks, ref ? static_cast<double>(beta_kl) : 0.0, loss, diag);
-    return cudaGetLastError();
+                             const int32_t* seq_offsets, const float* adv, const float* w_tilde, const int32_t* n_valid_seq, int64_t T,
+                             int S, int S_norm, float clip_eps, double* partials, uint32_t* ticket, float* coef, uint8_t* tile_flags,
+                             void* clear, size_t clear_bytes, float* loss, ais_diag* diag, const float* lse, cudaStream_t stream) {
+    LossArgs a = {};
+    a.lp_train = lp_train;
+    a.lp_old = lp_old;
+    a.lp_ref = (beta_kl != 0.f) ? lp_ref : nullptr;
+    a.lse = lse;
+    a.adv = adv;
+    a.w_tilde = w_tilde;
+    a.mask = mask;
+    a.seq_offsets = seq_offsets;
+    a.n_valid_seq = n_valid_seq;
+    a.T = T;
+    a.S = S;
+    a.S_norm = S_norm;
+    a.beta_kl = a.lp_ref ? static_cast<double>(beta_kl) : 0.0;
+    a.clip_eps = static_cast<double>(clip_eps);
+    a.partials = partials;
+    a.coef = coef;
+    a.tile_flags = tile_flags;
+    a.clear = static_cast<uint4*>(clear);
+    a.nclear = static_cast<int32_t>(clear_bytes / 16);
+    a.ticket = ticket;
+    a.loss = loss;
+    a.diag = diag;
+    return launch_pdl(vec4_ok(w_tilde, nullptr, nullptr, nullptr, mask) ? loss_coef_kernel<true> : loss_coef_kernel<false>, reduce_blocks(T, 4 * kDiagThreads),
+                      kDiagThreads, 0, stream, a);
 }
 
 }  // namespace ais

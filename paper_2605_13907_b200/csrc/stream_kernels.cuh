@@ -33,42 +33,48 @@ cudaError_t launch_quantize_mx(const void* x, int64_t rows, int64_t cols, int64_
 cudaError_t launch_quantize_tensor(const void* x, int64_t rows, int64_t cols, int64_t ld, uint8_t* codes, int64_t ldq,
                                    float* scale, cudaStream_t stream);
 
-// lp[t] = z_y - lse, lse[t] from nparts partial triples laid out [nparts][part_ld].
-cudaError_t launch_combine(const float* part_m, const float* part_s, const float* part_z, int nparts, int64_t part_ld,
-                           const uint8_t* mask, int64_t T, float* lp, float* lse, uint32_t* status, cudaStream_t stream);
+// One merge of partial triples laid out [nparts][part_ld]: lp[t] = z_y - lse, lse[t] (may be NULL).
+struct CombineJob {
+    const float *part_m, *part_s, *part_z;
+    int32_t nparts;
+    float *lp, *lse;
+};
+// One or two merges (the passes of one call) in one launch.
+cudaError_t launch_combine(const CombineJob* jobs, int njobs, int64_t part_ld, const uint8_t* mask, int64_t T, uint32_t* status,
+                           cudaStream_t stream);
 
-// flags[i] = 1 when rows 128 i .. 128 i + 127 contain a row with mask != 0 (resp. a non-zero gradient factor).
-cudaError_t launch_tile_flags_mask(const uint8_t* mask, int64_t T, uint8_t* flags, cudaStream_t stream);
-cudaError_t launch_tile_flags_coef(const float* coef, int64_t T, uint8_t* flags, cudaStream_t stream);
+// flags[i] = 1 when rows 128 i .. 128 i + 127 contain a row with mask != 0; clears `clear` (16-byte aligned, may be NULL).
+cudaError_t launch_tile_flags_mask(const uint8_t* mask, int64_t T, uint8_t* flags, void* clear, size_t clear_bytes, cudaStream_t stream);
 
-// n_valid_seq[s] = valid rows of sequence s.
-cudaError_t launch_seq_counts(const uint8_t* mask, const int32_t* seq_offsets, int S, int32_t* n_valid_seq, cudaStream_t stream);
-// adv[s] (group-relative advantages); zero_counts [S] (may be NULL) is cleared for the moments kernel to count into.
+// n_valid_seq[s] = valid rows of sequence s; zeroes `ticket` (the block counter of the reduction that follows).
+cudaError_t launch_seq_counts(const uint8_t* mask, const int32_t* seq_offsets, int S, int32_t* n_valid_seq, uint32_t* ticket, cudaStream_t stream);
+// adv[s] (group-relative advantages); zero_counts [S] (may be NULL) is cleared for the moments kernel to count into,
+// `ticket` for it to count its blocks.
 cudaError_t launch_advantages(const float* rewards, int S, int G, int adv_std_norm, float eps, float* adv, int32_t* zero_counts,
-                              cudaStream_t stream);
+                              uint32_t* ticket, cudaStream_t stream);
 
 // n_valid_seq (may be NULL) must have been cleared: the moments kernel adds every sequence's valid rows to it.
 cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
-                        const float* adv, int64_t T, int S, const ais_params& p, double* partials /*[kDiagBlocks][kNumMoments]*/,
+                        const float* adv, int64_t T, int S, const ais_params& p, double* partials /*[kDiagBlocks][kNumMoments]*/, uint32_t* ticket,
                         int32_t* n_valid_seq, float* seq_logw /* [S] scratch: non-NULL selects sequence-level weights */,
                         float* rho, float* w_tilde, ais_diag* diag, cudaStream_t stream);
 
 // The two halves of launch_diag: partial moments summed into `moments` [kNumMoments], and everything that follows
 // from a (possibly all-reduced) moment vector.
 cudaError_t launch_moments(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
-                           const float* adv, int64_t T, int S, const ais_params& p, double* partials, int32_t* n_valid_seq,
-                           float* seq_logw, double* moments, cudaStream_t stream);
+                           const float* adv, int64_t T, int S, const ais_params& p, double* partials, uint32_t* ticket,
+                           int32_t* n_valid_seq, float* seq_logw, double* moments, cudaStream_t stream);
 cudaError_t launch_finalize(const double* moments, const float* lp_train, const float* lp_roll, const uint8_t* mask, int64_t T,
                             const ais_params& p, float* rho, float* w_tilde, ais_diag* diag, const int32_t* seq_offsets, int S,
                             const float* seq_logw, cudaStream_t stream);
 
-// coef[t] and the loss; n_valid_seq must already hold the valid counts.  S_norm is the number of sequences the
-// objective averages over (all data-parallel ranks together).  Rows whose lse is not finite (marked by the forward
-// pass) contribute nothing.
+// coef[t], the row tiles that have a gradient, and the loss; n_valid_seq must already hold the valid counts, ticket zero.
+// S_norm is the number of sequences the objective averages over (all data-parallel ranks together).  Rows whose lse is not
+// finite (marked by the forward pass) contribute nothing.  Clears `clear` on the way.
 cudaError_t launch_loss_coef(const float* lp_train, const float* lp_old, const float* lp_ref, float beta_kl, const uint8_t* mask,
-                             const int32_t* seq_offsets,
-                             const float* adv, const float* w_tilde, const int32_t* n_valid_seq, int64_t T, int S, int S_norm,
-                             float clip_eps, double* partials /*[kDiagBlocks][2]*/, float* coef, float* loss, ais_diag* diag,
-                             const float* lse, cudaStream_t stream);
+                             const int32_t* seq_offsets, const float* adv, const float* w_tilde, const int32_t* n_valid_seq, int64_t T,
+                             int S, int S_norm, float clip_eps, double* partials /*[kDiagBlocks][2]*/, uint32_t* ticket, float* coef,
+                             uint8_t* tile_flags, void* clear, size_t clear_bytes, float* loss, ais_diag* diag, const float* lse,
+                             cudaStream_t stream);
 
 }  // namespace ais
