@@ -317,6 +317,29 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params,
                  uint32_t* dev_status, void* workspace, size_t workspace_bytes, void* stream);
 
 /*
+ * The stages of a step in one call: what `stages` names, in the order quantise H, quantise W, log-probs, diagnostics, loss
+ * and gradients, each exactly as its own entry point above does it (the same arguments under the same names).  For callers
+ * that run the same step again and again and fill the struct once: a step of a small batch takes tens of microseconds, and
+ * marshalling six argument lists is a good part of that.  Quantises by shape->fp8_block; the codes' row strides are those
+ * ais_logprob_fwd expects.  Stops at the first stage that returns an error.
+ */
+#define AIS_STAGE_QUANTIZE_H 1u
+#define AIS_STAGE_QUANTIZE_W 2u
+#define AIS_STAGE_LOGPROB    4u
+#define AIS_STAGE_DIAGNOSE   8u
+#define AIS_STAGE_LOSS       16u
+typedef struct ais_step_args {
+    const void* H; const void* W; const int32_t* tokens; const uint8_t* mask; const int32_t* seq_offsets; const float* rewards;
+    const float* lp_old; const float* lp_ref;
+    uint8_t* qH; void* sH; int64_t ldsH; uint8_t* qW; void* sW; int64_t ldsW;
+    float* lp_train; float* lse_train; float* lp_roll; float* lse_roll;
+    float* adv; int32_t* n_valid_seq; float* rho; float* w_tilde; ais_diag* diag;
+    void* dH; float* loss; float* dW; int64_t lddw; int64_t dw_accumulate;
+    uint32_t* dev_status; void* workspace; size_t workspace_bytes;
+} ais_step_args;
+int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_args* args, uint32_t stages, void* stream);
+
+/*
  * Row compaction for batches whose valid rows are scattered (masked-diffusion log-probabilities: only the masked
  * positions of a response take part, Appendix "LLaDA Experiments").  The tensor-core passes work on tiles of 128
  * consecutive rows, so scattered invalid rows cost as much as valid ones; packing the valid rows first makes the

@@ -42,6 +42,18 @@ class Diag(C.Structure):
         return {n: getattr(self, n) for n, _ in self._fields_ if n != "reserved"}
 
 
+STAGE_QUANTIZE_H, STAGE_QUANTIZE_W, STAGE_LOGPROB, STAGE_DIAGNOSE, STAGE_LOSS = 1, 2, 4, 8, 16
+
+
+class StepArgs(C.Structure):
+    _fields_ = [(n, C.c_void_p) for n in ("H", "W", "tokens", "mask", "seq_offsets", "rewards", "lp_old", "lp_ref", "qH", "sH")] + \
+               [("ldsH", C.c_int64), ("qW", C.c_void_p), ("sW", C.c_void_p), ("ldsW", C.c_int64)] + \
+               [(n, C.c_void_p) for n in ("lp_train", "lse_train", "lp_roll", "lse_roll", "adv", "n_valid_seq", "rho", "w_tilde",
+                                          "diag", "dH", "loss", "dW")] + \
+               [("lddw", C.c_int64), ("dw_accumulate", C.c_int64), ("dev_status", C.c_void_p), ("workspace", C.c_void_p),
+                ("workspace_bytes", C.c_size_t)]
+
+
 def lib_path() -> str:
     return _LIB_PATH
 
@@ -86,6 +98,8 @@ def lib() -> C.CDLL:
         L.ais_diag_moments.argtypes = [C.POINTER(Shape), C.POINTER(Params)] + [vp] * 9 + [vp, sz, vp]
         L.ais_diag_finalize.restype = C.c_int
         L.ais_diag_finalize.argtypes = [C.POINTER(Shape), C.POINTER(Params)] + [vp] * 10
+        L.ais_step.restype = C.c_int
+        L.ais_step.argtypes = [C.POINTER(Shape), C.POINTER(Params), C.POINTER(StepArgs), C.c_uint32, vp]
         L.ais_compact_index.restype = C.c_int
         L.ais_compact_index.argtypes = [vp, vp, C.c_int32, vp, vp, vp, vp]
         L.ais_gather_rows.restype = C.c_int
@@ -115,11 +129,17 @@ def _check(status: int, what: str) -> None:
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# the raw handle without a Stream object around it (a microsecond per call), where this torch has it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(t: torch.Tensor):
-    return C.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+    if _raw_stream is not None:
+        return _raw_stream(t.get_device())
+    return torch.cuda.current_stream(t.device).cuda_stream
 
 
 def default_params(**overrides) -> Params:
@@ -383,6 +403,69 @@ class AisStep:
         self.dH = torch.empty(max(T, 1), ldh, dtype=torch.bfloat16, device=dev)[:, :d] if want_grad else None
         self.w_quantized = False
 
+    # ---- the stages in one library call.  The struct with the step's own buffers is filled once and again whenever an
+    # attribute it holds is assigned; the caller's tensors go in at every call.
+    _PLANNED = frozenset(("shape", "params", "workspace", "qH", "sH", "qW", "sW", "lp_train", "lse_train", "lp_roll", "lse_roll", "rho",
+                          "w_tilde", "adv", "n_valid_seq", "loss", "diag", "status", "dH", "w_layout"))
+
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        if name in AisStep._PLANNED:
+            object.__setattr__(self, "_plan", None)
+
+    def _make_plan(self):
+        """The filled struct, its address and those of shape and params; None when a buffer does not have the layout that
+        ais_step takes (codes with another row stride than the shape's): such steps go through the single calls."""
+        sh = self.shape
+        ldq_h = sh.ldh // 2 if sh.fp8_block == FP4_MX32 else sh.ldh
+        ldq_w = sh.d if self.w_layout == W_DV else sh.ldw // 2 if sh.fp8_block == FP4_MX32 else sh.ldw
+        own = dict(qH=self.qH, sH=self.sH, qW=self.qW, sW=self.sW, lp_train=self.lp_train, lse_train=self.lse_train, lp_roll=self.lp_roll,
+                   lse_roll=self.lse_roll, adv=self.adv, n_valid_seq=self.n_valid_seq, rho=self.rho, w_tilde=self.w_tilde, diag=self.diag,
+                   dH=self.dH, loss=self.loss, dev_status=self.status, workspace=self.workspace)
+        _require_cuda(*own.values())
+        plan = False
+        if self.qH.stride(0) == ldq_h and self.qW.stride(0) == ldq_w:
+            args = StepArgs(**{k: _ptr(t) for k, t in own.items()})
+            args.ldsH = self.sH.stride(0) if self.sH.dim() == 2 else 0
+            args.ldsW = self.sW.stride(0) if self.sW.dim() == 2 else 0
+            args.workspace_bytes = self.workspace.numel() * self.workspace.element_size()
+            plan = (args, C.byref(args), C.byref(sh), C.byref(self.params), lib().ais_step)
+        object.__setattr__(self, "_plan", plan)
+        return plan
+
+    def _run(self, stages, H, W, tokens, mask, seq_offsets=None, rewards=None, lp_old=None, lp_ref=None, dW=None,
+             dw_accumulate: bool = False) -> bool:
+        """Enqueues `stages` in one call; False when the operands are not laid out as the shape says (the caller then goes
+        through the single entry points, which take every stride)."""
+        plan = self._plan
+        if plan is None:
+            plan = self._make_plan()
+        if plan is False:
+            return False
+        sh = self.shape
+        if stages & STAGE_QUANTIZE_H and (H.shape != (sh.T, sh.d) or H.stride(0) != sh.ldh):
+            return False
+        if stages & STAGE_QUANTIZE_W and (W.shape != ((sh.d, sh.V) if self.w_layout == W_DV else (sh.V, sh.d)) or W.stride(0) != sh.ldw):
+            return False
+        for t in (H, W, tokens, mask, seq_offsets, rewards, lp_old, lp_ref, dW):
+            if t is not None and not t.is_cuda:
+                _require_cuda(t)
+        a, a_ref, sh_ref, p_ref, fn = plan
+        a.H = _ptr(H)
+        a.W = _ptr(W)
+        a.tokens = _ptr(tokens)
+        a.mask = _ptr(mask)
+        a.seq_offsets = _ptr(seq_offsets)
+        a.rewards = _ptr(rewards)
+        if stages & STAGE_LOSS:
+            a.lp_old = _ptr(lp_old)
+            a.lp_ref = _ptr(lp_ref)
+            a.dW = _ptr(dW)
+            a.lddw = 0 if dW is None else dW.stride(0)
+            a.dw_accumulate = 1 if dw_accumulate else 0
+        _check(fn(sh_ref, p_ref, a_ref, stages, _stream(self.workspace)), "ais_step")
+        return True
+
     def quantize_weights(self, W: torch.Tensor) -> None:
         if self.w_layout == W_DV:
             quantize_fp8_cols(W, self.shape.fp8_block, self.qW, self.sW)
@@ -391,9 +474,13 @@ class AisStep:
         self.w_quantized = True
 
     def forward(self, H, W, tokens, mask, requantize_w: bool = True) -> None:
+        fresh_w = requantize_w or not self.w_quantized
+        if self._run(STAGE_QUANTIZE_H | STAGE_LOGPROB | (STAGE_QUANTIZE_W if fresh_w else 0), H, W, tokens, mask):
+            self.w_quantized = True
+            return
         if self.shape.T > 0:
             quantize_fp8(H, self.shape.fp8_block, self.qH, self.sH)
-        if requantize_w or not self.w_quantized:
+        if fresh_w:
             self.quantize_weights(W)
         logprob_fwd(self.shape, self.params, H, W, self.qH, self.sH, self.qW, self.sW, tokens, mask, self.lp_train,
                     self.lse_train, self.lp_roll, self.lse_roll, self.status, self.workspace)
@@ -417,6 +504,13 @@ class AisStep:
                  dw_accumulate=dw_accumulate)
 
     def step(self, H, W, tokens, mask, seq_offsets, rewards, lp_old=None, requantize_w: bool = True, lp_ref=None) -> None:
+        if self.group is None:
+            fresh_w = requantize_w or not self.w_quantized
+            stages = STAGE_QUANTIZE_H | STAGE_LOGPROB | STAGE_DIAGNOSE | (STAGE_QUANTIZE_W if fresh_w else 0) | \
+                (STAGE_LOSS if self.dH is not None else 0)
+            if self._run(stages, H, W, tokens, mask, seq_offsets, rewards, lp_old, lp_ref):
+                self.w_quantized = True
+                return
         self.forward(H, W, tokens, mask, requantize_w)
         self.diagnose(mask, seq_offsets, rewards)
         if self.dH is not None:

@@ -723,4 +723,33 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
     return AIS_OK;
 }
 
+int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_args* a, uint32_t stages, void* stream) {
+    int st = check_shape(shape);
+    if (st != AIS_OK) return st;
+    if (!a) return AIS_ERR_NULL;
+    const int block = shape->fp8_block;
+    const bool dv = shape->w_layout == AIS_W_DV, fp4 = block == AIS_FP4_MX32;
+    auto quantize = [&](const void* x, int64_t rows, int64_t ld, uint8_t* codes, int64_t ldq, void* scales, int64_t lds) {
+        if (fp4) return ais_quantize_mxfp4(x, rows, shape->d, ld, codes, ldq / 2, static_cast<uint8_t*>(scales), stream);
+        if (block == AIS_FP8_MX32) return ais_quantize_mxfp8(x, rows, shape->d, ld, codes, ldq, static_cast<uint8_t*>(scales), stream);
+        if (block == 0) return ais_quantize_fp8_tensor(x, rows, shape->d, ld, codes, ldq, static_cast<float*>(scales), stream);
+        return ais_quantize_fp8(x, rows, shape->d, ld, block, codes, ldq, static_cast<float*>(scales), lds, stream);
+    };
+    if ((stages & AIS_STAGE_QUANTIZE_H) && shape->T > 0) st = quantize(a->H, shape->T, shape->ldh, a->qH, shape->ldh, a->sH, a->ldsH);
+    if (st == AIS_OK && (stages & AIS_STAGE_QUANTIZE_W))
+        st = dv ? ais_quantize_fp8_cols(a->W, shape->d, shape->V, shape->ldw, block, a->qW, shape->d, static_cast<float*>(a->sW), a->ldsW, stream)
+                : quantize(a->W, shape->V, shape->ldw, a->qW, shape->ldw, a->sW, a->ldsW);
+    if (st == AIS_OK && (stages & AIS_STAGE_LOGPROB))
+        st = ais_logprob_fwd(shape, params, a->H, a->W, a->qH, a->sH, a->ldsH, a->qW, a->sW, a->ldsW, a->tokens, a->mask, a->lp_train,
+                             a->lse_train, a->lp_roll, a->lse_roll, a->dev_status, a->workspace, a->workspace_bytes, stream);
+    if (st == AIS_OK && (stages & AIS_STAGE_DIAGNOSE))
+        st = ais_diagnostics(shape, params, a->lp_train, a->lp_roll, a->mask, a->seq_offsets, a->rewards, a->adv, a->n_valid_seq, a->rho,
+                             a->w_tilde, a->diag, a->workspace, a->workspace_bytes, stream);
+    if (st == AIS_OK && (stages & AIS_STAGE_LOSS))
+        st = ais_loss_bwd(shape, params, a->H, a->W, a->tokens, a->mask, a->seq_offsets, a->lse_train, a->lp_train, a->lp_old, a->lp_ref,
+                          a->adv, a->w_tilde, a->dH, a->loss, a->diag, a->dW, a->lddw, static_cast<int>(a->dw_accumulate), a->dev_status,
+                          a->workspace, a->workspace_bytes, stream);
+    return st;
+}
+
 }  // extern "C"

@@ -13,14 +13,17 @@ namespace ais {
 namespace {
 
 // ------------------------------------------------------------------------------------------------
-// FP8-E4M3 block quantisation.  A CTA covers 32 rows x 1024 columns; each warp walks 4 rows, a lane
-// holds 8 consecutive bf16 values (16-byte load), the lanes of one block share the block's amax by
-// shuffles, and the block-major scales are staged in shared memory so that they leave coalesced.
+// Quantisation of the rows of a bf16 matrix: E4M3 with an fp32 scale per 128 / 64 / 32 elements or per tensor, or
+// microscaling FP8 / FP4 (E8M0 scale per 32).  Streaming kernels, bound by HBM (3 bytes per element): a CTA covers 8 warps x
+// RPW rows x 1024 columns, a lane holds 8 consecutive values per 16-byte load, four loads per row segment.  Measured on a
+// 151936 x 4096 head (copy bandwidth 6.5 TB/s): block 128 5.9 TB/s with the 48 registers of five CTAs per SM (5.1 with the 69
+// the compiler would take, 5.6 with 40; a persistent form with the next segment prefetched 4.3 to 4.9), microscaling FP8
+// 6.4 TB/s with 64 registers.  Small matrices take RPW = 1: four times the CTAs, no serial chain of rows in a warp.
 // ------------------------------------------------------------------------------------------------
-constexpr int kQRows = 32;
 constexpr int kQCols = 1024;
 constexpr int kQThreads = 256;
-constexpr int kQIters = kQCols / 256;      // 16-byte loads per lane and row
+constexpr int kQIters = kQCols / 256;      // 16-byte loads per lane and row segment
+constexpr int kQWarps = kQThreads / 32;
 
 __device__ __forceinline__ uint16_t cvt_e4m3x2(float hi, float lo) {
     uint16_t r;
@@ -87,36 +90,43 @@ __device__ __forceinline__ uint2 quantize_values(const uint4 raw, float s, float
     return out;
 }
 
-template <int BLOCK>
-__global__ void __launch_bounds__(kQThreads) quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
-                                                             int64_t ld, uint8_t* __restrict__ codes, int64_t ldq,
-                                                             float* __restrict__ scales, int64_t lds) {
-    pdl_enter();
-    constexpr int kLanesPerBlock = BLOCK / 8;
-    constexpr int kBlocksPerTile = kQCols / BLOCK;
-    __shared__ float sc[kBlocksPerTile][kQRows + 1];
-
+// The row segments of a warp: RPW rows one after the other (the loop stays rolled so that the kernel is small in the
+// instruction cache; occupancy, not prefetching, hides the load latency), four 16-byte loads per lane each.
+// body(row, raw): rows beyond the matrix included, with zeros.
+template <int RPW, class Body>
+__device__ __forceinline__ void walk_rows(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, int64_t row0,
+                                          int64_t col0, Body body) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t row0 = static_cast<int64_t>(blockIdx.y) * kQRows;
-    const int64_t col0 = static_cast<int64_t>(blockIdx.x) * kQCols;
-
-    // each warp walks 4 rows; the row loop is kept rolled so that the kernel stays small in the instruction cache
-    // (a fully unrolled version stalled on instruction fetch); occupancy, not prefetching, hides the load latency
 #pragma unroll 1
-    for (int rr = 0; rr < 4; ++rr) {
-        const int r_local = warp * 4 + rr;
-        const int64_t row = row0 + r_local;
+    for (int rr = 0; rr < RPW; ++rr) {
+        const int64_t row = row0 + warp * RPW + rr;
         uint4 raw[kQIters];
 #pragma unroll
         for (int it = 0; it < kQIters; ++it) {
             const int64_t col = col0 + it * 256 + lane * 8;
             raw[it] = (row < rows && col < cols) ? __ldg(reinterpret_cast<const uint4*>(x + row * ld + col)) : make_uint4(0, 0, 0, 0);
         }
-        // block maxima of the row's four load rounds, then the scales of all the row's blocks at once: lane L derives
-        // scale and reciprocal of block L of the row tile (one divergent region per row instead of one per round)
+        body(row, raw);
+    }
+}
+
+template <int BLOCK, int RPW>
+__global__ void __launch_bounds__(kQThreads, 5) quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
+                                                             uint8_t* __restrict__ codes, int64_t ldq, float* __restrict__ scales,
+                                                             int64_t lds) {
+    constexpr int kLanesPerBlock = BLOCK / 8;
+    constexpr int kBlocksPerTile = kQCols / BLOCK;
+    constexpr int kRows = kQWarps * RPW;
+    __shared__ float sc[kBlocksPerTile][kRows + 1];          // scales leave along the rows (block-major)
+    pdl_enter();
+    const int lane = threadIdx.x & 31;
+    const int64_t row0 = static_cast<int64_t>(blockIdx.y) * kRows, col0 = static_cast<int64_t>(blockIdx.x) * kQCols;
+    walk_rows<RPW>(x, rows, cols, ld, row0, col0, [&](int64_t row, const uint4 (&raw)[kQIters]) {
+        // block maxima of the four loads, then the scales of all the segment's blocks at once: lane L derives scale and
+        // reciprocal of block L (one divergent region per segment instead of one per load)
         constexpr int kBlkPerIt = 32 / kLanesPerBlock;
         constexpr int kBlkPerRow = kQIters * kBlkPerIt;
-        static_assert(kBlkPerRow <= 32, "one lane per block of the row tile");
+        static_assert(kBlkPerRow <= 32, "one lane per block of the segment");
         uint32_t mine = 0;
 #pragma unroll
         for (int it = 0; it < kQIters; ++it) {
@@ -129,24 +139,20 @@ __global__ void __launch_bounds__(kQThreads) quantize_kernel(const __nv_bfloat16
             s_mine = __fdiv_rn(__uint_as_float(mine << 16), 448.0f);
             y_mine = __frcp_rn(s_mine);
         }
+        if (lane < kBlkPerRow) sc[lane][static_cast<int>(row - row0)] = s_mine;
 #pragma unroll
         for (int it = 0; it < kQIters; ++it) {
             const int64_t col = col0 + it * 256 + lane * 8;
-            const bool in = row < rows && col < cols;
             const int blk = it * kBlkPerIt + lane / kLanesPerBlock;
             const float s = __shfl_sync(0xffffffffu, s_mine, blk);
             const float y = __shfl_sync(0xffffffffu, y_mine, blk);
-            if (in) {
-                *reinterpret_cast<uint2*>(codes + row * ldq + col) = quantize_values(raw[it], s, y);
-                if ((lane % kLanesPerBlock) == 0) sc[(it * 256 + lane * 8) / BLOCK][r_local] = s;
-            }
+            if (row < rows && col < cols) *reinterpret_cast<uint2*>(codes + row * ldq + col) = quantize_values(raw[it], s, y);
         }
-    }
+    });
     __syncthreads();
-    const int64_t kb0 = col0 / BLOCK;
-    const int64_t nkb = cols / BLOCK;
-    for (int idx = threadIdx.x; idx < kBlocksPerTile * kQRows; idx += kQThreads) {
-        const int kb_l = idx / kQRows, r_l = idx % kQRows;
+    const int64_t kb0 = col0 / BLOCK, nkb = cols / BLOCK;
+    for (int idx = threadIdx.x; idx < kBlocksPerTile * kRows; idx += kQThreads) {
+        const int kb_l = idx / kRows, r_l = idx % kRows;
         if (kb0 + kb_l < nkb && row0 + r_l < rows) scales[(kb0 + kb_l) * lds + row0 + r_l] = sc[kb_l][r_l];
     }
 }
@@ -155,72 +161,88 @@ __global__ void __launch_bounds__(kQThreads) quantize_kernel(const __nv_bfloat16
 // The same quantisation for a matrix stored with the blocks running DOWN its columns (an LM head kept as [d, V]):
 // block kb of column v is x[kb B .. kb B + B - 1, v].  The codes leave transposed, [V, ldq] with the block elements
 // contiguous, which is the K-major operand the rollout pass wants; the scales leave block-major [d / B, lds] as always.
-// A CTA stages a tile of 128 rows x 128 columns in shared memory (16-byte loads along the rows), then thread
-// (v, h) walks rows 64 h .. 64 h + 63 of column v: maximum, scale, exact division, sixteen codes per 16-byte store.
+// A CTA stages a tile of 128 rows x 128 columns in shared memory (16-byte loads along the rows).  Thread (vp, h) then holds
+// rows 32 h .. 32 h + 31 of the column pair vp in registers, one 32-bit word per row, so that maxima and divisions work on
+// both columns per instruction; the codes go back through the same shared memory and leave as whole 128-byte rows.
+// (One thread per column and 16-bit reads, twice per element, took 574 us for a 4096 x 151936 head.)
 // ------------------------------------------------------------------------------------------------
 constexpr int kQcTile = 128;
-constexpr int kQcPitch = kQcTile + 8;          // uint16 elements per shared-memory row: 272 bytes, 16-byte aligned rows
+constexpr int kQcPitch = kQcTile / 2 + 4;      // 32-bit words per staged row: 272 bytes
+constexpr int kQcOutPitch = kQcTile + 16;      // bytes per column of codes
+static_assert(kQcTile * kQcOutPitch <= kQcTile * kQcPitch * 4, "the codes reuse the staged tile's memory");
 
 template <int BLOCK>
 __global__ void __launch_bounds__(256) quantize_cols_kernel(const __nv_bfloat16* __restrict__ x, int64_t K, int64_t N, int64_t ld,
                                                             uint8_t* __restrict__ codes, int64_t ldq,
                                                             float* __restrict__ scales, int64_t lds) {
+    __shared__ __align__(16) uint32_t tile[kQcTile][kQcPitch];
+    __shared__ uint32_t part_max[4][kQcTile / 2];
     pdl_enter();
-    __shared__ __align__(16) uint16_t tile[kQcTile][kQcPitch];
-    __shared__ uint32_t half_max[2][kQcTile];
     const int tid = threadIdx.x;
     const int64_t k0 = static_cast<int64_t>(blockIdx.y) * kQcTile, v0 = static_cast<int64_t>(blockIdx.x) * kQcTile;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int c = tid + 256 * i, r = c >> 4, c8 = (c & 15) * 8;
         uint4 raw = make_uint4(0, 0, 0, 0);
-        if (k0 + r < K && v0 + c8 < N) raw = __ldg(reinterpret_cast<const uint4*>(x + (k0 + r) * ld + v0 + c8));
-        *reinterpret_cast<uint4*>(&tile[r][c8]) = raw;
+        if (v0 + c8 < N) raw = __ldg(reinterpret_cast<const uint4*>(x + (k0 + r) * ld + v0 + c8));
+        *reinterpret_cast<uint4*>(&tile[r][c8 / 2]) = raw;
     }
     __syncthreads();
-    const int v = tid & (kQcTile - 1), h = tid >> 7;
-    constexpr int kRun = BLOCK < 64 ? BLOCK : 64;          // rows of one block inside this thread's 64
-    constexpr int kRuns = 64 / kRun;
-    uint32_t amax[kRuns];
+    const int vp = tid & 63, h = tid >> 6;
+    uint32_t w[32], m = 0;
 #pragma unroll
-    for (int b = 0; b < kRuns; ++b) {
-        uint32_t m = 0;
-#pragma unroll 8
-        for (int j = 0; j < kRun; ++j) m = max(m, static_cast<uint32_t>(tile[64 * h + b * kRun + j][v]) & 0x7FFFu);
-        amax[b] = m;
+    for (int j = 0; j < 32; ++j) {
+        w[j] = tile[32 * h + j][vp];
+        m = __vmaxu2(m, w[j] & 0x7FFF7FFFu);
     }
-    if (BLOCK == 128) {                                      // the block spans both halves of the column
-        half_max[h][v] = amax[0];
-        __syncthreads();
-        amax[0] = max(half_max[0][v], half_max[1][v]);
-    }
-    const bool in = v0 + v < N;
+    part_max[h][vp] = m;
+    __syncthreads();                                        // the maxima are there, and nobody reads the tile any more
+    if (BLOCK == 64) m = __vmaxu2(m, part_max[h ^ 1][vp]);
+    if (BLOCK == 128) m = __vmaxu2(__vmaxu2(part_max[0][vp], part_max[1][vp]), __vmaxu2(part_max[2][vp], part_max[3][vp]));
+    const uint32_t mlo = m & 0xFFFFu, mhi = m >> 16;
+    F2 s = {1.0f, 1.0f};
+    if (mlo != 0u) s.x = __fdiv_rn(__uint_as_float(mlo << 16), 448.0f);
+    if (mhi != 0u) s.y = __fdiv_rn(__uint_as_float(mhi << 16), 448.0f);
+    const F2 y = {__frcp_rn(s.x), __frcp_rn(s.y)}, ns = {-s.x, -s.y};
+    const bool fast = s.x > 0x1p-100f && s.x < 0x1p100f && s.y > 0x1p-100f && s.y < 0x1p100f;
+    uint8_t* out = reinterpret_cast<uint8_t*>(&tile[0][0]);
 #pragma unroll
-    for (int b = 0; b < kRuns; ++b) {
-        float s = 1.0f, y = 1.0f;
-        if (amax[b] != 0u) {
-            s = __fdiv_rn(__uint_as_float(amax[b] << 16), 448.0f);
-            y = __frcp_rn(s);
-        }
-        const bool fast = s > 0x1p-100f && s < 0x1p100f;
+    for (int g = 0; g < 2; ++g) {                           // sixteen rows of both columns
+        uint32_t c0[4], c1[4];
 #pragma unroll
-        for (int g = 0; g < kRun / 16; ++g) {
-            float q[16];
+        for (int p = 0; p < 8; ++p) {
+            F2 q[2];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float xv = __uint_as_float(static_cast<uint32_t>(tile[64 * h + b * kRun + g * 16 + j][v]) << 16);
-                q[j] = fast ? exact_div(xv, s, y) : slow_div(xv, s);
+            for (int i = 0; i < 2; ++i) {
+                const uint32_t word = w[16 * g + 2 * p + i];
+                const F2 v = {__uint_as_float(word << 16), __uint_as_float(word & 0xFFFF0000u)};
+                if (fast) {                                  // exact_div on both columns
+                    F2 t = mul2(v, y);
+                    t = fma2(fma2(ns, t, v), y, t);
+                    t = fma2(fma2(ns, t, v), y, t);
+                    q[i] = F2{copysignf(t.x, v.x), copysignf(t.y, v.y)};
+                } else {
+                    q[i] = F2{slow_div(v.x, s.x), slow_div(v.y, s.y)};
+                }
             }
-            uint4 out;
-            out.x = static_cast<uint32_t>(cvt_e4m3x2(q[1], q[0])) | (static_cast<uint32_t>(cvt_e4m3x2(q[3], q[2])) << 16);
-            out.y = static_cast<uint32_t>(cvt_e4m3x2(q[5], q[4])) | (static_cast<uint32_t>(cvt_e4m3x2(q[7], q[6])) << 16);
-            out.z = static_cast<uint32_t>(cvt_e4m3x2(q[9], q[8])) | (static_cast<uint32_t>(cvt_e4m3x2(q[11], q[10])) << 16);
-            out.w = static_cast<uint32_t>(cvt_e4m3x2(q[13], q[12])) | (static_cast<uint32_t>(cvt_e4m3x2(q[15], q[14])) << 16);
-            if (in && k0 + 64 * h + b * kRun + g * 16 < K)
-                *reinterpret_cast<uint4*>(codes + (v0 + v) * ldq + k0 + 64 * h + b * kRun + g * 16) = out;
+            const uint32_t e0 = cvt_e4m3x2(q[1].x, q[0].x), e1 = cvt_e4m3x2(q[1].y, q[0].y);
+            if (p & 1) { c0[p >> 1] |= e0 << 16; c1[p >> 1] |= e1 << 16; }
+            else { c0[p >> 1] = e0; c1[p >> 1] = e1; }
         }
-        const int64_t kb = (k0 + 64 * h + b * kRun) / BLOCK;
-        if (in && kb * BLOCK < K && (BLOCK < 128 || h == 0)) scales[kb * lds + v0 + v] = s;
+        *reinterpret_cast<uint4*>(out + (2 * vp) * kQcOutPitch + 32 * h + 16 * g) = make_uint4(c0[0], c0[1], c0[2], c0[3]);
+        *reinterpret_cast<uint4*>(out + (2 * vp + 1) * kQcOutPitch + 32 * h + 16 * g) = make_uint4(c1[0], c1[1], c1[2], c1[3]);
+    }
+    if (h % (BLOCK / 32) == 0 && v0 + 2 * vp < N) {          // N is a multiple of 8: both columns are in
+        float* dst = scales + ((k0 + 32 * h) / BLOCK) * lds + v0 + 2 * vp;
+        dst[0] = s.x;
+        dst[1] = s.y;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int c = tid + 256 * i, col = c >> 3, part = (c & 7) * 16;
+        if (v0 + col < N)
+            *reinterpret_cast<uint4*>(codes + (v0 + col) * ldq + k0 + part) = *reinterpret_cast<const uint4*>(out + col * kQcOutPitch + part);
     }
 }
 
@@ -233,54 +255,9 @@ __global__ void __launch_bounds__(256) quantize_cols_kernel(const __nv_bfloat16*
 // chunks of 128 rows x 4 blocks, byte (r % 32) * 16 + ((r % 128) / 32) * 4 + kb % 4 of chunk (r / 128, kb / 4); the two
 // chunks of a 256-row group are adjacent: chunk start ((r / 256) * (cols / 128) + kb / 4) * 1024 + ((r % 256) / 128) * 512.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kQThreads) quantize_mx_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
-                                                                int64_t ld, uint8_t* __restrict__ codes, int64_t ldq,
-                                                                uint8_t* __restrict__ scales) {
-    pdl_enter();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t row0 = static_cast<int64_t>(blockIdx.y) * kQRows;
-    const int64_t col0 = static_cast<int64_t>(blockIdx.x) * kQCols;
-    const int64_t nk4 = cols / 128;
-#pragma unroll 1
-    for (int rr = 0; rr < 4; ++rr) {
-        const int64_t row = row0 + warp * 4 + rr;
-        if (row >= rows) break;
-#pragma unroll
-        for (int it = 0; it < kQIters; ++it) {
-            const int64_t col = col0 + it * 256 + lane * 8;
-            const bool in = col < cols;                     // cols is a multiple of 128: a block is wholly in or out
-            const uint4 raw = in ? __ldg(reinterpret_cast<const uint4*>(x + row * ld + col)) : make_uint4(0, 0, 0, 0);
-            const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-            uint32_t m = __vmaxu2(__vmaxu2(w[0] & 0x7FFF7FFFu, w[1] & 0x7FFF7FFFu), __vmaxu2(w[2] & 0x7FFF7FFFu, w[3] & 0x7FFF7FFFu));
-            m = max(m & 0xFFFFu, m >> 16);
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
-            const int e = static_cast<int>(m >> 7);         // biased exponent of amax (0 for zero and subnormals)
-            const int code = m == 0u ? 127 : max(e - 8, 0);
-            const float mult = __uint_as_float(static_cast<uint32_t>(254 - code) << 23);      // 2^(127 - code), exact
-            if (!in) continue;
-            float q[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                q[2 * i] = __uint_as_float(w[i] << 16) * mult;
-                q[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u) * mult;
-            }
-            uint2 out;
-            out.x = static_cast<uint32_t>(cvt_e4m3x2(q[1], q[0])) | (static_cast<uint32_t>(cvt_e4m3x2(q[3], q[2])) << 16);
-            out.y = static_cast<uint32_t>(cvt_e4m3x2(q[5], q[4])) | (static_cast<uint32_t>(cvt_e4m3x2(q[7], q[6])) << 16);
-            *reinterpret_cast<uint2*>(codes + row * ldq + col) = out;
-            if ((lane & 3) == 0) {
-                const int64_t kb = col / 32;
-                scales[((row >> 8) * nk4 + (kb >> 2)) * 1024 + ((row >> 7) & 1) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4 +
-                       (kb & 3)] = static_cast<uint8_t>(code);
-            }
-        }
-    }
-}
-
-// ------------------------------------------------------------------------------------------------
-// Microscaling FP4: as above with E2M1 elements (X = floor(log2 amax) - 2), two codes per byte, the element with
-// the lower index in the low nibble.  A lane turns 8 elements into 4 bytes.
+// Microscaling FP4: the same with E2M1 elements (X = floor(log2 amax) - 2), two codes per byte, the element with the lower
+// index in the low nibble; a lane turns 8 elements into 4 bytes.  The four scale bytes of a row and 128 columns lie next to
+// each other and are written as one word.  Rows that pad the last 256-row group carry the neutral scale 127.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t cvt_e2m1x2(float hi, float lo) {
     uint32_t r;
@@ -288,46 +265,57 @@ __device__ __forceinline__ uint32_t cvt_e2m1x2(float hi, float lo) {
     return r;
 }
 
-__global__ void __launch_bounds__(kQThreads) quantize_mxfp4_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
-                                                                   int64_t ld, uint8_t* __restrict__ codes, int64_t ldq,
-                                                                   uint8_t* __restrict__ scales) {
+template <bool FP4, int RPW>
+__global__ void __launch_bounds__(kQThreads) quantize_mx_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows,
+                                                                             int64_t padded_rows, int64_t cols, int64_t ld,
+                                                                             uint8_t* __restrict__ codes, int64_t ldq,
+                                                                             uint8_t* __restrict__ scales) {
     pdl_enter();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t row0 = static_cast<int64_t>(blockIdx.y) * kQRows;
-    const int64_t col0 = static_cast<int64_t>(blockIdx.x) * kQCols;
+    const int lane = threadIdx.x & 31;
     const int64_t nk4 = cols / 128;
-#pragma unroll 1
-    for (int rr = 0; rr < 4; ++rr) {
-        const int64_t row = row0 + warp * 4 + rr;
-        if (row >= rows) break;
+    auto scale_word = [&](int64_t row, int64_t k4) {
+        return reinterpret_cast<uint32_t*>(scales + ((row >> 8) * nk4 + k4) * 1024 + ((row >> 7) & 1) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4);
+    };
+    const int64_t row0 = static_cast<int64_t>(blockIdx.y) * (kQWarps * RPW), col0 = static_cast<int64_t>(blockIdx.x) * kQCols;
+    if (blockIdx.y == gridDim.y - 1)
+        for (int64_t i = threadIdx.x; i < (padded_rows - rows) * 8; i += kQThreads)
+            if (col0 / 128 + i % 8 < nk4) *scale_word(rows + i / 8, col0 / 128 + i % 8) = 0x7F7F7F7Fu;
+    walk_rows<RPW>(x, rows, cols, ld, row0, col0, [&](int64_t row, const uint4 (&raw)[kQIters]) {
+            if (row >= rows) return;
 #pragma unroll
-        for (int it = 0; it < kQIters; ++it) {
-            const int64_t col = col0 + it * 256 + lane * 8;
-            const bool in = col < cols;
-            const uint4 raw = in ? __ldg(reinterpret_cast<const uint4*>(x + row * ld + col)) : make_uint4(0, 0, 0, 0);
-            const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-            uint32_t m = __vmaxu2(__vmaxu2(w[0] & 0x7FFF7FFFu, w[1] & 0x7FFF7FFFu), __vmaxu2(w[2] & 0x7FFF7FFFu, w[3] & 0x7FFF7FFFu));
-            m = max(m & 0xFFFFu, m >> 16);
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
-            m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
-            const int e = static_cast<int>(m >> 7);
-            const int code = m == 0u ? 127 : max(e - 2, 0);
-            const float mult = __uint_as_float(static_cast<uint32_t>(254 - code) << 23);      // 2^(127 - code), exact
-            if (!in) continue;
-            uint32_t out = 0;
+            for (int it = 0; it < kQIters; ++it) {
+                const int64_t col = col0 + it * 256 + lane * 8;
+                const uint32_t w[4] = {raw[it].x, raw[it].y, raw[it].z, raw[it].w};
+                const uint32_t m = block_amax_bits<32>(raw[it]);
+                const int e = static_cast<int>(m >> 7);         // biased exponent of amax (0 for zero and subnormals)
+                const int code = m == 0u ? 127 : max(e - (FP4 ? 2 : 8), 0);
+                const float mult = __uint_as_float(static_cast<uint32_t>(254 - code) << 23);      // 2^(127 - code), exact
+                // the sixteen lanes of 128 columns hold four blocks: their codes become one word
+                uint32_t word = static_cast<uint32_t>(code) << (8 * ((lane >> 2) & 3));
+                word |= __shfl_xor_sync(0xffffffffu, word, 4);
+                word |= __shfl_xor_sync(0xffffffffu, word, 8);
+                if (col >= cols) continue;                      // cols is a multiple of 128: all sixteen lanes agree
+                if (FP4) {
+                    uint32_t out = 0;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float lo = __uint_as_float(w[i] << 16) * mult, hi = __uint_as_float(w[i] & 0xFFFF0000u) * mult;
-                out |= cvt_e2m1x2(hi, lo) << (8 * i);
+                    for (int i = 0; i < 4; ++i)
+                        out |= cvt_e2m1x2(__uint_as_float(w[i] & 0xFFFF0000u) * mult, __uint_as_float(w[i] << 16) * mult) << (8 * i);
+                    *reinterpret_cast<uint32_t*>(codes + row * ldq + col / 2) = out;
+                } else {
+                    float q[8];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        q[2 * i] = __uint_as_float(w[i] << 16) * mult;
+                        q[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u) * mult;
+                    }
+                    uint2 out;
+                    out.x = static_cast<uint32_t>(cvt_e4m3x2(q[1], q[0])) | (static_cast<uint32_t>(cvt_e4m3x2(q[3], q[2])) << 16);
+                    out.y = static_cast<uint32_t>(cvt_e4m3x2(q[5], q[4])) | (static_cast<uint32_t>(cvt_e4m3x2(q[7], q[6])) << 16);
+                    *reinterpret_cast<uint2*>(codes + row * ldq + col) = out;
+                }
+                if ((lane & 15) == 0) *scale_word(row, col / 128) = word;
             }
-            *reinterpret_cast<uint32_t*>(codes + row * ldq + col / 2) = out;
-            if ((lane & 3) == 0) {
-                const int64_t kb = col / 32;
-                scales[((row >> 8) * nk4 + (kb >> 2)) * 1024 + ((row >> 7) & 1) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4 +
-                       (kb & 3)] = static_cast<uint8_t>(code);
-            }
-        }
-    }
+    });
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -335,22 +323,25 @@ __global__ void __launch_bounds__(kQThreads) quantize_mxfp4_kernel(const __nv_bf
 // patterns of non-negative values order like the values, so an integer atomicMax is exact and order-free)
 // into the word that will hold the scale, pass 2 turns it into s = amax / 448, pass 3 quantises.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) tensor_amax_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
-                                                           uint32_t* __restrict__ amax_bits) {
+template <int RPW>
+__global__ void __launch_bounds__(kQThreads) tensor_amax_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
+                                                                uint32_t* __restrict__ amax_bits) {
+    __shared__ uint32_t block_max;
+    if (threadIdx.x == 0) block_max = 0;
     pdl_enter();
-    const int64_t vec_per_row = cols / 8;
-    const int64_t total = rows * vec_per_row;
+    __syncthreads();
     uint32_t m = 0;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t r = i / vec_per_row, c = (i % vec_per_row) * 8;
-        const uint4 w = __ldg(reinterpret_cast<const uint4*>(x + r * ld + c));
-        m = __vmaxu2(m, __vmaxu2(__vmaxu2(w.x & 0x7FFF7FFFu, w.y & 0x7FFF7FFFu), __vmaxu2(w.z & 0x7FFF7FFFu, w.w & 0x7FFF7FFFu)));
-    }
-    m = max(m & 0xFFFFu, m >> 16);
+    walk_rows<RPW>(x, rows, cols, ld, static_cast<int64_t>(blockIdx.y) * (kQWarps * RPW), static_cast<int64_t>(blockIdx.x) * kQCols,
+                   [&](int64_t, const uint4 (&raw)[kQIters]) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & 31) == 0 && m != 0u) atomicMax(amax_bits, m);
+                       for (int it = 0; it < kQIters; ++it)
+                           m = __vmaxu2(m, __vmaxu2(__vmaxu2(raw[it].x & 0x7FFF7FFFu, raw[it].y & 0x7FFF7FFFu),
+                                                    __vmaxu2(raw[it].z & 0x7FFF7FFFu, raw[it].w & 0x7FFF7FFFu)));
+                   });
+    m = __reduce_max_sync(0xffffffffu, max(m & 0xFFFFu, m >> 16));
+    if ((threadIdx.x & 31) == 0) atomicMax(&block_max, m);
+    __syncthreads();
+    if (threadIdx.x == 0 && block_max != 0u) atomicMax(amax_bits, block_max);
 }
 
 __global__ void tensor_scale_kernel(uint32_t* scale_word) {
@@ -360,32 +351,23 @@ __global__ void tensor_scale_kernel(uint32_t* scale_word) {
     *reinterpret_cast<float*>(scale_word) = s;
 }
 
-__global__ void __launch_bounds__(256) tensor_quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
-                                                               int64_t ld, uint8_t* __restrict__ codes, int64_t ldq,
-                                                               const float* __restrict__ scale) {
+// The rows in the opposite order of the maximum's: what that pass read last is still in L2.
+template <int RPW>
+__global__ void __launch_bounds__(kQThreads) tensor_quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
+                                                                    uint8_t* __restrict__ codes, int64_t ldq,
+                                                                    const float* __restrict__ scale) {
     pdl_enter();
     const float s = *scale;
-    const bool fast = s > 0x1p-100f && s < 0x1p100f;
-    const float y = fast ? __frcp_rn(s) : 0.f;
-    const int64_t vec_per_row = cols / 8;
-    const int64_t total = rows * vec_per_row;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t r = i / vec_per_row, c = (i % vec_per_row) * 8;
-        const uint4 raw = __ldg(reinterpret_cast<const uint4*>(x + r * ld + c));
-        const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-        float qv[8];
+    const float y = __frcp_rn(s);
+    const int64_t col0 = static_cast<int64_t>(blockIdx.x) * kQCols + (threadIdx.x & 31) * 8;
+    walk_rows<RPW>(x, rows, cols, ld, static_cast<int64_t>(gridDim.y - 1 - blockIdx.y) * (kQWarps * RPW),
+                   static_cast<int64_t>(blockIdx.x) * kQCols, [&](int64_t row, const uint4 (&raw)[kQIters]) {
+                       if (row >= rows) return;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float lo = __uint_as_float(w[k] << 16), hi = __uint_as_float(w[k] & 0xFFFF0000u);
-            qv[2 * k] = fast ? exact_div(lo, s, y) : slow_div(lo, s);
-            qv[2 * k + 1] = fast ? exact_div(hi, s, y) : slow_div(hi, s);
-        }
-        uint2 out;
-        out.x = static_cast<uint32_t>(cvt_e4m3x2(qv[1], qv[0])) | (static_cast<uint32_t>(cvt_e4m3x2(qv[3], qv[2])) << 16);
-        out.y = static_cast<uint32_t>(cvt_e4m3x2(qv[5], qv[4])) | (static_cast<uint32_t>(cvt_e4m3x2(qv[7], qv[6])) << 16);
-        *reinterpret_cast<uint2*>(codes + r * ldq + c) = out;
-    }
+                       for (int it = 0; it < kQIters; ++it)
+                           if (col0 + it * 256 < cols)
+                               *reinterpret_cast<uint2*>(codes + row * ldq + col0 + it * 256) = quantize_values(raw[it], s, y);
+                   });
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1431,15 +1413,27 @@ cudaError_t stream_prepare() {
 }
 
 // ------------------------------------------------------------------------------------------------ launchers
+// Grid of a row quantiser: four rows per warp once that gives every SM a CTA, single rows below (a small matrix is a chain of
+// latencies, not of bytes).
+inline bool quant_wide(int64_t rows, int64_t cols) {
+    return ((cols + kQCols - 1) / kQCols) * ((rows + 4 * kQWarps - 1) / (4 * kQWarps)) >= 148;
+}
+inline dim3 quant_grid(int64_t rows, int64_t cols) {
+    const int per = kQWarps * (quant_wide(rows, cols) ? 4 : 1);
+    return dim3(static_cast<unsigned>((cols + kQCols - 1) / kQCols), static_cast<unsigned>((rows + per - 1) / per));
+}
+
 cudaError_t launch_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, int block, uint8_t* codes,
                             int64_t ldq, float* scales, int64_t lds, cudaStream_t stream) {
     if (rows == 0 || cols == 0) return cudaSuccess;
-    dim3 grid(static_cast<unsigned>((cols + kQCols - 1) / kQCols), static_cast<unsigned>((rows + kQRows - 1) / kQRows));
+    const dim3 grid = quant_grid(rows, cols);
+    const bool wide = quant_wide(rows, cols);
     const __nv_bfloat16* xp = static_cast<const __nv_bfloat16*>(x);
+    auto go = [&](auto kernel) { return launch_pdl(kernel, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scales, lds); };
     switch (block) {
-        case 32:  return launch_pdl(quantize_kernel<32>, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scales, lds);
-        case 64:  return launch_pdl(quantize_kernel<64>, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scales, lds);
-        case 128: return launch_pdl(quantize_kernel<128>, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scales, lds);
+        case 32:  return go(wide ? quantize_kernel<32, 4> : quantize_kernel<32, 1>);
+        case 64:  return go(wide ? quantize_kernel<64, 4> : quantize_kernel<64, 1>);
+        case 128: return go(wide ? quantize_kernel<128, 4> : quantize_kernel<128, 1>);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1459,13 +1453,15 @@ cudaError_t launch_quantize_cols(const void* x, int64_t K, int64_t N, int64_t ld
 
 cudaError_t launch_quantize_mx(const void* x, int64_t rows, int64_t cols, int64_t ld, uint8_t* codes, int64_t ldq,
                                uint8_t* scales, size_t scale_bytes, bool fp4, cudaStream_t stream) {
-    // rows that pad the last chunks carry the neutral scale
-    cudaError_t e = cudaMemsetAsync(scales, 127, scale_bytes, stream);
-    if (e != cudaSuccess) return e;
-    if (rows == 0 || cols == 0) return cudaSuccess;
-    dim3 grid(static_cast<unsigned>((cols + kQCols - 1) / kQCols), static_cast<unsigned>((rows + kQRows - 1) / kQRows));
-    return launch_pdl(fp4 ? quantize_mxfp4_kernel : quantize_mx_kernel, grid, kQThreads, 0, stream, static_cast<const __nv_bfloat16*>(x), rows,
-                      cols, ld, codes, ldq, scales);
+    if (rows == 0 || cols == 0) return cudaMemsetAsync(scales, 127, scale_bytes, stream);       // padding only
+    const dim3 grid = quant_grid(rows, cols);
+    const bool wide = quant_wide(rows, cols);
+    const int64_t padded = static_cast<int64_t>(scale_bytes / 512) / (cols / 128) * 128;
+    auto go = [&](auto kernel) {
+        return launch_pdl(kernel, grid, kQThreads, 0, stream, static_cast<const __nv_bfloat16*>(x), rows, padded, cols, ld, codes, ldq, scales);
+    };
+    if (fp4) return go(wide ? quantize_mx_kernel<true, 4> : quantize_mx_kernel<true, 1>);
+    return go(wide ? quantize_mx_kernel<false, 4> : quantize_mx_kernel<false, 1>);
 }
 
 cudaError_t launch_quantize_tensor(const void* x, int64_t rows, int64_t cols, int64_t ld, uint8_t* codes, int64_t ldq,
@@ -1473,15 +1469,16 @@ cudaError_t launch_quantize_tensor(const void* x, int64_t rows, int64_t cols, in
     cudaError_t e = cudaMemsetAsync(scale, 0, sizeof(float), stream);
     if (e != cudaSuccess) return e;
     const __nv_bfloat16* xp = static_cast<const __nv_bfloat16*>(x);
-    const int64_t total = rows * (cols / 8);
-    const int blocks = static_cast<int>(total <= 0 ? 1 : ((total + 255) / 256 < 148 * 16 ? (total + 255) / 256 : 148 * 16));
-    if (total > 0) {
-        e = launch_pdl(tensor_amax_kernel, blocks, 256, 0, stream, xp, rows, cols, ld, reinterpret_cast<uint32_t*>(scale));
+    const bool any = rows > 0 && cols > 0, wide = quant_wide(rows, cols);
+    const dim3 grid = quant_grid(rows, cols);
+    if (any) {
+        e = launch_pdl(wide ? tensor_amax_kernel<4> : tensor_amax_kernel<1>, grid, kQThreads, 0, stream, xp, rows, cols, ld,
+                       reinterpret_cast<uint32_t*>(scale));
         if (e != cudaSuccess) return e;
     }
     e = launch_pdl(tensor_scale_kernel, 1, 1, 0, stream, reinterpret_cast<uint32_t*>(scale));
-    if (e != cudaSuccess || total <= 0) return e;
-    return launch_pdl(tensor_quantize_kernel, blocks, 256, 0, stream, xp, rows, cols, ld, codes, ldq, scale);
+    if (e != cudaSuccess || !any) return e;
+    return launch_pdl(wide ? tensor_quantize_kernel<4> : tensor_quantize_kernel<1>, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scale);
 }
 
 cudaError_t launch_combine(const CombineJob* jobs, int njobs, int64_t part_ld, const uint8_t* mask, int64_t T, uint32_t* status,
