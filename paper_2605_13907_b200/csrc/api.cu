@@ -145,6 +145,16 @@ int check_params(const ais_params* p) {
     return AIS_OK;
 }
 
+int check_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, int block, const uint8_t* codes, int64_t ldq,
+                   const float* scales, int64_t lds) {
+    if (!x || !codes || !scales) return AIS_ERR_NULL;
+    if (rows < 0 || cols < 0 || (block != 32 && block != 64 && block != 128)) return AIS_ERR_SHAPE;
+    if (cols % block != 0 || ld < cols || ldq < cols || lds < rows) return AIS_ERR_SHAPE;
+    if (ld % 8 != 0 || ldq % 8 != 0 || !aligned(x, 16) || !aligned(codes, 8) || !aligned(scales, 4)) return AIS_ERR_ALIGN;
+    if (rows > (int64_t(1) << 31) - 1024) return AIS_ERR_SHAPE;
+    return AIS_OK;
+}
+
 // vocab_chunk asks for its own ranges (at most 64); otherwise the pass gets what plan_ranges finds best.
 int pick_nsplit(const ais_shape* s, const ais_params* p, int64_t row_tiles, int n_col_tiles) {
     if (p->vocab_chunk <= 0) return plan_ranges(row_tiles, n_col_tiles, s->d, kMaxRanges);
@@ -248,6 +258,17 @@ bool arm_pace(LmheadArgs& a, uint8_t* ws, const Layout& L, int tiles_per_unit, i
     return a.pace != nullptr;
 }
 
+// What ais_step lets neighbouring stages share: a batch of a few hundred rows is a chain of launches, and these are the ones
+// whose work fits into a neighbour's.
+struct Fuse {
+    const QuantJob* quant = nullptr;     // log-probs: quantise these first, in the opening launch
+    int nquant = 0;
+    const AdvJob* adv = nullptr;         // log-probs: advantages in the merging launch; diagnostics: they are there already
+    bool rectify_later = false;          // diagnostics: the loss forms rho and w_tilde
+    const RectifyJob* rectify = nullptr; // loss: form them
+    const int32_t* counts = nullptr;     // loss: valid rows per sequence are there already, and so is its cleared ticket
+};
+
 }  // namespace
 
 extern "C" {
@@ -305,16 +326,13 @@ size_t ais_workspace_bytes(const ais_shape* shape, const ais_params* params) {
 
 int ais_quantize_fp8(const void* x, int64_t rows, int64_t cols, int64_t ld, int block, uint8_t* codes, int64_t ldq,
                      float* scales, int64_t lds, void* stream) {
-    if (!x || !codes || !scales) return AIS_ERR_NULL;
-    if (rows < 0 || cols < 0 || (block != 32 && block != 64 && block != 128)) return AIS_ERR_SHAPE;
-    if (cols % block != 0 || ld < cols || ldq < cols || lds < rows) return AIS_ERR_SHAPE;
-    if (ld % 8 != 0 || ldq % 8 != 0 || !aligned(x, 16) || !aligned(codes, 8) || !aligned(scales, 4)) return AIS_ERR_ALIGN;
-    if (rows > (int64_t(1) << 31) - 1024) return AIS_ERR_SHAPE;
-    int st = device_setup(nullptr);
+    int st = check_quantize(x, rows, cols, ld, block, codes, ldq, scales, lds);
     if (st != AIS_OK) return st;
-    return launch_quantize(x, rows, cols, ld, block, codes, ldq, scales, lds, static_cast<cudaStream_t>(stream)) == cudaSuccess
-               ? AIS_OK
-               : AIS_ERR_DEVICE;
+    st = device_setup(nullptr);
+    if (st != AIS_OK) return st;
+    if (rows == 0 || cols == 0) return AIS_OK;
+    const QuantJob job = {x, rows, ld, codes, ldq, scales, lds};
+    return launch_quantize(&job, 1, cols, block, nullptr, static_cast<cudaStream_t>(stream)) == cudaSuccess ? AIS_OK : AIS_ERR_DEVICE;
 }
 
 int ais_quantize_fp8_cols(const void* x, int64_t rows, int64_t cols, int64_t ld, int block, uint8_t* codes, int64_t ldq,
@@ -378,10 +396,10 @@ int ais_quantize_mxfp4(const void* x, int64_t rows, int64_t cols, int64_t ld, ui
                : AIS_ERR_DEVICE;
 }
 
-int ais_logprob_fwd(const ais_shape* shape, const ais_params* params, const void* H, const void* W, const uint8_t* qH,
-                    const void* sH_, int64_t ldsH, const uint8_t* qW, const void* sW_, int64_t ldsW, const int32_t* tokens,
-                    const uint8_t* mask, float* lp_train, float* lse_train, float* lp_roll, float* lse_roll,
-                    uint32_t* dev_status, void* workspace, size_t workspace_bytes, void* stream) {
+static int logprob_fwd(const ais_shape* shape, const ais_params* params, const void* H, const void* W, const uint8_t* qH,
+                       const void* sH_, int64_t ldsH, const uint8_t* qW, const void* sW_, int64_t ldsW, const int32_t* tokens,
+                       const uint8_t* mask, float* lp_train, float* lse_train, float* lp_roll, float* lse_roll,
+                       uint32_t* dev_status, void* workspace, size_t workspace_bytes, void* stream, const Fuse& fuse) {
     int st = check_shape(shape);
     if (st != AIS_OK) return st;
     st = check_params(params);
@@ -492,18 +510,27 @@ int ais_logprob_fwd(const ais_shape* shape, const ais_params* params, const void
                 make_tmap(&p.tmSB, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sW, V, nkb, ldsW * 4, kPairCols, sg, CU_TENSOR_MAP_SWIZZLE_NONE);
     }
     if (!maps) return AIS_ERR_DEVICE;
-    if (launch_tile_flags_mask(mask, T, ws + L.off_flags, paced ? ws + L.off_pace : nullptr, 2 * kPaceRingBytes, s) != cudaSuccess)
+    const FlagsJob flags = {mask, T, ws + L.off_flags, paced ? ws + L.off_pace : nullptr, 2 * kPaceRingBytes};
+    if ((fuse.nquant > 0 ? launch_quantize(fuse.quant, fuse.nquant, d, shape->fp8_block, &flags, s) : launch_flags(flags, s)) != cudaSuccess)
         return AIS_ERR_DEVICE;
     for (int i = 0; i < n; ++i)
         if (launch_lmhead(pass[i].mode, pass[i].tmA, pass[i].tmB, pass[i].tmSA, pass[i].tmSB, pass[i].a, pass[i].ctas, s) != cudaSuccess)
             return AIS_ERR_DEVICE;
-    if (launch_combine(jobs, n, L.t_ld, mask, T, dev_status, s) != cudaSuccess) return AIS_ERR_DEVICE;
+    if (launch_combine(jobs, n, L.t_ld, mask, T, dev_status, fuse.adv, s) != cudaSuccess) return AIS_ERR_DEVICE;
     return AIS_OK;
 }
 
-int ais_diagnostics(const ais_shape* shape, const ais_params* params, const float* lp_train, const float* lp_roll,
-                    const uint8_t* mask, const int32_t* seq_offsets, const float* rewards, float* adv, int32_t* n_valid_seq,
-                    float* rho, float* w_tilde, ais_diag* diag, void* workspace, size_t workspace_bytes, void* stream) {
+int ais_logprob_fwd(const ais_shape* shape, const ais_params* params, const void* H, const void* W, const uint8_t* qH,
+                    const void* sH, int64_t ldsH, const uint8_t* qW, const void* sW, int64_t ldsW, const int32_t* tokens,
+                    const uint8_t* mask, float* lp_train, float* lse_train, float* lp_roll, float* lse_roll,
+                    uint32_t* dev_status, void* workspace, size_t workspace_bytes, void* stream) {
+    return logprob_fwd(shape, params, H, W, qH, sH, ldsH, qW, sW, ldsW, tokens, mask, lp_train, lse_train, lp_roll, lse_roll,
+                       dev_status, workspace, workspace_bytes, stream, Fuse());
+}
+
+static int diagnostics(const ais_shape* shape, const ais_params* params, const float* lp_train, const float* lp_roll,
+                       const uint8_t* mask, const int32_t* seq_offsets, const float* rewards, float* adv, int32_t* n_valid_seq,
+                       float* rho, float* w_tilde, ais_diag* diag, void* workspace, size_t workspace_bytes, void* stream, const Fuse& fuse) {
     int st = check_shape(shape);
     if (st != AIS_OK) return st;
     st = check_params(params);
@@ -518,13 +545,22 @@ int ais_diagnostics(const ais_shape* shape, const ais_params* params, const floa
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int S = shape->P * shape->G;
-    if (launch_advantages(rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, reinterpret_cast<uint32_t*>(ws + L.off_ticket), s) != cudaSuccess)
+    uint32_t* tickets = reinterpret_cast<uint32_t*>(ws + L.off_ticket);
+    if (!fuse.adv &&
+        launch_advantages({rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, tickets}, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
-    if (launch_diag(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag),
-                    reinterpret_cast<uint32_t*>(ws + L.off_ticket), n_valid_seq, seq_level ? reinterpret_cast<float*>(ws + L.off_seqw) : nullptr, rho, w_tilde, diag, s) !=
-        cudaSuccess)
+    if (launch_diag(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag), tickets,
+                    n_valid_seq, seq_level ? reinterpret_cast<float*>(ws + L.off_seqw) : nullptr, rho, fuse.rectify_later ? nullptr : w_tilde,
+                    diag, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     return AIS_OK;
+}
+
+int ais_diagnostics(const ais_shape* shape, const ais_params* params, const float* lp_train, const float* lp_roll,
+                    const uint8_t* mask, const int32_t* seq_offsets, const float* rewards, float* adv, int32_t* n_valid_seq,
+                    float* rho, float* w_tilde, ais_diag* diag, void* workspace, size_t workspace_bytes, void* stream) {
+    return diagnostics(shape, params, lp_train, lp_roll, mask, seq_offsets, rewards, adv, n_valid_seq, rho, w_tilde, diag, workspace,
+                       workspace_bytes, stream, Fuse());
 }
 
 int ais_diag_moments(const ais_shape* shape, const ais_params* params, const float* lp_train, const float* lp_roll,
@@ -544,10 +580,11 @@ int ais_diag_moments(const ais_shape* shape, const ais_params* params, const flo
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int S = shape->P * shape->G;
-    if (launch_advantages(rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, reinterpret_cast<uint32_t*>(ws + L.off_ticket), s) != cudaSuccess)
+    uint32_t* tickets = reinterpret_cast<uint32_t*>(ws + L.off_ticket);
+    if (launch_advantages({rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, tickets}, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     if (launch_moments(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag),
-                       reinterpret_cast<uint32_t*>(ws + L.off_ticket), n_valid_seq, params->seq_level_weights != 0 ? seq_logw : nullptr, moments, s) != cudaSuccess)
+                       tickets, n_valid_seq, params->seq_level_weights != 0 ? seq_logw : nullptr, moments, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     return AIS_OK;
 }
@@ -571,11 +608,11 @@ int ais_diag_finalize(const ais_shape* shape, const ais_params* params, const do
     return AIS_OK;
 }
 
-int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H, const void* W, const int32_t* tokens,
-                 const uint8_t* mask, const int32_t* seq_offsets, const float* lse_train, const float* lp_train,
-                 const float* lp_old, const float* lp_ref, const float* adv, const float* w_tilde, void* dH, float* loss,
-                 ais_diag* diag, float* dW, int64_t lddw, int dw_accumulate,
-                 uint32_t* dev_status, void* workspace, size_t workspace_bytes, void* stream) {
+static int loss_bwd(const ais_shape* shape, const ais_params* params, const void* H, const void* W, const int32_t* tokens,
+                    const uint8_t* mask, const int32_t* seq_offsets, const float* lse_train, const float* lp_train,
+                    const float* lp_old, const float* lp_ref, const float* adv, const float* w_tilde, void* dH, float* loss,
+                    ais_diag* diag, float* dW, int64_t lddw, int dw_accumulate,
+                    uint32_t* dev_status, void* workspace, size_t workspace_bytes, void* stream, const Fuse& fuse) {
     int st = check_shape(shape);
     if (st != AIS_OK) return st;
     st = check_params(params);
@@ -595,14 +632,18 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int S = shape->P * shape->G;
     float* coef = reinterpret_cast<float*>(ws + L.off_coef);
-    int32_t* nseq = reinterpret_cast<int32_t*>(ws + L.off_nseq);
-    uint32_t* ticket = reinterpret_cast<uint32_t*>(ws + L.off_ticket);
-    if (launch_seq_counts(mask, seq_offsets, S, nseq, ticket, s) != cudaSuccess) return AIS_ERR_DEVICE;
+    const int32_t* nseq = fuse.counts;
+    uint32_t* ticket = reinterpret_cast<uint32_t*>(ws + L.off_ticket) + 1;
+    if (!nseq) {
+        int32_t* own = reinterpret_cast<int32_t*>(ws + L.off_nseq);
+        if (launch_seq_counts(mask, seq_offsets, S, own, ticket, s) != cudaSuccess) return AIS_ERR_DEVICE;
+        nseq = own;
+    }
     const int P_norm = shape->P_total > 0 ? shape->P_total : shape->P;
     // row tiles whose gradient factors are all zero (masked rows, zero advantage) are skipped by the recompute and dH passes
     if (launch_loss_coef(lp_train, lp_old, lp_ref, params->beta_kl, mask, seq_offsets, adv, w_tilde, nseq, shape->T, S, P_norm * shape->G,
                          params->clip_eps, reinterpret_cast<double*>(ws + L.off_diag), ticket, coef, ws + L.off_flags, ws + L.off_pace,
-                         2 * kPaceRingBytes, loss, diag, lse_train, s) != cudaSuccess)
+                         2 * kPaceRingBytes, loss, diag, lse_train, fuse.rectify, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     if (shape->T == 0) return AIS_OK;
 
@@ -723,32 +764,70 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H
     return AIS_OK;
 }
 
+int ais_loss_bwd(const ais_shape* shape, const ais_params* params, const void* H, const void* W, const int32_t* tokens,
+                 const uint8_t* mask, const int32_t* seq_offsets, const float* lse_train, const float* lp_train,
+                 const float* lp_old, const float* lp_ref, const float* adv, const float* w_tilde, void* dH, float* loss,
+                 ais_diag* diag, float* dW, int64_t lddw, int dw_accumulate,
+                 uint32_t* dev_status, void* workspace, size_t workspace_bytes, void* stream) {
+    return loss_bwd(shape, params, H, W, tokens, mask, seq_offsets, lse_train, lp_train, lp_old, lp_ref, adv, w_tilde, dH, loss, diag, dW,
+                    lddw, dw_accumulate, dev_status, workspace, workspace_bytes, stream, Fuse());
+}
+
 int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_args* a, uint32_t stages, void* stream) {
     int st = check_shape(shape);
+    if (st != AIS_OK) return st;
+    st = check_params(params);
     if (st != AIS_OK) return st;
     if (!a) return AIS_ERR_NULL;
     const int block = shape->fp8_block;
     const bool dv = shape->w_layout == AIS_W_DV, fp4 = block == AIS_FP4_MX32;
-    auto quantize = [&](const void* x, int64_t rows, int64_t ld, uint8_t* codes, int64_t ldq, void* scales, int64_t lds) {
+    const bool logprob = (stages & AIS_STAGE_LOGPROB) != 0, diag = (stages & AIS_STAGE_DIAGNOSE) != 0, loss = (stages & AIS_STAGE_LOSS) != 0;
+    const Layout L = make_layout(shape, params);
+    Fuse fuse;
+    // codes with fp32 block scales come from the launch that opens the log-probs ([d, V] heads have a quantiser of their own)
+    QuantJob quant[2];
+    auto quantize = [&](const void* x, int64_t rows, int64_t ld, uint8_t* codes, int64_t ldq, void* scales, int64_t lds) -> int {
         if (fp4) return ais_quantize_mxfp4(x, rows, shape->d, ld, codes, ldq / 2, static_cast<uint8_t*>(scales), stream);
         if (block == AIS_FP8_MX32) return ais_quantize_mxfp8(x, rows, shape->d, ld, codes, ldq, static_cast<uint8_t*>(scales), stream);
         if (block == 0) return ais_quantize_fp8_tensor(x, rows, shape->d, ld, codes, ldq, static_cast<float*>(scales), stream);
-        return ais_quantize_fp8(x, rows, shape->d, ld, block, codes, ldq, static_cast<float*>(scales), lds, stream);
+        float* sc = static_cast<float*>(scales);
+        if (!logprob || shape->T == 0) return ais_quantize_fp8(x, rows, shape->d, ld, block, codes, ldq, sc, lds, stream);
+        const int bad = check_quantize(x, rows, shape->d, ld, block, codes, ldq, sc, lds);
+        if (bad == AIS_OK) quant[fuse.nquant++] = {x, rows, ld, codes, ldq, sc, lds};
+        return bad;
     };
     if ((stages & AIS_STAGE_QUANTIZE_H) && shape->T > 0) st = quantize(a->H, shape->T, shape->ldh, a->qH, shape->ldh, a->sH, a->ldsH);
     if (st == AIS_OK && (stages & AIS_STAGE_QUANTIZE_W))
         st = dv ? ais_quantize_fp8_cols(a->W, shape->d, shape->V, shape->ldw, block, a->qW, shape->d, static_cast<float*>(a->sW), a->ldsW, stream)
                 : quantize(a->W, shape->V, shape->ldw, a->qW, shape->ldw, a->sW, a->ldsW);
-    if (st == AIS_OK && (stages & AIS_STAGE_LOGPROB))
-        st = ais_logprob_fwd(shape, params, a->H, a->W, a->qH, a->sH, a->ldsH, a->qW, a->sW, a->ldsW, a->tokens, a->mask, a->lp_train,
-                             a->lse_train, a->lp_roll, a->lse_roll, a->dev_status, a->workspace, a->workspace_bytes, stream);
-    if (st == AIS_OK && (stages & AIS_STAGE_DIAGNOSE))
-        st = ais_diagnostics(shape, params, a->lp_train, a->lp_roll, a->mask, a->seq_offsets, a->rewards, a->adv, a->n_valid_seq, a->rho,
-                             a->w_tilde, a->diag, a->workspace, a->workspace_bytes, stream);
-    if (st == AIS_OK && (stages & AIS_STAGE_LOSS))
-        st = ais_loss_bwd(shape, params, a->H, a->W, a->tokens, a->mask, a->seq_offsets, a->lse_train, a->lp_train, a->lp_old, a->lp_ref,
-                          a->adv, a->w_tilde, a->dH, a->loss, a->diag, a->dW, a->lddw, static_cast<int>(a->dw_accumulate), a->dev_status,
-                          a->workspace, a->workspace_bytes, stream);
+    if (st != AIS_OK) return st;
+    fuse.quant = quant;
+    const int S = shape->P * shape->G;
+    const AdvJob adv = {a->rewards, S, shape->G, params->adv_std_norm, params->eps, a->adv, a->n_valid_seq,
+                        reinterpret_cast<uint32_t*>(static_cast<uint8_t*>(a->workspace) + L.off_ticket)};
+    RectifyJob rectify;
+    // the diagnostics' advantages ride on the merge of the log-probs when there is one
+    if (logprob && diag && a->rewards && a->adv && a->lp_train && a->lp_roll && shape->T > 0) fuse.adv = &adv;
+    if (logprob)
+        st = logprob_fwd(shape, params, a->H, a->W, a->qH, a->sH, a->ldsH, a->qW, a->sW, a->ldsW, a->tokens, a->mask, a->lp_train,
+                         a->lse_train, a->lp_roll, a->lse_roll, a->dev_status, a->workspace, a->workspace_bytes, stream, fuse);
+    if (st != AIS_OK) return st;
+    if (diag) {
+        // the loss takes the counts from here and forms rho and w_tilde; the diagnostics' advantages have cleared its ticket
+        if (loss && a->n_valid_seq && shape->T > 0) {
+            fuse.counts = a->n_valid_seq;
+            fuse.rectify_later = true;
+            rectify = {a->lp_roll, params->C, a->diag, a->rho, a->w_tilde,
+                       params->seq_level_weights ? reinterpret_cast<const float*>(static_cast<uint8_t*>(a->workspace) + L.off_seqw) : nullptr};
+            fuse.rectify = &rectify;
+        }
+        st = diagnostics(shape, params, a->lp_train, a->lp_roll, a->mask, a->seq_offsets, a->rewards, a->adv, a->n_valid_seq, a->rho,
+                         a->w_tilde, a->diag, a->workspace, a->workspace_bytes, stream, fuse);
+    }
+    if (st == AIS_OK && loss)
+        st = loss_bwd(shape, params, a->H, a->W, a->tokens, a->mask, a->seq_offsets, a->lse_train, a->lp_train, a->lp_old, a->lp_ref,
+                      a->adv, a->w_tilde, a->dH, a->loss, a->diag, a->dW, a->lddw, static_cast<int>(a->dw_accumulate), a->dev_status,
+                      a->workspace, a->workspace_bytes, stream, fuse);
     return st;
 }
 

@@ -31,18 +31,6 @@ __device__ __forceinline__ uint16_t cvt_e4m3x2(float hi, float lo) {
     return r;
 }
 
-// Correctly rounded x / s from the correctly rounded reciprocal y = RN(1/s): two residual corrections with
-// fused multiply-adds; the first makes the quotient faithful, and a faithful quotient corrected once more with
-// the exact residual is the round-to-nearest quotient (Markstein's division theorem).  |x / s| <= 448 here, so
-// nothing overflows; a quotient that underflows encodes to zero either way; the sign of x is restored
-// explicitly because a zero residual sum would turn -0 into +0.
-__device__ __forceinline__ float exact_div(float x, float s, float y) {
-    float q = x * y;
-    q = __fmaf_rn(__fmaf_rn(-s, q, x), y, q);
-    q = __fmaf_rn(__fmaf_rn(-s, q, x), y, q);
-    return copysignf(q, x);
-}
-
 // IEEE division kept out of line: it is only reached for scales outside [2^-100, 2^100] and would otherwise
 // be inlined eight times into every copy of the hot loop.
 __device__ __noinline__ float slow_div(float x, float s) { return __fdiv_rn(x, s); }
@@ -69,7 +57,12 @@ __device__ __forceinline__ uint2 quantize_values(const uint4 raw, float s, float
         v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
     if (s > 0x1p-100f && s < 0x1p100f) {
-        // exact_div on two values per instruction (the packed fp32 forms round each half like the scalar ones)
+        // Correctly rounded x / s from the correctly rounded reciprocal y = RN(1/s), two values per instruction (the packed
+        // fp32 forms round each half like the scalar ones): two residual corrections with fused multiply-adds; the first
+        // makes the quotient faithful, and a faithful quotient corrected once more with the exact residual is the
+        // round-to-nearest quotient (Markstein's division theorem).  |x / s| <= 448 here, so nothing overflows; a quotient
+        // that underflows encodes to zero either way; the sign of x is restored explicitly because a zero residual sum would
+        // turn -0 into +0.
         const F2 ys = {y, y}, ns = {-s, -s};
 #pragma unroll
         for (int i = 0; i < 8; i += 2) {
@@ -110,17 +103,53 @@ __device__ __forceinline__ void walk_rows(const __nv_bfloat16* __restrict__ x, i
     }
 }
 
+// FlagsJob by blocks of 256 threads: one warp per 128-row tile.
+constexpr int kFlagTiles = kQThreads / 32;
+inline unsigned flag_blocks(const FlagsJob& f) { return static_cast<unsigned>(((f.T + 127) / 128 + kFlagTiles - 1) / kFlagTiles); }
+__device__ __forceinline__ void run_flags(const FlagsJob& f, unsigned block, unsigned nblocks) {
+    const int64_t tile = static_cast<int64_t>(block) * kFlagTiles + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (tile * 128 < f.T) {
+        bool any = false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int64_t t = tile * 128 + 32 * j + lane;
+            any |= t < f.T && f.mask[t] != 0;
+        }
+        any = __any_sync(0xffffffffu, any);
+        if (lane == 0) f.flags[tile] = any ? 1 : 0;
+    }
+    if (f.clear)
+        for (int64_t k = static_cast<int64_t>(block) * kQThreads + threadIdx.x; k < f.clear_bytes / 16; k += static_cast<int64_t>(nblocks) * kQThreads)
+            static_cast<uint4*>(f.clear)[k] = make_uint4(0, 0, 0, 0);
+}
+__global__ void __launch_bounds__(kQThreads) flags_kernel(const FlagsJob f) {
+    pdl_enter();
+    run_flags(f, blockIdx.x, gridDim.x);
+}
+
+// Blocks 0 .. n0 - 1 work on job0, the next n1 on job1, the rest on the flags.
 template <int BLOCK, int RPW>
-__global__ void __launch_bounds__(kQThreads, 5) quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
-                                                             uint8_t* __restrict__ codes, int64_t ldq, float* __restrict__ scales,
-                                                             int64_t lds) {
+__global__ void __launch_bounds__(kQThreads, 5) quantize_kernel(const QuantJob job0, const QuantJob job1, unsigned n0, unsigned n1,
+                                                                unsigned tiles_x, int64_t cols, const FlagsJob flags) {
     constexpr int kLanesPerBlock = BLOCK / 8;
     constexpr int kBlocksPerTile = kQCols / BLOCK;
     constexpr int kRows = kQWarps * RPW;
     __shared__ float sc[kBlocksPerTile][kRows + 1];          // scales leave along the rows (block-major)
     pdl_enter();
+    if (blockIdx.x >= n0 + n1) {
+        run_flags(flags, blockIdx.x - n0 - n1, gridDim.x - n0 - n1);
+        return;
+    }
+    const bool second = blockIdx.x >= n0;
+    const QuantJob& job = second ? job1 : job0;
+    const unsigned tile = second ? blockIdx.x - n0 : blockIdx.x;
+    const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(job.x);
+    const int64_t rows = job.rows, ld = job.ld, ldq = job.ldq, lds = job.lds;
+    uint8_t* codes = job.codes;
+    float* scales = job.scales;
     const int lane = threadIdx.x & 31;
-    const int64_t row0 = static_cast<int64_t>(blockIdx.y) * kRows, col0 = static_cast<int64_t>(blockIdx.x) * kQCols;
+    const int64_t row0 = static_cast<int64_t>(tile / tiles_x) * kRows, col0 = static_cast<int64_t>(tile % tiles_x) * kQCols;
     walk_rows<RPW>(x, rows, cols, ld, row0, col0, [&](int64_t row, const uint4 (&raw)[kQIters]) {
         // block maxima of the four loads, then the scales of all the segment's blocks at once: lane L derives scale and
         // reciprocal of block L (one divergent region per segment instead of one per load)
@@ -216,7 +245,7 @@ __global__ void __launch_bounds__(256) quantize_cols_kernel(const __nv_bfloat16*
             for (int i = 0; i < 2; ++i) {
                 const uint32_t word = w[16 * g + 2 * p + i];
                 const F2 v = {__uint_as_float(word << 16), __uint_as_float(word & 0xFFFF0000u)};
-                if (fast) {                                  // exact_div on both columns
+                if (fast) {                                  // as in quantize_values, both columns at once
                     F2 t = mul2(v, y);
                     t = fma2(fma2(ns, t, v), y, t);
                     t = fma2(fma2(ns, t, v), y, t);
@@ -370,6 +399,26 @@ __global__ void __launch_bounds__(kQThreads) tensor_quantize_kernel(const __nv_b
                    });
 }
 
+// Group-relative advantage of sequence s (Eq. grpo_adv), and what AdvJob clears for it.
+__device__ __forceinline__ void run_advantage(const AdvJob& j, int s) {
+    if (s == 0) j.tickets[0] = j.tickets[1] = 0;
+    if (j.zero_counts) j.zero_counts[s] = 0;
+    const int g0 = (s / j.G) * j.G;
+    double mean = 0.0;
+    for (int k = 0; k < j.G; ++k) mean += static_cast<double>(j.rewards[g0 + k]);
+    mean /= j.G;
+    double a = static_cast<double>(j.rewards[s]) - mean;
+    if (j.std_norm) {
+        double var = 0.0;
+        for (int k = 0; k < j.G; ++k) {
+            const double dlt = static_cast<double>(j.rewards[g0 + k]) - mean;
+            var += dlt * dlt;
+        }
+        a /= (sqrt(var / j.G) + static_cast<double>(j.eps));
+    }
+    j.adv[s] = static_cast<float>(a);
+}
+
 // ------------------------------------------------------------------------------------------------
 // Merge of the per-split (max, sum-exp, target-logit) triples into lp and lse.
 // ------------------------------------------------------------------------------------------------
@@ -377,9 +426,14 @@ __global__ void __launch_bounds__(kQThreads) tensor_quantize_kernel(const __nv_b
 // (max, sum) goes through shared memory to warp 0, in warp order.  With one thread per row the up to 296 parts of a small
 // batch were a chain of dependent loads.
 constexpr int kCombWarps = 8;
-__global__ void __launch_bounds__(32 * kCombWarps) combine_kernel(const CombineJob j0, const CombineJob j1, int64_t part_ld,
-                                                                  const uint8_t* __restrict__ mask, int64_t T, uint32_t* status) {
+__global__ void __launch_bounds__(32 * kCombWarps) combine_kernel(const CombineJob j0, const CombineJob j1, int njobs, int64_t part_ld,
+                                                                  const uint8_t* __restrict__ mask, int64_t T, uint32_t* status,
+                                                                  const AdvJob adv) {
     pdl_enter();
+    if (static_cast<int>(blockIdx.y) == njobs) {                 // the row of blocks behind the merges
+        for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < adv.S; s += gridDim.x * blockDim.x) run_advantage(adv, s);
+        return;
+    }
     const CombineJob job = blockIdx.y == 0 ? j0 : j1;
     const float *part_m = job.part_m, *part_s = job.part_s, *part_z = job.part_z;
     const int nparts = job.nparts;
@@ -526,30 +580,10 @@ __global__ void __launch_bounds__(256) seq_count_kernel(const uint8_t* __restric
     if (lane == 0) n_valid_seq[s] = cnt;
 }
 
-// Group-relative advantages (Eq. grpo_adv): one thread per sequence.  With `zero_counts` the per-sequence row
-// counts are cleared for the moments kernel, which adds them up.
-__global__ void adv_kernel(const float* __restrict__ rewards, int S, int G, int adv_std_norm, float eps, float* __restrict__ adv,
-                           int32_t* __restrict__ zero_counts, uint32_t* __restrict__ ticket) {
+__global__ void adv_kernel(const AdvJob job) {
     pdl_enter();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= S) return;
-    if (zero_counts) zero_counts[s] = 0;
-    if (!rewards || !adv) return;
-    const int g0 = (s / G) * G;
-    double mean = 0.0;
-    for (int j = 0; j < G; ++j) mean += static_cast<double>(rewards[g0 + j]);
-    mean /= G;
-    double a = static_cast<double>(rewards[s]) - mean;
-    if (adv_std_norm) {
-        double var = 0.0;
-        for (int j = 0; j < G; ++j) {
-            const double dlt = static_cast<double>(rewards[g0 + j]) - mean;
-            var += dlt * dlt;
-        }
-        a /= (sqrt(var / G) + static_cast<double>(eps));
-    }
-    adv[s] = static_cast<float>(a);
+    if (s < job.S) run_advantage(job, s);
 }
 
 // Sequence-level importance weight (Eq. is-weight): log w(x) = sum over the valid rows of a sequence of
@@ -566,20 +600,6 @@ __global__ void __launch_bounds__(256) seq_logw_kernel(const float* __restrict__
         if (mask[t]) acc += static_cast<double>(lp_train[t]) - static_cast<double>(lp_roll[t]);
     acc = warp_sum(acc);
     if (lane == 0) seq_logw[s] = static_cast<float>(acc);
-}
-
-// One byte per 128-row tile: does any row of the tile need computing?  (mask != 0 / gradient factor != 0)  The same launch
-// clears the pacing rings of the passes that follow (`clear`: uint4 words, may be NULL).
-template <typename T>
-__global__ void tile_flags_kernel(const T* __restrict__ pred, int64_t n, uint8_t* __restrict__ flags, uint4* __restrict__ clear,
-                                  int nclear) {
-    pdl_enter();
-    const int64_t tile = blockIdx.x;
-    const int64_t i = tile * 128 + threadIdx.x;
-    const int any = __syncthreads_or(i < n && pred[i] != T(0));
-    if (threadIdx.x == 0) flags[tile] = any ? 1 : 0;
-    if (clear)
-        for (int64_t k = i; k < nclear; k += static_cast<int64_t>(gridDim.x) * 128) clear[k] = make_uint4(0, 0, 0, 0);
 }
 
 __device__ __forceinline__ int seq_of_row(const int32_t* __restrict__ seq_offsets, int S, int64_t t) {
@@ -1212,6 +1232,13 @@ __global__ void moments_reduce_kernel(const double* __restrict__ partials, int n
     if (lane == 0) moments[i] = m;
 }
 
+// Ratio and rectification weight of a valid row; seq_logw: its sequence's log weight (sequence-level variant) or NULL.
+__device__ __forceinline__ void rectify_row(float lt, float lr, float alpha, float C, const float* seq_logw, float& r, float& wt) {
+    r = __expf(lt - lr);
+    const float w = seq_logw ? __expf(*seq_logw) : r;
+    wt = fmaf(alpha, fminf(w, C) - 1.0f, 1.0f);
+}
+
 template <int VEC>
 __global__ void __launch_bounds__(256) rectify_kernel(const float* __restrict__ lp_train, const float* __restrict__ lp_roll,
                                                       const uint8_t* __restrict__ mask, int64_t T, float C,
@@ -1230,12 +1257,7 @@ __global__ void __launch_bounds__(256) rectify_kernel(const float* __restrict__ 
     auto one = [&](float lt, float lr, uint8_t mk, float& r, float& wt, int64_t t) {
         r = 1.0f;
         wt = 1.0f;
-        if (mk) {
-            const float dl = lt - lr;
-            r = __expf(dl);
-            const float w = seq_logw ? __expf(seq_logw[seq_of_row(seq_offsets, S, t)]) : r;      // sequence-level variant
-            wt = fmaf(alpha, fminf(w, C) - 1.0f, 1.0f);
-        }
+        if (mk) rectify_row(lt, lr, alpha, C, seq_logw ? seq_logw + seq_of_row(seq_offsets, S, t) : nullptr, r, wt);
     };
     for (int64_t g = g0; g < ngroups; g += stride) {
         if (g != g0) in = load_group<VEC>(lp_train, lp_roll, mask, g);
@@ -1278,14 +1300,16 @@ struct LossArgs {
     uint32_t* ticket;
     float* loss;
     ais_diag* diag;
+    RectifyJob rectify;    // rectify.w_tilde != NULL: ratios and weights of the rows are formed here and written on the way
 };
 
-template <bool VEC>
+template <bool VEC, bool RECTIFY>
 __global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const LossArgs a) {
     __shared__ double scratch[2][32];
     __shared__ double totals[2];
     pdl_enter();
     const int lane = threadIdx.x & 31;
+    const float alpha = RECTIFY ? static_cast<float>(a.rectify.alpha_of->alpha) : 0.f;
     double J = 0.0, KL = 0.0;
     // one valid row of sequence sq: its share of the objective, of the KL estimate, and its gradient factor
     auto one = [&](int64_t t, int sq, float wtf) -> float {
@@ -1318,20 +1342,40 @@ __global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const LossArgs 
         uint32_t mk = 0;                                          // mask bytes of the four rows
         if (VEC && rows == 4) {
             mk = *reinterpret_cast<const uint32_t*>(a.mask + t0);
-            const float4 w4 = *reinterpret_cast<const float4*>(a.w_tilde + t0);
-            wt[0] = w4.x; wt[1] = w4.y; wt[2] = w4.z; wt[3] = w4.w;
+            if (!RECTIFY) {
+                const float4 w4 = *reinterpret_cast<const float4*>(a.w_tilde + t0);
+                wt[0] = w4.x; wt[1] = w4.y; wt[2] = w4.z; wt[3] = w4.w;
+            }
         } else {
             for (int j = 0; j < rows; ++j) {
                 mk |= static_cast<uint32_t>(a.mask[t0 + j]) << (8 * j);
-                wt[j] = a.w_tilde[t0 + j];
+                if (!RECTIFY) wt[j] = a.w_tilde[t0 + j];
             }
         }
+        float rho[4] = {1.f, 1.f, 1.f, 1.f};
+        if (RECTIFY) wt[0] = wt[1] = wt[2] = wt[3] = 1.f;
         if (mk != 0u) {
             int sq = seq_of_row(a.seq_offsets, a.S, t0);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 while (sq + 1 < a.S && static_cast<int64_t>(a.seq_offsets[sq + 1]) <= t0 + j) ++sq;
-                if ((mk >> (8 * j)) & 0xFFu) c[j] = one(t0 + j, sq, wt[j]);
+                if ((mk >> (8 * j)) & 0xFFu) {
+                    if (RECTIFY)
+                        rectify_row(a.lp_train[t0 + j], a.rectify.lp_roll[t0 + j], alpha, a.rectify.C, a.rectify.seq_logw ? a.rectify.seq_logw + sq : nullptr,
+                                    rho[j], wt[j]);
+                    c[j] = one(t0 + j, sq, wt[j]);
+                }
+            }
+        }
+        if (RECTIFY) {
+            if (VEC && rows == 4) {
+                if (a.rectify.rho) *reinterpret_cast<float4*>(a.rectify.rho + t0) = make_float4(rho[0], rho[1], rho[2], rho[3]);
+                *reinterpret_cast<float4*>(a.rectify.w_tilde + t0) = make_float4(wt[0], wt[1], wt[2], wt[3]);
+            } else {
+                for (int j = 0; j < rows; ++j) {
+                    if (a.rectify.rho) a.rectify.rho[t0 + j] = rho[j];
+                    a.rectify.w_tilde[t0 + j] = wt[j];
+                }
             }
         }
         if (rows == 4) *reinterpret_cast<float4*>(a.coef + t0) = make_float4(c[0], c[1], c[2], c[3]);     // workspace: aligned
@@ -1423,13 +1467,18 @@ inline dim3 quant_grid(int64_t rows, int64_t cols) {
     return dim3(static_cast<unsigned>((cols + kQCols - 1) / kQCols), static_cast<unsigned>((rows + per - 1) / per));
 }
 
-cudaError_t launch_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, int block, uint8_t* codes,
-                            int64_t ldq, float* scales, int64_t lds, cudaStream_t stream) {
-    if (rows == 0 || cols == 0) return cudaSuccess;
-    const dim3 grid = quant_grid(rows, cols);
+cudaError_t launch_quantize(const QuantJob* jobs, int njobs, int64_t cols, int block, const FlagsJob* flags, cudaStream_t stream) {
+    const unsigned tiles_x = static_cast<unsigned>((cols + kQCols - 1) / kQCols);
+    int64_t rows = 0;
+    for (int i = 0; i < njobs; ++i) rows += jobs[i].rows;
     const bool wide = quant_wide(rows, cols);
-    const __nv_bfloat16* xp = static_cast<const __nv_bfloat16*>(x);
-    auto go = [&](auto kernel) { return launch_pdl(kernel, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scales, lds); };
+    const int per = kQWarps * (wide ? 4 : 1);
+    unsigned n[2] = {0, 0};
+    for (int i = 0; i < njobs; ++i) n[i] = tiles_x * static_cast<unsigned>((jobs[i].rows + per - 1) / per);
+    const FlagsJob f = flags ? *flags : FlagsJob{};
+    const unsigned blocks = n[0] + n[1] + (flags ? flag_blocks(f) : 0);
+    if (blocks == 0) return cudaSuccess;
+    auto go = [&](auto kernel) { return launch_pdl(kernel, blocks, kQThreads, 0, stream, jobs[0], jobs[njobs - 1], n[0], n[1], tiles_x, cols, f); };
     switch (block) {
         case 32:  return go(wide ? quantize_kernel<32, 4> : quantize_kernel<32, 1>);
         case 64:  return go(wide ? quantize_kernel<64, 4> : quantize_kernel<64, 1>);
@@ -1482,25 +1531,23 @@ cudaError_t launch_quantize_tensor(const void* x, int64_t rows, int64_t cols, in
 }
 
 cudaError_t launch_combine(const CombineJob* jobs, int njobs, int64_t part_ld, const uint8_t* mask, int64_t T, uint32_t* status,
-                           cudaStream_t stream) {
-    if (T == 0) return cudaSuccess;
-    return launch_pdl(combine_kernel, dim3(static_cast<unsigned>((T + 31) / 32), static_cast<unsigned>(njobs)), 32 * kCombWarps, 0, stream, jobs[0],
-                      jobs[njobs - 1], part_ld, mask, T, status);
+                           const AdvJob* adv, cudaStream_t stream) {
+    if (T == 0) return adv ? launch_advantages(*adv, stream) : cudaSuccess;
+    const dim3 grid(static_cast<unsigned>((T + 31) / 32), static_cast<unsigned>(njobs + (adv ? 1 : 0)));
+    return launch_pdl(combine_kernel, grid, 32 * kCombWarps, 0, stream, jobs[0], jobs[njobs - 1], njobs, part_ld, mask, T, status,
+                      adv ? *adv : AdvJob{});
 }
 
-cudaError_t launch_tile_flags_mask(const uint8_t* mask, int64_t T, uint8_t* flags, void* clear, size_t clear_bytes, cudaStream_t stream) {
-    if (T <= 0) return cudaSuccess;
-    return launch_pdl(tile_flags_kernel<uint8_t>, static_cast<unsigned>((T + 127) / 128), 128, 0, stream, mask, T, flags,
-                      static_cast<uint4*>(clear), static_cast<int>(clear_bytes / 16));
+cudaError_t launch_flags(const FlagsJob& job, cudaStream_t stream) {
+    return job.T > 0 ? launch_pdl(flags_kernel, flag_blocks(job), kQThreads, 0, stream, job) : cudaSuccess;
 }
 
 cudaError_t launch_seq_counts(const uint8_t* mask, const int32_t* seq_offsets, int S, int32_t* n_valid_seq, uint32_t* ticket, cudaStream_t stream) {
     return launch_pdl(seq_count_kernel, (S + 7) / 8, 256, 0, stream, mask, seq_offsets, S, n_valid_seq, ticket);
 }
 
-cudaError_t launch_advantages(const float* rewards, int S, int G, int adv_std_norm, float eps, float* adv, int32_t* zero_counts,
-                              uint32_t* ticket, cudaStream_t stream) {
-    return launch_pdl(adv_kernel, (S + 255) / 256, 256, 0, stream, rewards, S, G, adv_std_norm, eps, adv, zero_counts, ticket);
+cudaError_t launch_advantages(const AdvJob& job, cudaStream_t stream) {
+    return launch_pdl(adv_kernel, (job.S + 255) / 256, 256, 0, stream, job);
 }
 
 cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
@@ -1508,7 +1555,7 @@ cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8
                         int32_t* n_valid_seq, float* seq_logw, float* rho, float* w_tilde, ais_diag* diag, cudaStream_t stream) {
     const DiagFinish fin = {p, diag, nullptr, ticket};
     const cudaError_t e = launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, fin, stream);
-    if (e != cudaSuccess || T == 0) return e;
+    if (e != cudaSuccess || T == 0 || w_tilde == nullptr) return e;
     return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, diag, rho, w_tilde, seq_offsets, S, seq_logw, stream);
 }
 
@@ -1530,7 +1577,8 @@ cudaError_t launch_finalize(const double* moments, const float* lp_train, const 
 cudaError_t launch_loss_coef(const float* lp_train, const float* lp_old, const float* lp_ref, float beta_kl, const uint8_t* mask,
                              const int32_t* seq_offsets, const float* adv, const float* w_tilde, const int32_t* n_valid_seq, int64_t T,
                              int S, int S_norm, float clip_eps, double* partials, uint32_t* ticket, float* coef, uint8_t* tile_flags,
-                             void* clear, size_t clear_bytes, float* loss, ais_diag* diag, const float* lse, cudaStream_t stream) {
+                             void* clear, size_t clear_bytes, float* loss, ais_diag* diag, const float* lse, const RectifyJob* rectify,
+                             cudaStream_t stream) {
     LossArgs a = {};
     a.lp_train = lp_train;
     a.lp_old = lp_old;
@@ -1554,7 +1602,13 @@ cudaError_t launch_loss_coef(const float* lp_train, const float* lp_old, const f
     a.ticket = ticket;
     a.loss = loss;
     a.diag = diag;
-    return launch_pdl(vec4_ok(w_tilde, nullptr, nullptr, nullptr, mask) ? loss_coef_kernel<true> : loss_coef_kernel<false>, reduce_blocks(T, 4 * kDiagThreads),
+    const int blocks = reduce_blocks(T, 4 * kDiagThreads);
+    if (rectify) {
+        a.rectify = *rectify;
+        return launch_pdl(vec4_ok(rectify->w_tilde, rectify->rho, nullptr, nullptr, mask) ? loss_coef_kernel<true, true> : loss_coef_kernel<false, true>,
+                          blocks, kDiagThreads, 0, stream, a);
+    }
+    return launch_pdl(vec4_ok(w_tilde, nullptr, nullptr, nullptr, mask) ? loss_coef_kernel<true, false> : loss_coef_kernel<false, false>, blocks,
                       kDiagThreads, 0, stream, a);
 }
 

@@ -13,11 +13,49 @@ constexpr int kDiagBlocks = 592;      // fixed grid of the batch reductions (kee
 constexpr int kDiagThreads = 256;
 constexpr int kNumMoments = 12;
 
+// One matrix for the row quantiser with fp32 block scales.
+struct QuantJob {
+    const void* x;
+    int64_t rows, ld;
+    uint8_t* codes;
+    int64_t ldq;
+    float* scales;
+    int64_t lds;
+};
+// Opening of a log-prob call: flags[i] = 1 when rows 128 i .. 128 i + 127 contain a row with mask != 0; `clear` (16-byte
+// words, may be NULL) is zeroed on the way.
+struct FlagsJob {
+    const uint8_t* mask;
+    int64_t T;
+    uint8_t* flags;
+    void* clear;
+    int64_t clear_bytes;
+};
+// Group-relative advantages adv[s]; zero_counts [S] (may be NULL) and the two tickets (block counters of the batch
+// reductions) are cleared for the kernels that count into them.
+struct AdvJob {
+    const float* rewards;
+    int32_t S, G, std_norm;
+    float eps;
+    float* adv;
+    int32_t* zero_counts;
+    uint32_t* tickets;
+};
+// The rectification of a batch (rho, w_tilde) as part of the loss kernel.
+struct RectifyJob {
+    const float* lp_roll;
+    float C;
+    const ais_diag* alpha_of;
+    float *rho, *w_tilde;
+    const float* seq_logw;
+};
+
 // Raises the dynamic shared-memory limit of the kernels here that need it (once per device).
 cudaError_t stream_prepare();
 
-cudaError_t launch_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, int block, uint8_t* codes,
-                            int64_t ldq, float* scales, int64_t lds, cudaStream_t stream);
+// Rows quantised with one fp32 scale per `block` elements; one or two matrices (of the same width) and, if not NULL, the
+// opening of the log-prob call that follows, in one launch.
+cudaError_t launch_quantize(const QuantJob* jobs, int njobs, int64_t cols, int block, const FlagsJob* flags, cudaStream_t stream);
 
 // Blocks running down the columns of x [K, ld] (K a multiple of 128): codes transposed [N, ldq], scales [K / block, lds].
 cudaError_t launch_quantize_cols(const void* x, int64_t K, int64_t N, int64_t ld, int block, uint8_t* codes, int64_t ldq,
@@ -39,25 +77,20 @@ struct CombineJob {
     int32_t nparts;
     float *lp, *lse;
 };
-// One or two merges (the passes of one call) in one launch.
+// One or two merges (the passes of one call) in one launch, and, if not NULL, the advantages of the diagnostics that follow.
 cudaError_t launch_combine(const CombineJob* jobs, int njobs, int64_t part_ld, const uint8_t* mask, int64_t T, uint32_t* status,
-                           cudaStream_t stream);
-
-// flags[i] = 1 when rows 128 i .. 128 i + 127 contain a row with mask != 0; clears `clear` (16-byte aligned, may be NULL).
-cudaError_t launch_tile_flags_mask(const uint8_t* mask, int64_t T, uint8_t* flags, void* clear, size_t clear_bytes, cudaStream_t stream);
+                           const AdvJob* adv, cudaStream_t stream);
+cudaError_t launch_flags(const FlagsJob& job, cudaStream_t stream);
 
 // n_valid_seq[s] = valid rows of sequence s; zeroes `ticket` (the block counter of the reduction that follows).
 cudaError_t launch_seq_counts(const uint8_t* mask, const int32_t* seq_offsets, int S, int32_t* n_valid_seq, uint32_t* ticket, cudaStream_t stream);
-// adv[s] (group-relative advantages); zero_counts [S] (may be NULL) is cleared for the moments kernel to count into,
-// `ticket` for it to count its blocks.
-cudaError_t launch_advantages(const float* rewards, int S, int G, int adv_std_norm, float eps, float* adv, int32_t* zero_counts,
-                              uint32_t* ticket, cudaStream_t stream);
+cudaError_t launch_advantages(const AdvJob& job, cudaStream_t stream);
 
 // n_valid_seq (may be NULL) must have been cleared: the moments kernel adds every sequence's valid rows to it.
 cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
                         const float* adv, int64_t T, int S, const ais_params& p, double* partials /*[kDiagBlocks][kNumMoments]*/, uint32_t* ticket,
                         int32_t* n_valid_seq, float* seq_logw /* [S] scratch: non-NULL selects sequence-level weights */,
-                        float* rho, float* w_tilde, ais_diag* diag, cudaStream_t stream);
+                        float* rho, float* w_tilde /* NULL: the loss kernel rectifies */, ais_diag* diag, cudaStream_t stream);
 
 // The two halves of launch_diag: partial moments summed into `moments` [kNumMoments], and everything that follows
 // from a (possibly all-reduced) moment vector.
@@ -75,6 +108,6 @@ cudaError_t launch_loss_coef(const float* lp_train, const float* lp_old, const f
                              const int32_t* seq_offsets, const float* adv, const float* w_tilde, const int32_t* n_valid_seq, int64_t T,
                              int S, int S_norm, float clip_eps, double* partials /*[kDiagBlocks][2]*/, uint32_t* ticket, float* coef,
                              uint8_t* tile_flags, void* clear, size_t clear_bytes, float* loss, ais_diag* diag, const float* lse,
-                             cudaStream_t stream);
+                             const RectifyJob* rectify /* NULL: w_tilde is there already */, cudaStream_t stream);
 
 }  // namespace ais
