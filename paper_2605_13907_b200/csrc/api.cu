@@ -81,10 +81,12 @@ bool make_tmap(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, ui
 // The units of a pass are (row tile, vocabulary range) pairs handed round robin to one persistent CTA per SM, so its time
 // is waves x tiles of the longest range.  Four ranges for everybody left a response of 613 rows (5 row tiles) on 20 of 148
 // SMs (3.2 ms per pass at d = 4096, V = 151936) and ran 79 row tiles as three waves where 2.1 were full.  The number of
-// ranges with the least waves x tiles wins, with a slight handicap for many ranges: the fewer row tiles are in flight, the
-// more often W is read.  From below it is bounded by L2: the hidden rows of the row tiles in flight are read again for
-// every column tile and should take no more than 40 MB of it.
-int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most) {
+// ranges with the least waves x tiles wins, with a handicap for many ranges: the fewer row tiles are in flight, the more
+// often W is read, and in the passes that run into the power cap an idle SM costs less than that (2,500 rows: 7 ranges in one
+// wave 2.44 ms, 22 in three better filled ones 2.75; 58,142 rows at d = 5120: 7 ranges 58.1 ms, 11 61.5).  The FP8 block
+// pass does not reach the cap and takes the balance (11 ranges 48.4 ms, 4 52.3).  From below the number is bounded by L2:
+// the hidden rows of the row tiles in flight are read again for every column tile and should take no more than 40 MB of it.
+int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most, bool pairs) {
     if (row_tiles < 1) row_tiles = 1;
     if (most > col_tiles) most = col_tiles;
     if (most < 1) most = 1;
@@ -93,9 +95,9 @@ int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most) {
     for (int s = 1; s <= most; ++s) {
         int64_t in_flight = kSms / s > 0 ? kSms / s : 1;
         if (in_flight > row_tiles) in_flight = row_tiles;
-        if (in_flight * kBM * d * 2 > (int64_t(40) << 20) && s < most) continue;
+        if (in_flight * 2 * kBM * d > (int64_t(40) << 20) && s < most) continue;
         const int64_t waves = (row_tiles * s + kSms - 1) / kSms;
-        const double cost = static_cast<double>(waves) * ((col_tiles + s - 1) / s) * (1.0 + s / 400.0);
+        const double cost = static_cast<double>(waves) * ((col_tiles + s - 1) / s) * (1.0 + s / (pairs ? 400.0 : 120.0));
         if (best_cost == 0.0 || cost < best_cost) { best = s; best_cost = cost; }
     }
     return best;
@@ -156,8 +158,8 @@ int check_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, int bl
 }
 
 // vocab_chunk asks for its own ranges (at most 64); otherwise the pass gets what plan_ranges finds best.
-int pick_nsplit(const ais_shape* s, const ais_params* p, int64_t row_tiles, int n_col_tiles) {
-    if (p->vocab_chunk <= 0) return plan_ranges(row_tiles, n_col_tiles, s->d, kMaxRanges);
+int pick_nsplit(const ais_shape* s, const ais_params* p, int64_t row_tiles, int n_col_tiles, bool pairs = false) {
+    if (p->vocab_chunk <= 0) return plan_ranges(row_tiles, n_col_tiles, s->d, kMaxRanges, pairs);
     int nsplit = (s->V + p->vocab_chunk - 1) / p->vocab_chunk;
     if (nsplit > 64) nsplit = 64;
     if (nsplit > n_col_tiles) nsplit = n_col_tiles;
@@ -210,7 +212,7 @@ Layout make_layout(const ais_shape* s, const ais_params* p) {
     Layout L;
     L.t_ld = static_cast<int64_t>(align_up(static_cast<size_t>(s->T > 0 ? s->T : 1), 64));
     L.nsplit = pick_nsplit(s, p, (s->T + kBM - 1) / kBM, (s->V + kBN - 1) / kBN);
-    L.nsplit_pair = pick_nsplit(s, p, (s->T + kPairRows - 1) / kPairRows, (s->V + kPairCols - 1) / kPairCols);
+    L.nsplit_pair = pick_nsplit(s, p, (s->T + kPairRows - 1) / kPairRows, (s->V + kPairCols - 1) / kPairCols, true);
     L.nparts = 2 * L.nsplit > kPairParts * L.nsplit_pair ? 2 * L.nsplit : kPairParts * L.nsplit_pair;
     size_t off = 0;
     L.part_bytes = align_up(static_cast<size_t>(L.nparts) * L.t_ld * sizeof(float), 256);

@@ -15,8 +15,8 @@ bool make_tmap(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, ui
                uint64_t stride1_bytes, uint32_t box0, uint32_t box1, CUtensorMapSwizzle swz);
 
 // How many vocabulary ranges a forward or recompute pass over `row_tiles` x `col_tiles` tiles splits each row tile into,
-// at most `most`; `d` is the hidden size.
-int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most);
+// at most `most`; `d` is the hidden size; `pairs`: the FP8 pass with tiles of two row tiles x 128 columns.
+int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most, bool pairs = false);
 
 // Bound of the kernels' device-side waits in clock ticks as set by ais_set_wait_cycles (0 = the kernels' default).
 int64_t wait_cycles();
