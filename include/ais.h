@@ -320,7 +320,10 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params,
  * The stages of a step in one call: what `stages` names, in the order quantise H, quantise W, log-probs, diagnostics, loss
  * and gradients, each exactly as its own entry point above does it (the same arguments under the same names).  For callers
  * that run the same step again and again and fill the struct once: a step of a small batch takes tens of microseconds, and
- * marshalling six argument lists is a good part of that.  Quantises by shape->fp8_block; the codes' row strides are those
+ * marshalling six argument lists is a good part of that.  Neighbouring stages share launches, and with AIS_STAGE_LOGPROB,
+ * AIS_STAGE_DIAGNOSE and AIS_STAGE_LOSS in one call (and no dW) the trainer pass leaves e^z (bf16) in the scratch rows that
+ * the workspace has for the backward pass, so that those rows' logits are not computed again; dH then has the same
+ * precision, but not the same bits, as the stages called one by one.  Quantises by shape->fp8_block; the codes' row strides are those
  * ais_logprob_fwd expects.  Stops at the first stage that returns an error.
  */
 #define AIS_STAGE_QUANTIZE_H 1u

@@ -199,6 +199,7 @@ struct Layout {
     size_t off_pace;                              // two rings of counters that keep the CTAs of a tensor-core launch in step
     size_t off_ticket;                            // block counter of the batch reductions
     size_t off_coef, off_nseq;                    // backward: c_t, valid rows per sequence
+    size_t off_scale, off_redo;                   // backward, exponent form: row factors, row tiles to recompute
     size_t off_seqw;                              // sequence-level variant: log weight per sequence
     size_t off_split;                             // dH: partial tiles of the split units
     int split_slots, ksplit;                      // how many there is room for; ksplit > 0: ranges fixed by the shape alone
@@ -223,6 +224,8 @@ Layout make_layout(const ais_shape* s, const ais_params* p) {
     L.off_diag = off;   off += align_up(static_cast<size_t>(kDiagBlocks) * kNumMoments * sizeof(double), 256);
     L.off_coef = off;   off += align_up(static_cast<size_t>(L.t_ld) * sizeof(float), 256);
     L.off_nseq = off;   off += align_up(static_cast<size_t>(s->P) * s->G * sizeof(int32_t), 256);
+    L.off_scale = off;  off += align_up(static_cast<size_t>(L.t_ld) * sizeof(float), 256);
+    L.off_redo = off;   off += align_up(static_cast<size_t>(L.t_ld / kBM + 2), 256);
     L.off_seqw = off;   off += align_up(static_cast<size_t>(s->P) * s->G * sizeof(float), 256);
     {
         // a batch whose dH tiles do not fill one wave gets its ranges from its size alone, so that the split (and with it
@@ -260,6 +263,13 @@ bool arm_pace(LmheadArgs& a, uint8_t* ws, const Layout& L, int tiles_per_unit, i
     return a.pace != nullptr;
 }
 
+// Rows of backward scratch that the workspace holds: whole row tiles, no more than the batch has.
+int64_t scratch_rows(const Layout& L, int64_t T, size_t workspace_bytes) {
+    const int64_t rows = static_cast<int64_t>((workspace_bytes - L.fixed_bytes) / L.u_row_bytes) / kBM * kBM;
+    const int64_t t_pad = static_cast<int64_t>(align_up(static_cast<size_t>(T), kBM));
+    return rows < t_pad ? rows : t_pad;
+}
+
 // What ais_step lets neighbouring stages share: a batch of a few hundred rows is a chain of launches, and these are the ones
 // whose work fits into a neighbour's.
 struct Fuse {
@@ -268,6 +278,7 @@ struct Fuse {
     const AdvJob* adv = nullptr;         // log-probs: advantages in the merging launch; diagnostics: they are there already
     bool rectify_later = false;          // diagnostics: the loss forms rho and w_tilde
     const RectifyJob* rectify = nullptr; // loss: form them
+    int64_t keep_rows = 0;               // log-probs: leave the exponentials of these rows in the scratch; loss: they are there
     const int32_t* counts = nullptr;     // loss: valid rows per sequence are there already, and so is its cleared ticket
 };
 
@@ -482,7 +493,11 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
     if (do_train) {
         // W [V, d]: K-major boxes of 64 hidden units x 256 vocabulary rows.  W [d, V]: the vocabulary is the contiguous
         // axis, boxes of 64 vocabulary columns x 64 hidden units (four of them per stage)
-        Pass& p = add(dv ? kFwdBf16Dv : kFwdBf16, kBM, kBN, L.nsplit, shape->d / 64, lp_train, lse_train);
+        const bool keep = fuse.keep_rows > 0;
+        Pass& p = add(keep ? (dv ? kFwdKeepDv : kFwdKeep) : dv ? kFwdBf16Dv : kFwdBf16, kBM, kBN, L.nsplit, shape->d / 64, lp_train, lse_train);
+        p.a.U = reinterpret_cast<__nv_bfloat16*>(ws + L.off_u);
+        p.a.ldU = L.ldU;
+        p.a.keep_tiles = static_cast<int32_t>((fuse.keep_rows + kBM - 1) / kBM);
         maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, H, d, T, shape->ldh * 2, 64, kBM, CU_TENSOR_MAP_SWIZZLE_128B) &&
                 (dv ? make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, V, d, shape->ldw * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
                     : make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, d, V, shape->ldw * 2, 64, kBN, CU_TENSOR_MAP_SWIZZLE_128B));
@@ -642,17 +657,17 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
         nseq = own;
     }
     const int P_norm = shape->P_total > 0 ? shape->P_total : shape->P;
+    float* scale = reinterpret_cast<float*>(ws + L.off_scale);
+    const KeepJob keep = {reinterpret_cast<__nv_bfloat16*>(ws + L.off_u), L.ldU, fuse.keep_rows, tokens, shape->V, scale, ws + L.off_redo, ticket + 1};
     // row tiles whose gradient factors are all zero (masked rows, zero advantage) are skipped by the recompute and dH passes
     if (launch_loss_coef(lp_train, lp_old, lp_ref, params->beta_kl, mask, seq_offsets, adv, w_tilde, nseq, shape->T, S, P_norm * shape->G,
                          params->clip_eps, reinterpret_cast<double*>(ws + L.off_diag), ticket, coef, ws + L.off_flags, ws + L.off_pace,
-                         2 * kPaceRingBytes, loss, diag, lse_train, fuse.rectify, s) != cudaSuccess)
+                         2 * kPaceRingBytes, loss, diag, lse_train, fuse.rectify, fuse.keep_rows > 0 ? &keep : nullptr, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     if (shape->T == 0) return AIS_OK;
 
-    // rows of scratch the workspace can hold (whole row tiles)
-    int64_t blk_rows = static_cast<int64_t>((workspace_bytes - L.fixed_bytes) / L.u_row_bytes) / kBM * kBM;
-    const int64_t t_pad = static_cast<int64_t>(align_up(static_cast<size_t>(shape->T), kBM));
-    if (blk_rows > t_pad) blk_rows = t_pad;
+    // the rows go through in passes of what the scratch holds
+    const int64_t blk_rows = scratch_rows(L, shape->T, workspace_bytes);
     __nv_bfloat16* U = reinterpret_cast<__nv_bfloat16*>(ws + L.off_u);
     const uint64_t V = static_cast<uint64_t>(shape->V), d = static_cast<uint64_t>(shape->d);
 
@@ -687,6 +702,8 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
         a.tokens = tokens;
         a.mask = mask;
         a.lse = lse_train;
+        a.lp = lp_train;
+        a.row_scale = fuse.keep_rows > 0 ? scale : nullptr;
         a.U = U;
         a.ldU = L.ldU;
         a.coef = coef;
@@ -695,7 +712,12 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
         a.status = dev_status;
         a.tile_active = ws + L.off_flags;
         a.sgroups = 1;
-        // recompute softmax - onehot into the scratch
+        // recompute softmax - onehot into the scratch; rows that the forward pass left there are only redone where they are
+        // outside the range of the exponent form (a launch that usually finds its gate closed)
+        if (r0 < fuse.keep_rows) {
+            a.tile_active = ws + L.off_redo;
+            a.gate = ticket + 1;
+        }
         a.ncols = shape->V;
         a.n_col_tiles = (shape->V + kBN - 1) / kBN;
         a.nsplit = pick_nsplit(shape, params, a.n_row_tiles, a.n_col_tiles);
@@ -707,6 +729,8 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
         if (launch_lmhead(dv ? kBwdPDv : kBwdP, tmH, tmW_k, tmH, tmW_k, a, ctas, s) != cudaSuccess)
             return AIS_ERR_DEVICE;
         // dH = c (.) (U W)
+        a.tile_active = ws + L.off_flags;
+        a.gate = nullptr;
         a.ncols = shape->d;
         a.n_col_tiles = (shape->d + kBN - 1) / kBN;
         a.n_row_tiles = static_cast<int32_t>((rows + kDhRows - 1) / kDhRows);
@@ -810,6 +834,9 @@ int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_ar
     RectifyJob rectify;
     // the diagnostics' advantages ride on the merge of the log-probs when there is one
     if (logprob && diag && a->rewards && a->adv && a->lp_train && a->lp_roll && shape->T > 0) fuse.adv = &adv;
+    // log-probs and loss in one call: the exponentials of the rows that the scratch holds stay there (dW wants plain form)
+    if (fuse.adv && loss && !a->dW && a->n_valid_seq && a->lse_train && a->dH && a->workspace_bytes >= L.fixed_bytes + static_cast<size_t>(kBM) * L.u_row_bytes)
+        fuse.keep_rows = scratch_rows(L, shape->T, a->workspace_bytes);
     if (logprob)
         st = logprob_fwd(shape, params, a->H, a->W, a->qH, a->sH, a->ldsH, a->qW, a->sW, a->ldsW, a->tokens, a->mask, a->lp_train,
                          a->lse_train, a->lp_roll, a->lse_roll, a->dev_status, a->workspace, a->workspace_bytes, stream, fuse);

@@ -19,6 +19,9 @@ namespace ais {
 
 namespace {
 
+// |reference| (log2 units) up to which the kept exponentials are relative to 0; just above exp_form's largest lse
+constexpr float kKeepRange = 86.0f;
+
 constexpr int threads_of(int mode) { return (mode == kFwdMx || mode == kFwdMx4) ? kMxThreads : kThreads; }
 
 template <int MODE>
@@ -56,6 +59,12 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int num_units = count_units<BASE>(a);
+    constexpr bool KEEP = (MODE == kFwdKeep || MODE == kFwdKeepDv);
+    const bool gated = BASE == kBwdP && a.gate != nullptr;
+    if (gated) {
+        enter_pass(a);
+        if (__ldcg(a.gate) == 0u) return;                 // no row tile needs this pass
+    }
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); mbar_init(&sfull[i], 4); }
@@ -71,7 +80,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
-    enter_pass(a);
+    if (!gated) enter_pass(a);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -294,7 +303,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                                 if (w.t0 * kBN + half * 128 + j * 8 < a.ncols) dst[j] = make_uint4(0, 0, 0, 0);
                         }
                     }
-                } else if (BASE == kBwdP) {
+                } else if (BASE == kBwdP && !gated) {
                     const int64_t lr = static_cast<int64_t>(w.rt) * kBM + r_in_tile;
                     if (lr < a.rows) {
                         for (int t = w.t0; t < w.t1; ++t) {
@@ -316,6 +325,8 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                     const int64_t lrow2 = static_cast<int64_t>(w.rt) * kDhRows + sub * kBM + r_in_tile;
                     const bool in = lrow2 < a.rows;
                     const int64_t grow2 = a.row0 + lrow2;
+                    // (the row's factor, or 1; rows with factor 0 may hold anything, so they are selected away)
+                    const float rs = (a.row_scale != nullptr && in) ? a.row_scale[grow2] : 1.f;
                     const uint32_t taddr2 = tmem_base + lane_addr + sub * kBN + half * 128;
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
@@ -336,7 +347,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                             uint32_t pk[16];
 #pragma unroll
                             for (int i = 0; i < 32; i += 2) {
-                                pk[i >> 1] = pack_bf16(__uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+                                pk[i >> 1] = rs != 0.f ? pack_bf16(__uint_as_float(v[i]) * rs, __uint_as_float(v[i + 1]) * rs) : 0u;
                             }
                             uint4* dst = reinterpret_cast<uint4*>(a.dH + grow2 * a.lddh + col0);
 #pragma unroll
@@ -402,11 +413,17 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             float m2 = kNegBig, s = 0.f, zy = -INFINITY;       // log2-domain running max, sum, target logit
             const float tscale = (MODE == kFwdFp8T) ? (*a.scale_a) * (*a.scale_b) : 1.f;
             float lse2 = 0.f;
-            float cf = 0.f;                                    // recompute: c_t, folded into the scratch
+            // recompute: U = mul (e^(z - off) - onehot) in plain form (off = lse, mul = c), mul = 1, off = 0 and `target` at
+            // the target column in exponent form
+            float mul = 0.f, target = 0.f;
+            bool ef = false;
             if (BASE == kBwdP && row_ok) {
-                lse2 = a.lse[grow] * kLog2e;
-                cf = a.coef[grow];
-                if (cf == 0.f) valid = false;                  // rows without gradient are written as exact zeros
+                const float lse = a.lse[grow];
+                mul = a.coef[grow];
+                if (mul == 0.f) valid = false;                 // rows without gradient are written as exact zeros
+                ef = a.row_scale != nullptr && exp_form(lse);
+                if (ef) { mul = 1.f; target = exp_form_target(a.lp[grow], lse); }
+                else lse2 = lse * kLog2e;
             }
 
             for (int t = w.t0; t < w.t1 && ok; ++t) {
@@ -460,10 +477,34 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                         float cm = x[0];
 #pragma unroll
                         for (int i = 1; i < 32; ++i) cm = fmaxf(cm, x[i]);
-                        const float m_new = fmaxf(m2, cm * kLog2e);
+                        float m_new = fmaxf(m2, cm * kLog2e);
+                        // reference 0 for every row within range, so that the terms of the sum are what the scratch wants
+                        if (KEEP && fabsf(m_new) <= kKeepRange) m_new = 0.f;
                         float add = 0.f;
+                        if (KEEP) {
+                            uint32_t pk[16];
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) add += ex2(fmaf(x[i], kLog2e, -m_new));
+                            for (int i = 0; i < 32; i += 2) {
+                                const float e0 = ex2(fmaf(x[i], kLog2e, -m_new)), e1 = ex2(fmaf(x[i + 1], kLog2e, -m_new));
+                                add += e0;
+                                add += e1;
+                                pk[i >> 1] = pack_bf16(e0, e1);
+                            }
+                            if (row_ok && w.rt < a.keep_tiles && col0 < a.ncols) {
+                                if (m_new != 0.f) {                // rare: this range of the row lies far below the rest, or above
+#pragma unroll
+                                    for (int i = 0; i < 32; i += 2)
+                                        pk[i >> 1] = pack_bf16(ex2(fmaf(x[i], kLog2e, -0.f)), ex2(fmaf(x[i + 1], kLog2e, -0.f)));
+                                }
+                                uint4* dst = reinterpret_cast<uint4*>(a.U + lrow * a.ldU + col0);
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    if (col0 + j * 8 < a.ncols) dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+                            }
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) add += ex2(fmaf(x[i], kLog2e, -m_new));
+                        }
                         s = fmaf(s, ex2(m2 - m_new), add);
                         m2 = m_new;
                     } else if (BASE == kBwdP) {
@@ -473,9 +514,9 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                             for (int i = 0; i < 32; i += 2) {
                                 float p0 = valid ? ex2(fmaf(x[i], kLog2e, -lse2)) : 0.f;
                                 float p1 = valid ? ex2(fmaf(x[i + 1], kLog2e, -lse2)) : 0.f;
-                                if (col0 + i == y) p0 -= 1.f;
-                                if (col0 + i + 1 == y) p1 -= 1.f;
-                                pk[i >> 1] = pack_bf16(valid ? cf * p0 : 0.f, valid ? cf * p1 : 0.f);
+                                if (col0 + i == y) p0 = ef ? target : p0 - 1.f;
+                                if (col0 + i + 1 == y) p1 = ef ? target : p1 - 1.f;
+                                pk[i >> 1] = pack_bf16(valid ? mul * p0 : 0.f, valid ? mul * p1 : 0.f);
                             }
                             uint4* dst = reinterpret_cast<uint4*>(a.U + lrow * a.ldU + col0);
 #pragma unroll
@@ -548,6 +589,12 @@ __global__ void __launch_bounds__(256) dh_reduce_kernel(const LmheadArgs a) {
             }
         }
     }
+    if (a.row_scale != nullptr) {
+        const float rs = a.row_scale[a.row0 + lr];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            acc[j] = rs != 0.f ? make_float4(acc[j].x * rs, acc[j].y * rs, acc[j].z * rs, acc[j].w * rs) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     uint4* dst = reinterpret_cast<uint4*>(a.dH + (a.row0 + lr) * a.lddh + col0);
 #pragma unroll
     for (int j = 0; j < 2; ++j)
@@ -582,33 +629,25 @@ cudaError_t launch_lmhead(int mode, const CUtensorMap& tmA, const CUtensorMap& t
         case kFwdBf16Dv: return launch_mode<kFwdBf16Dv>(tmA, tmB, args, num_ctas, stream);
         case kBwdPDv:    return launch_mode<kBwdPDv>(tmA, tmB, args, num_ctas, stream);
         case kBwdDhDv:   return launch_mode<kBwdDhDv>(tmA, tmB, args, num_ctas, stream);
+        case kFwdKeep:   return launch_mode<kFwdKeep>(tmA, tmB, args, num_ctas, stream);
+        case kFwdKeepDv: return launch_mode<kFwdKeepDv>(tmA, tmB, args, num_ctas, stream);
     }
     return cudaErrorInvalidValue;
 }
 
+template <int MODE>
+static cudaError_t prepare_mode() {
+    return cudaFuncSetAttribute(lmhead_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+}
+
 cudaError_t lmhead_prepare() {
-    cudaError_t e;
-    e = cudaFuncSetAttribute(lmhead_kernel<kFwdBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = lmhead_fp8_block_prepare();
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lmhead_kernel<kBwdP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lmhead_kernel<kBwdDh>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lmhead_kernel<kFwdFp8T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lmhead_kernel<kBwdDw>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lmhead_kernel<kFwdMx>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lmhead_kernel<kFwdBf16Dv>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lmhead_kernel<kBwdPDv>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lmhead_kernel<kBwdDhDv>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(lmhead_kernel<kFwdMx4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    const cudaError_t all[] = {lmhead_fp8_block_prepare(), prepare_mode<kFwdBf16>(), prepare_mode<kBwdP>(), prepare_mode<kBwdDh>(),
+                               prepare_mode<kFwdFp8T>(), prepare_mode<kBwdDw>(), prepare_mode<kFwdMx>(), prepare_mode<kFwdMx4>(),
+                               prepare_mode<kFwdBf16Dv>(), prepare_mode<kBwdPDv>(), prepare_mode<kBwdDhDv>(), prepare_mode<kFwdKeep>(),
+                               prepare_mode<kFwdKeepDv>()};
+    for (const cudaError_t e : all)
+        if (e != cudaSuccess) return e;
+    return cudaSuccess;
 }
 
 }  // namespace ais

@@ -21,16 +21,19 @@ enum LmheadMode : int {
     // K-major (like the forward passes of the other layout)
     kFwdBf16Dv = 8,
     kBwdPDv    = 9,
-    kBwdDhDv   = 10
+    kBwdDhDv   = 10,
+    // the trainer pass that also stores the exponentials of its logits in the scratch of the dH pass (see exp_form)
+    kFwdKeep   = 11,
+    kFwdKeepDv = 12
 };
 
 // What a mode computes (its epilogue and work-unit shape), whatever the layout of W.
 __host__ __device__ constexpr int base_mode(int mode) {
-    return mode == kFwdBf16Dv ? kFwdBf16 : mode == kBwdPDv ? kBwdP : mode == kBwdDhDv ? kBwdDh : mode;
+    return mode == kFwdBf16Dv || mode == kFwdKeep || mode == kFwdKeepDv ? kFwdBf16 : mode == kBwdPDv ? kBwdP : mode == kBwdDhDv ? kBwdDh : mode;
 }
 // B operand stored with the output column as the contiguous axis (MN-major)?
 __host__ __device__ constexpr bool b_mn_major(int mode) {
-    return mode == kBwdDh || mode == kBwdDw || mode == kFwdBf16Dv || mode == kBwdPDv;
+    return mode == kBwdDh || mode == kBwdDw || mode == kFwdBf16Dv || mode == kBwdPDv || mode == kFwdKeepDv;
 }
 
 constexpr int kSms = 148;                // SMs of the part; the work splits below are planned for it
@@ -65,6 +68,17 @@ constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kStages * kMxStageScal
 // dH: one partial tile of a split unit, 256 x 256 fp32, ordered for 16-byte accesses with the rows across the lanes:
 // [row half][group of 4 columns][128 rows][4 columns]
 constexpr int kPartTileFloats = kDhRows * kBN;
+
+// Exponent form of a scratch row.  The gradient of a row is c (softmax - onehot) W = c e^-lse (e^z - e^lse onehot) W, and the
+// factor in front does not depend on the column: with U = e^z off the target and (p - 1) e^lse at it, the dH pass only has
+// to scale its rows by c e^-lse at the end.  e^z is there before lse, c or alpha are known -- the forward pass forms it for
+// its sum -- so a step that runs log-probs and loss in one call stores it there and has no logits to recompute.  bf16 has
+// the exponent range of fp32, so the relative rounding is that of softmax itself as long as e^z neither overflows nor loses
+// terms that matter: rows with lse in [-20, 59] (terms below e^-67 of the row's sum vanish).  Other rows are in plain form,
+// U = c (softmax - onehot) and scale 1; their row tiles are recomputed.  p - 1 at the target comes from the log-prob
+// (expm1), so a nearly certain token loses nothing to cancellation.
+__host__ __device__ inline bool exp_form(float lse) { return lse >= -20.0f && lse <= 59.0f; }
+__device__ __forceinline__ float exp_form_target(float lp, float lse) { return expm1f(lp) * expf(lse); }
 
 // Pacing of the CTAs of a launch (lmhead_common.cuh): stage fills per announcement, counters in the ring.
 constexpr int kPaceFills = 16;
@@ -106,6 +120,10 @@ struct LmheadArgs {
     int32_t split_from;    // dH: units from here on are split along the contraction (the last, partial wave); others whole
     int32_t ksplit;        // dH: ranges of the contraction per split unit (1 = nothing is split)
     float* part_acc;       // dH: fp32 partial tiles of the split units, [slot][kPartTileFloats] (see dh_reduce_kernel)
+    int32_t keep_tiles;    // kFwdKeep: row tiles (from the first) whose exponentials go to U
+    const float* lp;       // recompute: log-probs of the targets (exponent form)
+    const float* row_scale;   // recompute: non-NULL selects the exponent form; dH: factor of every row (0: the row is zero)
+    const uint32_t* gate;  // recompute: non-NULL: run only if *gate != 0, and leave the rows of inactive tiles as they are
     uint32_t* pace;        // ring of kPaceRing zeroed counters that keeps the CTAs of the launch in step; NULL = no pacing
     uint32_t* pace_clear;  // ring of the next pass of the same call, cleared by this one; NULL = nothing to clear
     int32_t overlap;       // the pass needs nothing from the kernel before it (the other pass of the same call): it starts

@@ -3,6 +3,7 @@
 
 #include "stream_kernels.cuh"
 #include "launch.cuh"
+#include "lmhead.cuh"
 #include "ptx.cuh"
 
 #include <cuda_bf16.h>
@@ -401,7 +402,7 @@ __global__ void __launch_bounds__(kQThreads) tensor_quantize_kernel(const __nv_b
 
 // Group-relative advantage of sequence s (Eq. grpo_adv), and what AdvJob clears for it.
 __device__ __forceinline__ void run_advantage(const AdvJob& j, int s) {
-    if (s == 0) j.tickets[0] = j.tickets[1] = 0;
+    if (s == 0) j.tickets[0] = j.tickets[1] = j.tickets[2] = 0;
     if (j.zero_counts) j.zero_counts[s] = 0;
     const int g0 = (s / j.G) * j.G;
     double mean = 0.0;
@@ -1301,6 +1302,7 @@ struct LossArgs {
     float* loss;
     ais_diag* diag;
     RectifyJob rectify;    // rectify.w_tilde != NULL: ratios and weights of the rows are formed here and written on the way
+    KeepJob keep;          // keep.scale != NULL: the scratch is in exponent form (with `rectify` only)
 };
 
 template <bool VEC, bool RECTIFY>
@@ -1381,6 +1383,28 @@ __global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const LossArgs 
         if (rows == 4) *reinterpret_cast<float4*>(a.coef + t0) = make_float4(c[0], c[1], c[2], c[3]);     // workspace: aligned
         else
             for (int j = 0; j < rows; ++j) a.coef[t0 + j] = c[j];
+        if (RECTIFY && a.keep.scale != nullptr) {
+            bool redo = false;
+            for (int j = 0; j < rows; ++j) {
+                const int64_t t = t0 + j;
+                float scale = 0.f;
+                if (c[j] != 0.f) {
+                    const float lse = a.lse[t];
+                    const bool ef = exp_form(lse);
+                    scale = ef ? c[j] * expf(-lse) : 1.f;
+                    redo |= !ef;
+                    const int y = a.keep.tokens[t];
+                    if (ef && t < a.keep.rows && y >= 0 && y < a.keep.V)
+                        a.keep.U[t * a.keep.ldU + y] = __float2bfloat16(exp_form_target(a.lp_train[t], lse));
+                }
+                a.keep.scale[t] = scale;
+            }
+            redo = __any_sync(0xffffffffu, redo);
+            if (lane == 0) {
+                a.keep.redo_flags[tile] = redo ? 1 : 0;
+                if (redo) atomicAdd(a.keep.redo_count, 1u);
+            }
+        }
         const bool any = __any_sync(0xffffffffu, c[0] != 0.f || c[1] != 0.f || c[2] != 0.f || c[3] != 0.f);
         if (lane == 0) a.tile_flags[tile] = any ? 1 : 0;
     }
@@ -1578,7 +1602,7 @@ cudaError_t launch_loss_coef(const float* lp_train, const float* lp_old, const f
                              const int32_t* seq_offsets, const float* adv, const float* w_tilde, const int32_t* n_valid_seq, int64_t T,
                              int S, int S_norm, float clip_eps, double* partials, uint32_t* ticket, float* coef, uint8_t* tile_flags,
                              void* clear, size_t clear_bytes, float* loss, ais_diag* diag, const float* lse, const RectifyJob* rectify,
-                             cudaStream_t stream) {
+                             const KeepJob* keep, cudaStream_t stream) {
     LossArgs a = {};
     a.lp_train = lp_train;
     a.lp_old = lp_old;
@@ -1605,6 +1629,7 @@ cudaError_t launch_loss_coef(const float* lp_train, const float* lp_old, const f
     const int blocks = reduce_blocks(T, 4 * kDiagThreads);
     if (rectify) {
         a.rectify = *rectify;
+        if (keep) a.keep = *keep;
         return launch_pdl(vec4_ok(rectify->w_tilde, rectify->rho, nullptr, nullptr, mask) ? loss_coef_kernel<true, true> : loss_coef_kernel<false, true>,
                           blocks, kDiagThreads, 0, stream, a);
     }

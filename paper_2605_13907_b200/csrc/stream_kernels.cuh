@@ -2,6 +2,7 @@
 // the per-split log-sum-exp partials, segmented and whole-batch reductions, per-token loss coefficients.
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -31,8 +32,8 @@ struct FlagsJob {
     void* clear;
     int64_t clear_bytes;
 };
-// Group-relative advantages adv[s]; zero_counts [S] (may be NULL) and the two tickets (block counters of the batch
-// reductions) are cleared for the kernels that count into them.
+// Group-relative advantages adv[s]; zero_counts [S] (may be NULL) and the tickets (block counters of the two batch
+// reductions, count of row tiles to recompute) are cleared for the kernels that count into them.
 struct AdvJob {
     const float* rewards;
     int32_t S, G, std_norm;
@@ -48,6 +49,18 @@ struct RectifyJob {
     const ais_diag* alpha_of;
     float *rho, *w_tilde;
     const float* seq_logw;
+};
+
+// The scratch rows that the forward pass of the same call has filled with exponentials (exp_form in lmhead.cuh), as part of
+// the loss kernel: row factors, target columns, and which row tiles have to be recomputed.
+struct KeepJob {
+    __nv_bfloat16* U;
+    int64_t ldU, rows;         // rows kept (the ones after them are recomputed anyway)
+    const int32_t* tokens;
+    int32_t V;
+    float* scale;              // [T] factor of the row in the dH pass
+    uint8_t* redo_flags;       // per row tile
+    uint32_t* redo_count;      // zeroed before the launch
 };
 
 // Raises the dynamic shared-memory limit of the kernels here that need it (once per device).
@@ -108,6 +121,7 @@ cudaError_t launch_loss_coef(const float* lp_train, const float* lp_old, const f
                              const int32_t* seq_offsets, const float* adv, const float* w_tilde, const int32_t* n_valid_seq, int64_t T,
                              int S, int S_norm, float clip_eps, double* partials /*[kDiagBlocks][2]*/, uint32_t* ticket, float* coef,
                              uint8_t* tile_flags, void* clear, size_t clear_bytes, float* loss, ais_diag* diag, const float* lse,
-                             const RectifyJob* rectify /* NULL: w_tilde is there already */, cudaStream_t stream);
+                             const RectifyJob* rectify /* NULL: w_tilde is there already */,
+                             const KeepJob* keep /* NULL; only with rectify */, cudaStream_t stream);
 
 }  // namespace ais

@@ -56,3 +56,44 @@ def test_split_passes_match_the_oracle(case):
     lp = torch.empty(T, device="cuda")
     ais.logprob_train_static(step.shape, H, W, tok, msk, lp)
     assert np.max(np.abs(lp.cpu().numpy() - ref["lp_train"])) <= LP_ATOL
+
+
+@pytest.mark.parametrize("dv", [False, True])
+@pytest.mark.parametrize("rows", ["ordinary", "mixed"])
+def test_kept_exponentials_match_the_oracle(rows, dv):
+    """A step in one call keeps e^z of the forward pass for dH; rows whose log-sum-exp lies outside [-20, 59] are recomputed,
+    alone or beside ordinary rows of their tile.  With room for 128 rows only the first tile is kept: same bits."""
+    import paper_2605_13907_b200 as ais
+    d, V, P, G = 384, 1336, 2, 3
+    w = workloads.scaled(workloads.WORKLOADS["tiny"], d=d, V=V, P=P, G=G, lengths="uniform:90:130", w_std=d ** -0.5, seed=302)
+    b = workloads.make_batch(w, device="cpu")
+    T = b.T
+    if rows == "mixed":
+        b.W[:, 0] = 1.0
+        b.H[:, 0] = 0.0
+        b.H[0:3] *= 30.0                                    # logits beyond +-59 (first tile)
+        b.H[130:150, 0] = -50.0                             # log-sum-exp near -43
+        b.H[256:384:7, 0] = 70.0                            # near +77, scattered over a tile
+        b.tokens[0:3] = 5                                   # a target that is far from certain
+    b.mask[40:60] = 0
+    rewards = torch.zeros(P * G)
+    rewards[::2] = 1.0
+    b.rewards = rewards
+    a = workloads.to_numpy(b)
+    ref = oais.full_path(a["H"], a["W"], a["tokens"], a["mask"], a["seq_offsets"], a["rewards"], P, G, w.block)
+    Wx = (b.W.t().contiguous() if dv else b.W).cuda()
+    out = []
+    for cap in (None, 1):
+        step = ais.AisStep(T, d, V, P, G, w.block, workspace_bytes_cap=cap, w_layout=ais.W_DV if dv else ais.W_VD)
+        step.dH.fill_(7.0)
+        step.step(b.H.cuda(), Wx, b.tokens.cuda(), b.mask.cuda(), b.seq_offsets.cuda(), b.rewards.cuda())
+        torch.cuda.synchronize()
+        assert int(step.status.item()) == 0
+        # |z| up to 120: fp32 sums of d products and the rounding of the sum itself, 120 * 2^-23 * a few
+        assert np.max(np.abs(step.lse_train[:T].cpu().numpy() - ref["lse_train"])) <= LP_ATOL
+        out.append(step.dH[:T].clone())
+    dH = out[0].float().cpu().numpy().astype(np.float64)
+    assert np.all(dH[a["mask"] == 0] == 0)
+    for r in range(0, T, 128):
+        assert np.linalg.norm(dH[r:r + 128] - ref["dH"][r:r + 128]) <= DH_REL * np.linalg.norm(ref["dH"][r:r + 128]), r
+    assert torch.equal(out[0], out[1])
