@@ -568,7 +568,7 @@ static int diagnostics(const ais_shape* shape, const ais_params* params, const f
         return AIS_ERR_DEVICE;
     if (launch_diag(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag), tickets,
                     n_valid_seq, seq_level ? reinterpret_cast<float*>(ws + L.off_seqw) : nullptr, rho, fuse.rectify_later ? nullptr : w_tilde,
-                    diag, s) != cudaSuccess)
+                    diag, !fuse.adv, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     return AIS_OK;
 }

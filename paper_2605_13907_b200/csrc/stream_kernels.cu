@@ -612,6 +612,29 @@ __device__ __forceinline__ int seq_of_row(const int32_t* __restrict__ seq_offset
     return lo;
 }
 
+// The sequences of rows t_first and t_last (t_first <= t_last) found by a whole warp, 32 probes at a time: two rounds of loads
+// for up to 1,024 sequences where the binary search of a single thread is a chain of ten.
+__device__ __forceinline__ int2 seqs_of_rows_warp(const int32_t* __restrict__ seq_offsets, int S, int64_t t_first, int64_t t_last) {
+    const int lane = threadIdx.x & 31;
+    int lo[2] = {0, 0}, hi[2] = {S, S};
+    const int64_t t[2] = {t_first, t_last};
+    while (hi[0] - lo[0] > 1 || hi[1] - lo[1] > 1) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int step = (hi[k] - lo[k] + 31) / 32;
+            const int at = lo[k] + (lane + 1) * step;
+            const int n = __popc(__ballot_sync(0xffffffffu, at < hi[k] && static_cast<int64_t>(seq_offsets[at < hi[k] ? at : lo[k]]) <= t[k]));
+            lo[k] += n * step;
+            hi[k] = min(lo[k] + step, hi[k]);
+        }
+    }
+    return make_int2(lo[0], lo[1]);
+}
+// The largest s in [range.x, range.y] whose first row is not behind t.
+__device__ __forceinline__ int seq_in_range(const int32_t* __restrict__ seq_offsets, int2 range, int64_t t) {
+    return range.x == range.y ? range.x : range.x + seq_of_row(seq_offsets + range.x, range.y - range.x + 1, t);
+}
+
 // The diagnostics and alpha from the ten sums over the batch.
 __device__ __noinline__ void derive_diag(const double* m, const ais_params& p, ais_diag* __restrict__ diag) {
     ais_diag d;
@@ -918,7 +941,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
                                                                          const int32_t* __restrict__ seq_offsets,
                                                                          const float* __restrict__ adv, int T, int S, float C,
                                                                          double* partials, int32_t* __restrict__ n_valid_seq,
-                                                                         const float* __restrict__ seq_logw, const DiagFinish fin) {
+                                                                         const float* __restrict__ seq_logw, bool early, const DiagFinish fin) {
     static_assert(kDiagThreads * 8 == kMomRows, "one 8-row group per thread and tile");
     extern __shared__ __align__(128) uint8_t stages[];          // kMomStages stages, then the barriers
     uint64_t* full = reinterpret_cast<uint64_t*>(stages + kMomStages * kMomStageBytes);
@@ -927,7 +950,8 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
     __shared__ int abort_flag;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
-    const int ntiles = T / kMomRows;
+    const int nfull = T / kMomRows;                    // whole tiles; what is left is one more, read directly
+    const int ntiles = (T + kMomRows - 1) / kMomRows;
     const int per = (ntiles + gridDim.x - 1) / gridDim.x;
     const int tile0 = blockIdx.x * per < ntiles ? blockIdx.x * per : ntiles;
     const int tile1 = tile0 + per < ntiles ? tile0 + per : ntiles;
@@ -936,7 +960,6 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
         abort_flag = 0;
         fence_barrier_init();
     }
-    pdl_enter();
     __syncthreads();
     auto issue = [&](int tile, int st) {               // thread 0: the three copies of one tile onto the stage's barrier
         uint8_t* dst = stages + st * kMomStageBytes;
@@ -976,15 +999,12 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
         next_b = 0;
     };
     reset();
+    auto start_at = [&](int s0) {
+        sq = s0;
+        next_b = sq + 1 < S ? seq_offsets[sq + 1] : kNever;
+    };
     auto seek = [&](int t) {
-        if (sq < 0) {
-            sq = seq_of_row(seq_offsets, S, t);
-            next_b = sq + 1 < S ? seq_offsets[sq + 1] : kNever;
-        }
-        while (t >= next_b) {
-            ++sq;
-            next_b = sq + 1 < S ? seq_offsets[sq + 1] : kNever;
-        }
+        while (t >= next_b) start_at(sq + 1);
     };
     auto enter = [&]() {                                // the row's sequence becomes the current one
         if (sq != cur) {
@@ -1086,11 +1106,15 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
     // One walk over the block's tiles, the `base`-th tile of the stage ring first; the fast one also adds up the valid rows
     // per sequence on the way.
     bool failed = false;
+    int issued = tile0;                                 // first tile not yet requested (thread 0)
+    const int full1 = tile1 < nfull ? tile1 : nfull;    // tiles of the block that arrive by copy: tile0 .. full1 - 1
+    auto fill_ring = [&](int base) {
+        issued = tile0;
+        if (tid == 0)
+            for (; issued < full1 && issued < tile0 + kMomStages; ++issued) issue(issued, (base + issued - tile0) % kMomStages);
+    };
     auto walk = [&](auto exact, int base) {
         constexpr bool count = !decltype(exact)::value;
-        int issued = tile0;                             // first tile not yet requested (thread 0)
-        if (tid == 0)
-            for (; issued < tile1 && issued < tile0 + kMomStages; ++issued) issue(issued, (base + issued - tile0) % kMomStages);
         for (int tile = tile0; tile < tile1; ++tile) {
             const unsigned k = static_cast<unsigned>(base + tile - tile0);
             const unsigned st = k % kMomStages;
@@ -1100,17 +1124,31 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
             const bool single = t0 + 8 <= next_b;          // the usual case: the eight rows belong to one sequence
             if (single) enter();
             const uint32_t parity = (k / kMomStages) & 1u;
-            bool ok = mbar_try_wait(&full[st], parity);
+            bool ok = tile >= nfull || mbar_try_wait(&full[st], parity);
             if (!ok) ok = mbar_wait_slow(&full[st], parity, &abort_flag);
             int n = 0;
             if (ok) {
-                const uint8_t* src = stages + st * kMomStageBytes;
-                const float4* pa = reinterpret_cast<const float4*>(src) + 2 * tid;
-                const float4* pb = reinterpret_cast<const float4*>(src + kMomRows * 4) + 2 * tid;
-                const float4 a0 = pa[0], a1 = pa[1], b0 = pb[0], b1 = pb[1];
-                const uint2 mk = reinterpret_cast<const uint2*>(src + kMomRows * 8)[tid];
-                const float lt[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                const float lr[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                float lt[8], lr[8];
+                uint2 mk = make_uint2(0, 0);
+                if (tile < nfull) {
+                    const uint8_t* src = stages + st * kMomStageBytes;
+                    const float4* pa = reinterpret_cast<const float4*>(src) + 2 * tid;
+                    const float4* pb = reinterpret_cast<const float4*>(src + kMomRows * 4) + 2 * tid;
+                    const float4 a0 = pa[0], a1 = pa[1], b0 = pb[0], b1 = pb[1];
+                    mk = reinterpret_cast<const uint2*>(src + kMomRows * 8)[tid];
+                    lt[0] = a0.x; lt[1] = a0.y; lt[2] = a0.z; lt[3] = a0.w; lt[4] = a1.x; lt[5] = a1.y; lt[6] = a1.z; lt[7] = a1.w;
+                    lr[0] = b0.x; lr[1] = b0.y; lr[2] = b0.z; lr[3] = b0.w; lr[4] = b1.x; lr[5] = b1.y; lr[6] = b1.z; lr[7] = b1.w;
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const bool in = t0 + j < T;
+                        lt[j] = in ? lp_train[t0 + j] : 0.f;
+                        lr[j] = in ? lp_roll[t0 + j] : 0.f;
+                        const uint32_t m = in ? mask[t0 + j] : 0u;
+                        if (j < 4) mk.x |= m << (8 * j);
+                        else mk.y |= m << (8 * (j - 4));
+                    }
+                }
                 if (single) {
                     if ((mk.x | mk.y) != 0u) n = add_rows(exact, lt, lr, mk.x, mk.y);
                 } else if ((mk.x | mk.y) != 0u) {
@@ -1148,7 +1186,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
             }
             // everyone is done with the stage (or someone gave up): the stage can take the tile three ahead
             if (__syncthreads_or(ok ? 0 : 1)) { failed = true; break; }
-            if (tid == 0 && issued < tile1) { issue(issued, st); ++issued; }
+            if (tid == 0 && issued < full1) { issue(issued, st); ++issued; }
         }
         if (failed && tid == 0) {
             // let the copies still in flight land before the block's shared memory is given up
@@ -1159,23 +1197,27 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
                 }
         }
         if (count && n_valid_seq && lane == 0 && wsq >= 0 && wcnt > 0) atomicAdd(&n_valid_seq[wsq], wcnt);
-    // rows after the last whole tile: the first threads of the grid, one row each
-    for (int t = ntiles * kMomRows + static_cast<int>(blockIdx.x * blockDim.x) + tid; t < T; t += gridDim.x * blockDim.x) {
-        if (!mask[t]) continue;
-        sq = -1;
-        seek(t);
-        enter();
-        const float lt[8] = {lp_train[t], 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, lr[8] = {lp_roll[t], 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        add_rows(exact, lt, lr, 1u, 0u);
-        if (count && n_valid_seq) atomicAdd(&n_valid_seq[sq], 1);
-    }
     };
+    // The sequences of the warp's rows of the first tile, before the wait: the offsets are older than the kernel before this
+    // one.  So are the rows when that kernel only formed advantages (`early`): their copies start now, too.
+    int2 range = make_int2(0, 0);
+    if (tile0 < tile1) {
+        const int w0 = tile0 * kMomRows + (tid & ~31) * 8;
+        range = seqs_of_rows_warp(seq_offsets, S, w0 < T ? w0 : T - 1, w0 + 255 < T ? w0 + 255 : T - 1);
+    }
+    const int first_sq = seq_in_range(seq_offsets, range, tile0 * kMomRows + 8 * tid < T ? tile0 * kMomRows + 8 * tid : T - 1);
+    if (early) fill_ring(0);
+    pdl_enter();
+    if (!early) fill_ring(0);
+    start_at(first_sq);
     walk(std::false_type{}, 0);
     const bool any_big = __syncthreads_or(nbig) != 0;
     const bool any_small = __syncthreads_or(nsmall) != 0;
     if (!any_big && any_small && !__syncthreads_or(failed ? 1 : 0)) {
         reset();
-        walk(std::true_type{}, tile1 - tile0);
+        start_at(first_sq);
+        fill_ring(full1 - tile0);
+        walk(std::true_type{}, full1 - tile0);
     }
     constexpr int kSums = 10;                            // slots 10 and 11 are no moments
     double acc[kSums];
@@ -1200,9 +1242,26 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
     block_sums(acc, scratch, totals);
     if (tid < kSums) partials[blockIdx.x * kNumMoments + tid] = totals[tid];
     if (!last_block(fin.ticket)) return;
-    for (int i = tid >> 5; i < kNumMoments; i += kDiagThreads / 32) {
-        const double m = i < kSums ? warp_ordered_sum(partials, gridDim.x, kNumMoments, i, lane) : 0.0;
-        if (lane == 0) totals[i] = m;
+    // Totals over the blocks: thread (slice, moment) adds every 25th block's value in block order, ten threads add the slices.
+    constexpr int kSlices = kDiagThreads / kSums;
+    if (tid < kSlices * kSums) {
+        const int m = tid % kSums, nb = static_cast<int>(gridDim.x);
+        double acc2 = 0.0;
+        for (int b0 = tid / kSums; b0 < nb; b0 += 12 * kSlices) {
+            double v[12];
+#pragma unroll
+            for (int j = 0; j < 12; ++j) v[j] = b0 + j * kSlices < nb ? __ldcg(partials + (b0 + j * kSlices) * kNumMoments + m) : 0.0;
+#pragma unroll
+            for (int j = 0; j < 12; ++j) acc2 += v[j];
+        }
+        scratch[m][tid / kSums] = acc2;
+    }
+    __syncthreads();
+    if (tid < kNumMoments) {
+        double tot = 0.0;
+        if (tid < kSums)
+            for (int k = 0; k < kSlices; ++k) tot += scratch[tid][k];
+        totals[tid] = tot;
     }
     __syncthreads();
     if (fin.moments != nullptr && tid < kNumMoments) fin.moments[tid] = totals[tid];
@@ -1356,8 +1415,9 @@ __global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const LossArgs 
         }
         float rho[4] = {1.f, 1.f, 1.f, 1.f};
         if (RECTIFY) wt[0] = wt[1] = wt[2] = wt[3] = 1.f;
+        const int2 range = seqs_of_rows_warp(a.seq_offsets, a.S, tile * 128, tile * 128 + 127 < a.T ? tile * 128 + 127 : a.T - 1);
         if (mk != 0u) {
-            int sq = seq_of_row(a.seq_offsets, a.S, t0);
+            int sq = seq_in_range(a.seq_offsets, range, t0);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 while (sq + 1 < a.S && static_cast<int64_t>(a.seq_offsets[sq + 1]) <= t0 + j) ++sq;
@@ -1442,7 +1502,7 @@ inline int reduce_blocks(int64_t T, int rows) {
 // The masked sums of the batch into fin.diag and / or fin.moments.
 cudaError_t launch_moments_kernel(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
                                   const float* adv, int64_t T, int S, float C, double* partials, int32_t* n_valid_seq,
-                                  float* seq_logw, const DiagFinish& fin, cudaStream_t stream) {
+                                  float* seq_logw, bool early, const DiagFinish& fin, cudaStream_t stream) {
     cudaError_t e;
     if (seq_logw && S > 0) {
         e = launch_pdl(seq_logw_kernel, (S + 7) / 8, 256, 0, stream, lp_train, lp_roll, mask, seq_offsets, S, seq_logw);
@@ -1452,7 +1512,7 @@ cudaError_t launch_moments_kernel(const float* lp_train, const float* lp_roll, c
         const int blocks = reduce_blocks(T, kMomRows);
         const int Ti = static_cast<int>(T);
         return launch_pdl(seq_logw ? moments_staged_kernel<true> : moments_staged_kernel<false>, blocks, kDiagThreads, kMomSmemBytes, stream,
-                          lp_train, lp_roll, mask, seq_offsets, adv, Ti, S, C, partials, n_valid_seq, seq_logw, fin);
+                          lp_train, lp_roll, mask, seq_offsets, adv, Ti, S, C, partials, n_valid_seq, seq_logw, early && !seq_logw, fin);
     }
     e = launch_pdl(vec4_ok(lp_train, lp_roll, nullptr, nullptr, mask) ? moments_kernel<4> : moments_kernel<1>, kDiagBlocks, kDiagThreads, 0, stream,
                    lp_train, lp_roll, mask, seq_offsets, adv, T, S, C, partials, n_valid_seq, seq_logw);
@@ -1576,9 +1636,9 @@ cudaError_t launch_advantages(const AdvJob& job, cudaStream_t stream) {
 
 cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
                         const float* adv, int64_t T, int S, const ais_params& p, double* partials, uint32_t* ticket,
-                        int32_t* n_valid_seq, float* seq_logw, float* rho, float* w_tilde, ais_diag* diag, cudaStream_t stream) {
+                        int32_t* n_valid_seq, float* seq_logw, float* rho, float* w_tilde, ais_diag* diag, bool early, cudaStream_t stream) {
     const DiagFinish fin = {p, diag, nullptr, ticket};
-    const cudaError_t e = launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, fin, stream);
+    const cudaError_t e = launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, early, fin, stream);
     if (e != cudaSuccess || T == 0 || w_tilde == nullptr) return e;
     return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, diag, rho, w_tilde, seq_offsets, S, seq_logw, stream);
 }
@@ -1587,7 +1647,7 @@ cudaError_t launch_moments(const float* lp_train, const float* lp_roll, const ui
                            const float* adv, int64_t T, int S, const ais_params& p, double* partials, uint32_t* ticket,
                            int32_t* n_valid_seq, float* seq_logw, double* moments, cudaStream_t stream) {
     const DiagFinish fin = {p, nullptr, moments, ticket};
-    return launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, fin, stream);
+    return launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, true, fin, stream);
 }
 
 cudaError_t launch_finalize(const double* moments, const float* lp_train, const float* lp_roll, const uint8_t* mask, int64_t T,

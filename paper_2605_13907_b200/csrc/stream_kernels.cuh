@@ -103,7 +103,8 @@ cudaError_t launch_advantages(const AdvJob& job, cudaStream_t stream);
 cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
                         const float* adv, int64_t T, int S, const ais_params& p, double* partials /*[kDiagBlocks][kNumMoments]*/, uint32_t* ticket,
                         int32_t* n_valid_seq, float* seq_logw /* [S] scratch: non-NULL selects sequence-level weights */,
-                        float* rho, float* w_tilde /* NULL: the loss kernel rectifies */, ais_diag* diag, cudaStream_t stream);
+                        float* rho, float* w_tilde /* NULL: the loss kernel rectifies */, ais_diag* diag,
+                        bool early /* the log-probs are older than the kernel enqueued last */, cudaStream_t stream);
 
 // The two halves of launch_diag: partial moments summed into `moments` [kNumMoments], and everything that follows
 // from a (possibly all-reduced) moment vector.
