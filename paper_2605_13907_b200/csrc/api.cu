@@ -78,6 +78,16 @@ bool make_tmap(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, ui
     return r == CUDA_SUCCESS;
 }
 
+bool make_tmap_blocks(CUtensorMap* map, const void* base, uint64_t dim0, uint64_t dim1, uint64_t stride1_bytes) {
+    if (!g_encode) return false;
+    cuuint64_t dims[3] = {64, dim1, (dim0 + 63) / 64};
+    cuuint64_t strides[2] = {stride1_bytes, 128};
+    cuuint32_t box[3] = {64, 64, 4};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // The units of a pass are (row tile, vocabulary range) pairs handed round robin to one persistent CTA per SM, so its time
 // is waves x tiles of the longest range.  Four ranges for everybody left a response of 613 rows (5 row tiles) on 20 of 148
 // SMs (3.2 ms per pass at d = 4096, V = 151936) and ran 79 row tiles as three waves where 2.1 were full.  The number of
@@ -262,6 +272,9 @@ bool arm_pace(LmheadArgs& a, uint8_t* ws, const Layout& L, int tiles_per_unit, i
     a.pace_per_unit = static_cast<int32_t>((fills + kPaceFills - 1) / kPaceFills);
     return a.pace != nullptr;
 }
+
+// Width of a [d, V] head that its map of 64-column blocks covers (below 64 columns no tile uses that map).
+uint64_t whole_blocks(uint64_t V) { return V < 64 ? 64 : V / 64 * 64; }
 
 // Rows of backward scratch that the workspace holds: whole row tiles, no more than the batch has.
 int64_t scratch_rows(const Layout& L, int64_t T, size_t workspace_bytes) {
@@ -463,7 +476,7 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
         LmheadArgs a;
         CUtensorMap tmA, tmB, tmSA, tmSB;
         int mode, units, ctas;
-    } pass[2];
+    } pass[2] = {};
     CombineJob jobs[2];
     int n = 0;
     bool paced = false;
@@ -492,14 +505,16 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
     bool maps = true;
     if (do_train) {
         // W [V, d]: K-major boxes of 64 hidden units x 256 vocabulary rows.  W [d, V]: the vocabulary is the contiguous
-        // axis, boxes of 64 vocabulary columns x 64 hidden units (four of them per stage)
+        // axis, four blocks of 64 vocabulary columns x 64 hidden units per copy, and single boxes for the last tile
         const bool keep = fuse.keep_rows > 0;
         Pass& p = add(keep ? (dv ? kFwdKeepDv : kFwdKeep) : dv ? kFwdBf16Dv : kFwdBf16, kBM, kBN, L.nsplit, shape->d / 64, lp_train, lse_train);
         p.a.U = reinterpret_cast<__nv_bfloat16*>(ws + L.off_u);
         p.a.ldU = L.ldU;
+        p.a.block_tiles = static_cast<int32_t>(V / kBN);
         p.a.keep_tiles = static_cast<int32_t>((fuse.keep_rows + kBM - 1) / kBM);
         maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, H, d, T, shape->ldh * 2, 64, kBM, CU_TENSOR_MAP_SWIZZLE_128B) &&
-                (dv ? make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, V, d, shape->ldw * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
+                (dv ? make_tmap_blocks(&p.tmB, W, whole_blocks(V), d, shape->ldw * 2) &&
+                          make_tmap(&p.tmSA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, V, d, shape->ldw * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
                     : make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, d, V, shape->ldw * 2, 64, kBN, CU_TENSOR_MAP_SWIZZLE_128B));
     }
     if (do_roll && (mx || per_tensor)) {
@@ -672,15 +687,16 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
     const uint64_t V = static_cast<uint64_t>(shape->V), d = static_cast<uint64_t>(shape->d);
 
     // tmW_k: W for the recompute pass (contraction over d), tmW_n: W for the dH pass (contraction over V).  With W [V, d]
-    // the first is K-major (boxes of 64 hidden units x 256 vocabulary rows) and the second MN-major (64 x 64 boxes);
+    // the first is K-major (boxes of 64 hidden units x 256 vocabulary rows) and the second MN-major (blocks of 64 x 64);
     // with W [d, V] it is the other way round (64 x 64 boxes of vocabulary columns x hidden units; boxes of 64 vocabulary
     // columns x 256 hidden units).
     const bool dv = shape->w_layout == AIS_W_DV;
-    CUtensorMap tmW_k, tmW_n, tmU;
-    if (!(dv ? make_tmap(&tmW_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, V, d, shape->ldw * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
+    CUtensorMap tmW_k, tmW_n, tmW_tail, tmU;
+    if (!(dv ? make_tmap_blocks(&tmW_k, W, whole_blocks(V), d, shape->ldw * 2) &&
+                   make_tmap(&tmW_tail, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, V, d, shape->ldw * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
              : make_tmap(&tmW_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, d, V, shape->ldw * 2, 64, kBN, CU_TENSOR_MAP_SWIZZLE_128B)) ||
         !(dv ? make_tmap(&tmW_n, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, V, d, shape->ldw * 2, 64, kBN, CU_TENSOR_MAP_SWIZZLE_128B)
-             : make_tmap(&tmW_n, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, d, V, shape->ldw * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)) ||
+             : make_tmap_blocks(&tmW_n, W, d, V, shape->ldw * 2)) ||
         !make_tmap(&tmU, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, U, V, static_cast<uint64_t>(blk_rows), L.ldU * 2, 64, kBM,
                    CU_TENSOR_MAP_SWIZZLE_128B))
         return AIS_ERR_DEVICE;
@@ -722,11 +738,12 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
         a.n_col_tiles = (shape->V + kBN - 1) / kBN;
         a.nsplit = pick_nsplit(shape, params, a.n_row_tiles, a.n_col_tiles);
         a.ksteps = shape->d / 64;
+        a.block_tiles = shape->V / kBN;
         int units = a.n_row_tiles * a.nsplit;
         int ctas = units < num_sms ? units : num_sms;
         arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, units, ctas, pass, pass > 0);
         ++pass;
-        if (launch_lmhead(dv ? kBwdPDv : kBwdP, tmH, tmW_k, tmH, tmW_k, a, ctas, s) != cudaSuccess)
+        if (launch_lmhead(dv ? kBwdPDv : kBwdP, tmH, tmW_k, dv ? tmW_tail : tmH, tmW_k, a, ctas, s) != cudaSuccess)
             return AIS_ERR_DEVICE;
         // dH = c (.) (U W)
         a.tile_active = ws + L.off_flags;
@@ -760,10 +777,9 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
             // dW (+)= U^T H over the rows of this pass: both operands are read with the rows as contraction axis;
             // the maps end at `rows`, so rows the scratch still holds from an earlier pass read as zeros
             CUtensorMap tmU_t, tmH_t;
-            if (!make_tmap(&tmU_t, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, U, V, static_cast<uint64_t>(rows), L.ldU * 2, 64, 64,
-                           CU_TENSOR_MAP_SWIZZLE_128B) ||
-                !make_tmap(&tmH_t, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Hc, d, static_cast<uint64_t>(rows), shape->ldh * 2, 64, 64,
-                           CU_TENSOR_MAP_SWIZZLE_128B))
+            // (the scratch rows are padded to 64 columns; what the padding holds only reaches outputs that are not stored)
+            if (!make_tmap_blocks(&tmU_t, U, V, static_cast<uint64_t>(rows), L.ldU * 2) ||
+                !make_tmap_blocks(&tmH_t, Hc, d, static_cast<uint64_t>(rows), shape->ldh * 2))
                 return AIS_ERR_DEVICE;
             // output in W's layout: [V, d] = U^T H, or [d, V] = H^T U with the two operands changing places
             const int out_rows = dv ? shape->d : shape->V, out_cols = dv ? shape->V : shape->d;

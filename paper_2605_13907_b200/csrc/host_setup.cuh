@@ -14,6 +14,10 @@ int device_setup(int* num_sms);
 bool make_tmap(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, uint64_t dim0, uint64_t dim1,
                uint64_t stride1_bytes, uint32_t box0, uint32_t box1, CUtensorMapSwizzle swz);
 
+// The same matrix as [dim0 / 64][dim1][64] for boxes of four 64-column blocks x 64 rows (128-byte swizzle, one block after
+// the other in shared memory).  dim0 has to be a multiple of 64, or the rows long enough to hold the rounded-up width.
+bool make_tmap_blocks(CUtensorMap* map, const void* base, uint64_t dim0, uint64_t dim1, uint64_t stride1_bytes);
+
 // How many vocabulary ranges a forward or recompute pass over `row_tiles` x `col_tiles` tiles splits each row tile into,
 // at most `most`; `d` is the hidden size; `pairs`: the FP8 pass with tiles of two row tiles x 128 columns.
 int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most, bool pairs = false);

@@ -26,7 +26,8 @@ constexpr int threads_of(int mode) { return (mode == kFwdMx || mode == kFwdMx4) 
 
 template <int MODE>
 __global__ void __launch_bounds__(threads_of(MODE), 1)
-lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const LmheadArgs a) {
+lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+              const __grid_constant__ CUtensorMap tmB2, const LmheadArgs a) {
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte aligned start, as an offset from the array so that the compiler still knows the address space
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -132,19 +133,24 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                             tma_load_2d(sA, &tmA, &full[st.idx], kelem, w.rt * kDhRows);
                             tma_load_2d(sA + kAStageBytes, &tmA, &full[st.idx], kelem, w.rt * kDhRows + kBM);
                         } else if (BASE == kBwdDw) {
-                            // A is U[t, v]: the output row v is the contiguous axis -> four 64-wide boxes of 64 rows t
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                tma_load_2d(sA + j * (kAStageBytes / 2), &tmA, &full[st.idx], w.rt * kDhRows + j * 64, kelem);
+                            // A is U[t, v]: the output row v is the contiguous axis -> four 64-wide blocks of 64 rows t in one copy
+                            tma_load_3d(sA, &tmA, &full[st.idx], 0, kelem, w.rt * (kDhRows / 64));
                         } else {
                             tma_load_2d(sA, &tmA, &full[st.idx], kelem, w.rt * kBM);
                         }
                         if (B_MN) {
                             // B is stored with the output column as the contiguous axis (W[v, n] in the dH pass, H[t, n] in
-                            // the dW pass, W[k, v] in the forward passes over a [d, V] head) -> four 64-column boxes
+                            // the dW pass, W[k, v] in the forward passes over a [d, V] head): four blocks of 64 columns, one
+                            // after the other in shared memory.  One copy for the four: with a copy each the forward pass over a
+                            // [d, V] head took 14.2 Mcycles for 9,217 rows, 11.8 now (as much as the other layout).  The last,
+                            // partial tile of such a head keeps single boxes, which end at V.
+                            if (MODE == kBwdDh || MODE == kBwdDw || t < a.block_tiles) {
+                                tma_load_3d(sB, &tmB, &full[st.idx], 0, kelem, t * (kBN / 64));
+                            } else {
 #pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                tma_load_2d(sB + j * (kBStageBytes / 4), &tmB, &full[st.idx], t * kBN + j * 64, kelem);
+                                for (int j = 0; j < 4; ++j)
+                                    tma_load_2d(sB + j * (kBStageBytes / 4), &tmB2, &full[st.idx], t * kBN + j * 64, kelem);
+                            }
                         } else {
                             tma_load_2d(sB, &tmB, &full[st.idx], kelem, t * kBN);
                         }
@@ -610,27 +616,27 @@ cudaError_t launch_dh_reduce(const LmheadArgs& args, cudaStream_t stream) {
 }
 
 template <int MODE>
-static cudaError_t launch_mode(const CUtensorMap& tmA, const CUtensorMap& tmB, const LmheadArgs& args, int num_ctas,
+static cudaError_t launch_mode(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB2, const LmheadArgs& args, int num_ctas,
                                cudaStream_t stream) {
-    return launch_pdl(lmhead_kernel<MODE>, num_ctas, threads_of(MODE), kSmemBytes, stream, tmA, tmB, args);
+    return launch_pdl(lmhead_kernel<MODE>, num_ctas, threads_of(MODE), kSmemBytes, stream, tmA, tmB, tmB2, args);
 }
 
 cudaError_t launch_lmhead(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,
                           const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream) {
     switch (mode) {
-        case kFwdBf16: return launch_mode<kFwdBf16>(tmA, tmB, args, num_ctas, stream);
+        case kFwdBf16: return launch_mode<kFwdBf16>(tmA, tmB, tmSA, args, num_ctas, stream);
         case kFwdFp8:  return launch_lmhead_fp8_block(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
-        case kBwdP:    return launch_mode<kBwdP>(tmA, tmB, args, num_ctas, stream);
-        case kBwdDh:   return launch_mode<kBwdDh>(tmA, tmB, args, num_ctas, stream);
-        case kFwdFp8T: return launch_mode<kFwdFp8T>(tmA, tmB, args, num_ctas, stream);
-        case kBwdDw:   return launch_mode<kBwdDw>(tmA, tmB, args, num_ctas, stream);
-        case kFwdMx:   return launch_mode<kFwdMx>(tmA, tmB, args, num_ctas, stream);
-        case kFwdMx4:  return launch_mode<kFwdMx4>(tmA, tmB, args, num_ctas, stream);
-        case kFwdBf16Dv: return launch_mode<kFwdBf16Dv>(tmA, tmB, args, num_ctas, stream);
-        case kBwdPDv:    return launch_mode<kBwdPDv>(tmA, tmB, args, num_ctas, stream);
-        case kBwdDhDv:   return launch_mode<kBwdDhDv>(tmA, tmB, args, num_ctas, stream);
-        case kFwdKeep:   return launch_mode<kFwdKeep>(tmA, tmB, args, num_ctas, stream);
-        case kFwdKeepDv: return launch_mode<kFwdKeepDv>(tmA, tmB, args, num_ctas, stream);
+        case kBwdP:    return launch_mode<kBwdP>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kBwdDh:   return launch_mode<kBwdDh>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kFwdFp8T: return launch_mode<kFwdFp8T>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kBwdDw:   return launch_mode<kBwdDw>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kFwdMx:   return launch_mode<kFwdMx>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kFwdMx4:  return launch_mode<kFwdMx4>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kFwdBf16Dv: return launch_mode<kFwdBf16Dv>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kBwdPDv:    return launch_mode<kBwdPDv>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kBwdDhDv:   return launch_mode<kBwdDhDv>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kFwdKeep:   return launch_mode<kFwdKeep>(tmA, tmB, tmSA, args, num_ctas, stream);
+        case kFwdKeepDv: return launch_mode<kFwdKeepDv>(tmA, tmB, tmSA, args, num_ctas, stream);
     }
     return cudaErrorInvalidValue;
 }

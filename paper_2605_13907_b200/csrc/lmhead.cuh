@@ -93,6 +93,7 @@ struct LmheadArgs {
     int32_t n_col_tiles;
     int32_t ksteps;        // shared-memory stages per accumulator tile
     int32_t nsplit;        // forward / recompute: independent column ranges per row tile
+    int32_t block_tiles;   // MN-major B of a [d, V] head: column tiles below this are whole and come by one copy of four blocks
     int32_t sgroups;       // FP8: scale blocks per stage (128 / fp8_block)
     const uint8_t* tile_active;   // one byte per global 128-row tile: 0 = nothing to compute there (may be NULL)
     const int32_t* tokens;
@@ -131,7 +132,8 @@ struct LmheadArgs {
     int32_t pace_per_unit; // announcements per unit = ceil(largest number of stage fills of a unit / fills per announcement)
 };
 
-// Launches one pass.  tmSA / tmSB are only read in kFwdFp8 mode.
+// Launches one pass.  tmSA / tmSB are only read in kFwdFp8 mode; with an MN-major B tmB maps blocks of 64 columns
+// (make_tmap_blocks) and tmSA, for the last column tile of a [d, V] head, plain 64 x 64 boxes.
 cudaError_t launch_lmhead(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,
                           const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream);
 // Sums the partial tiles of a dH launch's split units (args as that launch got them) and writes their part of dH.

@@ -132,8 +132,15 @@ __device__ __forceinline__ Unit decode_unit(const LmheadArgs& a, int u) {
             w.k1 = static_cast<int>((static_cast<int64_t>(kr + 1) * a.ksteps) / a.ksplit);
             u = a.split_from + w.slot % tail;
         }
-        w.rt = u / a.n_col_tiles;
-        w.t0 = u % a.n_col_tiles;
+        if (MODE == kBwdDw && a.n_row_tiles < a.n_col_tiles) {
+            // dW of a [d, V] head: the few row tiles (their operand stays in L2) vary fastest, so that the scratch is read once;
+            // the other order read all of it for every row tile
+            w.rt = u % a.n_row_tiles;
+            w.t0 = u / a.n_row_tiles;
+        } else {
+            w.rt = u / a.n_col_tiles;
+            w.t0 = u % a.n_col_tiles;
+        }
         w.t1 = w.t0 + 1;
         w.part = 0;
     } else {

@@ -15,14 +15,16 @@ namespace {
 
 // ------------------------------------------------------------------------------------------------
 // Quantisation of the rows of a bf16 matrix: E4M3 with an fp32 scale per 128 / 64 / 32 elements or per tensor, or
-// microscaling FP8 / FP4 (E8M0 scale per 32).  Streaming kernels, bound by HBM (3 bytes per element): a CTA covers 8 warps x
-// RPW rows x 1024 columns, a lane holds 8 consecutive values per 16-byte load, four loads per row segment.  Measured on a
-// 151936 x 4096 head (copy bandwidth 6.5 TB/s): block 128 5.9 TB/s with the 48 registers of five CTAs per SM (5.1 with the 69
-// the compiler would take, 5.6 with 40; a persistent form with the next segment prefetched 4.3 to 4.9), microscaling FP8
-// 6.4 TB/s with 64 registers.  Small matrices take RPW = 1: four times the CTAs, no serial chain of rows in a warp.
+// microscaling FP8 / FP4 (E8M0 scale per 32).  Streaming kernels, bound by HBM (3 bytes per element) and close behind it by
+// instruction issue: a CTA covers 4 warps x RPW rows x 1024 columns, a lane holds 8 consecutive values per 16-byte load, four
+// loads per row segment.  Measured back to back on a 151936 x 4096 head (copy bandwidth 6.5 TB/s): block 128 380 -> 302 us
+// (6.3 TB/s) with one residual correction instead of two and the maxima of two loads per shuffle; ten CTAs of four warps per
+// SM (48 registers) against five of eight 302 / 305, four 311, six 337, eight 385; microscaling FP8 305, FP4 272 us; a
+// persistent form with the next segment prefetched 4.3 to 4.9 TB/s.  Small matrices take RPW = 1: four times the CTAs, no
+// serial chain of rows in a warp.
 // ------------------------------------------------------------------------------------------------
 constexpr int kQCols = 1024;
-constexpr int kQThreads = 256;
+constexpr int kQThreads = 128;
 constexpr int kQIters = kQCols / 256;      // 16-byte loads per lane and row segment
 constexpr int kQWarps = kQThreads / 32;
 
@@ -36,15 +38,18 @@ __device__ __forceinline__ uint16_t cvt_e4m3x2(float hi, float lo) {
 // be inlined eight times into every copy of the hot loop.
 __device__ __noinline__ float slow_div(float x, float s) { return __fdiv_rn(x, s); }
 
-// amax of the block a lane belongs to, on the bf16 bit patterns: |x| is the pattern without its sign bit, and patterns
-// of non-negative values order like the values, so packed 16-bit unsigned maxima do the work of eight float compares
+// Block maxima of two 16-byte loads at once, on the bf16 bit patterns: |x| is the pattern without its sign bit, and patterns
+// of non-negative values order like the values, so packed 16-bit unsigned maxima do the work of eight float compares.
+// Low half: the maximum over the lane's block in a, high half: in b.
 template <int BLOCK>
-__device__ __forceinline__ uint32_t block_amax_bits(const uint4 raw) {
+__device__ __forceinline__ uint32_t block_amax_pair(const uint4 a, const uint4 b) {
     constexpr int kLanesPerBlock = BLOCK / 8;
-    uint32_t m = __vmaxu2(__vmaxu2(raw.x & 0x7FFF7FFFu, raw.y & 0x7FFF7FFFu), __vmaxu2(raw.z & 0x7FFF7FFFu, raw.w & 0x7FFF7FFFu));
-    m = max(m & 0xFFFFu, m >> 16);
+    constexpr uint32_t k = 0x7FFF7FFFu;
+    const uint32_t ma = __vmaxu2(__vmaxu2(a.x & k, a.y & k), __vmaxu2(a.z & k, a.w & k));
+    const uint32_t mb = __vmaxu2(__vmaxu2(b.x & k, b.y & k), __vmaxu2(b.z & k, b.w & k));
+    uint32_t m = __vmaxu2(__byte_perm(ma, mb, 0x5410), __byte_perm(ma, mb, 0x7632));
 #pragma unroll
-    for (int off = 1; off < kLanesPerBlock; off <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
+    for (int off = 1; off < kLanesPerBlock; off <<= 1) m = __vmaxu2(m, __shfl_xor_sync(0xffffffffu, m, off));
     return m;
 }
 
@@ -52,28 +57,30 @@ __device__ __forceinline__ uint32_t block_amax_bits(const uint4 raw) {
 __device__ __forceinline__ uint2 quantize_values(const uint4 raw, float s, float y) {
     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
     float v[8], qv[8];
+    uint2 signs = make_uint2(0, 0);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         v[2 * i] = __uint_as_float(w[i] << 16);
         v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
     if (s > 0x1p-100f && s < 0x1p100f) {
-        // Correctly rounded x / s from the correctly rounded reciprocal y = RN(1/s), two values per instruction (the packed
-        // fp32 forms round each half like the scalar ones): two residual corrections with fused multiply-adds; the first
-        // makes the quotient faithful, and a faithful quotient corrected once more with the exact residual is the
-        // round-to-nearest quotient (Markstein's division theorem).  |x / s| <= 448 here, so nothing overflows; a quotient
-        // that underflows encodes to zero either way; the sign of x is restored explicitly because a zero residual sum would
-        // turn -0 into +0.
+        // x / s from the correctly rounded reciprocal y = RN(1/s), two values per instruction: q0 = RN(x y) is within 2^-23 of
+        // x / s, and q1 = RN(q0 + r y) with the residual r = x - s q0 rounds a value within 2^-46 of it.  The code of q1 is that
+        // of the correctly rounded quotient: they could only differ where a half-ulp neighbour h of an E4M3 midpoint lies
+        // within 2^-46 of x / s.  With S (24 bits) and X (8) the significands of s and x and M 2^20 +- 1, 16 <= M < 32, that of h,
+        // |S (M 2^20 +- 1) - X 2^40| <= 8 forces S = a 2^20 + b with |b| <= 8 and b M = -+ a, a <= 16: only S = 2^24 - 1, M = 16,
+        // where q1 is right (checked in exact arithmetic).  |x / s| <= 448, so nothing overflows; a quotient that underflows
+        // encodes to zero either way.  The sign is put back into the codes because a zero residual sum turns -0 into +0.
         const F2 ys = {y, y}, ns = {-s, -s};
 #pragma unroll
         for (int i = 0; i < 8; i += 2) {
             const F2 x = {v[i], v[i + 1]};
             F2 q = mul2(x, ys);
             q = fma2(fma2(ns, q, x), ys, q);
-            q = fma2(fma2(ns, q, x), ys, q);
-            qv[i] = copysignf(q.x, x.x);
-            qv[i + 1] = copysignf(q.y, x.y);
+            qv[i] = q.x;
+            qv[i + 1] = q.y;
         }
+        signs = make_uint2(__byte_perm(w[0], w[1], 0x7531) & 0x80808080u, __byte_perm(w[2], w[3], 0x7531) & 0x80808080u);
     } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i) qv[i] = slow_div(v[i], s);      // rare: scale outside the safe exponent range
@@ -81,6 +88,8 @@ __device__ __forceinline__ uint2 quantize_values(const uint4 raw, float s, float
     uint2 out;
     out.x = static_cast<uint32_t>(cvt_e4m3x2(qv[1], qv[0])) | (static_cast<uint32_t>(cvt_e4m3x2(qv[3], qv[2])) << 16);
     out.y = static_cast<uint32_t>(cvt_e4m3x2(qv[5], qv[4])) | (static_cast<uint32_t>(cvt_e4m3x2(qv[7], qv[6])) << 16);
+    out.x |= signs.x;
+    out.y |= signs.y;
     return out;
 }
 
@@ -104,7 +113,7 @@ __device__ __forceinline__ void walk_rows(const __nv_bfloat16* __restrict__ x, i
     }
 }
 
-// FlagsJob by blocks of 256 threads: one warp per 128-row tile.
+// FlagsJob by blocks of kQThreads threads: one warp per 128-row tile.
 constexpr int kFlagTiles = kQThreads / 32;
 inline unsigned flag_blocks(const FlagsJob& f) { return static_cast<unsigned>(((f.T + 127) / 128 + kFlagTiles - 1) / kFlagTiles); }
 __device__ __forceinline__ void run_flags(const FlagsJob& f, unsigned block, unsigned nblocks) {
@@ -131,7 +140,7 @@ __global__ void __launch_bounds__(kQThreads) flags_kernel(const FlagsJob f) {
 
 // Blocks 0 .. n0 - 1 work on job0, the next n1 on job1, the rest on the flags.
 template <int BLOCK, int RPW>
-__global__ void __launch_bounds__(kQThreads, 5) quantize_kernel(const QuantJob job0, const QuantJob job1, unsigned n0, unsigned n1,
+__global__ void __launch_bounds__(kQThreads, 10) quantize_kernel(const QuantJob job0, const QuantJob job1, unsigned n0, unsigned n1,
                                                                 unsigned tiles_x, int64_t cols, const FlagsJob flags) {
     constexpr int kLanesPerBlock = BLOCK / 8;
     constexpr int kBlocksPerTile = kQCols / BLOCK;
@@ -152,30 +161,22 @@ __global__ void __launch_bounds__(kQThreads, 5) quantize_kernel(const QuantJob j
     const int lane = threadIdx.x & 31;
     const int64_t row0 = static_cast<int64_t>(tile / tiles_x) * kRows, col0 = static_cast<int64_t>(tile % tiles_x) * kQCols;
     walk_rows<RPW>(x, rows, cols, ld, row0, col0, [&](int64_t row, const uint4 (&raw)[kQIters]) {
-        // block maxima of the four loads, then the scales of all the segment's blocks at once: lane L derives scale and
-        // reciprocal of block L (one divergent region per segment instead of one per load)
+        // block maxima of the four loads, then lane L of every block's lanes derives scale and reciprocal for load L % 4
         constexpr int kBlkPerIt = 32 / kLanesPerBlock;
-        constexpr int kBlkPerRow = kQIters * kBlkPerIt;
-        static_assert(kBlkPerRow <= 32, "one lane per block of the segment");
-        uint32_t mine = 0;
-#pragma unroll
-        for (int it = 0; it < kQIters; ++it) {
-            const uint32_t m = block_amax_bits<BLOCK>(raw[it]);
-            const uint32_t got = __shfl_sync(0xffffffffu, m, (lane % kBlkPerIt) * kLanesPerBlock);
-            if (lane / kBlkPerIt == it) mine = got;
-        }
+        const uint32_t m01 = block_amax_pair<BLOCK>(raw[0], raw[1]), m23 = block_amax_pair<BLOCK>(raw[2], raw[3]);
+        static_assert(kQIters == 4 && kLanesPerBlock >= 4, "a lane per load in every block");
+        const uint32_t mine = ((lane & 2) ? m23 : m01) >> ((lane & 1) ? 16 : 0) << 16;
         float s_mine = 1.0f, y_mine = 1.0f;
-        if (lane < kBlkPerRow && mine != 0u) {
-            s_mine = __fdiv_rn(__uint_as_float(mine << 16), 448.0f);
+        if (mine != 0u) {
+            s_mine = __fdiv_rn(__uint_as_float(mine), 448.0f);
             y_mine = __frcp_rn(s_mine);
         }
-        if (lane < kBlkPerRow) sc[lane][static_cast<int>(row - row0)] = s_mine;
+        if (lane % kLanesPerBlock < 4) sc[(lane & 3) * kBlkPerIt + lane / kLanesPerBlock][static_cast<int>(row - row0)] = s_mine;
 #pragma unroll
         for (int it = 0; it < kQIters; ++it) {
             const int64_t col = col0 + it * 256 + lane * 8;
-            const int blk = it * kBlkPerIt + lane / kLanesPerBlock;
-            const float s = __shfl_sync(0xffffffffu, s_mine, blk);
-            const float y = __shfl_sync(0xffffffffu, y_mine, blk);
+            const float s = __shfl_sync(0xffffffffu, s_mine, it, kLanesPerBlock);
+            const float y = __shfl_sync(0xffffffffu, y_mine, it, kLanesPerBlock);
             if (row < rows && col < cols) *reinterpret_cast<uint2*>(codes + row * ldq + col) = quantize_values(raw[it], s, y);
         }
     });
@@ -247,10 +248,9 @@ __global__ void __launch_bounds__(256) quantize_cols_kernel(const __nv_bfloat16*
                 const uint32_t word = w[16 * g + 2 * p + i];
                 const F2 v = {__uint_as_float(word << 16), __uint_as_float(word & 0xFFFF0000u)};
                 if (fast) {                                  // as in quantize_values, both columns at once
-                    F2 t = mul2(v, y);
-                    t = fma2(fma2(ns, t, v), y, t);
-                    t = fma2(fma2(ns, t, v), y, t);
-                    q[i] = F2{copysignf(t.x, v.x), copysignf(t.y, v.y)};
+                    const F2 t = mul2(v, y);
+                    const F2 u = fma2(fma2(ns, t, v), y, t);
+                    q[i] = F2{copysignf(u.x, v.x), copysignf(u.y, v.y)};
                 } else {
                     q[i] = F2{slow_div(v.x, s.x), slow_div(v.y, s.y)};
                 }
@@ -312,11 +312,13 @@ __global__ void __launch_bounds__(kQThreads) quantize_mx_kernel(const __nv_bfloa
             if (col0 / 128 + i % 8 < nk4) *scale_word(rows + i / 8, col0 / 128 + i % 8) = 0x7F7F7F7Fu;
     walk_rows<RPW>(x, rows, cols, ld, row0, col0, [&](int64_t row, const uint4 (&raw)[kQIters]) {
             if (row >= rows) return;
+            uint32_t pair = 0;
 #pragma unroll
             for (int it = 0; it < kQIters; ++it) {
+                if (it % 2 == 0) pair = block_amax_pair<32>(raw[it], raw[it + 1]);
                 const int64_t col = col0 + it * 256 + lane * 8;
                 const uint32_t w[4] = {raw[it].x, raw[it].y, raw[it].z, raw[it].w};
-                const uint32_t m = block_amax_bits<32>(raw[it]);
+                const uint32_t m = it % 2 == 0 ? pair & 0xFFFFu : pair >> 16;
                 const int e = static_cast<int>(m >> 7);         // biased exponent of amax (0 for zero and subnormals)
                 const int code = m == 0u ? 127 : max(e - (FP4 ? 2 : 8), 0);
                 const float mult = __uint_as_float(static_cast<uint32_t>(254 - code) << 23);      // 2^(127 - code), exact

@@ -97,3 +97,24 @@ def test_kept_exponentials_match_the_oracle(rows, dv):
     for r in range(0, T, 128):
         assert np.linalg.norm(dH[r:r + 128] - ref["dH"][r:r + 128]) <= DH_REL * np.linalg.norm(ref["dH"][r:r + 128]), r
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("V", [40, 64, 264, 520, 832])
+def test_d_by_v_head_at_the_edges_of_the_column_blocks(V):
+    """Heads stored [d, V] narrower than a 64-column block, and with whole and partial blocks and tiles at their end: the same
+    log-probs bit for bit as the [V, d] form, and dH within the rounding of bf16 (2^-8) of it."""
+    import paper_2605_13907_b200 as ais
+    d, P, G = 256, 1, 4
+    w = workloads.scaled(workloads.WORKLOADS["tiny"], d=d, V=V, P=P, G=G, lengths="uniform:30:80", w_std=d ** -0.5, seed=303)
+    b = workloads.make_batch(w, device="cpu")
+    out = []
+    for dv in (False, True):
+        step = ais.AisStep(b.T, d, V, P, G, w.block, w_layout=ais.W_DV if dv else ais.W_VD)
+        W = (b.W.t().contiguous() if dv else b.W).cuda()
+        step.step(b.H.cuda(), W, b.tokens.cuda(), b.mask.cuda(), b.seq_offsets.cuda(), torch.tensor([1.0, 0.0, 0.0, 1.0]).cuda())
+        torch.cuda.synchronize()
+        assert int(step.status.item()) == 0
+        out.append(step)
+    assert torch.equal(out[0].lp_train, out[1].lp_train) and torch.equal(out[0].lp_roll, out[1].lp_roll)
+    a, c = out[0].dH.double(), out[1].dH.double()
+    assert float((a - c).norm()) <= 2 ** -8 * float(a.norm())
