@@ -96,21 +96,35 @@ bool make_tmap_blocks(CUtensorMap* map, const void* base, uint64_t dim0, uint64_
 // wave 2.44 ms, 22 in three better filled ones 2.75; 58,142 rows at d = 5120: 7 ranges 58.1 ms, 11 61.5).  The FP8 block
 // pass does not reach the cap and takes the balance (11 ranges 48.4 ms, 4 52.3).  From below the number is bounded by L2:
 // the hidden rows of the row tiles in flight are read again for every column tile and should take no more than 40 MB of it.
-int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most, bool pairs) {
-    if (row_tiles < 1) row_tiles = 1;
+PassPlan plan_kind(TileKind kind, int64_t rows, int V, int d, int most, int forced, double* cost) {
+    const int unit_rows = kind == kTileOne ? kBM : kPairRows, tile_cols = kind == kTileBlock ? kPairCols : kBN;
+    const int64_t units = rows > 0 ? (rows + unit_rows - 1) / unit_rows : 1;
+    const int col_tiles = (V + tile_cols - 1) / tile_cols;
     if (most > col_tiles) most = col_tiles;
     if (most < 1) most = 1;
     int best = 1;
     double best_cost = 0.0;
     for (int s = 1; s <= most; ++s) {
+        if (forced > 0 && s != (forced < most ? forced : most)) continue;
         int64_t in_flight = kSms / s > 0 ? kSms / s : 1;
-        if (in_flight > row_tiles) in_flight = row_tiles;
-        if (in_flight * 2 * kBM * d > (int64_t(40) << 20) && s < most) continue;
-        const int64_t waves = (row_tiles * s + kSms - 1) / kSms;
-        const double cost = static_cast<double>(waves) * ((col_tiles + s - 1) / s) * (1.0 + s / (pairs ? 400.0 : 120.0));
-        if (best_cost == 0.0 || cost < best_cost) { best = s; best_cost = cost; }
+        if (in_flight > units) in_flight = units;
+        if (in_flight * (unit_rows / kBM) * d * (kind == kTileBlock ? 128 : 256) > (int64_t(40) << 20) && s < most && forced <= 0) continue;
+        const int64_t waves = (units * s + kSms - 1) / kSms;
+        const double c = static_cast<double>(waves) * ((col_tiles + s - 1) / s) * (1.0 + s / (kind == kTileBlock ? 400.0 : 120.0));
+        if (best_cost == 0.0 || c < best_cost) { best = s; best_cost = c; }
     }
-    return best;
+    // clocks of a tile: 512 per stage and row tile on the tensor cores at best.  One row tile: 620, and no less than its epilogue
+    // takes; two: 1,040 plus what the skew at the ends of a tile leaves exposed.
+    const double stages = d / 64.0;
+    const double tile = kind == kTileTwo ? fmax(1040.0 * stages + 700.0, 7500.0) : fmax(620.0 * stages, 3500.0);
+    if (cost) *cost = best_cost * tile;
+    return {kind == kTileTwo, best, unit_rows, tile_cols};
+}
+
+PassPlan plan_pass(int64_t rows, int V, int d, int most, int forced) {
+    double one = 0.0, two = 0.0;
+    const PassPlan a = plan_kind(kTileOne, rows, V, d, most, forced, &one), b = plan_kind(kTileTwo, rows, V, d, most, forced, &two);
+    return two < one ? b : a;
 }
 
 }  // namespace ais
@@ -167,13 +181,11 @@ int check_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, int bl
     return AIS_OK;
 }
 
-// vocab_chunk asks for its own ranges (at most 64); otherwise the pass gets what plan_ranges finds best.
-int pick_nsplit(const ais_shape* s, const ais_params* p, int64_t row_tiles, int n_col_tiles, bool pairs = false) {
-    if (p->vocab_chunk <= 0) return plan_ranges(row_tiles, n_col_tiles, s->d, kMaxRanges, pairs);
-    int nsplit = (s->V + p->vocab_chunk - 1) / p->vocab_chunk;
-    if (nsplit > 64) nsplit = 64;
-    if (nsplit > n_col_tiles) nsplit = n_col_tiles;
-    return nsplit < 1 ? 1 : nsplit;
+// vocab_chunk asks for its own number of ranges (at most 64); 0: the plan decides.
+int forced_ranges(const ais_shape* s, const ais_params* p) {
+    if (p->vocab_chunk <= 0) return 0;
+    const int n = (s->V + p->vocab_chunk - 1) / p->vocab_chunk;
+    return n > 64 ? 64 : n;
 }
 
 // dH: the last, partial wave of 256 x 256 output tiles would leave most SMs idle for the length of a whole contraction
@@ -201,8 +213,7 @@ constexpr size_t kPaceRingBytes = kPaceRing * sizeof(uint32_t);
 
 struct Layout {
     int64_t t_ld;          // padded length of per-row vectors
-    int nsplit, nsplit_pair;   // vocabulary ranges: one-row-tile passes, two-row-tile FP8 pass
-    int nparts;
+    PassPlan train, roll;  // how the two forward passes split
     size_t off_part[2], part_bytes;               // forward partials of the trainer and the rollout pass: max, sum, target planes
     size_t off_diag;                              // reduction partials (doubles)
     size_t off_flags;                             // one byte per 128-row tile: anything to compute there?
@@ -222,11 +233,14 @@ struct Layout {
 Layout make_layout(const ais_shape* s, const ais_params* p) {
     Layout L;
     L.t_ld = static_cast<int64_t>(align_up(static_cast<size_t>(s->T > 0 ? s->T : 1), 64));
-    L.nsplit = pick_nsplit(s, p, (s->T + kBM - 1) / kBM, (s->V + kBN - 1) / kBN);
-    L.nsplit_pair = pick_nsplit(s, p, (s->T + kPairRows - 1) / kPairRows, (s->V + kPairCols - 1) / kPairCols, true);
-    L.nparts = 2 * L.nsplit > kPairParts * L.nsplit_pair ? 2 * L.nsplit : kPairParts * L.nsplit_pair;
+    const int forced = forced_ranges(s, p);
+    L.train = plan_pass(s->T, s->V, s->d, kMaxRanges, forced);
+    L.roll = s->fp8_block > 0    ? plan_kind(kTileBlock, s->T, s->V, s->d, kMaxRanges, forced, nullptr)
+             : s->fp8_block == 0 ? plan_pass(s->T, s->V, s->d / 2, kMaxRanges, forced)
+                                 : plan_kind(kTileOne, s->T, s->V, s->d, kMaxRanges, forced, nullptr);
+    const int nparts = L.train.parts() > L.roll.parts() ? L.train.parts() : L.roll.parts();
     size_t off = 0;
-    L.part_bytes = align_up(static_cast<size_t>(L.nparts) * L.t_ld * sizeof(float), 256);
+    L.part_bytes = align_up(static_cast<size_t>(nparts) * L.t_ld * sizeof(float), 256);
     for (int i = 0; i < 2; ++i) { L.off_part[i] = off; off += 3 * L.part_bytes; }
     L.off_flags = off;  off += align_up(static_cast<size_t>(L.t_ld / kBM + 2), 256);
     L.off_pace = off;   off += 2 * kPaceRingBytes;
@@ -476,16 +490,19 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
         LmheadArgs a;
         CUtensorMap tmA, tmB, tmSA, tmSB;
         int mode, units, ctas;
+        bool two;
     } pass[2] = {};
     CombineJob jobs[2];
     int n = 0;
     bool paced = false;
-    auto add = [&](int mode, int64_t rows_per_tile, int cols_per_tile, int nsplit, int ksteps, float* lp, float* lse) -> Pass& {
+    auto add = [&](int mode, const PassPlan& plan, int ksteps, float* lp, float* lse) -> Pass& {
         Pass& p = pass[n];
         p.mode = mode;
+        p.two = plan.two;
         p.a = base;
-        p.a.n_row_tiles = static_cast<int32_t>((T + rows_per_tile - 1) / rows_per_tile);
-        p.a.n_col_tiles = static_cast<int32_t>((V + cols_per_tile - 1) / cols_per_tile);
+        const int nsplit = plan.ranges;
+        p.a.n_row_tiles = static_cast<int32_t>((T + plan.unit_rows - 1) / plan.unit_rows);
+        p.a.n_col_tiles = static_cast<int32_t>((V + plan.tile_cols - 1) / plan.tile_cols);
         p.a.nsplit = nsplit;
         p.a.ksteps = ksteps;
         p.a.sgroups = 1;
@@ -500,7 +517,7 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
         // passes come one after the other: CTAs that start early wait for the rest of their launch in the pacing ring
         // (9,217 rows, both passes: 16.32 ms overlapped, 16.26 not)
         p.a.overlap = n > 0 && pass[0].ctas + p.ctas <= num_sms ? 1 : 0;
-        jobs[n] = {p.a.part_m, p.a.part_s, p.a.part_z, (mode == kFwdFp8 ? kPairParts : 2) * nsplit, lp, lse};
+        jobs[n] = {p.a.part_m, p.a.part_s, p.a.part_z, plan.parts(), lp, lse};
         ++n;
         return p;
     };
@@ -509,12 +526,12 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
         // W [V, d]: K-major boxes of 64 hidden units x 256 vocabulary rows.  W [d, V]: the vocabulary is the contiguous
         // axis, four blocks of 64 vocabulary columns x 64 hidden units per copy, and single boxes for the last tile
         const bool keep = fuse.keep_rows > 0;
-        Pass& p = add(keep ? (dv ? kFwdKeepDv : kFwdKeep) : dv ? kFwdBf16Dv : kFwdBf16, kBM, kBN, L.nsplit, shape->d / 64, lp_train, lse_train);
+        Pass& p = add(keep ? (dv ? kFwdKeepDv : kFwdKeep) : dv ? kFwdBf16Dv : kFwdBf16, L.train, shape->d / 64, lp_train, lse_train);
         p.a.U = reinterpret_cast<__nv_bfloat16*>(ws + L.off_u);
         p.a.ldU = L.ldU;
         p.a.block_tiles = static_cast<int32_t>(V / kBN);
-        p.a.keep_tiles = static_cast<int32_t>((fuse.keep_rows + kBM - 1) / kBM);
-        maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, H, d, T, shape->ldh * 2, 64, kBM, CU_TENSOR_MAP_SWIZZLE_128B) &&
+        p.a.keep_rows = fuse.keep_rows;
+        maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, H, d, T, shape->ldh * 2, 64, L.train.unit_rows, CU_TENSOR_MAP_SWIZZLE_128B) &&
                 (dv ? make_tmap_blocks(&p.tmB, W, whole_blocks(V), d, shape->ldw * 2) &&
                           make_tmap(&p.tmSA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, V, d, shape->ldw * 2, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B)
                     : make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, d, V, shape->ldw * 2, 64, kBN, CU_TENSOR_MAP_SWIZZLE_128B));
@@ -524,19 +541,19 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
         // epilogue.  Either way the whole contraction stays in tensor memory.  FP4 codes are two per byte: the maps see
         // d / 2 bytes per row with half the row stride.
         const int64_t kb = fp4 ? d / 2 : d;
-        Pass& p = add(per_tensor ? kFwdFp8T : fp4 ? kFwdMx4 : kFwdMx, kBM, kBN, L.nsplit, static_cast<int>(kb / 128), lp_roll, lse_roll);
+        Pass& p = add(per_tensor ? kFwdFp8T : fp4 ? kFwdMx4 : kFwdMx, L.roll, static_cast<int>(kb / 128), lp_roll, lse_roll);
         p.a.sf_a = static_cast<const uint8_t*>(sH_);
         p.a.sf_b = static_cast<const uint8_t*>(sW_);
         p.a.nk4 = shape->d / 128;
         p.a.scale_a = sH;
         p.a.scale_b = sW;
-        maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, kb, T, fp4 ? shape->ldh / 2 : shape->ldh, 128, kBM, CU_TENSOR_MAP_SWIZZLE_128B) &&
+        maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, kb, T, fp4 ? shape->ldh / 2 : shape->ldh, 128, L.roll.unit_rows, CU_TENSOR_MAP_SWIZZLE_128B) &&
                 make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, qW, kb, V, fp4 ? shape->ldw / 2 : shape->ldw, 128, kBN, CU_TENSOR_MAP_SWIZZLE_128B);
     } else if (do_roll) {
         // tiles of 256 rows x 128 columns
         const int64_t nkb = d / shape->fp8_block;
         const int sg = 128 / shape->fp8_block;
-        Pass& p = add(kFwdFp8, kPairRows, kPairCols, L.nsplit_pair, shape->d / 128, lp_roll, lse_roll);
+        Pass& p = add(kFwdFp8, L.roll, shape->d / 128, lp_roll, lse_roll);
         p.a.sgroups = sg;
         maps &= make_tmap(&p.tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, qH, d, T, shape->ldh, 128, kPairRows, CU_TENSOR_MAP_SWIZZLE_128B) &&
                 make_tmap(&p.tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, qW, d, V, dv ? d : shape->ldw, 128, kPairCols, CU_TENSOR_MAP_SWIZZLE_128B) &&
@@ -548,7 +565,8 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
     if ((fuse.nquant > 0 ? launch_quantize(fuse.quant, fuse.nquant, d, shape->fp8_block, &flags, s) : launch_flags(flags, s)) != cudaSuccess)
         return AIS_ERR_DEVICE;
     for (int i = 0; i < n; ++i)
-        if (launch_lmhead(pass[i].mode, pass[i].tmA, pass[i].tmB, pass[i].tmSA, pass[i].tmSB, pass[i].a, pass[i].ctas, s) != cudaSuccess)
+        if ((pass[i].two ? launch_lmhead_pair(pass[i].mode, pass[i].tmA, pass[i].tmB, pass[i].tmSA, pass[i].a, pass[i].ctas, s)
+                         : launch_lmhead(pass[i].mode, pass[i].tmA, pass[i].tmB, pass[i].tmSA, pass[i].tmSB, pass[i].a, pass[i].ctas, s)) != cudaSuccess)
             return AIS_ERR_DEVICE;
     if (launch_combine(jobs, n, L.t_ld, mask, T, dev_status, fuse.adv, s) != cudaSuccess) return AIS_ERR_DEVICE;
     return AIS_OK;
@@ -708,7 +726,8 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
         const int64_t rows = (shape->T - r0) < blk_rows ? (shape->T - r0) : blk_rows;
         CUtensorMap tmH;
         const __nv_bfloat16* Hc = static_cast<const __nv_bfloat16*>(H) + r0 * shape->ldh;
-        if (!make_tmap(&tmH, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Hc, d, static_cast<uint64_t>(rows), shape->ldh * 2, 64, kBM,
+        const PassPlan plan = plan_pass(rows, shape->V, shape->d, kMaxRanges, forced_ranges(shape, params));
+        if (!make_tmap(&tmH, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Hc, d, static_cast<uint64_t>(rows), shape->ldh * 2, 64, plan.unit_rows,
                        CU_TENSOR_MAP_SWIZZLE_128B))
             return AIS_ERR_DEVICE;
         LmheadArgs a;
@@ -716,7 +735,6 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
         a.wait_cycles = wait_cycles();
         a.rows = rows;
         a.row0 = r0;
-        a.n_row_tiles = static_cast<int32_t>((rows + kBM - 1) / kBM);
         a.tokens = tokens;
         a.mask = mask;
         a.lse = lse_train;
@@ -738,14 +756,18 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
         }
         a.ncols = shape->V;
         a.n_col_tiles = (shape->V + kBN - 1) / kBN;
-        a.nsplit = pick_nsplit(shape, params, a.n_row_tiles, a.n_col_tiles);
+        a.n_row_tiles = static_cast<int32_t>((rows + plan.unit_rows - 1) / plan.unit_rows);
+        a.nsplit = plan.ranges;
         a.ksteps = shape->d / 64;
         a.block_tiles = shape->V / kBN;
         int units = a.n_row_tiles * a.nsplit;
         int ctas = units < num_sms ? units : num_sms;
         arm_pace(a, ws, L, (a.n_col_tiles + a.nsplit - 1) / a.nsplit, units, ctas, pass, pass > 0);
         ++pass;
-        if (launch_lmhead(dv ? kBwdPDv : kBwdP, tmH, tmW_k, dv ? tmW_tail : tmH, tmW_k, a, ctas, s) != cudaSuccess)
+        const CUtensorMap& tail_map = dv ? tmW_tail : tmH;
+        const int mode = dv ? kBwdPDv : kBwdP;
+        if ((plan.two ? launch_lmhead_pair(mode, tmH, tmW_k, tail_map, a, ctas, s) : launch_lmhead(mode, tmH, tmW_k, tail_map, tmW_k, a, ctas, s)) !=
+            cudaSuccess)
             return AIS_ERR_DEVICE;
         // dH = c (.) (U W)
         a.tile_active = ws + L.off_flags;

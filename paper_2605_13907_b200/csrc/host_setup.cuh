@@ -18,9 +18,19 @@ bool make_tmap(CUtensorMap* map, CUtensorMapDataType dtype, const void* base, ui
 // the other in shared memory).  dim0 has to be a multiple of 64, or the rows long enough to hold the rounded-up width.
 bool make_tmap_blocks(CUtensorMap* map, const void* base, uint64_t dim0, uint64_t dim1, uint64_t stride1_bytes);
 
-// How many vocabulary ranges a forward or recompute pass over `row_tiles` x `col_tiles` tiles splits each row tile into,
-// at most `most`; `d` is the hidden size; `pairs`: the FP8 pass with tiles of two row tiles x 128 columns.
-int plan_ranges(int64_t row_tiles, int col_tiles, int d, int most, bool pairs = false);
+// How a forward or recompute pass over `rows` x `V` splits: row tiles per CTA and vocabulary ranges per unit of rows (at most
+// `most`, or exactly `forced` if that is positive).
+enum TileKind { kTileOne, kTileTwo, kTileBlock };   // 128 x 256 (lmhead.cu), 256 x 256 (lmhead_pair.cu), 256 x 128 (lmhead_fp8.cu)
+struct PassPlan {
+    bool two;          // kTileTwo
+    int ranges;
+    int unit_rows;     // rows of a unit
+    int tile_cols;
+    int parts() const { return 2 * ranges; }
+};
+PassPlan plan_kind(TileKind kind, int64_t rows, int V, int d, int most, int forced, double* cost);
+// The better of kTileOne and kTileTwo.
+PassPlan plan_pass(int64_t rows, int V, int d, int most, int forced);
 
 // Bound of the kernels' device-side waits in clock ticks as set by ais_set_wait_cycles (0 = the kernels' default).
 int64_t wait_cycles();

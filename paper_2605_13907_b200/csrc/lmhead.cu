@@ -19,9 +19,6 @@ namespace ais {
 
 namespace {
 
-// |reference| (log2 units) up to which the kept exponentials are relative to 0; just above exp_form's largest lse
-constexpr float kKeepRange = 86.0f;
-
 constexpr int threads_of(int mode) { return (mode == kFwdMx || mode == kFwdMx4) ? kMxThreads : kThreads; }
 
 template <int MODE>
@@ -60,7 +57,6 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int num_units = count_units<BASE>(a);
-    constexpr bool KEEP = (MODE == kFwdKeep || MODE == kFwdKeepDv);
     const bool gated = BASE == kBwdP && a.gate != nullptr;
     if (gated) {
         enter_pass(a);
@@ -406,32 +402,9 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                 tb.advance();
                 continue;
             }
-            const int64_t lrow = static_cast<int64_t>(w.rt) * kBM + r_in_tile;   // row inside this launch
-            const bool row_ok = lrow < a.rows;
-            const int64_t grow = a.row0 + lrow;
-            int y = -1;
-            bool valid = false;
-            if (row_ok) {
-                y = a.tokens[grow];
-                valid = a.mask[grow] != 0;
-                if (valid && (y < 0 || y >= a.ncols)) { flags |= AIS_FLAG_TOKEN_RANGE; y = -1; }
-            }
-            float m2 = kNegBig, s = 0.f, zy = -INFINITY;       // log2-domain running max, sum, target logit
+            RowState r = begin_row<MODE>(a, static_cast<int64_t>(w.rt) * kBM + r_in_tile, flags);
+            const bool store = r.in && (BASE == kBwdP || r.lrow < a.keep_rows);
             const float tscale = (MODE == kFwdFp8T) ? (*a.scale_a) * (*a.scale_b) : 1.f;
-            float lse2 = 0.f;
-            // recompute: U = mul (e^(z - off) - onehot) in plain form (off = lse, mul = c), mul = 1, off = 0 and `target` at
-            // the target column in exponent form
-            float mul = 0.f, target = 0.f;
-            bool ef = false;
-            if (BASE == kBwdP && row_ok) {
-                const float lse = a.lse[grow];
-                mul = a.coef[grow];
-                if (mul == 0.f) valid = false;                 // rows without gradient are written as exact zeros
-                ef = a.row_scale != nullptr && exp_form(lse);
-                if (ef) { mul = 1.f; target = exp_form_target(a.lp[grow], lse); }
-                else lse2 = lse * kLog2e;
-            }
-
             for (int t = w.t0; t < w.t1 && ok; ++t) {
                 const int col_base = t * kBN + half * 128;    // first output column of this thread's half
                 {
@@ -469,67 +442,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                             for (int i = 0; i < 32; ++i) x[i] *= tscale;
                         }
                     }
-                    if (BASE == kFwdBf16 || MODE == kFwdFp8T || MX) {
-                        if (y >= col0 && y < col0 + 32) {
-#pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                if (col0 + i == y) zy = x[i];
-                        }
-                        if (col0 + 32 > a.ncols) {
-#pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                if (col0 + i >= a.ncols) x[i] = -INFINITY;
-                        }
-                        float cm = x[0];
-#pragma unroll
-                        for (int i = 1; i < 32; ++i) cm = fmaxf(cm, x[i]);
-                        float m_new = fmaxf(m2, cm * kLog2e);
-                        // reference 0 for every row within range, so that the terms of the sum are what the scratch wants
-                        if (KEEP && fabsf(m_new) <= kKeepRange) m_new = 0.f;
-                        float add = 0.f;
-                        if (KEEP) {
-                            uint32_t pk[16];
-#pragma unroll
-                            for (int i = 0; i < 32; i += 2) {
-                                const float e0 = ex2(fmaf(x[i], kLog2e, -m_new)), e1 = ex2(fmaf(x[i + 1], kLog2e, -m_new));
-                                add += e0;
-                                add += e1;
-                                pk[i >> 1] = pack_bf16(e0, e1);
-                            }
-                            if (row_ok && w.rt < a.keep_tiles && col0 < a.ncols) {
-                                if (m_new != 0.f) {                // rare: this range of the row lies far below the rest, or above
-#pragma unroll
-                                    for (int i = 0; i < 32; i += 2)
-                                        pk[i >> 1] = pack_bf16(ex2(fmaf(x[i], kLog2e, -0.f)), ex2(fmaf(x[i + 1], kLog2e, -0.f)));
-                                }
-                                uint4* dst = reinterpret_cast<uint4*>(a.U + lrow * a.ldU + col0);
-#pragma unroll
-                                for (int j = 0; j < 4; ++j)
-                                    if (col0 + j * 8 < a.ncols) dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
-                            }
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) add += ex2(fmaf(x[i], kLog2e, -m_new));
-                        }
-                        s = fmaf(s, ex2(m2 - m_new), add);
-                        m2 = m_new;
-                    } else if (BASE == kBwdP) {
-                        if (row_ok && col0 < a.ncols) {
-                            uint32_t pk[16];
-#pragma unroll
-                            for (int i = 0; i < 32; i += 2) {
-                                float p0 = valid ? ex2(fmaf(x[i], kLog2e, -lse2)) : 0.f;
-                                float p1 = valid ? ex2(fmaf(x[i + 1], kLog2e, -lse2)) : 0.f;
-                                if (col0 + i == y) p0 = ef ? target : p0 - 1.f;
-                                if (col0 + i + 1 == y) p1 = ef ? target : p1 - 1.f;
-                                pk[i >> 1] = pack_bf16(valid ? mul * p0 : 0.f, valid ? mul * p1 : 0.f);
-                            }
-                            uint4* dst = reinterpret_cast<uint4*>(a.U + lrow * a.ldU + col0);
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                if (col0 + j * 8 < a.ncols) dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
-                        }
-                    }
+                    row_slice<MODE>(a, r, col0, x, store);
                 }
                 if (!MX) {
                     tc_fence_before();
@@ -538,12 +451,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                 }
                 tb.advance();
             }
-            if (ok && row_ok && (BASE == kFwdBf16 || MODE == kFwdFp8T || MX)) {
-                const int64_t o = static_cast<int64_t>(w.part * 2 + half) * a.part_ld + grow;
-                a.part_m[o] = m2 * kLn2;
-                a.part_s[o] = s;
-                a.part_z[o] = zy;
-            }
+            if (ok && BASE != kBwdP) end_row(a, r, w.part * 2 + half);
         }
         if (flags && a.status) atomicOr(a.status, flags);
     }
@@ -647,7 +555,7 @@ static cudaError_t prepare_mode() {
 }
 
 cudaError_t lmhead_prepare() {
-    const cudaError_t all[] = {lmhead_fp8_block_prepare(), prepare_mode<kFwdBf16>(), prepare_mode<kBwdP>(), prepare_mode<kBwdDh>(),
+    const cudaError_t all[] = {lmhead_fp8_block_prepare(), lmhead_pair_prepare(), prepare_mode<kFwdBf16>(), prepare_mode<kBwdP>(), prepare_mode<kBwdDh>(),
                                prepare_mode<kFwdFp8T>(), prepare_mode<kBwdDw>(), prepare_mode<kFwdMx>(), prepare_mode<kFwdMx4>(),
                                prepare_mode<kFwdBf16Dv>(), prepare_mode<kBwdPDv>(), prepare_mode<kBwdDhDv>(), prepare_mode<kFwdKeep>(),
                                prepare_mode<kFwdKeepDv>()};

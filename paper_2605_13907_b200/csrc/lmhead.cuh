@@ -53,7 +53,6 @@ constexpr int kDhStages = 3;
 // shared memory serves two rows of a thread
 constexpr int kPairRows = 2 * kBM;
 constexpr int kPairCols = 128;
-constexpr int kPairParts = 2;            // partial triples per row and vocabulary range: one per column group of the promotion warps
 static_assert(kDhStages * kDhStageBytes <= kStages * kStageBytes, "the dH stage ring must fit the same shared memory");
 constexpr int kNumBarriers = 3 * kStages + 4 + 1;
 // microscaling passes: per 128-byte K stage one 512-byte scale chunk for the 128 rows of A and two for the 256 rows of B
@@ -121,7 +120,7 @@ struct LmheadArgs {
     int32_t split_from;    // dH: units from here on are split along the contraction (the last, partial wave); others whole
     int32_t ksplit;        // dH: ranges of the contraction per split unit (1 = nothing is split)
     float* part_acc;       // dH: fp32 partial tiles of the split units, [slot][kPartTileFloats] (see dh_reduce_kernel)
-    int32_t keep_tiles;    // kFwdKeep: row tiles (from the first) whose exponentials go to U
+    int64_t keep_rows;     // kFwdKeep: rows (from the first) whose exponentials go to U
     const float* lp;       // recompute: log-probs of the targets (exponent form)
     const float* row_scale;   // recompute: non-NULL selects the exponent form; dH: factor of every row (0: the row is zero)
     const uint32_t* gate;  // recompute: non-NULL: run only if *gate != 0, and leave the rows of inactive tiles as they are
@@ -145,5 +144,11 @@ cudaError_t lmhead_prepare();   // sets the dynamic shared-memory attribute of e
 cudaError_t launch_lmhead_fp8_block(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,
                                     const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream);
 cudaError_t lmhead_fp8_block_prepare();
+
+// The forward and recompute passes (no microscaling) with two row tiles per CTA: n_row_tiles counts 256-row units, tmA has boxes
+// of 256 rows.
+cudaError_t launch_lmhead_pair(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB2, const LmheadArgs& args,
+                               int num_ctas, cudaStream_t stream);
+cudaError_t lmhead_pair_prepare();
 
 }  // namespace ais

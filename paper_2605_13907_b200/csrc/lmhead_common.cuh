@@ -2,6 +2,7 @@
 // register re-splitting, work-unit decoding and the test for row tiles without work.
 #pragma once
 
+#include "../../include/ais.h"
 #include "launch.cuh"
 #include "lmhead.cuh"
 #include "ptx.cuh"
@@ -186,6 +187,122 @@ __device__ __forceinline__ void enter_pass(const LmheadArgs& a) {
 // Its end, by every thread: a pass that did not wait at the start completes only after the kernel before it has.
 __device__ __forceinline__ void leave_pass(const LmheadArgs& a) {
     if (a.overlap) pdl_wait();
+}
+
+// ------------------------------------------------------------------ epilogue of the forward and recompute passes
+// One output row of a thread: what its epilogue knows about it and, in the forward passes, its streaming log-sum-exp
+// (log2-domain running reference, sum of 2^(z log2e - reference), target logit).
+// Recompute: U = mul (e^(z - off) - onehot) in plain form (off = lse, mul = c), mul = 1, off = 0 and `target` at the target
+// column in exponent form (exp_form).
+constexpr __host__ __device__ bool keep_mode(int mode) { return mode == kFwdKeep || mode == kFwdKeepDv; }
+// |reference| (log2 units) up to which the kept exponentials are relative to 0; just above exp_form's largest lse
+constexpr float kKeepRange = 86.0f;
+
+struct RowState {
+    int64_t lrow, grow;              // row inside the launch, row of the batch
+    bool in, valid;
+    int y;                           // target column, -1: none
+    float m2, s, zy;
+    float off2, mul, target;
+    bool ef;
+};
+
+template <int MODE>
+__device__ __forceinline__ RowState begin_row(const LmheadArgs& a, int64_t lrow, uint32_t& flags) {
+    constexpr int BASE = base_mode(MODE);
+    RowState r;
+    r.lrow = lrow;
+    r.in = lrow < a.rows;
+    r.grow = a.row0 + lrow;
+    r.y = -1;
+    r.valid = false;
+    r.m2 = kNegBig;
+    r.s = 0.f;
+    r.zy = -INFINITY;
+    r.off2 = r.mul = r.target = 0.f;
+    r.ef = false;
+    if (!r.in) return r;
+    r.y = a.tokens[r.grow];
+    r.valid = a.mask[r.grow] != 0;
+    if (r.valid && (r.y < 0 || r.y >= a.ncols)) { flags |= AIS_FLAG_TOKEN_RANGE; r.y = -1; }
+    if (BASE == kBwdP) {
+        const float lse = a.lse[r.grow];
+        r.mul = a.coef[r.grow];
+        if (r.mul == 0.f) r.valid = false;             // rows without gradient are written as exact zeros
+        r.ef = a.row_scale != nullptr && exp_form(lse);
+        if (r.ef) { r.mul = 1.f; r.target = exp_form_target(a.lp[r.grow], lse); }
+        else r.off2 = lse * kLog2e;
+    }
+    return r;
+}
+
+// 32 consecutive logits of the row, from column col0 on.  `store`: the row's scratch is wanted (kFwdKeep, recompute).
+template <int MODE>
+__device__ __forceinline__ void row_slice(const LmheadArgs& a, RowState& r, int col0, float (&x)[32], bool store) {
+    constexpr bool KEEP = keep_mode(MODE);
+    uint32_t pk[16];
+    if (base_mode(MODE) == kBwdP) {
+        if (!store || col0 >= a.ncols) return;
+#pragma unroll
+        for (int i = 0; i < 32; i += 2) {
+            float p0 = r.valid ? ex2(fmaf(x[i], kLog2e, -r.off2)) : 0.f;
+            float p1 = r.valid ? ex2(fmaf(x[i + 1], kLog2e, -r.off2)) : 0.f;
+            if (col0 + i == r.y) p0 = r.ef ? r.target : p0 - 1.f;
+            if (col0 + i + 1 == r.y) p1 = r.ef ? r.target : p1 - 1.f;
+            pk[i >> 1] = pack_bf16(r.valid ? r.mul * p0 : 0.f, r.valid ? r.mul * p1 : 0.f);
+        }
+    } else {
+        if (r.y >= col0 && r.y < col0 + 32) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (col0 + i == r.y) r.zy = x[i];
+        }
+        if (col0 + 32 > a.ncols) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (col0 + i >= a.ncols) x[i] = -INFINITY;
+        }
+        float cm = x[0];
+#pragma unroll
+        for (int i = 1; i < 32; ++i) cm = fmaxf(cm, x[i]);
+        float m_new = fmaxf(r.m2, cm * kLog2e);
+        // reference 0 for every row within range, so that the terms of the sum are what the scratch wants
+        if (KEEP && fabsf(m_new) <= kKeepRange) m_new = 0.f;
+        float add = 0.f;
+        if (KEEP) {
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) {
+                const float e0 = ex2(fmaf(x[i], kLog2e, -m_new)), e1 = ex2(fmaf(x[i + 1], kLog2e, -m_new));
+                add += e0;
+                add += e1;
+                pk[i >> 1] = pack_bf16(e0, e1);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) add += ex2(fmaf(x[i], kLog2e, -m_new));
+        }
+        r.s = fmaf(r.s, ex2(r.m2 - m_new), add);
+        r.m2 = m_new;
+        if (!KEEP || !store || col0 >= a.ncols) return;
+        if (m_new != 0.f) {                            // rare: this range of the row lies far below the rest, or above
+#pragma unroll
+            for (int i = 0; i < 32; i += 2)
+                pk[i >> 1] = pack_bf16(ex2(fmaf(x[i], kLog2e, -0.f)), ex2(fmaf(x[i + 1], kLog2e, -0.f)));
+        }
+    }
+    uint4* dst = reinterpret_cast<uint4*>(a.U + r.lrow * a.ldU + col0);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (col0 + j * 8 < a.ncols) dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+}
+
+// Forward passes: the row's partial triple for one vocabulary range and column half.
+__device__ __forceinline__ void end_row(const LmheadArgs& a, const RowState& r, int part) {
+    if (!r.in) return;
+    const int64_t o = static_cast<int64_t>(part) * a.part_ld + r.grow;
+    a.part_m[o] = r.m2 * kLn2;
+    a.part_s[o] = r.s;
+    a.part_z[o] = r.zy;
 }
 
 // After every role has left its loops: if the CTA gave up on a wait, the tile copies that the producer issued last

@@ -65,13 +65,14 @@ extern "C" int ais_logprob_train_static(const ais_shape* shape, const void* H, c
     const int n_col_tiles = (shape->V + kBN - 1) / kBN;
     const int64_t ld = (shape->T + 63) / 64 * 64;                  // rows of one part
     const int64_t room = static_cast<int64_t>(kStaticPlane) / (2 * ld);
-    const int nsplit = plan_ranges((shape->T + kBM - 1) / kBM, n_col_tiles, shape->d, room < kMaxRanges ? static_cast<int>(room) : kMaxRanges);
+    const PassPlan plan = plan_pass(shape->T, shape->V, shape->d, room < kMaxRanges ? static_cast<int>(room) : kMaxRanges, 0);
+    const int nsplit = plan.ranges;
     LmheadArgs a;
     memset(&a, 0, sizeof(a));
     a.wait_cycles = wait_cycles();
     a.rows = shape->T;
     a.row0 = 0;
-    a.n_row_tiles = static_cast<int32_t>((shape->T + kBM - 1) / kBM);
+    a.n_row_tiles = static_cast<int32_t>((shape->T + plan.unit_rows - 1) / plan.unit_rows);
     a.ncols = shape->V;
     a.n_col_tiles = n_col_tiles;
     a.ksteps = shape->d / 64;
@@ -86,7 +87,7 @@ extern "C" int ais_logprob_train_static(const ais_shape* shape, const void* H, c
     a.status = dev_status;
     CUtensorMap tmA, tmB;
     if (!make_tmap(&tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, H, static_cast<uint64_t>(shape->d), static_cast<uint64_t>(shape->T),
-                   shape->ldh * 2, 64, kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
+                   shape->ldh * 2, 64, plan.unit_rows, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_tmap(&tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, static_cast<uint64_t>(shape->d), static_cast<uint64_t>(shape->V),
                    shape->ldw * 2, 64, kBN, CU_TENSOR_MAP_SWIZZLE_128B))
         return AIS_ERR_DEVICE;
@@ -94,7 +95,8 @@ extern "C" int ais_logprob_train_static(const ais_shape* shape, const void* H, c
     const int units = a.n_row_tiles * nsplit;
     // Every slot of the scratch that the merge reads (parts 0 .. 2*nsplit-1, rows 0 .. T-1) is written by the
     // pass just before it, so nothing left over from an earlier call is ever read and nothing needs zeroing.
-    if (launch_lmhead(kFwdBf16, tmA, tmB, tmA, tmB, a, units < num_sms ? units : num_sms, s) != cudaSuccess)
+    const int ctas = units < num_sms ? units : num_sms;
+    if ((plan.two ? launch_lmhead_pair(kFwdBf16, tmA, tmB, tmA, a, ctas, s) : launch_lmhead(kFwdBf16, tmA, tmB, tmA, tmB, a, ctas, s)) != cudaSuccess)
         return AIS_ERR_DEVICE;
     const CombineJob job = {a.part_m, a.part_s, a.part_z, nsplit * 2, lp_train, lse_train};
     if (launch_combine(&job, 1, ld, mask, shape->T, dev_status, nullptr, s) != cudaSuccess) return AIS_ERR_DEVICE;

@@ -118,3 +118,55 @@ def test_d_by_v_head_at_the_edges_of_the_column_blocks(V):
     assert torch.equal(out[0].lp_train, out[1].lp_train) and torch.equal(out[0].lp_roll, out[1].lp_roll)
     a, c = out[0].dH.double(), out[1].dH.double()
     assert float((a - c).norm()) <= 2 ** -8 * float(a.norm())
+
+
+@pytest.mark.parametrize("variant", ["vd", "dv", "per_tensor"])
+def test_two_row_tiles_per_cta_match_the_oracle(variant):
+    """Enough row tiles for 256-row units: pairs with either row tile masked, both masked, a ragged last pair with one row tile,
+    rows outside the exponent form in one tile of a pair; the step in one call and the stages on their own."""
+    import paper_2605_13907_b200 as ais
+    d, V, P, G = 1280, 2568, 2, 4
+    block = 0 if variant == "per_tensor" else 128
+    dv = variant == "dv"
+    w = workloads.scaled(workloads.WORKLOADS["tiny"], d=d, V=V, P=P, G=G, lengths="uniform:265:285", w_std=d ** -0.5, seed=304, block=block)
+    b = workloads.make_batch(w, device="cpu")
+    T = b.T
+    assert T % 256 != 0
+    b.mask[128:256] = 0                                     # second tile of pair 0
+    b.mask[256:384] = 0                                     # first tile of pair 1
+    b.mask[512:768] = 0                                     # pair 2
+    b.W[:, 0] = 1.0
+    b.H[:, 0] = 0.0
+    b.H[900:910, 0] = 70.0                                  # second tile of pair 3: log-sum-exp near +77
+    rewards = torch.zeros(P * G)
+    rewards[::2] = 1.0
+    b.rewards = rewards
+    a = workloads.to_numpy(b)
+    ref = oais.full_path(a["H"], a["W"], a["tokens"], a["mask"], a["seq_offsets"], a["rewards"], P, G, block)
+    # every MMA step (16 of the d products, d / 16 of them) may cut the accumulator off at one unit of its last place: 2^-17 for
+    # the logits near 77, so d / 16 * 2^-17 = 6.1e-4 there; the other rows as above
+    atol = LP_ATOL + np.where(np.abs(ref["lse_train"]) > 32, d / 16 * 2.0 ** -17, 0.0)
+    W = (b.W.t().contiguous() if dv else b.W).cuda()
+    H, tok, msk, offs, rew = b.H.cuda(), b.tokens.cuda(), b.mask.cuda(), b.seq_offsets.cuda(), b.rewards.cuda()
+    step = ais.AisStep(T, d, V, P, G, block, w_layout=ais.W_DV if dv else ais.W_VD)
+
+    def check():
+        torch.cuda.synchronize()
+        assert int(step.status.item()) == 0
+        for name in ("lp_train", "lp_roll", "lse_train"):
+            assert np.all(np.abs(getattr(step, name)[:T].cpu().numpy() - ref[name]) <= atol), name
+        dH = step.dH[:T].float().cpu().numpy().astype(np.float64)
+        assert np.all(dH[a["mask"] == 0] == 0)
+        for r in range(0, T, 128):
+            assert np.linalg.norm(dH[r:r + 128] - ref["dH"][r:r + 128]) <= DH_REL * max(np.linalg.norm(ref["dH"][r:r + 128]), 1e-12), r
+
+    step.dH.fill_(7.0)
+    step.step(H, W, tok, msk, offs, rew)
+    check()
+    step.dH.fill_(7.0)
+    step.backward(H, W, tok, msk, offs)
+    check()
+    lp = torch.empty(T, device="cuda")
+    if not dv:
+        ais.logprob_train_static(step.shape, H, W, tok, msk, lp)
+        assert np.all(np.abs(lp.cpu().numpy() - ref["lp_train"]) <= atol)
