@@ -215,10 +215,10 @@ struct Layout {
     int64_t t_ld;          // padded length of per-row vectors
     PassPlan train, roll;  // how the two forward passes split
     size_t off_part[2], part_bytes;               // forward partials of the trainer and the rollout pass: max, sum, target planes
-    size_t off_diag;                              // reduction partials (doubles)
+    size_t off_diag, off_loss;                    // partial sums of the batch moments and of the loss (doubles)
     size_t off_flags;                             // one byte per 128-row tile: anything to compute there?
     size_t off_pace;                              // two rings of counters that keep the CTAs of a tensor-core launch in step
-    size_t off_ticket;                            // block counter of the batch reductions
+    size_t off_ticket;                            // counters of the loss kernel
     size_t off_coef, off_nseq;                    // backward: c_t, valid rows per sequence
     size_t off_scale, off_redo;                   // backward, exponent form: row factors, row tiles to recompute
     size_t off_seqw;                              // sequence-level variant: log weight per sequence
@@ -246,6 +246,7 @@ Layout make_layout(const ais_shape* s, const ais_params* p) {
     L.off_pace = off;   off += 2 * kPaceRingBytes;
     L.off_ticket = off; off += 256;
     L.off_diag = off;   off += align_up(static_cast<size_t>(kDiagBlocks) * kNumMoments * sizeof(double), 256);
+    L.off_loss = off;   off += align_up(static_cast<size_t>(kDiagBlocks) * 2 * sizeof(double), 256);
     L.off_coef = off;   off += align_up(static_cast<size_t>(L.t_ld) * sizeof(float), 256);
     L.off_nseq = off;   off += align_up(static_cast<size_t>(s->P) * s->G * sizeof(int32_t), 256);
     L.off_scale = off;  off += align_up(static_cast<size_t>(L.t_ld) * sizeof(float), 256);
@@ -303,7 +304,7 @@ struct Fuse {
     const QuantJob* quant = nullptr;     // log-probs: quantise these first, in the opening launch
     int nquant = 0;
     const AdvJob* adv = nullptr;         // log-probs: advantages in the merging launch; diagnostics: they are there already
-    bool rectify_later = false;          // diagnostics: the loss forms rho and w_tilde
+    TotalsJob* totals = nullptr;         // diagnostics: leave the end (alpha, rho, w_tilde) to the loss, described here
     const RectifyJob* rectify = nullptr; // loss: form them
     int64_t keep_rows = 0;               // log-probs: leave the exponentials of these rows in the scratch; loss: they are there
     const int32_t* counts = nullptr;     // loss: valid rows per sequence are there already, and so is its cleared ticket
@@ -597,13 +598,12 @@ static int diagnostics(const ais_shape* shape, const ais_params* params, const f
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int S = shape->P * shape->G;
-    uint32_t* tickets = reinterpret_cast<uint32_t*>(ws + L.off_ticket);
     if (!fuse.adv &&
-        launch_advantages({rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, tickets}, s) != cudaSuccess)
+        launch_advantages({rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, reinterpret_cast<uint32_t*>(ws + L.off_ticket)}, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
-    if (launch_diag(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag), tickets,
-                    n_valid_seq, seq_level ? reinterpret_cast<float*>(ws + L.off_seqw) : nullptr, rho, fuse.rectify_later ? nullptr : w_tilde,
-                    diag, !fuse.adv, s) != cudaSuccess)
+    if (launch_diag(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag),
+                    n_valid_seq, seq_level ? reinterpret_cast<float*>(ws + L.off_seqw) : nullptr, rho, w_tilde,
+                    diag, !fuse.adv, fuse.totals, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     return AIS_OK;
 }
@@ -632,11 +632,10 @@ int ais_diag_moments(const ais_shape* shape, const ais_params* params, const flo
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int S = shape->P * shape->G;
-    uint32_t* tickets = reinterpret_cast<uint32_t*>(ws + L.off_ticket);
-    if (launch_advantages({rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, tickets}, s) != cudaSuccess)
+    if (launch_advantages({rewards, S, shape->G, params->adv_std_norm, params->eps, adv, n_valid_seq, nullptr}, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     if (launch_moments(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag),
-                       tickets, n_valid_seq, params->seq_level_weights != 0 ? seq_logw : nullptr, moments, s) != cudaSuccess)
+                       n_valid_seq, params->seq_level_weights != 0 ? seq_logw : nullptr, moments, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     return AIS_OK;
 }
@@ -685,7 +684,7 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
     const int S = shape->P * shape->G;
     float* coef = reinterpret_cast<float*>(ws + L.off_coef);
     const int32_t* nseq = fuse.counts;
-    uint32_t* ticket = reinterpret_cast<uint32_t*>(ws + L.off_ticket) + 1;
+    uint32_t* ticket = reinterpret_cast<uint32_t*>(ws + L.off_ticket);
     if (!nseq) {
         int32_t* own = reinterpret_cast<int32_t*>(ws + L.off_nseq);
         if (launch_seq_counts(mask, seq_offsets, S, own, ticket, s) != cudaSuccess) return AIS_ERR_DEVICE;
@@ -696,7 +695,7 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
     const KeepJob keep = {reinterpret_cast<__nv_bfloat16*>(ws + L.off_u), L.ldU, fuse.keep_rows, tokens, shape->V, scale, ws + L.off_redo, ticket + 1};
     // row tiles whose gradient factors are all zero (masked rows, zero advantage) are skipped by the recompute and dH passes
     if (launch_loss_coef(lp_train, lp_old, lp_ref, params->beta_kl, mask, seq_offsets, adv, w_tilde, nseq, shape->T, S, P_norm * shape->G,
-                         params->clip_eps, reinterpret_cast<double*>(ws + L.off_diag), ticket, coef, ws + L.off_flags, ws + L.off_pace,
+                         params->clip_eps, reinterpret_cast<double*>(ws + L.off_loss), ticket, coef, ws + L.off_flags, ws + L.off_pace,
                          2 * kPaceRingBytes, loss, diag, lse_train, fuse.rectify, fuse.keep_rows > 0 ? &keep : nullptr, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     if (shape->T == 0) return AIS_OK;
@@ -885,10 +884,10 @@ int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_ar
         // the loss takes the counts from here and forms rho and w_tilde; the diagnostics' advantages have cleared its ticket
         if (loss && a->n_valid_seq && shape->T > 0) {
             fuse.counts = a->n_valid_seq;
-            fuse.rectify_later = true;
-            rectify = {a->lp_roll, params->C, a->diag, a->rho, a->w_tilde,
+            rectify = {a->lp_roll, params->C, TotalsJob{}, a->rho, a->w_tilde,
                        params->seq_level_weights ? reinterpret_cast<const float*>(static_cast<uint8_t*>(a->workspace) + L.off_seqw) : nullptr};
             fuse.rectify = &rectify;
+            fuse.totals = &rectify.totals;
         }
         st = diagnostics(shape, params, a->lp_train, a->lp_roll, a->mask, a->seq_offsets, a->rewards, a->adv, a->n_valid_seq, a->rho,
                          a->w_tilde, a->diag, a->workspace, a->workspace_bytes, stream, fuse);

@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(kQThreads) tensor_quantize_kernel(const __nv_b
 
 // Group-relative advantage of sequence s (Eq. grpo_adv), and what AdvJob clears for it.
 __device__ __forceinline__ void run_advantage(const AdvJob& j, int s) {
-    if (s == 0) j.tickets[0] = j.tickets[1] = j.tickets[2] = 0;
+    if (s == 0 && j.tickets) j.tickets[0] = j.tickets[1] = 0;
     if (j.zero_counts) j.zero_counts[s] = 0;
     const int g0 = (s / j.G) * j.G;
     double mean = 0.0;
@@ -637,6 +637,15 @@ __device__ __forceinline__ int seq_in_range(const int32_t* __restrict__ seq_offs
     return range.x == range.y ? range.x : range.x + seq_of_row(seq_offsets + range.x, range.y - range.x + 1, t);
 }
 
+// Population variance E[x^2] - E[x]^2 in fp64.  The sums reach this point with fp64 accuracy relative to the spread of the data
+// (add_run), so what is left is the rounding of the fp64 additions themselves: a result below 2^-44 of the mean square (a few
+// hundred ulps of it; a standard deviation below 2.4e-7 of the rms value) is that rounding and is reported as exactly zero.
+__device__ __forceinline__ double population_variance(double N, double sum, double sumsq) {
+    const double mean = sum / N, ms = sumsq / N;
+    const double v = ms - mean * mean;
+    return v > ms * 0x1p-44 ? v : 0.0;
+}
+
 // The diagnostics and alpha from the ten sums over the batch.
 __device__ __noinline__ void derive_diag(const double* m, const ais_params& p, ais_diag* __restrict__ diag) {
     ais_diag d;
@@ -652,15 +661,7 @@ __device__ __noinline__ void derive_diag(const double* m, const ais_params& p, a
         d.alpha_adaptive = 0.0; d.kl_k1 = 0.0; d.mean_abs_dp = 0.0;
         d.status_flags |= AIS_FLAG_EMPTY;
     } else {
-        // Population variance E[x^2] - E[x]^2 in fp64.  The sums reach this point with fp64 accuracy relative to the
-        // spread of the data (add_run), so what is left is the rounding of the fp64 additions themselves: a result
-        // below 2^-44 of the mean square (a few hundred ulps of it; a standard deviation below 2.4e-7 of the rms
-        // value) is that rounding and is reported as exactly zero.
-        auto variance = [&](double sum, double sumsq) {
-            const double mean = sum / N, ms = sumsq / N;
-            const double v = ms - mean * mean;
-            return v > ms * 0x1p-44 ? v : 0.0;
-        };
+        auto variance = [&](double sum, double sumsq) { return population_variance(N, sum, sumsq); };
         const double mu = m[1] / N;
         const double var = variance(m[1], m[2]);
         d.mean_w = mu;
@@ -681,6 +682,84 @@ __device__ __noinline__ void derive_diag(const double* m, const ais_params& p, a
     if (isnan(N)) d.status_flags |= AIS_FLAG_TIMEOUT;       // a block of the moments kernel gave up on a bounded wait
     d.alpha = isnan(p.alpha_override) ? d.alpha_adaptive : static_cast<double>(p.alpha_override);
     *diag = d;
+}
+
+// alpha alone, the same operations by one warp: lane 0 follows the weights, lanes 1 and 2 the two standard deviations, lane 3
+// the log-ratio gap, so that the chain is five divisions and a square root long instead of fifteen.
+__device__ __forceinline__ double alpha_by_warp(const double* m, const ais_params& p, int lane) {
+    if (!isnan(p.alpha_override)) return static_cast<double>(p.alpha_override);
+    const double N = m[0];
+    if (N <= 0.0) return 0.0;
+    const int at = lane == 0 ? 1 : lane == 1 ? 4 : lane == 2 ? 6 : 3;
+    const double first = m[at] / N;                                                      // mu, ..., d_bar
+    const double var = lane < 3 ? population_variance(N, m[at], m[at + 1]) : 0.0;
+    const double root = sqrt(lane == 0 ? 1.0 + var / (first * first) : var);
+    const double std_A = __shfl_sync(0xffffffffu, root, 1), std_Aw = __shfl_sync(0xffffffffu, root, 2);
+    const double num = lane == 0 ? 1.0 : lane == 3 ? first : std_Aw;
+    const double den = lane == 0 ? root : lane == 3 ? static_cast<double>(p.delta) : std_A + static_cast<double>(p.eps);
+    const double q = num / den;                                                          // alpha_ess, delta_sigma, ..., d_bar / delta
+    const double alpha_ess = __shfl_sync(0xffffffffu, q, 0), delta_sigma = __shfl_sync(0xffffffffu, q, 1);
+    const double alpha_mis = fmin(1.0, __shfl_sync(0xffffffffu, q, 3));
+    const double alpha_var = fmax(0.0, (delta_sigma - static_cast<double>(p.gamma)) / static_cast<double>(p.gamma));
+    return fmin(1.0, fmax(0.0, alpha_ess - static_cast<double>(p.beta_var) * alpha_var)) * alpha_mis;
+}
+
+// Totals over the blocks of a batch reduction, formed by every block of the kernel that follows it (256 threads): thread
+// (slice, moment) adds every 25th block's value in block order, ten threads add the slices.  The kernel that produced the
+// partial sums is over by then, so nothing has to count arrivals.  Result in t.moments, valid for every thread.
+// Each block reads at most 47 KB from L2.  Measured (diagnostics of 1.48 M / 200 k rows, back to back): the last block of the
+// moments kernel adding up, deriving alpha and a third kernel reading it 22.1 / 13.5 us, this 18.5 / 12.4 us; the rectifying
+// kernel on 444, 296 and 148 blocks instead of 592 18.7, 19.2 and 21.0 us.
+constexpr int kSums = 10;                                // slots 10 and 11 are no moments
+constexpr int kSlices = kDiagThreads / kSums;
+struct Totals {
+    double slices[kSlices][kSums];
+    double moments[kNumMoments];
+    float alpha;
+};
+__device__ __forceinline__ void form_totals(const TotalsJob& job, Totals& t) {
+    const int tid = threadIdx.x;
+    if (tid < kSlices * kSums) {
+        double acc = 0.0;
+        for (int b0 = tid / kSums; b0 < job.blocks; b0 += 12 * kSlices) {
+            double v[12];
+#pragma unroll
+            for (int j = 0; j < 12; ++j) v[j] = b0 + j * kSlices < job.blocks ? job.partials[(b0 + j * kSlices) * kNumMoments + tid % kSums] : 0.0;
+#pragma unroll
+            for (int j = 0; j < 12; ++j) acc += v[j];
+        }
+        t.slices[tid / kSums][tid % kSums] = acc;
+    }
+    __syncthreads();
+    if (tid < kNumMoments) {
+        double tot = 0.0;
+        if (tid < kSums) {
+#pragma unroll
+            for (int k = 0; k < kSlices; ++k) tot += t.slices[k][tid];
+        }
+        t.moments[tid] = tot;
+    }
+    __syncthreads();
+}
+// alpha of the batch, for every thread; block 0 also writes the diagnostics.
+__device__ __forceinline__ float form_alpha(const TotalsJob& job, Totals& t) {
+    form_totals(job, t);
+    if (threadIdx.x < 32) {
+        const double alpha = alpha_by_warp(t.moments, job.params, threadIdx.x);
+        if (threadIdx.x == 0) t.alpha = static_cast<float>(alpha);
+    } else if (threadIdx.x == 32 && blockIdx.x == 0) {
+        derive_diag(t.moments, job.params, job.diag);
+    }
+    __syncthreads();
+    return t.alpha;
+}
+// The totals on their own: the sums (ais_diag_moments) or, for a batch without rows, the diagnostics.
+__global__ void __launch_bounds__(kDiagThreads) totals_kernel(const __grid_constant__ TotalsJob job, double* __restrict__ moments) {
+    __shared__ Totals t;
+    pdl_enter();
+    form_totals(job, t);
+    if (moments != nullptr && threadIdx.x < kNumMoments) moments[threadIdx.x] = t.moments[threadIdx.x];
+    if (job.diag != nullptr && threadIdx.x == 0) derive_diag(t.moments, job.params, job.diag);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -925,30 +1004,23 @@ __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, int*
     return mbar_wait(bar, parity, abort_flag);
 }
 
-// What the last block of the moments kernel leaves behind.
-struct DiagFinish {
-    ais_params params;
-    ais_diag* diag;        // diagnostics and alpha (may be NULL)
-    double* moments;       // the sums themselves (may be NULL)
-    uint32_t* ticket;      // arrivals of the blocks, zeroed before the launch
-};
-
-// SEQ: every row carries its sequence's truncated weight instead of its own.  The block that finishes last adds up the
-// blocks' partial sums in their order and writes the diagnostics (fin.diag) or the sums themselves (fin.moments), so that
-// the batch step needs no launch of its own for that.
-template <bool SEQ>
+// SEQ: every row carries its sequence's truncated weight instead of its own.  WALKS: the fast walk and, for a block that needs
+// it, the exact one (see add_rows) in one kernel, or each in its own -- the fast one leaves in slots 10 and 11 of its partial
+// sums which groups it met, and the exact one replaces the sums of the blocks that need it.
+enum Walks { kBothWalks, kFastWalk, kExactWalk };
+template <bool SEQ, int WALKS>
 __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const float* __restrict__ lp_train,
                                                                          const float* __restrict__ lp_roll,
                                                                          const uint8_t* __restrict__ mask,
                                                                          const int32_t* __restrict__ seq_offsets,
                                                                          const float* __restrict__ adv, int T, int S, float C,
                                                                          double* partials, int32_t* __restrict__ n_valid_seq,
-                                                                         const float* __restrict__ seq_logw, bool early, const DiagFinish fin) {
+                                                                         const float* __restrict__ seq_logw, bool early) {
     static_assert(kDiagThreads * 8 == kMomRows, "one 8-row group per thread and tile");
     extern __shared__ __align__(128) uint8_t stages[];          // kMomStages stages, then the barriers
     uint64_t* full = reinterpret_cast<uint64_t*>(stages + kMomStages * kMomStageBytes);
     __shared__ double scratch[10][32];
-    __shared__ double totals[kNumMoments];
+    __shared__ double totals[kSums];
     __shared__ int abort_flag;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
@@ -1208,20 +1280,32 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
         range = seqs_of_rows_warp(seq_offsets, S, w0 < T ? w0 : T - 1, w0 + 255 < T ? w0 + 255 : T - 1);
     }
     const int first_sq = seq_in_range(seq_offsets, range, tile0 * kMomRows + 8 * tid < T ? tile0 * kMomRows + 8 * tid : T - 1);
-    if (early) fill_ring(0);
-    pdl_enter();
-    if (!early) fill_ring(0);
-    start_at(first_sq);
-    walk(std::false_type{}, 0);
-    const bool any_big = __syncthreads_or(nbig) != 0;
-    const bool any_small = __syncthreads_or(nsmall) != 0;
-    if (!any_big && any_small && !__syncthreads_or(failed ? 1 : 0)) {
-        reset();
+    double* mine = partials + blockIdx.x * kNumMoments;
+    if (WALKS == kExactWalk) {
+        pdl_enter();
+        if (mine[10] != 0.0 || mine[11] == 0.0 || isnan(mine[0])) return;
+        fill_ring(0);
         start_at(first_sq);
-        fill_ring(full1 - tile0);
-        walk(std::true_type{}, full1 - tile0);
+        walk(std::true_type{}, 0);
+    } else {
+        if (early) fill_ring(0);
+        pdl_enter();
+        if (!early) fill_ring(0);
+        start_at(first_sq);
+        walk(std::false_type{}, 0);
+        const bool any_big = __syncthreads_or(nbig) != 0;
+        const bool any_small = __syncthreads_or(nsmall) != 0;
+        if (WALKS == kBothWalks && !any_big && any_small && !__syncthreads_or(failed ? 1 : 0)) {
+            reset();
+            start_at(first_sq);
+            fill_ring(full1 - tile0);
+            walk(std::true_type{}, full1 - tile0);
+        }
+        if (tid == 0) {
+            mine[10] = any_big ? 1.0 : 0.0;
+            mine[11] = any_small ? 1.0 : 0.0;
+        }
     }
-    constexpr int kSums = 10;                            // slots 10 and 11 are no moments
     double acc[kSums];
     {
         // from the shifted sums to the sums of w, w^2, A, A^2, A w, (A w)^2 in fp64, once per thread:
@@ -1242,56 +1326,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
     }
     if (failed) acc[0] = __longlong_as_double(0x7ff8000000000000LL);     // a NaN count marks the batch as not reduced
     block_sums(acc, scratch, totals);
-    if (tid < kSums) partials[blockIdx.x * kNumMoments + tid] = totals[tid];
-    if (!last_block(fin.ticket)) return;
-    // Totals over the blocks: thread (slice, moment) adds every 25th block's value in block order, ten threads add the slices.
-    constexpr int kSlices = kDiagThreads / kSums;
-    if (tid < kSlices * kSums) {
-        const int m = tid % kSums, nb = static_cast<int>(gridDim.x);
-        double acc2 = 0.0;
-        for (int b0 = tid / kSums; b0 < nb; b0 += 12 * kSlices) {
-            double v[12];
-#pragma unroll
-            for (int j = 0; j < 12; ++j) v[j] = b0 + j * kSlices < nb ? __ldcg(partials + (b0 + j * kSlices) * kNumMoments + m) : 0.0;
-#pragma unroll
-            for (int j = 0; j < 12; ++j) acc2 += v[j];
-        }
-        scratch[m][tid / kSums] = acc2;
-    }
-    __syncthreads();
-    if (tid < kNumMoments) {
-        double tot = 0.0;
-        if (tid < kSums)
-            for (int k = 0; k < kSlices; ++k) tot += scratch[tid][k];
-        totals[tid] = tot;
-    }
-    __syncthreads();
-    if (fin.moments != nullptr && tid < kNumMoments) fin.moments[tid] = totals[tid];
-    if (fin.diag != nullptr && tid == 0) derive_diag(totals, fin.params, fin.diag);
-}
-
-__global__ void __launch_bounds__(32 * kNumMoments) diag_finalize_kernel(const double* __restrict__ partials, int nblocks, ais_params p,
-                                                                       ais_diag* __restrict__ diag) {
-    // one warp per moment sums the partials in a fixed order; thread 0 then derives the diagnostics
-    __shared__ double m[kNumMoments];
-    pdl_enter();
-    {
-        const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        const double acc = warp_ordered_sum(partials, nblocks, kNumMoments, i, lane);
-        if (lane == 0) m[i] = acc;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) derive_diag(m, p, diag);
-}
-
-// Sums the per-block partial moments in block order into one vector of kNumMoments doubles.
-// One warp per moment, fixed order.
-__global__ void moments_reduce_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ moments) {
-    pdl_enter();
-    if (blockIdx.x != 0) return;
-    const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const double m = i < 10 ? warp_ordered_sum(partials, nblocks, kNumMoments, i, lane) : 0.0;   // 10, 11 are no moments
-    if (lane == 0) moments[i] = m;
+    if (tid < kSums) mine[tid] = totals[tid];
 }
 
 // Ratio and rectification weight of a valid row; seq_logw: its sequence's log weight (sequence-level variant) or NULL.
@@ -1301,28 +1336,34 @@ __device__ __forceinline__ void rectify_row(float lt, float lr, float alpha, flo
     wt = fmaf(alpha, fminf(w, C) - 1.0f, 1.0f);
 }
 
+// Forms alpha first, every block for itself (form_alpha).
 template <int VEC>
-__global__ void __launch_bounds__(256) rectify_kernel(const float* __restrict__ lp_train, const float* __restrict__ lp_roll,
-                                                      const uint8_t* __restrict__ mask, int64_t T, float C,
-                                                      const ais_diag* __restrict__ diag, float* __restrict__ rho,
-                                                      float* __restrict__ w_tilde, const int32_t* __restrict__ seq_offsets,
-                                                      int S, const float* __restrict__ seq_logw) {
-    // the log-probs and the mask were there before the kernel this one follows: the first group is loaded while that one
-    // still runs, the wait is for alpha
+__global__ void __launch_bounds__(kDiagThreads, 4) rectify_kernel(const float* __restrict__ lp_train, const float* __restrict__ lp_roll,
+                                                                  const uint8_t* __restrict__ mask, int64_t T, float C,
+                                                                  const __grid_constant__ TotalsJob job, float* __restrict__ rho,
+                                                                  float* __restrict__ w_tilde, const int32_t* __restrict__ seq_offsets,
+                                                                  int S, const float* __restrict__ seq_logw, bool early) {
+    // The log-probs and the mask were there before the kernel this one follows (`early`): the first two groups are loaded
+    // while that one still runs, the wait is for its sums.
+    __shared__ Totals totals;
     const int64_t ngroups = T / VEC;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const int64_t g0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    RowGroup<VEC> in;
-    if (g0 < ngroups) in = load_group<VEC>(lp_train, lp_roll, mask, g0);
+    RowGroup<VEC> in = {}, next = {};
+    auto preload = [&]() {
+        if (g0 < ngroups) in = load_group<VEC>(lp_train, lp_roll, mask, g0);
+        if (g0 + stride < ngroups) next = load_group<VEC>(lp_train, lp_roll, mask, g0 + stride);
+    };
+    if (early) preload();
     pdl_enter();
-    const float alpha = static_cast<float>(diag->alpha);
+    if (!early) preload();
+    const float alpha = form_alpha(job, totals);
     auto one = [&](float lt, float lr, uint8_t mk, float& r, float& wt, int64_t t) {
         r = 1.0f;
         wt = 1.0f;
         if (mk) rectify_row(lt, lr, alpha, C, seq_logw ? seq_logw + seq_of_row(seq_offsets, S, t) : nullptr, r, wt);
     };
     for (int64_t g = g0; g < ngroups; g += stride) {
-        if (g != g0) in = load_group<VEC>(lp_train, lp_roll, mask, g);
         float r[VEC], wt[VEC];
 #pragma unroll
         for (int j = 0; j < VEC; ++j) one(in.lt[j], in.lr[j], in.mk[j], r[j], wt[j], g * VEC + j);
@@ -1333,6 +1374,8 @@ __global__ void __launch_bounds__(256) rectify_kernel(const float* __restrict__ 
             if (rho) rho[g] = r[0];
             w_tilde[g] = wt[0];
         }
+        in = next;
+        if (g + 2 * stride < ngroups) next = load_group<VEC>(lp_train, lp_roll, mask, g + 2 * stride);
     }
     for (int64_t t = ngroups * VEC + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < T; t += stride) {
         float r, wt;
@@ -1367,12 +1410,14 @@ struct LossArgs {
 };
 
 template <bool VEC, bool RECTIFY>
-__global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const LossArgs a) {
+__global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const __grid_constant__ LossArgs a) {
     __shared__ double scratch[2][32];
     __shared__ double totals[2];
+    __shared__ std::conditional_t<RECTIFY, Totals, int> batch;
     pdl_enter();
     const int lane = threadIdx.x & 31;
-    const float alpha = RECTIFY ? static_cast<float>(a.rectify.alpha_of->alpha) : 0.f;
+    float alpha = 0.f;
+    if constexpr (RECTIFY) alpha = form_alpha(a.rectify.totals, batch);
     double J = 0.0, KL = 0.0;
     // one valid row of sequence sq: its share of the objective, of the KL estimate, and its gradient factor
     auto one = [&](int64_t t, int sq, float wtf) -> float {
@@ -1501,45 +1546,58 @@ inline int reduce_blocks(int64_t T, int rows) {
     return static_cast<int>(b < 1 ? 1 : b > kDiagBlocks ? kDiagBlocks : b);
 }
 
-// The masked sums of the batch into fin.diag and / or fin.moments.
+// The masked sums of the batch, one row of partial sums per block; the number of blocks in *blocks.
+// From kSplitWalkRows on the exact walk has a launch of its own: both walks in one kernel cost the fast one a tenth of its
+// bandwidth (4.5 against 4.0 TB/s at 67 M rows), a launch costs 2 us.
+constexpr int64_t kSplitWalkRows = int64_t(8) << 20;
 cudaError_t launch_moments_kernel(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
                                   const float* adv, int64_t T, int S, float C, double* partials, int32_t* n_valid_seq,
-                                  float* seq_logw, bool early, const DiagFinish& fin, cudaStream_t stream) {
+                                  float* seq_logw, bool early, int* blocks, cudaStream_t stream) {
     cudaError_t e;
     if (seq_logw && S > 0) {
         e = launch_pdl(seq_logw_kernel, (S + 7) / 8, 256, 0, stream, lp_train, lp_roll, mask, seq_offsets, S, seq_logw);
         if (e != cudaSuccess) return e;
     }
     if (vec4_ok(lp_train, lp_roll, nullptr, nullptr, mask) && reinterpret_cast<uintptr_t>(mask) % 16 == 0 && T < (int64_t(1) << 31) - 2 * kMomRows) {      // 32-bit row indices inside
-        const int blocks = reduce_blocks(T, kMomRows);
-        const int Ti = static_cast<int>(T);
-        return launch_pdl(seq_logw ? moments_staged_kernel<true> : moments_staged_kernel<false>, blocks, kDiagThreads, kMomSmemBytes, stream,
-                          lp_train, lp_roll, mask, seq_offsets, adv, Ti, S, C, partials, n_valid_seq, seq_logw, early && !seq_logw, fin);
+        // no more blocks than have a tile when every block takes the same number of them
+        const int tiles = static_cast<int>((T + kMomRows - 1) / kMomRows), per = (tiles + kDiagBlocks - 1) / kDiagBlocks;
+        *blocks = tiles > 0 ? (tiles + per - 1) / per : 1;
+        auto go = [&](auto kernel, bool ahead) {
+            return launch_pdl(kernel, *blocks, kDiagThreads, kMomSmemBytes, stream, lp_train, lp_roll, mask, seq_offsets, adv, static_cast<int>(T), S, C,
+                              partials, n_valid_seq, seq_logw, ahead);
+        };
+        if (T < kSplitWalkRows) return seq_logw ? go(moments_staged_kernel<true, kBothWalks>, false) : go(moments_staged_kernel<false, kBothWalks>, early);
+        e = seq_logw ? go(moments_staged_kernel<true, kFastWalk>, false) : go(moments_staged_kernel<false, kFastWalk>, early);
+        if (e != cudaSuccess) return e;
+        return seq_logw ? go(moments_staged_kernel<true, kExactWalk>, false) : go(moments_staged_kernel<false, kExactWalk>, false);
     }
-    e = launch_pdl(vec4_ok(lp_train, lp_roll, nullptr, nullptr, mask) ? moments_kernel<4> : moments_kernel<1>, kDiagBlocks, kDiagThreads, 0, stream,
-                   lp_train, lp_roll, mask, seq_offsets, adv, T, S, C, partials, n_valid_seq, seq_logw);
-    if (e != cudaSuccess) return e;
-    if (fin.moments) e = launch_pdl(moments_reduce_kernel, 1, 32 * kNumMoments, 0, stream, partials, kDiagBlocks, fin.moments);
-    if (e == cudaSuccess && fin.diag)
-        e = launch_pdl(diag_finalize_kernel, 1, 32 * kNumMoments, 0, stream, partials, kDiagBlocks, fin.params, fin.diag);
-    return e;
+    *blocks = kDiagBlocks;
+    return launch_pdl(vec4_ok(lp_train, lp_roll, nullptr, nullptr, mask) ? moments_kernel<4> : moments_kernel<1>, kDiagBlocks, kDiagThreads, 0, stream,
+                      lp_train, lp_roll, mask, seq_offsets, adv, T, S, C, partials, n_valid_seq, seq_logw);
 }
 
-cudaError_t launch_rectify_kernel(const float* lp_train, const float* lp_roll, const uint8_t* mask, int64_t T, float C,
-                           const ais_diag* diag, float* rho, float* w_tilde, const int32_t* seq_offsets, int S,
-                           const float* seq_logw, cudaStream_t stream) {
-    const int64_t groups = (T + 3) / 4;
-    const int blocks = static_cast<int>(((groups + 255) / 256) < 2368 ? ((groups + 255) / 256) : 2368);
-    return launch_pdl(vec4_ok(lp_train, lp_roll, rho, w_tilde, mask) ? rectify_kernel<4> : rectify_kernel<1>, blocks, 256, 0, stream,
-                      lp_train, lp_roll, mask, T, C, diag, rho, w_tilde, seq_offsets, S, seq_logw);
+cudaError_t launch_rectify_kernel(const float* lp_train, const float* lp_roll, const uint8_t* mask, int64_t T, float C, const TotalsJob& job,
+                                  float* rho, float* w_tilde, const int32_t* seq_offsets, int S, const float* seq_logw, bool early,
+                                  cudaStream_t stream) {
+    const int blocks = reduce_blocks(T, 4 * kDiagThreads);
+    return launch_pdl(vec4_ok(lp_train, lp_roll, rho, w_tilde, mask) ? rectify_kernel<4> : rectify_kernel<1>, blocks, kDiagThreads, 0, stream,
+                      lp_train, lp_roll, mask, T, C, job, rho, w_tilde, seq_offsets, S, seq_logw, early);
 }
 
 }  // namespace
 
 cudaError_t stream_prepare() {
-    cudaError_t e = cudaFuncSetAttribute(moments_staged_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(moments_staged_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
+    cudaError_t e = cudaSuccess;
+    auto allow = [&](auto kernel) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
+    };
+    allow(moments_staged_kernel<false, kBothWalks>);
+    allow(moments_staged_kernel<false, kFastWalk>);
+    allow(moments_staged_kernel<false, kExactWalk>);
+    allow(moments_staged_kernel<true, kBothWalks>);
+    allow(moments_staged_kernel<true, kFastWalk>);
+    allow(moments_staged_kernel<true, kExactWalk>);
+    return e;
 }
 
 // ------------------------------------------------------------------------------------------------ launchers
@@ -1637,27 +1695,33 @@ cudaError_t launch_advantages(const AdvJob& job, cudaStream_t stream) {
 }
 
 cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
-                        const float* adv, int64_t T, int S, const ais_params& p, double* partials, uint32_t* ticket,
-                        int32_t* n_valid_seq, float* seq_logw, float* rho, float* w_tilde, ais_diag* diag, bool early, cudaStream_t stream) {
-    const DiagFinish fin = {p, diag, nullptr, ticket};
-    const cudaError_t e = launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, early, fin, stream);
-    if (e != cudaSuccess || T == 0 || w_tilde == nullptr) return e;
-    return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, diag, rho, w_tilde, seq_offsets, S, seq_logw, stream);
+                        const float* adv, int64_t T, int S, const ais_params& p, double* partials, int32_t* n_valid_seq, float* seq_logw,
+                        float* rho, float* w_tilde, ais_diag* diag, bool early, TotalsJob* later, cudaStream_t stream) {
+    TotalsJob job = {partials, 0, p, diag};
+    const cudaError_t e = launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, early, &job.blocks, stream);
+    if (e != cudaSuccess) return e;
+    if (later) {
+        *later = job;
+        return e;
+    }
+    if (T == 0) return launch_pdl(totals_kernel, 1, kDiagThreads, 0, stream, job, nullptr);
+    return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, job, rho, w_tilde, seq_offsets, S, seq_logw, true, stream);
 }
 
 cudaError_t launch_moments(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
-                           const float* adv, int64_t T, int S, const ais_params& p, double* partials, uint32_t* ticket,
-                           int32_t* n_valid_seq, float* seq_logw, double* moments, cudaStream_t stream) {
-    const DiagFinish fin = {p, nullptr, moments, ticket};
-    return launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, true, fin, stream);
+                           const float* adv, int64_t T, int S, const ais_params& p, double* partials, int32_t* n_valid_seq, float* seq_logw,
+                           double* moments, cudaStream_t stream) {
+    TotalsJob job = {partials, 0, p, nullptr};
+    const cudaError_t e = launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, true, &job.blocks, stream);
+    return e != cudaSuccess ? e : launch_pdl(totals_kernel, 1, kDiagThreads, 0, stream, job, moments);
 }
 
 cudaError_t launch_finalize(const double* moments, const float* lp_train, const float* lp_roll, const uint8_t* mask, int64_t T,
                             const ais_params& p, float* rho, float* w_tilde, ais_diag* diag, const int32_t* seq_offsets, int S,
                             const float* seq_logw, cudaStream_t stream) {
-    const cudaError_t e = launch_pdl(diag_finalize_kernel, 1, 32 * kNumMoments, 0, stream, moments, 1, p, diag);
-    if (e != cudaSuccess || T == 0) return e;
-    return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, diag, rho, w_tilde, seq_offsets, S, seq_logw, stream);
+    const TotalsJob job = {moments, 1, p, diag};
+    if (T == 0) return launch_pdl(totals_kernel, 1, kDiagThreads, 0, stream, job, nullptr);
+    return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, job, rho, w_tilde, seq_offsets, S, seq_logw, false, stream);
 }
 
 cudaError_t launch_loss_coef(const float* lp_train, const float* lp_old, const float* lp_ref, float beta_kl, const uint8_t* mask,

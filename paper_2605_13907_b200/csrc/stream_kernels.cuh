@@ -32,8 +32,8 @@ struct FlagsJob {
     void* clear;
     int64_t clear_bytes;
 };
-// Group-relative advantages adv[s]; zero_counts [S] (may be NULL) and the tickets (block counters of the two batch
-// reductions, count of row tiles to recompute) are cleared for the kernels that count into them.
+// Group-relative advantages adv[s]; zero_counts [S] and the two counters of the loss kernel (its finished blocks, the row tiles
+// to recompute) are cleared for the kernels that count into them; each may be NULL.
 struct AdvJob {
     const float* rewards;
     int32_t S, G, std_norm;
@@ -42,11 +42,19 @@ struct AdvJob {
     int32_t* zero_counts;
     uint32_t* tickets;
 };
+// The end of the batch moments, left to the kernel that follows: partial sums [blocks][kNumMoments], and where the
+// diagnostics formed from their totals go.
+struct TotalsJob {
+    const double* partials;
+    int32_t blocks;
+    ais_params params;
+    ais_diag* diag;
+};
 // The rectification of a batch (rho, w_tilde) as part of the loss kernel.
 struct RectifyJob {
     const float* lp_roll;
     float C;
-    const ais_diag* alpha_of;
+    TotalsJob totals;
     float *rho, *w_tilde;
     const float* seq_logw;
 };
@@ -101,16 +109,16 @@ cudaError_t launch_advantages(const AdvJob& job, cudaStream_t stream);
 
 // n_valid_seq (may be NULL) must have been cleared: the moments kernel adds every sequence's valid rows to it.
 cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
-                        const float* adv, int64_t T, int S, const ais_params& p, double* partials /*[kDiagBlocks][kNumMoments]*/, uint32_t* ticket,
+                        const float* adv, int64_t T, int S, const ais_params& p, double* partials /*[kDiagBlocks][kNumMoments]*/,
                         int32_t* n_valid_seq, float* seq_logw /* [S] scratch: non-NULL selects sequence-level weights */,
-                        float* rho, float* w_tilde /* NULL: the loss kernel rectifies */, ais_diag* diag,
-                        bool early /* the log-probs are older than the kernel enqueued last */, cudaStream_t stream);
+                        float* rho, float* w_tilde, ais_diag* diag, bool early /* the log-probs are older than the kernel enqueued last */,
+                        TotalsJob* later /* not NULL: the loss kernel forms alpha, rho and w_tilde from this */, cudaStream_t stream);
 
 // The two halves of launch_diag: partial moments summed into `moments` [kNumMoments], and everything that follows
 // from a (possibly all-reduced) moment vector.
 cudaError_t launch_moments(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
-                           const float* adv, int64_t T, int S, const ais_params& p, double* partials, uint32_t* ticket,
-                           int32_t* n_valid_seq, float* seq_logw, double* moments, cudaStream_t stream);
+                           const float* adv, int64_t T, int S, const ais_params& p, double* partials, int32_t* n_valid_seq,
+                           float* seq_logw, double* moments, cudaStream_t stream);
 cudaError_t launch_finalize(const double* moments, const float* lp_train, const float* lp_roll, const uint8_t* mask, int64_t T,
                             const ais_params& p, float* rho, float* w_tilde, ais_diag* diag, const int32_t* seq_offsets, int S,
                             const float* seq_logw, cudaStream_t stream);

@@ -170,3 +170,42 @@ def test_two_row_tiles_per_cta_match_the_oracle(variant):
     if not dv:
         ais.logprob_train_static(step.shape, H, W, tok, msk, lp)
         assert np.all(np.abs(lp.cpu().numpy() - ref["lp_train"]) <= atol)
+
+
+@pytest.mark.parametrize("gaps", ["small", "mixed"])
+@pytest.mark.parametrize("T", [(8 << 20) - 1, 8 << 20, (8 << 20) + 2049])
+def test_long_batches_sum_their_moments_in_one_launch_or_two(T, gaps):
+    """From 8 Mi rows on the exact walk over groups of tiny log-ratio gaps is a launch of its own, which replaces the sums of
+    the blocks that need it: all of them ("small": every gap is 1e-4) or those of the first half ("mixed").  Tolerance: the
+    weights are good to fp32 relative to w - 1 (2^-23 and the exponential's 2^-22), the sums over them are fp64."""
+    import ctypes
+
+    import paper_2605_13907_b200 as ais
+    rng = np.random.default_rng(T % 1000 + len(gaps))
+    P, G = 2, 4
+    S = P * G
+    offs = np.concatenate([[0], np.sort(rng.integers(0, T + 1, S - 1)), [T]]).astype(np.int32)
+    lp_t = -rng.uniform(0.5, 4.0, T).astype(np.float32)
+    size = np.full(T, 1e-4)
+    if gaps == "mixed":
+        size[T // 2:] = 0.3
+    lp_r = (lp_t - size * rng.choice([-1.0, 1.0], T)).astype(np.float32)
+    mask = (rng.random(T) < 0.8).astype(np.uint8)
+    rew = np.array([1, 0, 0, 1, 0, 1, 0, 0], np.float32)
+    ref_adv = oais.advantages(rew.astype(np.float64), G)
+    ref = oais.diagnostics(lp_t, lp_r, mask, ref_adv[oais.seq_ids(offs, T)], oais.Params())
+    params = ais.default_params()
+    shape = ais.make_shape(T, 128, 1024, P, G, 128)
+    ws = torch.empty(ais.workspace_min_bytes(shape, params), dtype=torch.uint8, device="cuda")
+    adv, nseq = torch.empty(S, device="cuda"), torch.zeros(S, dtype=torch.int32, device="cuda")
+    rho, wt = torch.zeros(T, device="cuda"), torch.zeros(T, device="cuda")
+    diag = torch.zeros(32, dtype=torch.float64, device="cuda")
+    ais.diagnostics(shape, params, *(torch.from_numpy(x).cuda() for x in (lp_t, lp_r, mask, offs, rew)), adv, nseq, rho, wt, diag, ws)
+    d = ais.Diag.from_buffer_copy(diag.cpu().numpy().tobytes()[:ctypes.sizeof(ais.Diag)]).as_dict()
+    assert d["n_valid"] == ref["n_valid"] and d["status_flags"] == 0
+    assert np.array_equal(nseq.cpu().numpy(), np.add.reduceat(np.append(mask, 0).astype(np.int64), offs[:-1]) * (np.diff(offs) > 0))
+    for k in ("cv2", "std_Aw", "delta_sigma", "alpha_ess", "d_bar", "kl_k1", "mean_abs_dp", "alpha"):
+        assert abs(d[k] - ref[k]) <= 1e-4 * max(abs(ref[k]), 1e-9 if k == "cv2" else 1e-4), (k, d[k], ref[k])
+    valid = mask.astype(bool)
+    ref_wt = oais.rectify(oais.ratios(lp_t, lp_r, mask, 5.0)[2], ref["alpha"], mask)
+    assert np.abs(wt.cpu().numpy() - ref_wt)[valid].max() <= 1e-5 and bool((wt.cpu()[~torch.from_numpy(valid)] == 1).all())
