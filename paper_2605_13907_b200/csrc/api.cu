@@ -809,6 +809,7 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
             LmheadArgs w = a;
             w.rows = out_rows;
             w.row0 = 0;
+            w.tile_active = nullptr;         // it contracts over the rows: nothing to skip
             w.n_row_tiles = static_cast<int32_t>((out_rows + kDhRows - 1) / kDhRows);
             w.ncols = out_cols;
             w.n_col_tiles = (out_cols + kBN - 1) / kBN;
@@ -822,7 +823,7 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
             ctas = units < num_sms ? units : num_sms;
             arm_pace(w, ws, L, 1, units, ctas, pass, true);
             ++pass;
-            if (launch_lmhead(kBwdDw, tmRow, tmCol, tmRow, tmCol, w, ctas, s) != cudaSuccess)
+            if (launch_lmhead_pair(kBwdDw, tmRow, tmCol, tmCol, w, ctas, s) != cudaSuccess)
                 return AIS_ERR_DEVICE;
         }
     }

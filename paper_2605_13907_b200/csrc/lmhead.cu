@@ -43,7 +43,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 
     constexpr int BASE = base_mode(MODE);                                       // what is computed, whatever W's layout
     constexpr bool B_MN = b_mn_major(MODE);                                     // B tile arrives as four 64-column boxes
-    constexpr bool TWO_ACC = (BASE == kBwdDh || BASE == kBwdDw);                // two 128-row tiles per CTA, one B slice
+    constexpr bool TWO_ACC = BASE == kBwdDh;                                    // two 128-row tiles per CTA, one B slice
     constexpr int STG = TWO_ACC ? kDhStages : kStages;                          // depth of the stage ring
     constexpr int STG_BYTES = TWO_ACC ? kDhStageBytes : kStageBytes;
     constexpr int A_BYTES = TWO_ACC ? 2 * kAStageBytes : kAStageBytes;
@@ -128,9 +128,6 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                         if (BASE == kBwdDh) {
                             tma_load_2d(sA, &tmA, &full[st.idx], kelem, w.rt * kDhRows);
                             tma_load_2d(sA + kAStageBytes, &tmA, &full[st.idx], kelem, w.rt * kDhRows + kBM);
-                        } else if (BASE == kBwdDw) {
-                            // A is U[t, v]: the output row v is the contiguous axis -> four 64-wide blocks of 64 rows t in one copy
-                            tma_load_3d(sA, &tmA, &full[st.idx], 0, kelem, w.rt * (kDhRows / 64));
                         } else {
                             tma_load_2d(sA, &tmA, &full[st.idx], kelem, w.rt * kBM);
                         }
@@ -140,7 +137,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                             // after the other in shared memory.  One copy for the four: with a copy each the forward pass over a
                             // [d, V] head took 14.2 Mcycles for 9,217 rows, 11.8 now (as much as the other layout).  The last,
                             // partial tile of such a head keeps single boxes, which end at V.
-                            if (MODE == kBwdDh || MODE == kBwdDw || t < a.block_tiles) {
+                            if (MODE == kBwdDh || t < a.block_tiles) {
                                 tma_load_3d(sB, &tmB, &full[st.idx], 0, kelem, t * (kBN / 64));
                             } else {
 #pragma unroll
@@ -166,7 +163,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         if (lane == 0) {
             constexpr uint32_t idesc =
                 (MODE == kFwdFp8T || MX) ? make_idesc(kFmtE4M3, kFmtE4M3, kBM, kBN, 0, 0)
-                                  : make_idesc(kFmtBF16, kFmtBF16, kBM, kBN, BASE == kBwdDw ? 1 : 0, B_MN ? 1 : 0);
+                                  : make_idesc(kFmtBF16, kFmtBF16, kBM, kBN, 0, B_MN ? 1 : 0);
             Pipe st(STG), tb(NBUF);
             bool ok = true;
             for (int u = blockIdx.x; u < num_units && ok; u += gridDim.x) {
@@ -189,17 +186,6 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                                 const uint32_t accum = (ks > w.k0 || j > 0) ? 1u : 0u;
                                 mma_f16(tmem_base, smem_desc_sw128(sA + j * 32, 16, 1024), bdesc, idesc, accum);
                                 mma_f16(tmem_base + kBN, smem_desc_sw128(sA + kAStageBytes + j * 32, 16, 1024), bdesc, idesc, accum);
-                            }
-                        } else if (BASE == kBwdDw) {
-                            // both operands have the contraction axis t as rows of 128 bytes: 16 rows (2048 bytes) per
-                            // MMA; 64-wide chunks of the output axis are 8 KB apart
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const uint64_t bdesc = smem_desc_sw128(sB + j * 2048, kBStageBytes / 4, 1024);
-                                const uint32_t accum = (ks > w.k0 || j > 0) ? 1u : 0u;
-                                mma_f16(tmem_base, smem_desc_sw128(sA + j * 2048, kAStageBytes / 2, 1024), bdesc, idesc, accum);
-                                mma_f16(tmem_base + kBN, smem_desc_sw128(sA + kAStageBytes + j * 2048, kAStageBytes / 2, 1024), bdesc,
-                                        idesc, accum);
                             }
                         } else if (MX) {
                             // the scale warps have put this stage's scales into its column set: A's chunks first (4 columns
@@ -364,44 +350,6 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                 tb.advance();
                 continue;
             }
-            if (BASE == kBwdDw) {
-                // one unit = 256 vocabulary rows x 256 columns of dW after the contraction over this launch's rows
-                if (!mbar_wait_warp(&tfull[0], tb.phase, abort_flag, a.wait_cycles)) { ok = false; break; }
-                tc_fence_after();
-#pragma unroll
-                for (int sub = 0; sub < 2; ++sub) {
-                    const int64_t vrow = static_cast<int64_t>(w.rt) * kDhRows + sub * kBM + r_in_tile;
-                    const bool in = vrow < a.rows;
-                    const uint32_t taddr2 = tmem_base + lane_addr + sub * kBN + half * 128;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const int col0 = w.t0 * kBN + half * 128 + c * 32;
-                        uint32_t v[32];
-                        tmem_ld32(taddr2 + c * 32, v);
-                        tmem_ld_wait(v);
-                        if (in && col0 < a.ncols) {
-                            float4* dst = reinterpret_cast<float4*>(a.dW + vrow * a.lddw + col0);
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                if (col0 + j * 4 < a.ncols) {
-                                    float4 o = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                                           __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
-                                    if (a.dw_accumulate) {
-                                        const float4 old = dst[j];
-                                        o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w;
-                                    }
-                                    dst[j] = o;
-                                }
-                            }
-                        }
-                    }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[0]);
-                tb.advance();
-                continue;
-            }
             RowState r = begin_row<MODE>(a, static_cast<int64_t>(w.rt) * kBM + r_in_tile, flags);
             const bool store = r.in && (BASE == kBwdP || r.lrow < a.keep_rows);
             const float tscale = (MODE == kFwdFp8T) ? (*a.scale_a) * (*a.scale_b) : 1.f;
@@ -537,7 +485,6 @@ cudaError_t launch_lmhead(int mode, const CUtensorMap& tmA, const CUtensorMap& t
         case kBwdP:    return launch_mode<kBwdP>(tmA, tmB, tmSA, args, num_ctas, stream);
         case kBwdDh:   return launch_mode<kBwdDh>(tmA, tmB, tmSA, args, num_ctas, stream);
         case kFwdFp8T: return launch_mode<kFwdFp8T>(tmA, tmB, tmSA, args, num_ctas, stream);
-        case kBwdDw:   return launch_mode<kBwdDw>(tmA, tmB, tmSA, args, num_ctas, stream);
         case kFwdMx:   return launch_mode<kFwdMx>(tmA, tmB, tmSA, args, num_ctas, stream);
         case kFwdMx4:  return launch_mode<kFwdMx4>(tmA, tmB, tmSA, args, num_ctas, stream);
         case kFwdBf16Dv: return launch_mode<kFwdBf16Dv>(tmA, tmB, tmSA, args, num_ctas, stream);
@@ -556,7 +503,7 @@ static cudaError_t prepare_mode() {
 
 cudaError_t lmhead_prepare() {
     const cudaError_t all[] = {lmhead_fp8_block_prepare(), lmhead_pair_prepare(), prepare_mode<kFwdBf16>(), prepare_mode<kBwdP>(), prepare_mode<kBwdDh>(),
-                               prepare_mode<kFwdFp8T>(), prepare_mode<kBwdDw>(), prepare_mode<kFwdMx>(), prepare_mode<kFwdMx4>(),
+                               prepare_mode<kFwdFp8T>(), prepare_mode<kFwdMx>(), prepare_mode<kFwdMx4>(),
                                prepare_mode<kFwdBf16Dv>(), prepare_mode<kBwdPDv>(), prepare_mode<kBwdDhDv>(), prepare_mode<kFwdKeep>(),
                                prepare_mode<kFwdKeepDv>()};
     for (const cudaError_t e : all)

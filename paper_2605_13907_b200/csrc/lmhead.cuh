@@ -145,8 +145,8 @@ cudaError_t launch_lmhead_fp8_block(const CUtensorMap& tmA, const CUtensorMap& t
                                     const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream);
 cudaError_t lmhead_fp8_block_prepare();
 
-// The forward and recompute passes (no microscaling) with two row tiles per CTA: n_row_tiles counts 256-row units, tmA has boxes
-// of 256 rows.
+// The forward and recompute passes (no microscaling) with two row tiles per CTA, and the dW pass: n_row_tiles counts 256-row
+// units, tmA has boxes of 256 rows (dW: blocks, make_tmap_blocks).
 cudaError_t launch_lmhead_pair(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB2, const LmheadArgs& args,
                                int num_ctas, cudaStream_t stream);
 cudaError_t lmhead_pair_prepare();

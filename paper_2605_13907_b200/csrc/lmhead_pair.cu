@@ -1,4 +1,4 @@
-// Forward and recompute passes with two row tiles per CTA: 256 rows x 256 columns, both accumulators of tensor memory, every
+// Forward, recompute and dW passes with two row tiles per CTA: 256 rows x 256 columns, both accumulators of tensor memory, every
 // slice of W that a CTA fetches used for two row tiles.  Per 64 K-elements a stage of 64 KB feeds 1,024 clocks of MMAs where
 // the one-row-tile kernel (lmhead.cu) needs 48 KB for 512, which is more than L2 delivers to all SMs at that rate: its main
 // loop runs at 82% of the tensor rate.  The price is that no third accumulator is left for the next tile while the epilogue
@@ -10,6 +10,11 @@
 // 20,000 rows at d = 5120, V = 129112 21.6 -> 19.1 ms, 1,024 rows 1.08 -> 1.01 ms.  Without the epilogue's arithmetic it would
 // take 2% less, so the skew hides nearly all of it (head 3 / tail 2: 8.01 ms, no tail 8.04, head 1 8.12, head 2 8.13); what is
 // left is the power cap.  Batches of few row tiles stay with the other kernel (plan_pass): a CTA per pair halves the units.
+//
+// The dW pass (256 x 256 of dW per unit, contracted over the rows of the launch) has the same shape with both operands MN-major,
+// and an epilogue per 64-row K steps of the batch: at 1,500 rows every 24 stages.  With the epilogue behind the MMAs of both
+// accumulators it took 2,540 us for 1,500 rows, 4,275 us for 4,000 and 8.61 ms for 9,217 (d = 4096, V = 151936); drained in turn
+// 2,260, 3,950 and 8.32 ms.
 //
 // Roles as in lmhead.cu: warp 0 copies, warp 1 issues the MMAs, warps 4..11 are the epilogue (lane quarter w % 4, column half
 // (w - 4) / 4 of both accumulators: two rows per thread).  The first warpgroup hands registers to the other two
@@ -26,6 +31,21 @@ constexpr int kPairStageBytes = kDhStageBytes;
 constexpr int kPairBars = 2 * kPairStages + 4 + 1;
 constexpr int kPairSmem = 1024 + kPairStages * kPairStageBytes + kPairBars * 8 + 64;
 constexpr int kPairTail = 2;                     // stages at the end of a tile that the first row tile gets ahead of the second
+
+// 32 consecutive columns of one row of dW.
+__device__ __forceinline__ void store_dw(const LmheadArgs& a, int64_t row, int col0, const uint32_t (&v)[32]) {
+    float4* dst = reinterpret_cast<float4*>(a.dW + row * a.lddw + col0);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        if (col0 + j * 4 >= a.ncols) continue;
+        float4 o = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]), __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+        if (a.dw_accumulate) {
+            const float4 old = dst[j];
+            o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w;
+        }
+        dst[j] = o;
+    }
+}
 
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -46,9 +66,10 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     constexpr int BASE = base_mode(MODE);
     constexpr bool B_MN = b_mn_major(MODE);
     constexpr bool FP8 = MODE == kFwdFp8T;
-    constexpr int UNIT = kFwdFp8;                // units of two row tiles, for decode_unit / unit_active
+    constexpr bool DW = MODE == kBwdDw;
+    constexpr int UNIT = DW ? kBwdDw : kFwdFp8;  // units of two row tiles, for decode_unit / unit_active
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int num_units = a.n_row_tiles * a.nsplit;
+    const int num_units = count_units<UNIT>(a);
     const bool gated = BASE == kBwdP && a.gate != nullptr;
     if (gated) {
         enter_pass(a);
@@ -100,10 +121,16 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                         uint8_t* sB = sA + 2 * kAStageBytes;
                         mbar_expect_tx(&full[st.idx], kPairStageBytes);
                         const int kelem = FP8 ? ks * 128 : ks * 64;
-                        tma_load_2d(sA, &tmA, &full[st.idx], kelem, w.rt * kPairRows);          // one box of 256 rows
+                        // dW: the output row is the contiguous axis of A (U[t, v]), four 64-wide blocks of 64 rows t in one copy;
+                        // otherwise one box of 256 rows
+                        if (DW) tma_load_3d(sA, &tmA, &full[st.idx], 0, kelem, w.rt * (kPairRows / 64));
+                        else tma_load_2d(sA, &tmA, &full[st.idx], kelem, w.rt * kPairRows);
+                        // MN-major B (H[t, n] of dW, a [d, V] head): four blocks of 64 columns in one copy, except in the last,
+                        // partial tile of such a head, whose single boxes end at V.  With a copy for each block the forward pass
+                        // over a [d, V] head took 14.2 Mcycles for 9,217 rows instead of 11.8.
                         if (!B_MN) {
                             tma_load_2d(sB, &tmB, &full[st.idx], kelem, t * kBN);
-                        } else if (t < a.block_tiles) {
+                        } else if (DW || t < a.block_tiles) {
                             tma_load_3d(sB, &tmB, &full[st.idx], 0, kelem, t * (kBN / 64));
                         } else {
 #pragma unroll
@@ -122,7 +149,7 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         } else if (warp == 1 && lane == 0) {
             // -------------------------------------------------------------- MMA issuer
             constexpr uint32_t idesc = FP8 ? make_idesc(kFmtE4M3, kFmtE4M3, kBM, kBN, 0, 0)
-                                           : make_idesc(kFmtBF16, kFmtBF16, kBM, kBN, 0, B_MN ? 1 : 0);
+                                           : make_idesc(kFmtBF16, kFmtBF16, kBM, kBN, DW ? 1 : 0, B_MN ? 1 : 0);
             const int K = a.ksteps;
             const int head = K < kPairStages ? K : kPairStages;                 // stages that the first row tile gets alone
             const int tail = K - head < kPairTail ? K - head : kPairTail;
@@ -146,7 +173,9 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 const uint32_t sB = sA + 2 * kAStageBytes;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const uint64_t adesc = smem_desc_sw128(sA + i * kAStageBytes + j * 32, 16, 1024);
+                    // MN-major operands: 16 K rows of 128 bytes per instruction, 64-wide blocks of the output axis 8 KB apart
+                    const uint64_t adesc = DW ? smem_desc_sw128(sA + i * kAStageBytes + j * 2048, kAStageBytes / 2, 1024)
+                                              : smem_desc_sw128(sA + i * kAStageBytes + j * 32, 16, 1024);
                     const uint64_t bdesc = B_MN ? smem_desc_sw128(sB + j * 2048, kBStageBytes / 4, 1024) : smem_desc_sw128(sB + j * 32, 16, 1024);
                     if (FP8) mma_f8(tmem_base + i * kBN, adesc, bdesc, idesc, (k > 0 || j > 0) ? 1u : 0u);
                     else mma_f16(tmem_base + i * kBN, adesc, bdesc, idesc, (k > 0 || j > 0) ? 1u : 0u);
@@ -229,7 +258,7 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             RowState r[2];
             bool store[2];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
+            for (int i = 0; i < 2 && !DW; ++i) {
                 r[i] = begin_row<MODE>(a, lrow0 + i * kBM, flags);
                 // a gated pass leaves the rows of a tile alone that was not marked, even beside one that was
                 const bool mine = !gated || (a.tile_active[a.row0 / kBM + 2 * static_cast<int64_t>(w.rt) + i * (r[i].in ? 1 : 0)] != 0);
@@ -264,6 +293,15 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&tempty[i]);
+                    if (DW) {
+                        const int64_t row = lrow0 + i * kBM;
+                        if (row < a.rows) {
+#pragma unroll
+                            for (int c = 0; c < 4; ++c)
+                                store_dw(a, row, col_base + c * 32, v[c]);
+                        }
+                        continue;
+                    }
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         float x[32];
@@ -273,7 +311,7 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                     }
                 }
             }
-            if (ok && BASE != kBwdP) {
+            if (ok && BASE != kBwdP && !DW) {
                 end_row(a, r[0], w.part * 2 + half);
                 end_row(a, r[1], w.part * 2 + half);
             }
@@ -319,13 +357,14 @@ cudaError_t launch_lmhead_pair(int mode, const CUtensorMap& tmA, const CUtensorM
         case kBwdP:      return launch<kBwdP>(tmA, tmB, tmB2, args, num_ctas, stream);
         case kBwdPDv:    return launch<kBwdPDv>(tmA, tmB, tmB2, args, num_ctas, stream);
         case kFwdFp8T:   return launch<kFwdFp8T>(tmA, tmB, tmB2, args, num_ctas, stream);
+        case kBwdDw:     return launch<kBwdDw>(tmA, tmB, tmB2, args, num_ctas, stream);
     }
     return cudaErrorInvalidValue;
 }
 
 cudaError_t lmhead_pair_prepare() {
     const cudaError_t all[] = {prepare<kFwdBf16>(), prepare<kFwdBf16Dv>(), prepare<kFwdKeep>(), prepare<kFwdKeepDv>(),
-                               prepare<kBwdP>(),    prepare<kBwdPDv>(),    prepare<kFwdFp8T>()};
+                               prepare<kBwdP>(),    prepare<kBwdPDv>(),    prepare<kFwdFp8T>(),   prepare<kBwdDw>()};
     for (const cudaError_t e : all)
         if (e != cudaSuccess) return e;
     return cudaSuccess;

@@ -209,3 +209,30 @@ def test_long_batches_sum_their_moments_in_one_launch_or_two(T, gaps):
     valid = mask.astype(bool)
     ref_wt = oais.rectify(oais.ratios(lp_t, lp_r, mask, 5.0)[2], ref["alpha"], mask)
     assert np.abs(wt.cpu().numpy() - ref_wt)[valid].max() <= 1e-5 and bool((wt.cpu()[~torch.from_numpy(valid)] == 1).all())
+
+
+@pytest.mark.parametrize("dv", [False, True])
+@pytest.mark.parametrize("length", [5, 17, 25, 50])
+def test_weight_gradient_with_few_and_many_k_steps(length, dv):
+    """dW of 40, 136, 200 and 400 rows: fewer 64-row K steps than the stage ring holds (1, 3), one more (4), and enough for the
+    whole order of row tiles (7); 237 units of 256 x 256, so that CTAs have a second one; a last unit with one row tile and a
+    ragged column tile.  dW is fp32 from bf16 gradients (2^-9)."""
+    import paper_2605_13907_b200 as ais
+    d, V, P, G = 640, 20104, 2, 4
+    w = workloads.scaled(workloads.WORKLOADS["tiny"], d=d, V=V, P=P, G=G, lengths=f"const:{length}", w_std=d ** -0.5, seed=305)
+    b = workloads.make_batch(w, device="cpu")
+    a = workloads.to_numpy(b)
+    ref = oais.full_path(a["H"], a["W"], a["tokens"], a["mask"], a["seq_offsets"], a["rewards"], P, G, w.block)
+    W = (b.W.t().contiguous() if dv else b.W).cuda()
+    H, tok, msk, offs, rew = b.H.cuda(), b.tokens.cuda(), b.mask.cuda(), b.seq_offsets.cuda(), b.rewards.cuda()
+    step = ais.AisStep(b.T, d, V, P, G, w.block, w_layout=ais.W_DV if dv else ais.W_VD)
+    dW = torch.full((d, V) if dv else (V, d), 7.0, device="cuda")
+    step.forward(H, W, tok, msk)
+    step.diagnose(msk, offs, rew)
+    for accumulate in (False, True):
+        step.backward(H, W, tok, msk, offs, dW=dW, dw_accumulate=accumulate)
+        torch.cuda.synchronize()
+        assert int(step.status.item()) == 0
+        got = (dW.t() if dv else dW).double().cpu().numpy() / (2.0 if accumulate else 1.0)
+        for c in range(0, V, 256):
+            assert np.linalg.norm(got[c:c + 256] - ref["dW"][c:c + 256]) <= DH_REL * np.linalg.norm(ref["dW"][c:c + 256]), c
