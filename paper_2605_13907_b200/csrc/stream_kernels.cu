@@ -528,9 +528,9 @@ __device__ __forceinline__ double warp_ordered_sum(const double* partials, int n
 }
 
 // The same sums for N values at once (same order each): two barriers for all of them instead of two for each; results in
-// out[0 .. N-1], valid for every thread after the call.
+// out[0 .. N-1], valid for every thread after the call.  Blocks of kDiagThreads.
 template <int N>
-__device__ __forceinline__ void block_sums(double (&v)[N], double (*scratch)[32] /*[N][32]*/, double* out) {
+__device__ __forceinline__ void block_sums(double (&v)[N], double (*scratch)[kDiagThreads / 32] /*[N]*/, double* out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -540,8 +540,8 @@ __device__ __forceinline__ void block_sums(double (&v)[N], double (*scratch)[32]
     __syncthreads();
     if (threadIdx.x < N) {
         double tot = 0.0;
-        const int nw = (blockDim.x + 31) >> 5;
-        for (int i = 0; i < nw; ++i) tot += scratch[threadIdx.x][i];
+#pragma unroll
+        for (int i = 0; i < kDiagThreads / 32; ++i) tot += scratch[threadIdx.x][i];
         out[threadIdx.x] = tot;
     }
     __syncthreads();
@@ -989,6 +989,9 @@ constexpr int kMomRows = 2048;
 constexpr int kMomStages = 3;
 constexpr int kMomStageBytes = kMomRows * 9;
 constexpr int kMomSmemBytes = kMomStages * kMomStageBytes + 128;
+// 228 KB per SM, 1 KB of it reserved per block: four blocks fit, and all 592 run at once (with three per SM 67 M rows took
+// 3.5 TB/s instead of 4.9)
+static_assert(4 * (kMomSmemBytes + 1024 + 10 * (kDiagThreads / 32 + 1) * 8 + 64) <= 228 * 1024, "four blocks per SM");
 
 
 // (add2 / sub2 / mul2 / fma2: the packed two-element fp32 instructions, ptx.cuh.)  The staged kernel is bound by
@@ -1019,16 +1022,15 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
     static_assert(kDiagThreads * 8 == kMomRows, "one 8-row group per thread and tile");
     extern __shared__ __align__(128) uint8_t stages[];          // kMomStages stages, then the barriers
     uint64_t* full = reinterpret_cast<uint64_t*>(stages + kMomStages * kMomStageBytes);
-    __shared__ double scratch[10][32];
+    __shared__ double scratch[kSums][kDiagThreads / 32];
     __shared__ double totals[kSums];
     __shared__ int abort_flag;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int nfull = T / kMomRows;                    // whole tiles; what is left is one more, read directly
     const int ntiles = (T + kMomRows - 1) / kMomRows;
-    const int per = (ntiles + gridDim.x - 1) / gridDim.x;
-    const int tile0 = blockIdx.x * per < ntiles ? blockIdx.x * per : ntiles;
-    const int tile1 = tile0 + per < ntiles ? tile0 + per : ntiles;
+    const int tile0 = static_cast<int>(static_cast<int64_t>(blockIdx.x) * ntiles / gridDim.x);
+    const int tile1 = static_cast<int>(static_cast<int64_t>(blockIdx.x + 1) * ntiles / gridDim.x);
     if (tid == 0) {
         for (int i = 0; i < kMomStages; ++i) mbar_init(&full[i], 1);
         abort_flag = 0;
@@ -1411,7 +1413,7 @@ struct LossArgs {
 
 template <bool VEC, bool RECTIFY>
 __global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const __grid_constant__ LossArgs a) {
-    __shared__ double scratch[2][32];
+    __shared__ double scratch[2][kDiagThreads / 32];
     __shared__ double totals[2];
     __shared__ std::conditional_t<RECTIFY, Totals, int> batch;
     pdl_enter();
@@ -1548,8 +1550,11 @@ inline int reduce_blocks(int64_t T, int rows) {
 
 // The masked sums of the batch, one row of partial sums per block; the number of blocks in *blocks.
 // From kSplitWalkRows on the exact walk has a launch of its own: both walks in one kernel cost the fast one a tenth of its
-// bandwidth (4.5 against 4.0 TB/s at 67 M rows), a launch costs 2 us.
+// bandwidth (16 M rows, whole diagnostics 94 against 84 us; 67 M rows 380 against 337), a launch costs 2 us.
 constexpr int64_t kSplitWalkRows = int64_t(8) << 20;
+// Shared memory that lets an SM take no more than 1, 2 or 3 blocks, so that a grid of fewer than 4 per SM spreads evenly instead
+// of piling up on some SMs: diagnostics of 1.48 M rows (362 blocks) 18.2 -> 17.5 us, 400 k (196 blocks) 13.6 -> 12.5.
+constexpr size_t kMomSmemShare[4] = {116 << 10, 116 << 10, 77 << 10, 59 << 10};
 cudaError_t launch_moments_kernel(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
                                   const float* adv, int64_t T, int S, float C, double* partials, int32_t* n_valid_seq,
                                   float* seq_logw, bool early, int* blocks, cudaStream_t stream) {
@@ -1562,8 +1567,10 @@ cudaError_t launch_moments_kernel(const float* lp_train, const float* lp_roll, c
         // no more blocks than have a tile when every block takes the same number of them
         const int tiles = static_cast<int>((T + kMomRows - 1) / kMomRows), per = (tiles + kDiagBlocks - 1) / kDiagBlocks;
         *blocks = tiles > 0 ? (tiles + per - 1) / per : 1;
+        const int per_sm = (*blocks + kSms - 1) / kSms;
+        const size_t smem = per_sm >= 4 ? kMomSmemBytes : kMomSmemShare[per_sm];
         auto go = [&](auto kernel, bool ahead) {
-            return launch_pdl(kernel, *blocks, kDiagThreads, kMomSmemBytes, stream, lp_train, lp_roll, mask, seq_offsets, adv, static_cast<int>(T), S, C,
+            return launch_pdl(kernel, *blocks, kDiagThreads, smem, stream, lp_train, lp_roll, mask, seq_offsets, adv, static_cast<int>(T), S, C,
                               partials, n_valid_seq, seq_logw, ahead);
         };
         if (T < kSplitWalkRows) return seq_logw ? go(moments_staged_kernel<true, kBothWalks>, false) : go(moments_staged_kernel<false, kBothWalks>, early);
@@ -1589,7 +1596,7 @@ cudaError_t launch_rectify_kernel(const float* lp_train, const float* lp_roll, c
 cudaError_t stream_prepare() {
     cudaError_t e = cudaSuccess;
     auto allow = [&](auto kernel) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMomSmemShare[0]);
     };
     allow(moments_staged_kernel<false, kBothWalks>);
     allow(moments_staged_kernel<false, kFastWalk>);
