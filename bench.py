@@ -37,10 +37,10 @@ sys.path.insert(0, ROOT)
 import workloads  # noqa: E402
 
 # DRAM bytes (read + write) of one launch of each tensor-core kernel on a bench workload, from a one-pass profiler capture
-# of the full-size step (the two DRAM byte counters alone need no replay): the two backward kernels are taken together
-# because one call enqueues both.  None for workloads, variants and kernels that were not captured.
+# of the full-size step (the two DRAM byte counters alone need no replay).  None for workloads, variants and kernels that were
+# not captured (the step in one call runs other forms of the trainer pass and of the recompute pass than the stages alone).
 TRAFFIC = {
-    "qwen3_8b": {"fwd_train_bf16": 19.28e9, "fwd_roll_fp8": 9.95e9, "bwd": (31.03e9 + 21.50e9) + (66.69e9 + 0.57e9)},
+    "qwen3_8b": {"fwd_roll_fp8": 9.96e9},
 }
 METRIC = "AIS-corrected fwd+bwd tokens/sec"
 UNIT = "tokens/s"
@@ -271,14 +271,23 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
     # variant (not the headline step): also produce the LM-head weight gradient, one more T x d x V pass
     dW_buf = torch.empty((w.d, w.V) if args.w_dv else (w.V, w.d), dtype=torch.float32, device=dev) if args.with_dw else None
 
-    def one_step(ev=None):
+    def one_step():
+        """The step as a training program runs it: one library call (data parallel: the stages around the all-reduce)."""
+        if dW_buf is None:
+            step.step(batch.H, batch.W, batch.tokens, batch.mask, offs, rew)
+        else:
+            step.forward(batch.H, batch.W, batch.tokens, batch.mask)
+            step.diagnose(batch.mask, offs, rew)
+            step.backward(batch.H, batch.W, batch.tokens, batch.mask, offs, dW=dW_buf)
+
+    def staged_step(ev):
+        """The stages called one by one, with an event between them: what each costs on its own."""
         marks = []
 
         def mark():
-            if ev is not None:
-                e = torch.cuda.Event(enable_timing=True)
-                e.record(stream)
-                marks.append(e)
+            e = torch.cuda.Event(enable_timing=True)
+            e.record(stream)
+            marks.append(e)
         mark()
         ais.quantize_fp8(batch.H, w.block, step.qH, step.sH)
         mark()
@@ -294,8 +303,7 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
         mark()
         step.backward(batch.H, batch.W, batch.tokens, batch.mask, offs, dW=dW_buf)
         mark()
-        if ev is not None:
-            ev.append(marks)
+        ev.append(marks)
 
     def barrier():
         if world > 1:
@@ -311,12 +319,11 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
         one_step()
     barrier()
     sampler = ClockSampler(local) if rank == 0 else None
-    events = []
     t_start = torch.cuda.Event(enable_timing=True)
     t_end = torch.cuda.Event(enable_timing=True)
     t_start.record(stream)
     for _ in range(args.steps):
-        one_step(events)
+        one_step()
     t_end.record(stream)
     barrier()
     total_ms = t_start.elapsed_time(t_end)
@@ -326,12 +333,18 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
         raise RuntimeError(f"device status word {status}")
     diag = step.read_diag()
 
+    # the stages one by one, right behind the timed steps (same clocks and temperature)
+    events = []
+    seg_steps = max(1, min(args.steps, 3))
+    for _ in range(seg_steps):
+        staged_step(events)
+    barrier()
     names = ["quantize_H", "quantize_W", "fwd_train_bf16", "fwd_roll_fp8", "diagnostics", "loss_bwd"]
     seg = {n: 0.0 for n in names}
     for marks in events:
         for i, n in enumerate(names):
             seg[n] += marks[i].elapsed_time(marks[i + 1])
-    seg = {n: v / args.steps for n, v in seg.items()}
+    seg = {n: v / seg_steps for n, v in seg.items()}
 
     # ---- end to end through host buffers
     pin = dict(H=batch.H.cpu().pin_memory(), tokens=batch.tokens.cpu().pin_memory(), mask=batch.mask.cpu().pin_memory(),
@@ -346,12 +359,15 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
 
     # Every step copies its inputs in from pinned host memory and its results (dH, diagnostics, loss) out.  The copies
     # run on two side streams so that a step's input copy and the previous step's result copy overlap the tensor-core
-    # passes: two device buffers for H alternate, and the backward waits until the previous dH has left the device.
+    # passes: two device buffers for H and two for dH alternate.
     in_s, out_s = torch.cuda.Stream(device=dev), torch.cuda.Stream(device=dev)
     Hbuf = [H2, torch.empty_like(batch.H)]
     ev_in = [torch.cuda.Event(), torch.cuda.Event()]
     ev_used = [torch.cuda.Event(), torch.cuda.Event()]      # the step that read Hbuf[i] has finished
-    ev_bwd, ev_out = torch.cuda.Event(), torch.cuda.Event()
+    ev_bwd = torch.cuda.Event()
+    ev_out = [torch.cuda.Event(), torch.cuda.Event()]       # dHbuf[i] and its step's small results have reached the host
+    dHbuf = [step.dH, torch.empty_like(step.dH)]
+    small_dev = [torch.empty(small_host.numel(), dtype=torch.float64, device=dev) for _ in range(2)]
 
     def e2e_prefetch(i):
         with torch.cuda.stream(in_s):
@@ -368,23 +384,30 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
         offs2.copy_(pin["offs"], non_blocking=True)
         rew2.copy_(pin["rew"], non_blocking=True)
         Hi = Hbuf[i % 2]
-        step.forward(Hi, batch.W, tok2, msk2)
-        step.diagnose(msk2, offs2, rew2)
-        stream.wait_event(ev_out)                           # dH and the diagnostics of the previous step are on the host
-        step.backward(Hi, batch.W, tok2, msk2, offs2)
+        stream.wait_event(ev_out[i % 2])                    # the results of the step before the last are on the host
+        step.dH = dHbuf[i % 2]
+        if dW_buf is None:
+            step.step(Hi, batch.W, tok2, msk2, offs2, rew2)
+        else:
+            step.forward(Hi, batch.W, tok2, msk2)
+            step.diagnose(msk2, offs2, rew2)
+            step.backward(Hi, batch.W, tok2, msk2, offs2)
+        small = small_dev[i % 2]
+        small[:-1].copy_(step.diag)
+        small[-1:].copy_(step.loss)
         ev_bwd.record(stream)
         ev_used[i % 2].record(stream)
         with torch.cuda.stream(out_s):
             out_s.wait_event(ev_bwd)
-            dH_host.copy_(step.dH, non_blocking=True)
-            small_host[:-1].copy_(step.diag, non_blocking=True)
-            small_host[-1:].copy_(step.loss.double(), non_blocking=True)
-            ev_out.record(out_s)
+            dH_host.copy_(dHbuf[i % 2], non_blocking=True)
+            small_host.copy_(small, non_blocking=True)
+            ev_out[i % 2].record(out_s)
 
     e2e_steps = max(1, min(args.steps, 5))
     ev_used[0].record(stream)
     ev_used[1].record(stream)
-    ev_out.record(stream)
+    ev_out[0].record(stream)
+    ev_out[1].record(stream)
     e2e_prefetch(0)
     e2e_step(0, True)                                       # warm-up
     barrier()
@@ -394,7 +417,8 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
     e2e_prefetch(0)
     for i in range(e2e_steps):
         e2e_step(i, i == e2e_steps - 1)
-    stream.wait_event(ev_out)                               # the last results have reached the host
+    for e in ev_out:                                        # the last results have reached the host
+        stream.wait_event(e)
     e1.record(stream)
     barrier()
     e2e_ms = e0.elapsed_time(e1) / e2e_steps
@@ -414,7 +438,12 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
     blk_rows = (step.workspace.numel() - fixed) // (_ld_u(w.V) * 2) // 128 * 128
     blk_rows = max(128, min(blk_rows, (T + 127) // 128 * 128))
     chunks = -(-T // blk_rows)
-    launches = (6 if w.block == 0 else 4 if w.block < 0 else 2) + 3 + 3 + (4 if world == 1 else 5) + 4 + (3 if args.with_dw else 2) * chunks
+    # kernels per step: quantisers with the opening of the log-probs, two passes, their merge with the advantages, moments, loss;
+    # then per row chunk recompute (or the launch that finds nothing to recompute), dH and dW.  Data parallel: advantages,
+    # totals, rectification and the sequence counts are launches of their own.
+    launches = (6 if w.block == 0 else 3 if w.block < 0 else 2 if args.w_dv else 1) + 5 + (3 if args.with_dw else 2) * chunks
+    if world > 1 or args.with_dw:
+        launches += 4 if world > 1 else 3
     return dict(ms_per_step=total_ms / args.steps, e2e_ms=e2e_ms, n_valid=n_valid, T=T, seg=seg, clocks=clocks, diag=diag,
                 h2d=h2d, d2h=d2h, streaming=streaming, zero_rows=int(T - live.sum() - (batch.mask.cpu().numpy() == 0).sum()),
                 rows_recompute=rows_recompute, rows_dh=rows_dh, bwd_row_chunks=chunks, launches_per_step=launches,
@@ -466,11 +495,11 @@ def assemble_line(args, world: int, local: dict, glob: dict) -> dict:
     per_kernel = {"fwd_train_bf16": seg["fwd_train_bf16"], "fwd_roll_fp8": seg["fwd_roll_fp8"], "bwd": seg["loss_bwd"] / n_bwd}
     top = max(per_kernel, key=per_kernel.get)
     kernel_names = {
-        "fwd_train_bf16": "lmhead_kernel<bf16 forward> (trainer log-probs)",
-        "fwd_roll_fp8": {0: "lmhead_kernel<per-tensor FP8 forward>", -32: "lmhead_kernel<microscaling FP8 forward>",
+        "fwd_train_bf16": "lmhead_kernel<bf16 forward> with two row tiles per CTA (lmhead_pair_kernel; trainer log-probs)",
+        "fwd_roll_fp8": {0: "lmhead_pair_kernel<per-tensor FP8 forward>", -32: "lmhead_kernel<microscaling FP8 forward>",
                          -4: "lmhead_kernel<microscaling FP4 forward>"}.get(
             w.block, "lmhead_fp8_block_kernel (rollout log-probs, E4M3 with fp32 scales per %d elements)" % w.block),
-        "bwd": "lmhead_kernel<recompute> and lmhead_kernel<dH> (average of the two launches)",
+        "bwd": "lmhead_pair_kernel<recompute> and lmhead_kernel<dH> (average of the two launches)",
     }
     tp = passes[top]
     roofline = {"bound": "tensor", "kernel": kernel_names[top], "achieved": tp["tflops"], "peak": tp["peak"], "unit": "TFLOP/s",
@@ -497,6 +526,8 @@ def assemble_line(args, world: int, local: dict, glob: dict) -> dict:
                    "parallelism": f"dp{world} (whole prompts per GPU, LM head replicated, one all-reduce of 12 moments for alpha)",
                    "bwd_row_chunks": local["bwd_row_chunks"], "alpha": local["diag"]["alpha"], "d_bar": local["diag"]["d_bar"]},
         "segments_ms": seg,
+        "segments_note": "the stages called one by one in separate steps (their sum is above ms_per_step: a step in one call has no "
+                         "recompute pass, the forward pass leaves its exponentials for dH)",
         "roofline": roofline,
         "e2e": {"value": glob["tokens_all"] / (glob["e2e_ms"] * 1e-3), "unit": UNIT, "h2d_bytes_per_step": local["h2d"],
                 "d2h_bytes_per_step": local["d2h"],
