@@ -132,8 +132,8 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                             tma_load_2d(sA, &tmA, &full[st.idx], kelem, w.rt * kBM);
                         }
                         if (B_MN) {
-                            // B is stored with the output column as the contiguous axis (W[v, n] in the dH pass, H[t, n] in
-                            // the dW pass, W[k, v] in the forward passes over a [d, V] head): four blocks of 64 columns, one
+                            // B is stored with the output column as the contiguous axis (W[v, n] in the dH pass, W[k, v] in
+                            // the forward passes over a [d, V] head): four blocks of 64 columns, one
                             // after the other in shared memory.  One copy for the four: with a copy each the forward pass over a
                             // [d, V] head took 14.2 Mcycles for 9,217 rows, 11.8 now (as much as the other layout).  The last,
                             // partial tile of such a head keeps single boxes, which end at V.
