@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 import torch
 
+import loss_bound
 import workloads
 from oracle import ais as oais
 
@@ -55,10 +56,12 @@ def test_non_finite_hidden_state_raises_the_flag_and_neutralises_the_row():
     # loss and gradient: the row is left out (its count still normalises its sequence)
     _, _, wbar = oais.ratios(lp_t, lp_r, a["mask"], 5.0)
     w_tilde = oais.rectify(wbar, diag["alpha"], a["mask"])
-    loss, c = oais.loss_and_coeff(lp_t, lp_t, a["mask"], a["seq_offsets"], adv, w_tilde, w.P, w.G, 0.2)
+    _, c = oais.loss_and_coeff(lp_t, lp_t, a["mask"], a["seq_offsets"], adv, w_tilde, w.P, w.G, 0.2)
     n_s = oais.valid_counts(a["mask"], a["seq_offsets"])[sid[bad]]
-    loss_without = loss + w_tilde[bad] * adv[sid[bad]] / (w.P * w.G * n_s)
-    assert abs(float(step.loss.item()) - loss_without) <= 1e-3 * max(1.0, abs(loss_without))
+    g_wt = step.w_tilde[:T].cpu().numpy().astype(np.float64)
+    loss, terms = loss_bound.reference(lp_t, a["mask"], a["seq_offsets"], adv, g_wt, w.P, w.G)
+    loss_without = loss + g_wt[bad] * adv[sid[bad]] / (w.P * w.G * n_s)
+    assert abs(float(step.loss.item()) - loss_without) <= 2.0 ** -23 * abs(loss_without) + 1e-10 * terms
     c[bad] = 0.0
     dH_ref = oais.grad_hidden(a["H"], a["W"], a["tokens"], c)
     dH = step.dH[:T].float().cpu().numpy().astype(np.float64)

@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 import torch
 
+import loss_bound
 import workloads
 from oracle import ais as oais
 
@@ -46,8 +47,12 @@ def test_padded_sequences_equal_packed_sequences():
         assert torch.equal(getattr(packed, name)[:b.T].cpu(), getattr(padded, name).cpu()[r]), name
     dp, dq = packed.read_diag(), padded.read_diag()
     assert dp["n_valid"] == dq["n_valid"] == float(b.mask.sum())
-    for k in ("alpha", "d_bar", "cv2", "ess", "delta_sigma", "loss"):
+    for k in ("alpha", "d_bar", "cv2", "ess", "delta_sigma"):
         assert abs(dp[k] - dq[k]) <= 1e-6 * max(1.0, abs(dp[k])), k
+    # the weights differ by alpha's 1e-6 and their own rounding, the losses by that times their terms
+    _, terms = loss_bound.reference(packed.lp_train[:b.T].cpu().numpy(), b.mask.numpy(), offs, packed.adv.cpu().numpy(), np.ones(b.T), w.P, w.G)
+    assert abs(dp["loss"] - dq["loss"]) <= 5e-6 * terms
+    loss_bound.check_step(packed, dict(mask=b.mask.numpy(), seq_offsets=offs), w.P, w.G, b.T)
     assert torch.equal(packed.n_valid_seq.cpu(), padded.n_valid_seq.cpu())
     dH_packed = packed.dH[:b.T].float().cpu()
     dH_padded = padded.dH.float().cpu()
