@@ -113,6 +113,18 @@ __device__ __forceinline__ void walk_rows(const __nv_bfloat16* __restrict__ x, i
     }
 }
 
+// Row and column of a block's tile: tiles are numbered along the rows first, on grid.x alone (grid.y ends at 65,535 blocks,
+// a million rows).
+struct QuantTile {
+    int64_t row0, col0;
+    bool last_rows;          // one of the tiles with the last rows
+};
+template <int RPW>
+__device__ __forceinline__ QuantTile quant_tile(unsigned tiles_x) {
+    const unsigned row = blockIdx.x / tiles_x;
+    return {static_cast<int64_t>(row) * (kQWarps * RPW), static_cast<int64_t>(blockIdx.x % tiles_x) * kQCols, row == (gridDim.x - 1) / tiles_x};
+}
+
 // FlagsJob by blocks of kQThreads threads: one warp per 128-row tile.
 constexpr int kFlagTiles = kQThreads / 32;
 inline unsigned flag_blocks(const FlagsJob& f) { return static_cast<unsigned>(((f.T + 127) / 128 + kFlagTiles - 1) / kFlagTiles); }
@@ -299,18 +311,19 @@ template <bool FP4, int RPW>
 __global__ void __launch_bounds__(kQThreads) quantize_mx_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows,
                                                                              int64_t padded_rows, int64_t cols, int64_t ld,
                                                                              uint8_t* __restrict__ codes, int64_t ldq,
-                                                                             uint8_t* __restrict__ scales) {
+                                                                             uint8_t* __restrict__ scales, unsigned tiles_x) {
     pdl_enter();
     const int lane = threadIdx.x & 31;
     const int64_t nk4 = cols / 128;
     auto scale_word = [&](int64_t row, int64_t k4) {
         return reinterpret_cast<uint32_t*>(scales + ((row >> 8) * nk4 + k4) * 1024 + ((row >> 7) & 1) * 512 + (row & 31) * 16 + ((row & 127) >> 5) * 4);
     };
-    const int64_t row0 = static_cast<int64_t>(blockIdx.y) * (kQWarps * RPW), col0 = static_cast<int64_t>(blockIdx.x) * kQCols;
-    if (blockIdx.y == gridDim.y - 1)
+    const QuantTile tile = quant_tile<RPW>(tiles_x);
+    const int64_t col0 = tile.col0;
+    if (tile.last_rows)
         for (int64_t i = threadIdx.x; i < (padded_rows - rows) * 8; i += kQThreads)
             if (col0 / 128 + i % 8 < nk4) *scale_word(rows + i / 8, col0 / 128 + i % 8) = 0x7F7F7F7Fu;
-    walk_rows<RPW>(x, rows, cols, ld, row0, col0, [&](int64_t row, const uint4 (&raw)[kQIters]) {
+    walk_rows<RPW>(x, rows, cols, ld, tile.row0, col0, [&](int64_t row, const uint4 (&raw)[kQIters]) {
             if (row >= rows) return;
             uint32_t pair = 0;
 #pragma unroll
@@ -357,13 +370,14 @@ __global__ void __launch_bounds__(kQThreads) quantize_mx_kernel(const __nv_bfloa
 // ------------------------------------------------------------------------------------------------
 template <int RPW>
 __global__ void __launch_bounds__(kQThreads) tensor_amax_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
-                                                                uint32_t* __restrict__ amax_bits) {
+                                                                uint32_t* __restrict__ amax_bits, unsigned tiles_x) {
     __shared__ uint32_t block_max;
     if (threadIdx.x == 0) block_max = 0;
     pdl_enter();
     __syncthreads();
     uint32_t m = 0;
-    walk_rows<RPW>(x, rows, cols, ld, static_cast<int64_t>(blockIdx.y) * (kQWarps * RPW), static_cast<int64_t>(blockIdx.x) * kQCols,
+    const QuantTile tile = quant_tile<RPW>(tiles_x);
+    walk_rows<RPW>(x, rows, cols, ld, tile.row0, tile.col0,
                    [&](int64_t, const uint4 (&raw)[kQIters]) {
 #pragma unroll
                        for (int it = 0; it < kQIters; ++it)
@@ -387,13 +401,13 @@ __global__ void tensor_scale_kernel(uint32_t* scale_word) {
 template <int RPW>
 __global__ void __launch_bounds__(kQThreads) tensor_quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
                                                                     uint8_t* __restrict__ codes, int64_t ldq,
-                                                                    const float* __restrict__ scale) {
+                                                                    const float* __restrict__ scale, unsigned tiles_x) {
     pdl_enter();
     const float s = *scale;
     const float y = __frcp_rn(s);
-    const int64_t col0 = static_cast<int64_t>(blockIdx.x) * kQCols + (threadIdx.x & 31) * 8;
-    walk_rows<RPW>(x, rows, cols, ld, static_cast<int64_t>(gridDim.y - 1 - blockIdx.y) * (kQWarps * RPW),
-                   static_cast<int64_t>(blockIdx.x) * kQCols, [&](int64_t row, const uint4 (&raw)[kQIters]) {
+    const QuantTile tile = quant_tile<RPW>(tiles_x);
+    const int64_t col0 = tile.col0 + (threadIdx.x & 31) * 8;
+    walk_rows<RPW>(x, rows, cols, ld, static_cast<int64_t>((gridDim.x - 1) / tiles_x) * (kQWarps * RPW) - tile.row0, tile.col0, [&](int64_t row, const uint4 (&raw)[kQIters]) {
                        if (row >= rows) return;
 #pragma unroll
                        for (int it = 0; it < kQIters; ++it)
@@ -1613,19 +1627,19 @@ cudaError_t stream_prepare() {
 inline bool quant_wide(int64_t rows, int64_t cols) {
     return ((cols + kQCols - 1) / kQCols) * ((rows + 4 * kQWarps - 1) / (4 * kQWarps)) >= 148;
 }
-inline dim3 quant_grid(int64_t rows, int64_t cols) {
-    const int per = kQWarps * (quant_wide(rows, cols) ? 4 : 1);
-    return dim3(static_cast<unsigned>((cols + kQCols - 1) / kQCols), static_cast<unsigned>((rows + per - 1) / per));
+inline unsigned quant_tiles_x(int64_t cols) { return static_cast<unsigned>((cols + kQCols - 1) / kQCols); }
+inline unsigned quant_blocks(int64_t rows, int64_t cols, bool wide) {
+    const int per = kQWarps * (wide ? 4 : 1);
+    return quant_tiles_x(cols) * static_cast<unsigned>((rows + per - 1) / per);
 }
 
 cudaError_t launch_quantize(const QuantJob* jobs, int njobs, int64_t cols, int block, const FlagsJob* flags, cudaStream_t stream) {
-    const unsigned tiles_x = static_cast<unsigned>((cols + kQCols - 1) / kQCols);
+    const unsigned tiles_x = quant_tiles_x(cols);
     int64_t rows = 0;
     for (int i = 0; i < njobs; ++i) rows += jobs[i].rows;
     const bool wide = quant_wide(rows, cols);
-    const int per = kQWarps * (wide ? 4 : 1);
     unsigned n[2] = {0, 0};
-    for (int i = 0; i < njobs; ++i) n[i] = tiles_x * static_cast<unsigned>((jobs[i].rows + per - 1) / per);
+    for (int i = 0; i < njobs; ++i) n[i] = quant_blocks(jobs[i].rows, cols, wide);
     const FlagsJob f = flags ? *flags : FlagsJob{};
     const unsigned blocks = n[0] + n[1] + (flags ? flag_blocks(f) : 0);
     if (blocks == 0) return cudaSuccess;
@@ -1654,11 +1668,11 @@ cudaError_t launch_quantize_cols(const void* x, int64_t K, int64_t N, int64_t ld
 cudaError_t launch_quantize_mx(const void* x, int64_t rows, int64_t cols, int64_t ld, uint8_t* codes, int64_t ldq,
                                uint8_t* scales, size_t scale_bytes, bool fp4, cudaStream_t stream) {
     if (rows == 0 || cols == 0) return cudaMemsetAsync(scales, 127, scale_bytes, stream);       // padding only
-    const dim3 grid = quant_grid(rows, cols);
     const bool wide = quant_wide(rows, cols);
+    const unsigned tiles_x = quant_tiles_x(cols), blocks = quant_blocks(rows, cols, wide);
     const int64_t padded = static_cast<int64_t>(scale_bytes / 512) / (cols / 128) * 128;
     auto go = [&](auto kernel) {
-        return launch_pdl(kernel, grid, kQThreads, 0, stream, static_cast<const __nv_bfloat16*>(x), rows, padded, cols, ld, codes, ldq, scales);
+        return launch_pdl(kernel, blocks, kQThreads, 0, stream, static_cast<const __nv_bfloat16*>(x), rows, padded, cols, ld, codes, ldq, scales, tiles_x);
     };
     if (fp4) return go(wide ? quantize_mx_kernel<true, 4> : quantize_mx_kernel<true, 1>);
     return go(wide ? quantize_mx_kernel<false, 4> : quantize_mx_kernel<false, 1>);
@@ -1670,15 +1684,16 @@ cudaError_t launch_quantize_tensor(const void* x, int64_t rows, int64_t cols, in
     if (e != cudaSuccess) return e;
     const __nv_bfloat16* xp = static_cast<const __nv_bfloat16*>(x);
     const bool any = rows > 0 && cols > 0, wide = quant_wide(rows, cols);
-    const dim3 grid = quant_grid(rows, cols);
+    const unsigned tiles_x = quant_tiles_x(cols), blocks = quant_blocks(rows, cols, wide);
     if (any) {
-        e = launch_pdl(wide ? tensor_amax_kernel<4> : tensor_amax_kernel<1>, grid, kQThreads, 0, stream, xp, rows, cols, ld,
-                       reinterpret_cast<uint32_t*>(scale));
+        e = launch_pdl(wide ? tensor_amax_kernel<4> : tensor_amax_kernel<1>, blocks, kQThreads, 0, stream, xp, rows, cols, ld,
+                       reinterpret_cast<uint32_t*>(scale), tiles_x);
         if (e != cudaSuccess) return e;
     }
     e = launch_pdl(tensor_scale_kernel, 1, 1, 0, stream, reinterpret_cast<uint32_t*>(scale));
     if (e != cudaSuccess || !any) return e;
-    return launch_pdl(wide ? tensor_quantize_kernel<4> : tensor_quantize_kernel<1>, grid, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scale);
+    return launch_pdl(wide ? tensor_quantize_kernel<4> : tensor_quantize_kernel<1>, blocks, kQThreads, 0, stream, xp, rows, cols, ld, codes, ldq, scale,
+                      tiles_x);
 }
 
 cudaError_t launch_combine(const CombineJob* jobs, int njobs, int64_t part_ld, const uint8_t* mask, int64_t T, uint32_t* status,
