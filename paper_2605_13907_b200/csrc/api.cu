@@ -599,9 +599,10 @@ int ais_logprob_fwd(const ais_shape* shape, const ais_params* params, const void
                        dev_status, workspace, workspace_bytes, stream, Fuse());
 }
 
-static int diagnostics(const ais_shape* shape, const ais_params* params, const float* lp_train, const float* lp_roll,
-                       const uint8_t* mask, const int32_t* seq_offsets, const float* rewards, float* adv, int32_t* n_valid_seq,
-                       float* rho, float* w_tilde, ais_diag* diag, void* workspace, size_t workspace_bytes, void* stream, const Fuse& fuse) {
+// What ais_diagnostics refuses.
+static int check_diagnostics(const ais_shape* shape, const ais_params* params, const void* lp_train, const void* lp_roll, const void* mask,
+                             const void* seq_offsets, const void* rewards, const void* adv, const void* w_tilde, const void* diag,
+                             const void* workspace, size_t workspace_bytes) {
     int st = check_shape(shape);
     if (st != AIS_OK) return st;
     st = check_params(params);
@@ -609,10 +610,20 @@ static int diagnostics(const ais_shape* shape, const ais_params* params, const f
     if (!lp_train || !lp_roll || !mask || !seq_offsets || !rewards || !adv || !w_tilde || !diag) return AIS_ERR_NULL;
     if (!aligned(diag, 8)) return AIS_ERR_ALIGN;
     const Layout L = make_layout(shape, params);
-    const bool seq_level = params->seq_level_weights != 0;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < (seq_level ? L.off_split : L.off_coef)) return AIS_ERR_WORKSPACE;
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < (params->seq_level_weights != 0 ? L.off_split : L.off_coef))
+        return AIS_ERR_WORKSPACE;
+    return AIS_OK;
+}
+
+static int diagnostics(const ais_shape* shape, const ais_params* params, const float* lp_train, const float* lp_roll,
+                       const uint8_t* mask, const int32_t* seq_offsets, const float* rewards, float* adv, int32_t* n_valid_seq,
+                       float* rho, float* w_tilde, ais_diag* diag, void* workspace, size_t workspace_bytes, void* stream, const Fuse& fuse) {
+    int st = check_diagnostics(shape, params, lp_train, lp_roll, mask, seq_offsets, rewards, adv, w_tilde, diag, workspace, workspace_bytes);
+    if (st != AIS_OK) return st;
     st = device_setup(nullptr);
     if (st != AIS_OK) return st;
+    const Layout L = make_layout(shape, params);
+    const bool seq_level = params->seq_level_weights != 0;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const int S = shape->P * shape->G;
@@ -890,8 +901,12 @@ int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_ar
     const AdvJob adv = {a->rewards, S, shape->G, params->adv_std_norm, params->eps, a->adv, a->n_valid_seq,
                         reinterpret_cast<uint32_t*>(static_cast<uint8_t*>(a->workspace) + L.off_ticket)};
     RectifyJob rectify;
-    // the diagnostics' advantages ride on the merge of the log-probs when there is one
-    if (logprob && diag && a->rewards && a->adv && a->lp_train && a->lp_roll && shape->T > 0) fuse.adv = &adv;
+    // The diagnostics' advantages ride on the merge of the log-probs when there is one -- and when the diagnostics are going to
+    // run: the merge is checked for what the log-probs need, and the counters that the advantages clear lie behind that.
+    if (logprob && diag && shape->T > 0 &&
+        check_diagnostics(shape, params, a->lp_train, a->lp_roll, a->mask, a->seq_offsets, a->rewards, a->adv, a->w_tilde, a->diag, a->workspace,
+                          a->workspace_bytes) == AIS_OK)
+        fuse.adv = &adv;
     // log-probs and loss in one call: the exponentials of the rows that the scratch holds stay there (dW wants plain form)
     if (fuse.adv && loss && !a->dW && a->n_valid_seq && a->lse_train && a->dH && a->workspace_bytes >= L.fixed_bytes + static_cast<size_t>(kBM) * L.u_row_bytes)
         fuse.keep_rows = scratch_rows(L, shape->T, a->workspace_bytes);
