@@ -688,11 +688,10 @@ int ais_diag_finalize(const ais_shape* shape, const ais_params* params, const do
     return AIS_OK;
 }
 
-static int loss_bwd(const ais_shape* shape, const ais_params* params, const void* H, const void* W, const int32_t* tokens,
-                    const uint8_t* mask, const int32_t* seq_offsets, const float* lse_train, const float* lp_train,
-                    const float* lp_old, const float* lp_ref, const float* adv, const float* w_tilde, void* dH, float* loss,
-                    ais_diag* diag, float* dW, int64_t lddw, int dw_accumulate,
-                    uint32_t* dev_status, void* workspace, size_t workspace_bytes, void* stream, const Fuse& fuse) {
+// What ais_loss_bwd refuses.
+static int check_loss(const ais_shape* shape, const ais_params* params, const void* H, const void* W, const void* tokens, const void* mask,
+                      const void* seq_offsets, const void* lse_train, const void* lp_train, const void* adv, const void* w_tilde, const void* dH,
+                      const void* dW, int64_t lddw, const void* workspace, size_t workspace_bytes) {
     int st = check_shape(shape);
     if (st != AIS_OK) return st;
     st = check_params(params);
@@ -704,9 +703,20 @@ static int loss_bwd(const ais_shape* shape, const ais_params* params, const void
     const Layout L = make_layout(shape, params);
     if (!workspace || !aligned(workspace, 256) || workspace_bytes < L.fixed_bytes + static_cast<size_t>(kBM) * L.u_row_bytes)
         return AIS_ERR_WORKSPACE;
+    return AIS_OK;
+}
+
+static int loss_bwd(const ais_shape* shape, const ais_params* params, const void* H, const void* W, const int32_t* tokens,
+                    const uint8_t* mask, const int32_t* seq_offsets, const float* lse_train, const float* lp_train,
+                    const float* lp_old, const float* lp_ref, const float* adv, const float* w_tilde, void* dH, float* loss,
+                    ais_diag* diag, float* dW, int64_t lddw, int dw_accumulate,
+                    uint32_t* dev_status, void* workspace, size_t workspace_bytes, void* stream, const Fuse& fuse) {
+    int st = check_loss(shape, params, H, W, tokens, mask, seq_offsets, lse_train, lp_train, adv, w_tilde, dH, dW, lddw, workspace, workspace_bytes);
+    if (st != AIS_OK) return st;
     int num_sms = 0;
     st = device_setup(&num_sms);
     if (st != AIS_OK) return st;
+    const Layout L = make_layout(shape, params);
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
@@ -907,8 +917,12 @@ int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_ar
         check_diagnostics(shape, params, a->lp_train, a->lp_roll, a->mask, a->seq_offsets, a->rewards, a->adv, a->w_tilde, a->diag, a->workspace,
                           a->workspace_bytes) == AIS_OK)
         fuse.adv = &adv;
+    // What the loss takes over from earlier stages it takes over only when it is going to run.
+    const bool loss_runs = loss && shape->T > 0 &&
+                           check_loss(shape, params, a->H, a->W, a->tokens, a->mask, a->seq_offsets, a->lse_train, a->lp_train, a->adv, a->w_tilde,
+                                      a->dH, a->dW, a->lddw, a->workspace, a->workspace_bytes) == AIS_OK;
     // log-probs and loss in one call: the exponentials of the rows that the scratch holds stay there (dW wants plain form)
-    if (fuse.adv && loss && !a->dW && a->n_valid_seq && a->lse_train && a->dH && a->workspace_bytes >= L.fixed_bytes + static_cast<size_t>(kBM) * L.u_row_bytes)
+    if (fuse.adv && loss_runs && !a->dW && a->n_valid_seq)
         fuse.keep_rows = scratch_rows(L, shape->T, a->workspace_bytes);
     if (logprob)
         st = logprob_fwd(shape, params, a->H, a->W, a->qH, a->sH, a->ldsH, a->qW, a->sW, a->ldsW, a->tokens, a->mask, a->lp_train,
@@ -916,7 +930,7 @@ int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_ar
     if (st != AIS_OK) return st;
     if (diag) {
         // the loss takes the counts from here and forms rho and w_tilde; the diagnostics' advantages have cleared its ticket
-        if (loss && a->n_valid_seq && shape->T > 0) {
+        if (loss_runs && a->n_valid_seq) {
             fuse.counts = a->n_valid_seq;
             rectify = {a->lp_roll, params->C, TotalsJob{}, a->rho, a->w_tilde,
                        params->seq_level_weights ? reinterpret_cast<const float*>(static_cast<uint8_t*>(a->workspace) + L.off_seqw) : nullptr};

@@ -77,3 +77,18 @@ def test_a_workspace_for_the_log_probs_alone_is_not_written_behind():
         assert bool((c.out[name] == 7).all()), name
     for name in ("lp_train", "lse_train", "lp_roll", "lse_roll"):
         assert torch.equal(c.out[name], ref.out[name]), name
+
+
+@pytest.mark.parametrize("refused", ["dH", "lse_train", "workspace", "lddw"])
+def test_a_refused_loss_leaves_the_stages_before_it_whole(refused):
+    """The diagnostics of a call whose loss stage is refused: the same bits as without that stage."""
+    before = _stages("QUANTIZE_H", "QUANTIZE_W", "LOGPROB", "DIAGNOSE")
+    c, ref = Call(), Call()
+    assert ref.run(before) == 0
+    dW = torch.empty(1032, 256, device="cuda")
+    changed = {"dH": dict(dH=None), "lse_train": dict(lse_train=None), "lddw": dict(dW=dW.data_ptr(), lddw=128),
+               "workspace": dict(workspace_bytes=c.ais.workspace_min_bytes(c.step.shape, c.step.params) - 1)}[refused]
+    assert c.run(before | _stages("LOSS"), **changed) < 0
+    for name in ("lp_train", "lp_roll", "adv", "n_valid_seq", "rho", "w_tilde", "diag"):
+        assert torch.equal(c.out[name], ref.out[name]), name
+    assert bool((c.out["dH"] == 7).all()) and float(c.out["loss"]) == 7.0
