@@ -320,7 +320,7 @@ int64_t scratch_rows(const Layout& L, int64_t T, size_t workspace_bytes) {
 // whose work fits into a neighbour's.
 struct Fuse {
     const QuantJob* quant = nullptr;     // log-probs: quantise these first, in the opening launch
-    int nquant = 0;
+    int* nquant = nullptr;               // how many; zeroed by that launch
     const AdvJob* adv = nullptr;         // log-probs: advantages in the merging launch; diagnostics: they are there already
     TotalsJob* totals = nullptr;         // diagnostics: leave the end (alpha, rho, w_tilde) to the loss, described here
     const RectifyJob* rectify = nullptr; // loss: form them
@@ -581,8 +581,10 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
     }
     if (!maps) return AIS_ERR_DEVICE;
     const FlagsJob flags = {mask, T, ws + L.off_flags, paced ? ws + L.off_pace : nullptr, 2 * kPaceRingBytes};
-    if ((fuse.nquant > 0 ? launch_quantize(fuse.quant, fuse.nquant, d, shape->fp8_block, &flags, s) : launch_flags(flags, s)) != cudaSuccess)
+    const int nquant = fuse.nquant ? *fuse.nquant : 0;
+    if ((nquant > 0 ? launch_quantize(fuse.quant, nquant, d, shape->fp8_block, &flags, s) : launch_flags(flags, s)) != cudaSuccess)
         return AIS_ERR_DEVICE;
+    if (nquant > 0) *fuse.nquant = 0;
     for (int i = 0; i < n; ++i)
         if ((pass[i].two ? launch_lmhead_pair(pass[i].mode, pass[i].tmA, pass[i].tmB, pass[i].tmSA, pass[i].a, pass[i].ctas, s)
                          : launch_lmhead(pass[i].mode, pass[i].tmA, pass[i].tmB, pass[i].tmSA, pass[i].tmSB, pass[i].a, pass[i].ctas, s)) != cudaSuccess)
@@ -891,6 +893,7 @@ int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_ar
     Fuse fuse;
     // codes with fp32 block scales come from the launch that opens the log-probs ([d, V] heads have a quantiser of their own)
     QuantJob quant[2];
+    int nquant = 0;
     auto quantize = [&](const void* x, int64_t rows, int64_t ld, uint8_t* codes, int64_t ldq, void* scales, int64_t lds) -> int {
         if (fp4) return ais_quantize_mxfp4(x, rows, shape->d, ld, codes, ldq / 2, static_cast<uint8_t*>(scales), stream);
         if (block == AIS_FP8_MX32) return ais_quantize_mxfp8(x, rows, shape->d, ld, codes, ldq, static_cast<uint8_t*>(scales), stream);
@@ -898,15 +901,28 @@ int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_ar
         float* sc = static_cast<float*>(scales);
         if (!logprob || shape->T == 0) return ais_quantize_fp8(x, rows, shape->d, ld, block, codes, ldq, sc, lds, stream);
         const int bad = check_quantize(x, rows, shape->d, ld, block, codes, ldq, sc, lds);
-        if (bad == AIS_OK) quant[fuse.nquant++] = {x, rows, ld, codes, ldq, sc, lds};
+        if (bad == AIS_OK) quant[nquant++] = {x, rows, ld, codes, ldq, sc, lds};
         return bad;
     };
     if ((stages & AIS_STAGE_QUANTIZE_H) && shape->T > 0) st = quantize(a->H, shape->T, shape->ldh, a->qH, shape->ldh, a->sH, a->ldsH);
     if (st == AIS_OK && (stages & AIS_STAGE_QUANTIZE_W))
         st = dv ? ais_quantize_fp8_cols(a->W, shape->d, shape->V, shape->ldw, block, a->qW, shape->d, static_cast<float*>(a->sW), a->ldsW, stream)
                 : quantize(a->W, shape->V, shape->ldw, a->qW, shape->ldw, a->sW, a->ldsW);
-    if (st != AIS_OK) return st;
+    // the quantisations that wait for the log-probs' opening launch, when it does not come
+    auto flush_quantize = [&]() -> int {
+        const int n = nquant;
+        nquant = 0;
+        if (n == 0) return AIS_OK;
+        const int ready = device_setup(nullptr);
+        if (ready != AIS_OK) return ready;
+        return launch_quantize(quant, n, shape->d, block, nullptr, static_cast<cudaStream_t>(stream)) == cudaSuccess ? AIS_OK : AIS_ERR_DEVICE;
+    };
+    if (st != AIS_OK) {                                     // W is refused; H may have been accepted
+        const int flushed = flush_quantize();
+        return flushed != AIS_OK ? flushed : st;
+    }
     fuse.quant = quant;
+    fuse.nquant = &nquant;
     const int S = shape->P * shape->G;
     const AdvJob adv = {a->rewards, S, shape->G, params->adv_std_norm, params->eps, a->adv, a->n_valid_seq,
                         reinterpret_cast<uint32_t*>(static_cast<uint8_t*>(a->workspace) + L.off_ticket)};
@@ -927,6 +943,8 @@ int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_ar
     if (logprob)
         st = logprob_fwd(shape, params, a->H, a->W, a->qH, a->sH, a->ldsH, a->qW, a->sW, a->ldsW, a->tokens, a->mask, a->lp_train,
                          a->lse_train, a->lp_roll, a->lse_roll, a->dev_status, a->workspace, a->workspace_bytes, stream, fuse);
+    const int flushed = flush_quantize();                   // the log-probs were refused, or none were asked for
+    if (flushed != AIS_OK) return flushed;
     if (st != AIS_OK) return st;
     if (diag) {
         // the loss takes the counts from here and forms rho and w_tilde; the diagnostics' advantages have cleared its ticket

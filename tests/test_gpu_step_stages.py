@@ -92,3 +92,19 @@ def test_a_refused_loss_leaves_the_stages_before_it_whole(refused):
     for name in ("lp_train", "lp_roll", "adv", "n_valid_seq", "rho", "w_tilde", "diag"):
         assert torch.equal(c.out[name], ref.out[name]), name
     assert bool((c.out["dH"] == 7).all()) and float(c.out["loss"]) == 7.0
+
+
+@pytest.mark.parametrize("block", [128, 0])
+@pytest.mark.parametrize("why", ["no pass asked for", "log-probs refused", "codes of W refused"])
+def test_codes_are_written_whatever_becomes_of_the_log_probs(why, block):
+    """Quantisers that ais_step merges into the log-probs' opening launch run without it, too."""
+    c, ref = Call(block), Call(block)
+    assert ref.run(_stages("QUANTIZE_H", "QUANTIZE_W")) == 0
+    changed = {"no pass asked for": dict(lp_train=None, lp_roll=None), "log-probs refused": dict(tokens=None),
+               "codes of W refused": dict(qW=None)}[why]
+    st = c.run(_stages("QUANTIZE_H", "QUANTIZE_W", "LOGPROB"), **changed)
+    assert (st == 0) == (why == "no pass asked for")
+    for name in ("qH", "sH") + (("qW", "sW") if why != "codes of W refused" else ()):
+        assert torch.equal(c.out[name], ref.out[name]), name
+    for name in ("lp_train", "lp_roll"):
+        assert bool((c.out[name] == 7).all()), name
