@@ -161,7 +161,8 @@ void ais_default_params(ais_params* p);
 
 /* Recommended workspace size in bytes for all entry points on this shape (host pointers in).
  * Any 256-byte aligned workspace of at least ais_workspace_min_bytes() is accepted; a larger one
- * lets ais_loss_bwd process more rows per pass.  Returns 0 for an invalid shape. */
+ * lets ais_loss_bwd process more rows per pass.  Neither size falls as T grows, so a workspace sized for a program's
+ * largest batch serves its shorter ones.  Returns 0 for an invalid shape. */
 size_t ais_workspace_bytes(const ais_shape* shape, const ais_params* params);
 size_t ais_workspace_min_bytes(const ais_shape* shape, const ais_params* params);
 

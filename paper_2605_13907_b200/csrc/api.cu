@@ -96,8 +96,14 @@ bool make_tmap_blocks(CUtensorMap* map, const void* base, uint64_t dim0, uint64_
 // wave 2.44 ms, 22 in three better filled ones 2.75; 58,142 rows at d = 5120: 7 ranges 58.1 ms, 11 61.5).  The FP8 block
 // pass does not reach the cap and takes the balance (11 ranges 48.4 ms, 4 52.3).  From below the number is bounded by L2:
 // the hidden rows of the row tiles in flight are read again for every column tile and should take no more than 40 MB of it.
+int unit_rows_of(TileKind kind) { return kind == kTileOne ? kBM : kPairRows; }
+int tile_cols_of(TileKind kind) { return kind == kTileBlock ? kPairCols : kBN; }
+double range_handicap(TileKind kind) { return kind == kTileBlock ? 400.0 : 120.0; }
+bool ranges_fit_l2(TileKind kind, int64_t in_flight, int d) {
+    return in_flight * (unit_rows_of(kind) / kBM) * d * (kind == kTileBlock ? 128 : 256) <= (int64_t(40) << 20);
+}
 PassPlan plan_kind(TileKind kind, int64_t rows, int V, int d, int most, int forced, double* cost) {
-    const int unit_rows = kind == kTileOne ? kBM : kPairRows, tile_cols = kind == kTileBlock ? kPairCols : kBN;
+    const int unit_rows = unit_rows_of(kind), tile_cols = tile_cols_of(kind);
     const int64_t units = rows > 0 ? (rows + unit_rows - 1) / unit_rows : 1;
     const int col_tiles = (V + tile_cols - 1) / tile_cols;
     if (most > col_tiles) most = col_tiles;
@@ -108,9 +114,9 @@ PassPlan plan_kind(TileKind kind, int64_t rows, int V, int d, int most, int forc
         if (forced > 0 && s != (forced < most ? forced : most)) continue;
         int64_t in_flight = kSms / s > 0 ? kSms / s : 1;
         if (in_flight > units) in_flight = units;
-        if (in_flight * (unit_rows / kBM) * d * (kind == kTileBlock ? 128 : 256) > (int64_t(40) << 20) && s < most && forced <= 0) continue;
+        if (!ranges_fit_l2(kind, in_flight, d) && s < most && forced <= 0) continue;
         const int64_t waves = (units * s + kSms - 1) / kSms;
-        const double c = static_cast<double>(waves) * ((col_tiles + s - 1) / s) * (1.0 + s / (kind == kTileBlock ? 400.0 : 120.0));
+        const double c = static_cast<double>(waves) * ((col_tiles + s - 1) / s) * (1.0 + s / range_handicap(kind));
         if (best_cost == 0.0 || c < best_cost) { best = s; best_cost = c; }
     }
     // clocks of a tile: 512 per stage and row tile on the tensor cores at best.  One row tile: 620, and no less than its epilogue
@@ -119,6 +125,24 @@ PassPlan plan_kind(TileKind kind, int64_t rows, int V, int d, int most, int forc
     const double tile = kind == kTileTwo ? fmax(1040.0 * stages + 700.0, 7500.0) : fmax(620.0 * stages, 3500.0);
     if (cost) *cost = best_cost * tile;
     return {kind == kTileTwo, best, unit_rows, tile_cols};
+}
+
+// Rows x ranges that plan_kind does not exceed for any batch of up to `rows` rows.  Its own choice does not grow with the batch
+// (5 row tiles take more ranges than 6), and a workspace sized by it for the largest batch would be too small for a shorter
+// one.  The choice s costs no less than units x col_tiles / kSms x (1 + s / h) and no more than that of any t within the L2
+// bound, less than (units x t / kSms + 1) x (col_tiles / t + 1) x (1 + t / h); so units x s stays below a line in units for
+// every t, and the least of these rises with units.
+int64_t most_range_rows(TileKind kind, int64_t rows, int V, int d, int most, int forced) {
+    const int64_t units = rows > 0 ? (rows + unit_rows_of(kind) - 1) / unit_rows_of(kind) : 1;
+    const int col_tiles = (V + tile_cols_of(kind) - 1) / tile_cols_of(kind);
+    if (most > col_tiles) most = col_tiles;
+    if (forced > 0) return (forced < most ? forced : most) * units * unit_rows_of(kind);
+    const double h = range_handicap(kind), u = static_cast<double>(units);
+    double s_u = most * u;
+    for (int t = 1; t <= most; ++t)
+        if (t == most || ranges_fit_l2(kind, kSms / t, d))
+            s_u = fmin(s_u, h * ((u + static_cast<double>(kSms) / t) * (1.0 + static_cast<double>(t) / col_tiles) * (1.0 + t / h) - u));
+    return static_cast<int64_t>(ceil(s_u * unit_rows_of(kind)));
 }
 
 PassPlan plan_pass(int64_t rows, int V, int d, int most, int forced) {
@@ -195,9 +219,19 @@ int forced_ranges(const ais_shape* s, const ais_params* p) {
 // and read per partial tile at 6 TB/s plus the extra launch.  A range keeps at least four stage fills (the depth of the
 // ring plus one), and the partial tiles number at most kSplitSlots (116 MB).
 constexpr int kSplitSlots = 3 * kSms;
+constexpr double kFillUs = 0.83, kSplitUs = 6.0, kSlotUs = 0.087;
 double split_cost(int tiles, int ks, int ksteps) {
     const double waves = (static_cast<int64_t>(tiles) * ks + kSms - 1) / kSms;
-    return waves * ((ksteps + ks - 1) / ks) * 0.83 + (ks > 1 ? 6.0 + tiles * ks * 0.087 : 0.0);
+    return waves * ((ksteps + ks - 1) / ks) * kFillUs + (ks > 1 ? kSplitUs + tiles * ks * kSlotUs : 0.0);
+}
+// Partial tiles that no pass over up to `tiles` output tiles asks pick_ksplit for: a split has to pay for its partial tiles
+// within the ksteps x kFillUs of the tail as it is.  Like most_range_rows, for a workspace that serves shorter batches.
+int most_split_slots(int64_t tiles, int ksteps) {
+    const int64_t tail = tiles < kSms ? tiles : kSms - 1;
+    const int64_t ks = ksteps / 4 < 64 ? ksteps / 4 : 64;
+    const double paid = (ksteps * kFillUs - kSplitUs) / kSlotUs;
+    const double slots = fmin(fmin(static_cast<double>(tail * ks), paid), static_cast<double>(kSplitSlots));
+    return ks < 2 || slots < 2.0 ? 0 : static_cast<int>(slots);
 }
 int pick_ksplit(int tiles, int ksteps, int slots) {
     int best = 1;
@@ -238,9 +272,22 @@ Layout compute_layout(const ais_shape* s, const ais_params* p) {
     L.roll = s->fp8_block > 0    ? plan_kind(kTileBlock, s->T, s->V, s->d, kMaxRanges, forced, nullptr)
              : s->fp8_block == 0 ? plan_pass(s->T, s->V, s->d / 2, kMaxRanges, forced)
                                  : plan_kind(kTileOne, s->T, s->V, s->d, kMaxRanges, forced, nullptr);
-    const int nparts = L.train.parts() > L.roll.parts() ? L.train.parts() : L.roll.parts();
+    // every size below is one that a batch of fewer rows does not exceed
+    int64_t range_rows = 0;
+    auto reserve = [&](TileKind kind, int d) {
+        const int64_t r = most_range_rows(kind, s->T, s->V, d, kMaxRanges, forced);
+        if (r > range_rows) range_rows = r;
+    };
+    reserve(kTileOne, s->d);
+    reserve(kTileTwo, s->d);
+    if (s->fp8_block > 0) {
+        reserve(kTileBlock, s->d);
+    } else if (s->fp8_block == 0) {
+        reserve(kTileOne, s->d / 2);
+        reserve(kTileTwo, s->d / 2);
+    }
     size_t off = 0;
-    L.part_bytes = align_up(static_cast<size_t>(nparts) * L.t_ld * sizeof(float), 256);
+    L.part_bytes = align_up(2 * static_cast<size_t>(range_rows) * sizeof(float), 256);
     for (int i = 0; i < 2; ++i) { L.off_part[i] = off; off += 3 * L.part_bytes; }
     L.off_flags = off;  off += align_up(static_cast<size_t>(L.t_ld / kBM + 2), 256);
     L.off_pace = off;   off += 2 * kPaceRingBytes;
@@ -257,12 +304,8 @@ Layout compute_layout(const ais_shape* s, const ais_params* p) {
         // every bit of dH) is the same whatever the workspace lets a pass hold
         const int64_t tiles = ((s->T + kDhRows - 1) / kDhRows) * ((s->d + kBN - 1) / kBN);
         const int ksteps = (s->V + 63) / 64;
-        L.ksplit = 0;
-        L.split_slots = kSplitSlots;
-        if (tiles < kSms) {
-            L.ksplit = tiles > 0 ? pick_ksplit(static_cast<int>(tiles), ksteps, kSplitSlots) : 1;
-            L.split_slots = L.ksplit > 1 ? static_cast<int>(tiles) * L.ksplit : 0;
-        }
+        L.split_slots = most_split_slots(tiles, ksteps);
+        L.ksplit = tiles >= kSms ? 0 : tiles > 0 ? pick_ksplit(static_cast<int>(tiles), ksteps, L.split_slots) : 1;
     }
     L.off_split = off;  off += static_cast<size_t>(L.split_slots) * kPartTileFloats * sizeof(float);
     L.off_u = off;
