@@ -403,8 +403,9 @@ class AisStep:
         self.dH = torch.empty(max(T, 1), ldh, dtype=torch.bfloat16, device=dev)[:, :d] if want_grad else None
         self.w_quantized = False
 
-    # ---- the stages in one library call.  The struct with the step's own buffers is filled once and again whenever an
-    # attribute it holds is assigned; the caller's tensors go in at every call.
+    # ---- the stages in one library call.  The struct with the step's own buffers is filled once, and again whenever an
+    # attribute it holds is assigned or a call finds a tensor's storage or strides changed (resize_, set_, .data); the
+    # caller's tensors go in at every call.
     _PLANNED = frozenset(("shape", "params", "workspace", "qH", "sH", "qW", "sW", "lp_train", "lse_train", "lp_roll", "lse_roll", "rho",
                           "w_tilde", "adv", "n_valid_seq", "loss", "diag", "status", "dH", "w_layout"))
 
@@ -413,9 +414,14 @@ class AisStep:
         if name in AisStep._PLANNED:
             object.__setattr__(self, "_plan", None)
 
+    def _layout(self):
+        sh = self.shape
+        return sh.ldh, sh.ldw, sh.fp8_block, sh.d
+
     def _make_plan(self):
-        """The filled struct, its address and those of shape and params; None when a buffer does not have the layout that
-        ais_step takes (codes with another row stride than the shape's): such steps go through the single calls."""
+        """(probes, what they gave, the shape's layout, the filled struct): a probe is a method of one of the step's tensors
+        whose answer is in the struct.  The struct is None when a buffer does not have the layout that ais_step takes (codes with
+        another row stride than the shape's): such steps go through the single calls."""
         sh = self.shape
         ldq_h = sh.ldh // 2 if sh.fp8_block == FP4_MX32 else sh.ldh
         ldq_w = sh.d if self.w_layout == W_DV else sh.ldw // 2 if sh.fp8_block == FP4_MX32 else sh.ldw
@@ -423,13 +429,16 @@ class AisStep:
                    lse_roll=self.lse_roll, adv=self.adv, n_valid_seq=self.n_valid_seq, rho=self.rho, w_tilde=self.w_tilde, diag=self.diag,
                    dH=self.dH, loss=self.loss, dev_status=self.status, workspace=self.workspace)
         _require_cuda(*own.values())
-        plan = False
+        probes = [t.data_ptr for t in own.values() if t is not None]
+        probes += [t.stride for t in (self.qH, self.sH, self.qW, self.sW)] + [self.workspace.numel, self.workspace.element_size]
+        found = [probe() for probe in probes]
+        args = None
         if self.qH.stride(0) == ldq_h and self.qW.stride(0) == ldq_w:
             args = StepArgs(**{k: _ptr(t) for k, t in own.items()})
             args.ldsH = self.sH.stride(0) if self.sH.dim() == 2 else 0
             args.ldsW = self.sW.stride(0) if self.sW.dim() == 2 else 0
             args.workspace_bytes = self.workspace.numel() * self.workspace.element_size()
-            plan = (args, C.byref(args), C.byref(sh), C.byref(self.params), lib().ais_step)
+        plan = (probes, found, self._layout(), args)
         object.__setattr__(self, "_plan", plan)
         return plan
 
@@ -438,9 +447,10 @@ class AisStep:
         """Enqueues `stages` in one call; False when the operands are not laid out as the shape says (the caller then goes
         through the single entry points, which take every stride)."""
         plan = self._plan
-        if plan is None:
+        if plan is None or [probe() for probe in plan[0]] != plan[1] or self._layout() != plan[2]:
             plan = self._make_plan()
-        if plan is False:
+        a = plan[3]
+        if a is None:
             return False
         sh = self.shape
         if stages & STAGE_QUANTIZE_H and (H.shape != (sh.T, sh.d) or H.stride(0) != sh.ldh):
@@ -450,7 +460,6 @@ class AisStep:
         for t in (H, W, tokens, mask, seq_offsets, rewards, lp_old, lp_ref, dW):
             if t is not None and not t.is_cuda:
                 _require_cuda(t)
-        a, a_ref, sh_ref, p_ref, fn = plan
         a.H = _ptr(H)
         a.W = _ptr(W)
         a.tokens = _ptr(tokens)
@@ -463,7 +472,7 @@ class AisStep:
             a.dW = _ptr(dW)
             a.lddw = 0 if dW is None else dW.stride(0)
             a.dw_accumulate = 1 if dw_accumulate else 0
-        _check(fn(sh_ref, p_ref, a_ref, stages, _stream(self.workspace)), "ais_step")
+        _check(lib().ais_step(C.byref(sh), C.byref(self.params), C.byref(a), stages, _stream(self.workspace)), "ais_step")
         return True
 
     def quantize_weights(self, W: torch.Tensor) -> None:
