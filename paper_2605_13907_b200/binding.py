@@ -414,6 +414,10 @@ class AisStep:
         if name in AisStep._PLANNED:
             object.__setattr__(self, "_plan", None)
 
+    def __getstate__(self):
+        """Copies and pickles go without the struct: it holds addresses."""
+        return {**self.__dict__, "_plan": None}
+
     def _layout(self):
         sh = self.shape
         return sh.ldh, sh.ldw, sh.fp8_block, sh.d

@@ -87,3 +87,17 @@ def test_strides_of_the_scales_are_read_at_every_call(recorder):
     step.sW.set_(wide)
     step.step(**x)
     assert recorder.calls[1]["ldsW"] == wide.stride(0)
+
+
+@pytest.mark.parametrize("how", ["copy", "deepcopy", "pickle"])
+def test_a_step_that_has_run_can_be_copied(recorder, how):
+    """A copy shares the tensors, a deep copy and a pickled one have their own."""
+    import copy
+    import pickle
+    step, x = _step(), _step_inputs()
+    step.step(**x)
+    other = {"copy": copy.copy, "deepcopy": copy.deepcopy, "pickle": lambda s: pickle.loads(pickle.dumps(s))}[how](step)
+    other.step(**x)
+    for name in ("workspace", "lp_train", "dH"):
+        assert recorder.calls[1][name] == getattr(other, name).data_ptr()
+        assert (recorder.calls[1][name] == recorder.calls[0][name]) == (how == "copy")
