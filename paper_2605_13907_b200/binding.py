@@ -414,6 +414,11 @@ class AisStep:
         if name in AisStep._PLANNED:
             object.__setattr__(self, "_plan", None)
 
+    def _own(self, *stages) -> bool:
+        """Are these stages the ones written here (not a subclass's, nor ones put in their place)?"""
+        cls, mine = type(self), self.__dict__
+        return all(getattr(cls, n) is _STAGES[n] and n not in mine for n in stages)
+
     def __getstate__(self):
         """Copies and pickles go without the struct: it holds addresses."""
         return {**self.__dict__, "_plan": None}
@@ -488,7 +493,8 @@ class AisStep:
 
     def forward(self, H, W, tokens, mask, requantize_w: bool = True) -> None:
         fresh_w = requantize_w or not self.w_quantized
-        if self._run(STAGE_QUANTIZE_H | STAGE_LOGPROB | (STAGE_QUANTIZE_W if fresh_w else 0), H, W, tokens, mask):
+        if self._own("quantize_weights") and \
+                self._run(STAGE_QUANTIZE_H | STAGE_LOGPROB | (STAGE_QUANTIZE_W if fresh_w else 0), H, W, tokens, mask):
             self.w_quantized = True
             return
         if self.shape.T > 0:
@@ -517,7 +523,7 @@ class AisStep:
                  dw_accumulate=dw_accumulate)
 
     def step(self, H, W, tokens, mask, seq_offsets, rewards, lp_old=None, requantize_w: bool = True, lp_ref=None) -> None:
-        if self.group is None:
+        if self.group is None and self._own("quantize_weights", "forward", "diagnose", "backward"):
             fresh_w = requantize_w or not self.w_quantized
             stages = STAGE_QUANTIZE_H | STAGE_LOGPROB | STAGE_DIAGNOSE | (STAGE_QUANTIZE_W if fresh_w else 0) | \
                 (STAGE_LOSS if self.dH is not None else 0)
@@ -531,3 +537,6 @@ class AisStep:
 
     def read_diag(self) -> dict:
         return read_diag(self.diag)
+
+
+_STAGES = {n: getattr(AisStep, n) for n in ("quantize_weights", "forward", "diagnose", "backward")}

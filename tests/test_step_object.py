@@ -101,3 +101,32 @@ def test_a_step_that_has_run_can_be_copied(recorder, how):
     for name in ("workspace", "lp_train", "dH"):
         assert recorder.calls[1][name] == getattr(other, name).data_ptr()
         assert (recorder.calls[1][name] == recorder.calls[0][name]) == (how == "copy")
+
+
+@pytest.mark.parametrize("where", ["subclass", "instance"])
+@pytest.mark.parametrize("name", ["quantize_weights", "forward", "diagnose", "backward"])
+def test_a_stage_that_was_replaced_is_called(recorder, monkeypatch, name, where):
+    """step() is made of the four stages: one that a subclass or a program puts its own in place of is run."""
+    from paper_2605_13907_b200 import binding
+    for f in ("quantize_fp8", "logprob_fwd", "diagnostics", "loss_bwd"):
+        monkeypatch.setattr(binding, f, lambda *a, **k: None)
+    seen = []
+    if where == "subclass":
+        cls = type("Own", (binding.AisStep,), {name: lambda self, *a, **k: seen.append(name)})
+        step = cls(T, D, V, P, G, 128, device="cpu")
+    else:
+        step = _step()
+        setattr(step, name, lambda *a, **k: seen.append(name))
+    step.step(**_step_inputs())
+    assert seen == [name]
+
+
+def test_replaced_weight_quantiser_is_called_by_forward(recorder, monkeypatch):
+    from paper_2605_13907_b200 import binding
+    for f in ("quantize_fp8", "logprob_fwd"):
+        monkeypatch.setattr(binding, f, lambda *a, **k: None)
+    step, seen = _step(), []
+    step.quantize_weights = seen.append
+    x = _inputs()
+    step.forward(**x)
+    assert seen == [x["W"]]
