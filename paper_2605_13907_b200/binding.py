@@ -458,8 +458,7 @@ class AisStep:
         plan = self._plan
         if plan is None or [probe() for probe in plan[0]] != plan[1] or self._layout() != plan[2]:
             plan = self._make_plan()
-        a = plan[3]
-        if a is None:
+        if plan[3] is None:
             return False
         sh = self.shape
         if stages & STAGE_QUANTIZE_H and (H.shape != (sh.T, sh.d) or H.stride(0) != sh.ldh):
@@ -469,6 +468,7 @@ class AisStep:
         for t in (H, W, tokens, mask, seq_offsets, rewards, lp_old, lp_ref, dW):
             if t is not None and not t.is_cuda:
                 _require_cuda(t)
+        a = StepArgs.from_buffer_copy(plan[3])           # the call's own: another thread may be calling this step, too
         a.H = _ptr(H)
         a.W = _ptr(W)
         a.tokens = _ptr(tokens)

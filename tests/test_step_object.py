@@ -130,3 +130,28 @@ def test_replaced_weight_quantiser_is_called_by_forward(recorder, monkeypatch):
     x = _inputs()
     step.forward(**x)
     assert seen == [x["W"]]
+
+
+def test_two_threads_calls_do_not_share_their_arguments(recorder):
+    """A call that is still inside the library (which runs without the interpreter's lock) keeps its own inputs when another
+    thread calls the same step."""
+    import threading
+    step, inside, go = _step(), threading.Event(), threading.Event()
+    x, y = _step_inputs(), _step_inputs()
+    note = recorder.ais_step
+
+    def slow(shape, params, args, stages, stream):
+        if threading.current_thread() is not threading.main_thread():
+            inside.set()
+            assert go.wait(20)
+        return note(shape, params, args, stages, stream)
+
+    recorder.ais_step = slow
+    step.step(**_step_inputs())
+    t = threading.Thread(target=lambda: step.step(**x))
+    t.start()
+    assert inside.wait(20)
+    step.step(**y)
+    go.set()
+    t.join()
+    assert [c["H"] for c in recorder.calls[1:]] == [y["H"].data_ptr(), x["H"].data_ptr()]
