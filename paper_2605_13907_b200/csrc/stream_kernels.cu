@@ -401,7 +401,7 @@ __global__ void tensor_scale_kernel(uint32_t* scale_word) {
 template <int RPW>
 __global__ void __launch_bounds__(kQThreads) tensor_quantize_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, int64_t ld,
                                                                     uint8_t* __restrict__ codes, int64_t ldq,
-                                                                    const float* __restrict__ scale, unsigned tiles_x) {
+                                                                    const float* scale, unsigned tiles_x) {
     pdl_enter();
     const float s = *scale;
     const float y = __frcp_rn(s);
@@ -605,7 +605,7 @@ __global__ void adv_kernel(const AdvJob job) {
 
 // Sequence-level importance weight (Eq. is-weight): log w(x) = sum over the valid rows of a sequence of
 // lp_train - lp_roll.  One warp per sequence, double accumulation in a fixed order.
-__global__ void __launch_bounds__(256) seq_logw_kernel(const float* __restrict__ lp_train, const float* __restrict__ lp_roll,
+__global__ void __launch_bounds__(256) seq_logw_kernel(const float* lp_train, const float* lp_roll,
                                                         const uint8_t* __restrict__ mask, const int32_t* __restrict__ seq_offsets,
                                                         int S, float* __restrict__ seq_logw) {
     pdl_enter();
@@ -835,7 +835,7 @@ struct RowGroup {
     bool any;
 };
 template <int VEC>
-__device__ __forceinline__ RowGroup<VEC> load_group(const float* __restrict__ lp_train, const float* __restrict__ lp_roll,
+__device__ __forceinline__ RowGroup<VEC> load_group(const float* lp_train, const float* lp_roll,
                                                     const uint8_t* __restrict__ mask, int64_t g) {
     RowGroup<VEC> r;
     if (VEC == 4) {
@@ -855,12 +855,12 @@ __device__ __forceinline__ RowGroup<VEC> load_group(const float* __restrict__ lp
 }
 
 template <int VEC>
-__global__ void __launch_bounds__(kDiagThreads) moments_kernel(const float* __restrict__ lp_train, const float* __restrict__ lp_roll,
+__global__ void __launch_bounds__(kDiagThreads) moments_kernel(const float* lp_train, const float* lp_roll,
                                                                 const uint8_t* __restrict__ mask,
                                                                 const int32_t* __restrict__ seq_offsets,
-                                                                const float* __restrict__ adv, int64_t T, int S, float C,
+                                                                const float* adv, int64_t T, int S, float C,
                                                                 double* __restrict__ partials, int32_t* __restrict__ n_valid_seq,
-                                                                const float* __restrict__ seq_logw) {
+                                                                const float* seq_logw) {
     pdl_enter();
     __shared__ double scratch[32];
     double acc[kNumMoments];
@@ -1026,13 +1026,12 @@ __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, int*
 // sums which groups it met, and the exact one replaces the sums of the blocks that need it.
 enum Walks { kBothWalks, kFastWalk, kExactWalk };
 template <bool SEQ, int WALKS>
-__global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const float* __restrict__ lp_train,
-                                                                         const float* __restrict__ lp_roll,
+__global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const float* lp_train, const float* lp_roll,
                                                                          const uint8_t* __restrict__ mask,
                                                                          const int32_t* __restrict__ seq_offsets,
-                                                                         const float* __restrict__ adv, int T, int S, float C,
+                                                                         const float* adv, int T, int S, float C,
                                                                          double* partials, int32_t* __restrict__ n_valid_seq,
-                                                                         const float* __restrict__ seq_logw, bool early) {
+                                                                         const float* seq_logw, bool early) {
     static_assert(kDiagThreads * 8 == kMomRows, "one 8-row group per thread and tile");
     extern __shared__ __align__(128) uint8_t stages[];          // kMomStages stages, then the barriers
     uint64_t* full = reinterpret_cast<uint64_t*>(stages + kMomStages * kMomStageBytes);
