@@ -437,16 +437,18 @@ class AisStep:
         own = dict(qH=self.qH, sH=self.sH, qW=self.qW, sW=self.sW, lp_train=self.lp_train, lse_train=self.lse_train, lp_roll=self.lp_roll,
                    lse_roll=self.lse_roll, adv=self.adv, n_valid_seq=self.n_valid_seq, rho=self.rho, w_tilde=self.w_tilde, diag=self.diag,
                    dH=self.dH, loss=self.loss, dev_status=self.status, workspace=self.workspace)
+        own = {k: t for k, t in own.items() if t is not None}
         _require_cuda(*own.values())
-        probes = [t.data_ptr for t in own.values() if t is not None]
+        probes = [t.data_ptr for t in own.values()]
         probes += [t.stride for t in (self.qH, self.sH, self.qW, self.sW)] + [self.workspace.numel, self.workspace.element_size]
         found = [probe() for probe in probes]
         args = None
         if self.qH.stride(0) == ldq_h and self.qW.stride(0) == ldq_w:
-            args = StepArgs(**{k: _ptr(t) for k, t in own.items()})
-            args.ldsH = self.sH.stride(0) if self.sH.dim() == 2 else 0
-            args.ldsW = self.sW.stride(0) if self.sW.dim() == 2 else 0
-            args.workspace_bytes = self.workspace.numel() * self.workspace.element_size()
+            lds_h, lds_w, count, size = found[-5], found[-3], found[-2], found[-1]
+            args = StepArgs(**dict(zip(own, found)))
+            args.ldsH = lds_h[0] if len(lds_h) == 2 else 0
+            args.ldsW = lds_w[0] if len(lds_w) == 2 else 0
+            args.workspace_bytes = count * size
         plan = (probes, found, self._layout(), args)
         object.__setattr__(self, "_plan", plan)
         return plan
