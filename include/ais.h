@@ -323,9 +323,12 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params,
  * that run the same step again and again and fill the struct once: a step of a small batch takes tens of microseconds, and
  * marshalling six argument lists is a good part of that.  Neighbouring stages share launches, and with AIS_STAGE_LOGPROB,
  * AIS_STAGE_DIAGNOSE and AIS_STAGE_LOSS in one call (and no dW) the trainer pass leaves e^z (bf16) in the scratch rows that
- * the workspace has for the backward pass, so that those rows' logits are not computed again; dH then has the same
- * precision, but not the same bits, as the stages called one by one.  Quantises by shape->fp8_block; the codes' row strides are those
- * ais_logprob_fwd expects.  Stops at the first stage that returns an error.
+ * the workspace has for the backward pass, so that those rows' logits are not computed again.  lse_train, lp_train, what
+ * follows from them and dH then have the same precision, but not the same bits, as the stages called one by one: the
+ * exponentials are summed about 0 instead of their maximum, and dH's scratch is rounded to bf16 before its row factor
+ * instead of after it.  (The loss is a sum that cancels to a small part of its terms; two such results agree to about
+ * 1e-7 of the sum of the terms' absolute values, not of the loss.)  Quantises by shape->fp8_block; the codes' row strides
+ * are those ais_logprob_fwd expects.  Stops at the first stage that returns an error; the stages before it have run.
  */
 #define AIS_STAGE_QUANTIZE_H 1u
 #define AIS_STAGE_QUANTIZE_W 2u

@@ -140,7 +140,7 @@ cudaError_t launch_dh_reduce(const LmheadArgs& args, cudaStream_t stream);
 cudaError_t lmhead_prepare();   // sets the dynamic shared-memory attribute of every instantiation
 
 // The rollout pass with per-block scales (mode kFwdFp8; args.sgroups = 128 / block = 1, 2 or 4).  tmSA / tmSB map the
-// block-major scale arrays with boxes of (128 rows, sgroups) and (256 rows, sgroups).
+// block-major scale arrays with boxes of kPairRows (256) and kPairCols (128) rows, each times sgroups blocks.
 cudaError_t launch_lmhead_fp8_block(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,
                                     const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream);
 cudaError_t lmhead_fp8_block_prepare();

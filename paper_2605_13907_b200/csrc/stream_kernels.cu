@@ -18,7 +18,7 @@ namespace {
 // microscaling FP8 / FP4 (E8M0 scale per 32).  Streaming kernels, bound by HBM (3 bytes per element) and close behind it by
 // instruction issue: a CTA covers 4 warps x RPW rows x 1024 columns, a lane holds 8 consecutive values per 16-byte load, four
 // loads per row segment.  Measured back to back on a 151936 x 4096 head (copy bandwidth 6.5 TB/s): block 128 380 -> 302 us
-// (6.3 TB/s) with one residual correction instead of two and the maxima of two loads per shuffle; ten CTAs of four warps per
+// (1.89 GB: 6.2 TB/s; 319 us when three heads take turns, so that nothing of one is left in L2) with one residual correction instead of two and the maxima of two loads per shuffle; ten CTAs of four warps per
 // SM (48 registers) against five of eight 302 / 305, four 311, six 337, eight 385; microscaling FP8 305, FP4 272 us; a
 // persistent form with the next segment prefetched 4.3 to 4.9 TB/s.  Small matrices take RPW = 1: four times the CTAs, no
 // serial chain of rows in a warp.
@@ -1064,7 +1064,7 @@ __global__ void __launch_bounds__(kDiagThreads, 4) moments_staged_kernel(const f
     // thread's own data -- v = (w - 1) - pivot for the weights, dA = A - A_pivot for the advantages, and
     // x = A w - A_pivot (1 + pivot) = A v + dA (1 + pivot) for their product -- so that the fp32 roundings scale with the
     // spread of the data and not with its size, and are exactly zero when all rows are equal.  A thread sees at most
-    // T / 151,552 rows.
+    // 8 ceil(tiles / kDiagBlocks) rows: 16 of 1.48 M, 448 of 67 M.
     float f3, f9, g_v, g_v2, g_dA, g_dA2, g_x, g_x2;
     F2 f8p;                                             // sum of D, two rows at a time
     int nrows;                                          // valid rows of the thread

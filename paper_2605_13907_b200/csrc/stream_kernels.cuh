@@ -83,7 +83,7 @@ cudaError_t launch_quantize_cols(const void* x, int64_t K, int64_t N, int64_t ld
                                  float* scales, int64_t lds, cudaStream_t stream);
 
 // Microscaling: E8M0 scale per 32 elements, packed in 512-byte chunks of 128 rows x 4 blocks; `scale_bytes` is the
-// size of the whole packed array (rows padded to a multiple of 256), filled with the neutral code first.
+// size of the whole packed array (rows padded to a multiple of 256); the padding rows get the neutral code.
 cudaError_t launch_quantize_mx(const void* x, int64_t rows, int64_t cols, int64_t ld, uint8_t* codes, int64_t ldq,
                                uint8_t* scales, size_t scale_bytes, bool fp4 /* E2M1 elements, two per byte */,
                                cudaStream_t stream);
