@@ -4,6 +4,7 @@ from __future__ import annotations
 
 import ctypes as C
 import math
+import operator
 import os
 
 import torch
@@ -414,10 +415,10 @@ class AisStep:
         if name in AisStep._PLANNED:
             object.__setattr__(self, "_plan", None)
 
-    def _own(self, *stages) -> bool:
-        """Are these stages the ones written here (not a subclass's, nor ones put in their place)?"""
-        cls, mine = type(self), self.__dict__
-        return all(getattr(cls, n) is _STAGES[n] and n not in mine for n in stages)
+    def _own_stages(self) -> bool:
+        """Are the four stages the ones written here (not a subclass's, nor ones put in their place)?"""
+        cls = type(self)
+        return (cls.quantize_weights, cls.forward, cls.diagnose, cls.backward) == _STAGES and _STAGE_NAMES.isdisjoint(self.__dict__)
 
     def __getstate__(self):
         """Copies and pickles go without the struct: it holds addresses."""
@@ -441,7 +442,7 @@ class AisStep:
         _require_cuda(*own.values())
         probes = [t.data_ptr for t in own.values()]
         probes += [t.stride for t in (self.qH, self.sH, self.qW, self.sW)] + [self.workspace.numel, self.workspace.element_size]
-        found = [probe() for probe in probes]
+        found = list(map(operator.call, probes))
         args = None
         if self.qH.stride(0) == ldq_h and self.qW.stride(0) == ldq_w:
             lds_h, lds_w, count, size = found[-5], found[-3], found[-2], found[-1]
@@ -458,7 +459,7 @@ class AisStep:
         """Enqueues `stages` in one call; False when the operands are not laid out as the shape says (the caller then goes
         through the single entry points, which take every stride)."""
         plan = self._plan
-        if plan is None or [probe() for probe in plan[0]] != plan[1] or self._layout() != plan[2]:
+        if plan is None or list(map(operator.call, plan[0])) != plan[1] or self._layout() != plan[2]:
             plan = self._make_plan()
         if plan[3] is None:
             return False
@@ -495,7 +496,7 @@ class AisStep:
 
     def forward(self, H, W, tokens, mask, requantize_w: bool = True) -> None:
         fresh_w = requantize_w or not self.w_quantized
-        if self._own("quantize_weights") and \
+        if self._own_stages() and \
                 self._run(STAGE_QUANTIZE_H | STAGE_LOGPROB | (STAGE_QUANTIZE_W if fresh_w else 0), H, W, tokens, mask):
             self.w_quantized = True
             return
@@ -525,7 +526,7 @@ class AisStep:
                  dw_accumulate=dw_accumulate)
 
     def step(self, H, W, tokens, mask, seq_offsets, rewards, lp_old=None, requantize_w: bool = True, lp_ref=None) -> None:
-        if self.group is None and self._own("quantize_weights", "forward", "diagnose", "backward"):
+        if self.group is None and self._own_stages():
             fresh_w = requantize_w or not self.w_quantized
             stages = STAGE_QUANTIZE_H | STAGE_LOGPROB | STAGE_DIAGNOSE | (STAGE_QUANTIZE_W if fresh_w else 0) | \
                 (STAGE_LOSS if self.dH is not None else 0)
@@ -541,4 +542,5 @@ class AisStep:
         return read_diag(self.diag)
 
 
-_STAGES = {n: getattr(AisStep, n) for n in ("quantize_weights", "forward", "diagnose", "backward")}
+_STAGES = (AisStep.quantize_weights, AisStep.forward, AisStep.diagnose, AisStep.backward)
+_STAGE_NAMES = frozenset(("quantize_weights", "forward", "diagnose", "backward"))
