@@ -88,7 +88,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (MX) reg_dealloc<32>();
-        if (lane == 0) {
+        if (elect_one()) {
             Pipe st(STG);
             uint32_t issued = 0;
             bool ok = true;
@@ -160,7 +160,7 @@ lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (MX) reg_dealloc<32>();
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc =
                 (MODE == kFwdFp8T || MX) ? make_idesc(kFmtE4M3, kFmtE4M3, kBM, kBN, 0, 0)
                                   : make_idesc(kFmtBF16, kFmtBF16, kBM, kBN, 0, B_MN ? 1 : 0);

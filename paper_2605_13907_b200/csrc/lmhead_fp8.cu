@@ -23,6 +23,17 @@
 // against 1,000 clocks per scale block.  Passing a barrier that completed long ago costs a warp about 250 clocks, which is
 // why the next block's barrier is tested before the last arithmetic of this one (block 32: 1,090 -> 1,000).  Sixteen and
 // twelve promotion warps (32 columns each) and scale loads hoisted above the waits measured slower or the same.
+// With several blocks per stage the two buffers alternate inside a stage, so the loop over its blocks is unrolled by two and
+// every tensor-memory address and barrier of a block is a constant offset: block 32 1,005 -> 962 clocks per scale block (8.15 ->
+// 7.80 ms, 9,216 rows, d = 4096, 65,536 columns), block 64 4.53 -> 4.35 ms; unrolled by four 1,038 (instruction fetch).
+// What the promotion contends for is the path out of shared memory: a broadcast 16-byte load returns 512 bytes, four clocks of
+// it, and the MMAs take all of it while they run (8 KB of operands per 64 clocks).  In a copy of the loop with real MMAs and
+// without the rest of the kernel a block takes 753 clocks with no MMA, 840 with the two of block 32 and 1,187 with the eight of
+// block 128, against 687, 720 and 791 with the column scales taken as constants; operand copies add nothing to that.  Loads of
+// scales by shuffle (1,232), 16x256b tensor-memory loads (eight rows x 16 columns per thread, a third of the scale traffic, but
+// half the tensor-memory rate: 1,137) and 128 x 256 tiles of them (1,141) do not get below it.
+// The roles with one thread are entered through elect.sync: with `lane == 0` a stage's copies and a block's MMAs took 10% to 20%
+// longer to issue (hand-overs alone, no promotion: 928 -> 847 clocks per block, block 32 414 -> 343).
 #include <type_traits>
 
 #include "lmhead_common.cuh"
@@ -100,7 +111,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         reg_dealloc<40>();
         if (warp == 0) {
             // ------------------------------------------------------------------ TMA producer
-            if (lane == 0) {
+            if (elect_one()) {
                 Pipe st(kStages), sc(C::kSlots);
                 uint32_t issued = 0;
                 bool ok = true;
@@ -143,7 +154,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             // block (block n of the CTA goes to buffer n % 2).  One thread cannot keep up: it shares its scheduler with
             // two promotion warps, and wait + four MMAs + two commits took it about 1,300 clocks per block against the
             // 542 the tensor core needs.  The two threads are independent: different buffers, different barriers.
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t me = warp - 1;
                 constexpr uint32_t idesc = make_idesc(kFmtE4M3, kFmtE4M3, kBM, kPairCols, 0, 0);
                 const uint64_t desc0 = smem_desc_sw128(0, 16, 1024);           // descriptor of address 0: add (address >> 4)
@@ -227,8 +238,9 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 for (int n = 0; n < kHalfCols / 2; ++n) acc[0][n] = acc[1][n] = F2{0.f, 0.f};
                 for (int ks = 0; ks < a.ksteps && ok; ++ks) {
                     const float* sS = reinterpret_cast<const float*>(scale_base + sc.idx * C::kSlotBytes);
-#pragma unroll 1
+#pragma unroll(SG > 1 ? 2 : 1)
                     for (int g = 0; g < SG; ++g) {
+                        if (SG > 1) tb.idx = g & 1;       // a stage starts with buffer 0: known when the loop is unrolled by two
                         if (!ready && !mbar_wait_warp_spin(&tfull[tb.idx], tb.phase, abort_flag, a.wait_cycles)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t buf = tb.idx;
@@ -269,7 +281,12 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&tempty[buf]);
-                        tb.advance();
+                        if (SG > 1) {
+                            tb.idx = (g + 1) & 1;
+                            tb.phase ^= g & 1;
+                        } else {
+                            tb.advance();
+                        }
                         // ask for the next block's barrier now: the answer comes back behind the last arithmetic
                         const bool seen = mbar_test_wait(&tfull[tb.idx], tb.phase);
                         promote(I3{}, vb);

@@ -98,7 +98,7 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
 
     if (warp < 4) {
         reg_dealloc<40>();
-        if (warp == 0 && lane == 0) {
+        if (warp == 0 && elect_one()) {
             // -------------------------------------------------------------- TMA producer
             Pipe st(kPairStages);
             uint32_t issued = 0;
@@ -146,7 +146,7 @@ lmhead_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             if (pacer.ring)                                     // units of the last wave that this CTA does not have
                 for (const int waves = (num_units + gridDim.x - 1) / gridDim.x; n < waves; ++n) pacer.top_up(n, 0);
             *issued_slot = issued;
-        } else if (warp == 1 && lane == 0) {
+        } else if (warp == 1 && elect_one()) {
             // -------------------------------------------------------------- MMA issuer
             constexpr uint32_t idesc = FP8 ? make_idesc(kFmtE4M3, kFmtE4M3, kBM, kBN, 0, 0)
                                            : make_idesc(kFmtBF16, kFmtBF16, kBM, kBN, DW ? 1 : 0, B_MN ? 1 : 0);
