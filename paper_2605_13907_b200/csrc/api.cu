@@ -365,6 +365,8 @@ struct Fuse {
     const QuantJob* quant = nullptr;     // log-probs: quantise these first, in the opening launch
     int* nquant = nullptr;               // how many; zeroed by that launch
     const AdvJob* adv = nullptr;         // log-probs: advantages in the merging launch; diagnostics: they are there already
+    const MomentsJob* moments = nullptr; // log-probs: advantages in the opening launch, batch moments in the merging one;
+                                         // diagnostics: their partial sums are there already
     TotalsJob* totals = nullptr;         // diagnostics: leave the end (alpha, rho, w_tilde) to the loss, described here
     const RectifyJob* rectify = nullptr; // loss: form them
     int64_t keep_rows = 0;               // log-probs: leave the exponentials of these rows in the scratch; loss: they are there
@@ -623,7 +625,7 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
                 make_tmap(&p.tmSB, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sW, V, nkb, ldsW * 4, kPairCols, sg, CU_TENSOR_MAP_SWIZZLE_NONE);
     }
     if (!maps) return AIS_ERR_DEVICE;
-    const FlagsJob flags = {mask, T, ws + L.off_flags, paced ? ws + L.off_pace : nullptr, 2 * kPaceRingBytes};
+    const FlagsJob flags = {mask, T, ws + L.off_flags, paced ? ws + L.off_pace : nullptr, 2 * kPaceRingBytes, fuse.moments ? *fuse.adv : AdvJob{}};
     const int nquant = fuse.nquant ? *fuse.nquant : 0;
     if ((nquant > 0 ? launch_quantize(fuse.quant, nquant, d, shape->fp8_block, &flags, s) : launch_flags(flags, s)) != cudaSuccess)
         return AIS_ERR_DEVICE;
@@ -632,7 +634,7 @@ static int logprob_fwd(const ais_shape* shape, const ais_params* params, const v
         if ((pass[i].two ? launch_lmhead_pair(pass[i].mode, pass[i].tmA, pass[i].tmB, pass[i].tmSA, pass[i].a, pass[i].ctas, s)
                          : launch_lmhead(pass[i].mode, pass[i].tmA, pass[i].tmB, pass[i].tmSA, pass[i].tmSB, pass[i].a, pass[i].ctas, s)) != cudaSuccess)
             return AIS_ERR_DEVICE;
-    if (launch_combine(jobs, n, L.t_ld, mask, T, dev_status, fuse.adv, s) != cudaSuccess) return AIS_ERR_DEVICE;
+    if (launch_combine(jobs, n, L.t_ld, mask, T, dev_status, fuse.adv, fuse.moments, s) != cudaSuccess) return AIS_ERR_DEVICE;
     return AIS_OK;
 }
 
@@ -677,7 +679,7 @@ static int diagnostics(const ais_shape* shape, const ais_params* params, const f
         return AIS_ERR_DEVICE;
     if (launch_diag(lp_train, lp_roll, mask, seq_offsets, adv, shape->T, S, *params, reinterpret_cast<double*>(ws + L.off_diag),
                     n_valid_seq, seq_level ? reinterpret_cast<float*>(ws + L.off_seqw) : nullptr, rho, w_tilde,
-                    diag, !fuse.adv, fuse.totals, s) != cudaSuccess)
+                    diag, !fuse.adv, fuse.moments ? merge_moment_blocks(shape->T) : 0, fuse.totals, s) != cudaSuccess)
         return AIS_ERR_DEVICE;
     return AIS_OK;
 }
@@ -976,6 +978,10 @@ int ais_step(const ais_shape* shape, const ais_params* params, const ais_step_ar
         check_diagnostics(shape, params, a->lp_train, a->lp_roll, a->mask, a->seq_offsets, a->rewards, a->adv, a->w_tilde, a->diag, a->workspace,
                           a->workspace_bytes) == AIS_OK)
         fuse.adv = &adv;
+    // Up to kMergeMomentRows rows the merge forms the batch moments as well (merge_moments_kernel), and the advantages, which
+    // they need, ride on the opening launch instead.
+    MomentsJob moments = {a->seq_offsets, a->adv, S, params->C, reinterpret_cast<double*>(static_cast<uint8_t*>(a->workspace) + L.off_diag), a->n_valid_seq};
+    if (fuse.adv && shape->T <= kMergeMomentRows && params->seq_level_weights == 0) fuse.moments = &moments;
     // What the loss takes over from earlier stages it takes over only when it is going to run.
     const bool loss_runs = loss && shape->T > 0 &&
                            check_loss(shape, params, a->H, a->W, a->tokens, a->mask, a->seq_offsets, a->lse_train, a->lp_train, a->adv, a->w_tilde,

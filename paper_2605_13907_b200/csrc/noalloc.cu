@@ -99,6 +99,6 @@ extern "C" int ais_logprob_train_static(const ais_shape* shape, const void* H, c
     if ((plan.two ? launch_lmhead_pair(kFwdBf16, tmA, tmB, tmA, a, ctas, s) : launch_lmhead(kFwdBf16, tmA, tmB, tmA, tmB, a, ctas, s)) != cudaSuccess)
         return AIS_ERR_DEVICE;
     const CombineJob job = {a.part_m, a.part_s, a.part_z, nsplit * 2, lp_train, lse_train};
-    if (launch_combine(&job, 1, ld, mask, shape->T, dev_status, nullptr, s) != cudaSuccess) return AIS_ERR_DEVICE;
+    if (launch_combine(&job, 1, ld, mask, shape->T, dev_status, nullptr, nullptr, s) != cudaSuccess) return AIS_ERR_DEVICE;
     return AIS_OK;
 }

@@ -125,6 +125,26 @@ __device__ __forceinline__ QuantTile quant_tile(unsigned tiles_x) {
     return {static_cast<int64_t>(row) * (kQWarps * RPW), static_cast<int64_t>(blockIdx.x % tiles_x) * kQCols, row == (gridDim.x - 1) / tiles_x};
 }
 
+// Group-relative advantage of sequence s (Eq. grpo_adv), and what AdvJob clears for it.
+__device__ __forceinline__ void run_advantage(const AdvJob& j, int s) {
+    if (s == 0 && j.tickets) j.tickets[0] = j.tickets[1] = 0;
+    if (j.zero_counts) j.zero_counts[s] = 0;
+    const int g0 = (s / j.G) * j.G;
+    double mean = 0.0;
+    for (int k = 0; k < j.G; ++k) mean += static_cast<double>(j.rewards[g0 + k]);
+    mean /= j.G;
+    double a = static_cast<double>(j.rewards[s]) - mean;
+    if (j.std_norm) {
+        double var = 0.0;
+        for (int k = 0; k < j.G; ++k) {
+            const double dlt = static_cast<double>(j.rewards[g0 + k]) - mean;
+            var += dlt * dlt;
+        }
+        a /= (sqrt(var / j.G) + static_cast<double>(j.eps));
+    }
+    j.adv[s] = static_cast<float>(a);
+}
+
 // FlagsJob by blocks of kQThreads threads: one warp per 128-row tile.
 constexpr int kFlagTiles = kQThreads / 32;
 inline unsigned flag_blocks(const FlagsJob& f) { return static_cast<unsigned>(((f.T + 127) / 128 + kFlagTiles - 1) / kFlagTiles); }
@@ -144,6 +164,7 @@ __device__ __forceinline__ void run_flags(const FlagsJob& f, unsigned block, uns
     if (f.clear)
         for (int64_t k = static_cast<int64_t>(block) * kQThreads + threadIdx.x; k < f.clear_bytes / 16; k += static_cast<int64_t>(nblocks) * kQThreads)
             static_cast<uint4*>(f.clear)[k] = make_uint4(0, 0, 0, 0);
+    for (int s = block * kQThreads + threadIdx.x; s < f.adv.S; s += nblocks * kQThreads) run_advantage(f.adv, s);
 }
 __global__ void __launch_bounds__(kQThreads) flags_kernel(const FlagsJob f) {
     pdl_enter();
@@ -416,26 +437,6 @@ __global__ void __launch_bounds__(kQThreads) tensor_quantize_kernel(const __nv_b
                    });
 }
 
-// Group-relative advantage of sequence s (Eq. grpo_adv), and what AdvJob clears for it.
-__device__ __forceinline__ void run_advantage(const AdvJob& j, int s) {
-    if (s == 0 && j.tickets) j.tickets[0] = j.tickets[1] = 0;
-    if (j.zero_counts) j.zero_counts[s] = 0;
-    const int g0 = (s / j.G) * j.G;
-    double mean = 0.0;
-    for (int k = 0; k < j.G; ++k) mean += static_cast<double>(j.rewards[g0 + k]);
-    mean /= j.G;
-    double a = static_cast<double>(j.rewards[s]) - mean;
-    if (j.std_norm) {
-        double var = 0.0;
-        for (int k = 0; k < j.G; ++k) {
-            const double dlt = static_cast<double>(j.rewards[g0 + k]) - mean;
-            var += dlt * dlt;
-        }
-        a /= (sqrt(var / j.G) + static_cast<double>(j.eps));
-    }
-    j.adv[s] = static_cast<float>(a);
-}
-
 // ------------------------------------------------------------------------------------------------
 // Merge of the per-split (max, sum-exp, target-logit) triples into lp and lse.
 // ------------------------------------------------------------------------------------------------
@@ -443,22 +444,13 @@ __device__ __forceinline__ void run_advantage(const AdvJob& j, int s) {
 // (max, sum) goes through shared memory to warp 0, in warp order.  With one thread per row the up to 296 parts of a small
 // batch were a chain of dependent loads.
 constexpr int kCombWarps = 8;
-__global__ void __launch_bounds__(32 * kCombWarps) combine_kernel(const CombineJob j0, const CombineJob j1, int njobs, int64_t part_ld,
-                                                                  const uint8_t* __restrict__ mask, int64_t T, uint32_t* status,
-                                                                  const AdvJob adv) {
-    pdl_enter();
-    if (static_cast<int>(blockIdx.y) == njobs) {                 // the row of blocks behind the merges
-        for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < adv.S; s += gridDim.x * blockDim.x) run_advantage(adv, s);
-        return;
-    }
-    const CombineJob job = blockIdx.y == 0 ? j0 : j1;
+struct MergeState {
+    float m[kCombWarps][kMergeRows], s[kCombWarps][kMergeRows], z[kCombWarps][kMergeRows];
+};
+// One warp's share of the parts of row t (a lane's own).
+__device__ __forceinline__ void merge_parts(const CombineJob& job, int64_t part_ld, int64_t t, bool live, int warp, MergeState& st) {
     const float *part_m = job.part_m, *part_s = job.part_s, *part_z = job.part_z;
-    const int nparts = job.nparts;
-    float *lp = job.lp, *lse = job.lse;
-    __shared__ float sm[kCombWarps][32], ss[kCombWarps][32], sz[kCombWarps][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t t = static_cast<int64_t>(blockIdx.x) * 32 + lane;
-    const bool live = t < T && mask[t] != 0;
+    const int nparts = job.nparts, lane = threadIdx.x & 31;
     float M = -INFINITY, S = 0.f, Z = -INFINITY;
     if (live) {
 #pragma unroll 4
@@ -470,22 +462,25 @@ __global__ void __launch_bounds__(32 * kCombWarps) combine_kernel(const CombineJ
             M = n;
         }
     }
-    sm[warp][lane] = M;
-    ss[warp][lane] = S;
-    sz[warp][lane] = Z;
-    __syncthreads();
-    if (warp != 0 || t >= T) return;
+    st.m[warp][lane] = M;
+    st.s[warp][lane] = S;
+    st.z[warp][lane] = Z;
+}
+struct MergedRow { float lp, lse; };
+// One warp, behind a barrier: the shares of the eight warps in their order, written to lp and lse (t < T).
+__device__ __forceinline__ MergedRow merge_finish(const CombineJob& job, int64_t t, bool live, uint32_t* status, const MergeState& st) {
+    const int lane = threadIdx.x & 31;
     float out_lp = 0.f, out_lse = 0.f;
     if (live) {
+        float M = st.m[0][lane], Z = st.z[0][lane], S = 0.f;
 #pragma unroll
         for (int w = 1; w < kCombWarps; ++w) {
-            M = fmaxf(M, sm[w][lane]);
-            Z = fmaxf(Z, sz[w][lane]);
+            M = fmaxf(M, st.m[w][lane]);
+            Z = fmaxf(Z, st.z[w][lane]);
         }
-        S = 0.f;
 #pragma unroll
         for (int w = 0; w < kCombWarps; ++w)
-            if (w < nparts) S += ss[w][lane] * expf(sm[w][lane] - M);
+            if (w < job.nparts) S += st.s[w][lane] * expf(st.m[w][lane] - M);
         out_lse = M + logf(S);
         out_lp = Z == -INFINITY ? 0.f : Z - out_lse;    // no target logit: token id out of range, flagged by the producer kernel
         if (!isfinite(out_lse) || !isfinite(out_lp)) {
@@ -496,8 +491,28 @@ __global__ void __launch_bounds__(32 * kCombWarps) combine_kernel(const CombineJ
             out_lse = __int_as_float(0x7fc00000);
         }
     }
-    lp[t] = out_lp;
-    if (lse) lse[t] = out_lse;
+    job.lp[t] = out_lp;
+    if (job.lse) job.lse[t] = out_lse;
+    return {out_lp, out_lse};
+}
+
+__global__ void __launch_bounds__(32 * kCombWarps) combine_kernel(const CombineJob j0, const CombineJob j1, int njobs, int64_t part_ld,
+                                                                  const uint8_t* __restrict__ mask, int64_t T, uint32_t* status,
+                                                                  const AdvJob adv) {
+    pdl_enter();
+    if (static_cast<int>(blockIdx.y) == njobs) {                 // the row of blocks behind the merges
+        for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < adv.S; s += gridDim.x * blockDim.x) run_advantage(adv, s);
+        return;
+    }
+    __shared__ MergeState st;
+    const CombineJob job = blockIdx.y == 0 ? j0 : j1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t t = static_cast<int64_t>(blockIdx.x) * kMergeRows + lane;
+    const bool live = t < T && mask[t] != 0;
+    merge_parts(job, part_ld, t, live, warp, st);
+    __syncthreads();
+    if (warp != 0 || t >= T) return;
+    merge_finish(job, t, live, status, st);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -826,6 +841,71 @@ __device__ __forceinline__ void add_run(double* acc, int n, float p, float sv, f
     acc[5] = fma(Ad * Ad, nd, acc[5]);
     acc[6] = fma(Ad, sw, acc[6]);
     acc[7] = fma(Ad * Ad, sw2, acc[7]);
+}
+
+// The merge of both passes and the batch moments in one kernel, for batches of up to kMergeMomentRows rows: the sixteen warps
+// merge 32 rows as combine_kernel does (eight warps per pass, the same order), then one warp forms the terms of its 32 rows
+// and their sums in fp64, one row of partial sums per block.  A small batch is a chain of launches, and the moments kernel (start,
+// walk, fp64 sums) is one of them, while every row's log-probs are in a register here: a step of 512 rows 46.4 -> 42.5 us, of
+// 3,001 rows (d = 512, V = 4096) 90.5 -> 86.7.  The limit is the number of partial sums that the totals behind it are formed from,
+// no more than the moments kernel leaves.
+__global__ void __launch_bounds__(2 * 32 * kCombWarps) merge_moments_kernel(const CombineJob j0, const CombineJob j1, int64_t part_ld,
+                                                                            const uint8_t* __restrict__ mask, int64_t T, uint32_t* status,
+                                                                            const MomentsJob mj) {
+    __shared__ MergeState st[2];
+    __shared__ float lp_roll[kMergeRows];
+    __shared__ int2 range;
+    pdl_enter();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, pass = warp / kCombWarps;
+    const int64_t t0 = static_cast<int64_t>(blockIdx.x) * kMergeRows, t = t0 + lane;
+    const int64_t last = t0 + kMergeRows <= T ? t0 + kMergeRows - 1 : T - 1;
+    const bool live = t < T && mask[t] != 0;
+    if (warp == 1) {
+        const int2 r = seqs_of_rows_warp(mj.seq_offsets, mj.S, t0, last);
+        if (lane == 0) range = r;
+    }
+    merge_parts(pass == 0 ? j0 : j1, part_ld, t, live, warp % kCombWarps, st[pass]);
+    __syncthreads();
+    MergedRow row = {0.f, 0.f};
+    if (warp % kCombWarps == 0 && t < T) {
+        row = merge_finish(pass == 0 ? j0 : j1, t, live, status, st[pass]);
+        if (pass == 1) lp_roll[lane] = row.lp;
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    const int sq = seq_in_range(mj.seq_offsets, range, t <= last ? t : last);
+    double v[kSums] = {};
+    if (live) {
+        const float lr = lp_roll[lane], x[1] = {row.lp - lr};
+        float u[1];
+        rho_minus_one(x, u);
+        const double w = 1.0 + static_cast<double>(fminf(u[0], mj.C - 1.0f)), A = mj.adv[sq];
+        v[0] = 1.0;
+        v[1] = w;
+        v[2] = w * w;
+        v[3] = fabsf(x[0]);
+        v[4] = A;
+        v[5] = A * A;
+        v[6] = A * w;
+        v[7] = (A * w) * (A * w);
+        v[8] = -x[0];
+        v[9] = __expf(lr) * fabsf(u[0]);
+    }
+    if (mj.n_valid_seq) {
+        const int sq0 = __shfl_sync(0xffffffffu, sq, 0);
+        if (__all_sync(0xffffffffu, sq == sq0)) {
+            const int n = __popc(__ballot_sync(0xffffffffu, live));
+            if (lane == 0 && n > 0) atomicAdd(&mj.n_valid_seq[sq0], n);
+        } else if (live) {
+            atomicAdd(&mj.n_valid_seq[sq], 1);
+        }
+    }
+    double* mine = mj.partials + static_cast<int64_t>(blockIdx.x) * kNumMoments;
+#pragma unroll
+    for (int i = 0; i < kSums; ++i) {
+        v[i] = warp_sum(v[i]);
+        if (lane == 0) mine[i] = v[i];
+    }
 }
 
 template <int VEC>
@@ -1696,9 +1776,11 @@ cudaError_t launch_quantize_tensor(const void* x, int64_t rows, int64_t cols, in
 }
 
 cudaError_t launch_combine(const CombineJob* jobs, int njobs, int64_t part_ld, const uint8_t* mask, int64_t T, uint32_t* status,
-                           const AdvJob* adv, cudaStream_t stream) {
+                           const AdvJob* adv, const MomentsJob* moments, cudaStream_t stream) {
     if (T == 0) return adv ? launch_advantages(*adv, stream) : cudaSuccess;
-    const dim3 grid(static_cast<unsigned>((T + 31) / 32), static_cast<unsigned>(njobs + (adv ? 1 : 0)));
+    if (moments)
+        return launch_pdl(merge_moments_kernel, merge_moment_blocks(T), 2 * 32 * kCombWarps, 0, stream, jobs[0], jobs[1], part_ld, mask, T, status, *moments);
+    const dim3 grid(static_cast<unsigned>((T + kMergeRows - 1) / kMergeRows), static_cast<unsigned>(njobs + (adv ? 1 : 0)));
     return launch_pdl(combine_kernel, grid, 32 * kCombWarps, 0, stream, jobs[0], jobs[njobs - 1], njobs, part_ld, mask, T, status,
                       adv ? *adv : AdvJob{});
 }
@@ -1717,16 +1799,18 @@ cudaError_t launch_advantages(const AdvJob& job, cudaStream_t stream) {
 
 cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,
                         const float* adv, int64_t T, int S, const ais_params& p, double* partials, int32_t* n_valid_seq, float* seq_logw,
-                        float* rho, float* w_tilde, ais_diag* diag, bool early, TotalsJob* later, cudaStream_t stream) {
-    TotalsJob job = {partials, 0, p, diag};
-    const cudaError_t e = launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, early, &job.blocks, stream);
-    if (e != cudaSuccess) return e;
+                        float* rho, float* w_tilde, ais_diag* diag, bool early, int merged_blocks, TotalsJob* later, cudaStream_t stream) {
+    TotalsJob job = {partials, merged_blocks, p, diag};
+    if (merged_blocks == 0) {
+        const cudaError_t e = launch_moments_kernel(lp_train, lp_roll, mask, seq_offsets, adv, T, S, p.C, partials, n_valid_seq, seq_logw, early, &job.blocks, stream);
+        if (e != cudaSuccess) return e;
+    }
     if (later) {
         *later = job;
-        return e;
+        return cudaSuccess;
     }
     if (T == 0) return launch_pdl(totals_kernel, 1, kDiagThreads, 0, stream, job, nullptr);
-    return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, job, rho, w_tilde, seq_offsets, S, seq_logw, true, stream);
+    return launch_rectify_kernel(lp_train, lp_roll, mask, T, p.C, job, rho, w_tilde, seq_offsets, S, seq_logw, merged_blocks == 0, stream);
 }
 
 cudaError_t launch_moments(const float* lp_train, const float* lp_roll, const uint8_t* mask, const int32_t* seq_offsets,

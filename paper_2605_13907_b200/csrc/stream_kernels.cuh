@@ -23,15 +23,6 @@ struct QuantJob {
     float* scales;
     int64_t lds;
 };
-// Opening of a log-prob call: flags[i] = 1 when rows 128 i .. 128 i + 127 contain a row with mask != 0; `clear` (16-byte
-// words, may be NULL) is zeroed on the way.
-struct FlagsJob {
-    const uint8_t* mask;
-    int64_t T;
-    uint8_t* flags;
-    void* clear;
-    int64_t clear_bytes;
-};
 // Group-relative advantages adv[s]; zero_counts [S] and the two counters of the loss kernel (its finished blocks, the row tiles
 // to recompute) are cleared for the kernels that count into them; each may be NULL.
 struct AdvJob {
@@ -41,6 +32,16 @@ struct AdvJob {
     float* adv;
     int32_t* zero_counts;
     uint32_t* tickets;
+};
+// Opening of a log-prob call: flags[i] = 1 when rows 128 i .. 128 i + 127 contain a row with mask != 0; `clear` (16-byte
+// words, may be NULL) is zeroed on the way, and the advantages of the diagnostics that follow are formed (adv.S = 0: none).
+struct FlagsJob {
+    const uint8_t* mask;
+    int64_t T;
+    uint8_t* flags;
+    void* clear;
+    int64_t clear_bytes;
+    AdvJob adv;
 };
 // The end of the batch moments, left to the kernel that follows: partial sums [blocks][kNumMoments], and where the
 // diagnostics formed from their totals go.
@@ -98,9 +99,23 @@ struct CombineJob {
     int32_t nparts;
     float *lp, *lse;
 };
-// One or two merges (the passes of one call) in one launch, and, if not NULL, the advantages of the diagnostics that follow.
+// The batch moments as part of the merge of both passes (batches of at most kMergeMomentRows rows): partial sums
+// [merge_moment_blocks(T)][kNumMoments].  adv is there already and n_valid_seq (may be NULL) has been cleared.
+constexpr int kMergeRows = 32;                                           // rows of a merging block
+constexpr int64_t kMergeMomentRows = int64_t(kDiagBlocks) * kMergeRows;
+inline int merge_moment_blocks(int64_t T) { return static_cast<int>((T + kMergeRows - 1) / kMergeRows); }
+struct MomentsJob {
+    const int32_t* seq_offsets;
+    const float* adv;
+    int32_t S;
+    float C;
+    double* partials;
+    int32_t* n_valid_seq;
+};
+// One or two merges (the passes of one call) in one launch, and, if not NULL, the batch moments (two merges, trainer first) or
+// the advantages of the diagnostics that follow.
 cudaError_t launch_combine(const CombineJob* jobs, int njobs, int64_t part_ld, const uint8_t* mask, int64_t T, uint32_t* status,
-                           const AdvJob* adv, cudaStream_t stream);
+                           const AdvJob* adv, const MomentsJob* moments, cudaStream_t stream);
 cudaError_t launch_flags(const FlagsJob& job, cudaStream_t stream);
 
 // n_valid_seq[s] = valid rows of sequence s; zeroes `ticket` (the block counter of the reduction that follows).
@@ -112,6 +127,7 @@ cudaError_t launch_diag(const float* lp_train, const float* lp_roll, const uint8
                         const float* adv, int64_t T, int S, const ais_params& p, double* partials /*[kDiagBlocks][kNumMoments]*/,
                         int32_t* n_valid_seq, float* seq_logw /* [S] scratch: non-NULL selects sequence-level weights */,
                         float* rho, float* w_tilde, ais_diag* diag, bool early /* the log-probs are older than the kernel enqueued last */,
+                        int merged_blocks /* > 0: the merge of the log-probs has left this many rows of partial sums */,
                         TotalsJob* later /* not NULL: the loss kernel forms alpha, rho and w_tilde from this */, cudaStream_t stream);
 
 // The two halves of launch_diag: partial moments summed into `moments` [kNumMoments], and everything that follows
