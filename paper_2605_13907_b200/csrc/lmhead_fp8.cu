@@ -56,7 +56,12 @@ struct Fp8Cfg {
 };
 static_assert(Fp8Cfg<4>::kSmem <= 232448 && Fp8Cfg<1>::kSmem <= 232448, "shared memory of the FP8 pass");
 
-template <int SG>
+// TILES: row tiles that are promoted, 2, or 1 for a batch of no more than one (kBM rows): half the tensor-memory loads and
+// arithmetic, the same scale loads.  100 rows at d = 4096, V = 151936 190 -> 159 us, block 32 (65,536 columns) 264 -> 172.  The last,
+// half pair of a longer batch stays with the others: behind whole pairs the launch ends with those, and giving it fewer, longer
+// ranges cost more than it saved (613 rows 525 -> 545 us, 1,100 rows 885 -> 926), because pairs that do not walk the vocabulary
+// together do not share its codes through L2.
+template <int SG, int TILES>
 __global__ void __launch_bounds__(kThreads, 1)
 lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmSA, const __grid_constant__ CUtensorMap tmSB,
@@ -208,11 +213,11 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         uint32_t flags = 0;
         uint32_t va[32], vb[32];
         bool ready = false;                           // the next block was seen complete before its turn
-        // piece p: 16 columns of both row tiles
+        // piece p: 16 columns of every row tile
         auto ld_piece = [&](uint32_t buf, int p, uint32_t (&v)[32]) {
             const uint32_t at = tmem_base + lane_base + buf * (2 * kPairCols) + half * kHalfCols + p * 16;
             tmem_ld16(at, v, 0);
-            tmem_ld16(at + kPairCols, v, 16);
+            if (TILES == 2) tmem_ld16(at + kPairCols, v, 16);
         };
         for (int u = blockIdx.x; u < num_units && ok; u += gridDim.x) {
             const Unit w = decode_unit<MODE>(a, u);
@@ -221,7 +226,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             bool rok[2];
             int y[2];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
+            for (int i = 0; i < TILES; ++i) {
                 const int64_t lr = static_cast<int64_t>(w.rt) * kPairRows + i * kBM + q * 32 + lane;
                 rok[i] = lr < a.rows;
                 grow[i] = a.row0 + lr;
@@ -233,9 +238,9 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             }
             float m_run[2] = {kNegBig, kNegBig}, s_run[2] = {0.f, 0.f}, zy[2] = {-INFINITY, -INFINITY};
             for (int t = w.t0; t < w.t1 && ok; ++t) {
-                F2 acc[2][kHalfCols / 2];                  // columns 2 n, 2 n + 1 of this thread's half, rows of both tiles
+                F2 acc[TILES][kHalfCols / 2];                  // columns 2 n, 2 n + 1 of this thread's half, rows of both tiles
 #pragma unroll
-                for (int n = 0; n < kHalfCols / 2; ++n) acc[0][n] = acc[1][n] = F2{0.f, 0.f};
+                for (int n = 0; n < kHalfCols / 2; ++n) acc[0][n] = acc[TILES - 1][n] = F2{0.f, 0.f};
                 for (int ks = 0; ks < a.ksteps && ok; ++ks) {
                     const float* sS = reinterpret_cast<const float*>(scale_base + sc.idx * C::kSlotBytes);
 #pragma unroll(SG > 1 ? 2 : 1)
@@ -245,7 +250,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         tc_fence_after();
                         const uint32_t buf = tb.idx;
                         ld_piece(buf, 0, va);
-                        const float sh0 = sS[g * kPairRows + q * 32 + lane], sh1 = sS[g * kPairRows + kBM + q * 32 + lane];
+                        const float sh0 = sS[g * kPairRows + q * 32 + lane], sh1 = sS[g * kPairRows + (TILES - 1) * kBM + q * 32 + lane];
                         const F2 r0 = {sh0, sh0}, r1 = {sh1, sh1};
                         // every lane reads the same column scales: broadcast 16-byte loads, each used for two rows
                         const float4* sw4 = reinterpret_cast<const float4*>(sS + (C::kSlotBOffset / 4) + g * kPairCols + half * kHalfCols);
@@ -256,9 +261,10 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                                 const float4 swf = sw4[pp * 4 + j];
                                 const F2 c0 = {swf.x, swf.y}, c1 = {swf.z, swf.w};
                                 F2* p0 = &acc[0][pp * 8 + 2 * j];
-                                F2* p1 = &acc[1][pp * 8 + 2 * j];
+                                F2* p1 = &acc[TILES - 1][pp * 8 + 2 * j];
                                 p0[0] = fma2(mul2(F2{__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1])}, r0), c0, p0[0]);
                                 p0[1] = fma2(mul2(F2{__uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])}, r0), c1, p0[1]);
+                                if (TILES == 1) continue;
                                 p1[0] = fma2(mul2(F2{__uint_as_float(v[16 + 4 * j]), __uint_as_float(v[17 + 4 * j])}, r1), c0, p1[0]);
                                 p1[1] = fma2(mul2(F2{__uint_as_float(v[18 + 4 * j]), __uint_as_float(v[19 + 4 * j])}, r1), c1, p1[1]);
                             }
@@ -301,7 +307,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 // streaming log-sum-exp over this thread's columns of its two rows
                 const int cbase = t * kPairCols + half * kHalfCols;        // column of acc[.][0].x
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
+                for (int i = 0; i < TILES; ++i) {
                     const int yy = y[i] - cbase;
                     if (yy >= 0 && yy < kHalfCols) {
                         // written as a running maximum on purpose: a chain of "if (k == n) z = acc[n]" is folded by
@@ -332,7 +338,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 }
             }
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < TILES; ++i)
                 if (ok && rok[i]) {
                     const int64_t o = static_cast<int64_t>(w.part * 2 + half) * a.part_ld + grow[i];
                     a.part_m[o] = m_run[i] * kLn2;
@@ -362,23 +368,35 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 
 }  // namespace
 
+template <int SG>
+static cudaError_t launch_sg(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA, const CUtensorMap& tmSB, const LmheadArgs& args,
+                             int num_ctas, cudaStream_t stream) {
+    return launch_pdl(args.rows <= kBM ? lmhead_fp8_block_kernel<SG, 1> : lmhead_fp8_block_kernel<SG, 2>, num_ctas, kThreads, Fp8Cfg<SG>::kSmem, stream, tmA,
+                      tmB, tmSA, tmSB, args);
+}
+
 cudaError_t launch_lmhead_fp8_block(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,
                                     const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream) {
     switch (args.sgroups) {
-        case 1: return launch_pdl(lmhead_fp8_block_kernel<1>, num_ctas, kThreads, Fp8Cfg<1>::kSmem, stream, tmA, tmB, tmSA, tmSB, args);
-        case 2: return launch_pdl(lmhead_fp8_block_kernel<2>, num_ctas, kThreads, Fp8Cfg<2>::kSmem, stream, tmA, tmB, tmSA, tmSB, args);
-        case 4: return launch_pdl(lmhead_fp8_block_kernel<4>, num_ctas, kThreads, Fp8Cfg<4>::kSmem, stream, tmA, tmB, tmSA, tmSB, args);
+        case 1: return launch_sg<1>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
+        case 2: return launch_sg<2>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
+        case 4: return launch_sg<4>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
         default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t lmhead_fp8_block_prepare() {
-    cudaError_t e;
-    e = cudaFuncSetAttribute(lmhead_fp8_block_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fp8Cfg<1>::kSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lmhead_fp8_block_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fp8Cfg<2>::kSmem);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(lmhead_fp8_block_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Fp8Cfg<4>::kSmem);
+    cudaError_t e = cudaSuccess;
+    auto allow = [&](auto kernel, int bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    allow(lmhead_fp8_block_kernel<1, 1>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<1, 2>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<2, 1>, Fp8Cfg<2>::kSmem);
+    allow(lmhead_fp8_block_kernel<2, 2>, Fp8Cfg<2>::kSmem);
+    allow(lmhead_fp8_block_kernel<4, 1>, Fp8Cfg<4>::kSmem);
+    allow(lmhead_fp8_block_kernel<4, 2>, Fp8Cfg<4>::kSmem);
+    return e;
 }
 
 }  // namespace ais
