@@ -440,12 +440,15 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
     blk_rows = max(128, min(blk_rows, (T + 127) // 128 * 128))
     chunks = -(-T // blk_rows)
     rows_recompute_one_call = int(rows_in_tile[live_tiles & (128 * np.arange(len(live_tiles)) >= blk_rows)].sum())
-    # kernels per step: quantisers with the opening of the log-probs, two passes, their merge with the advantages, moments, loss;
+    # kernels per step: quantisers with the opening of the log-probs, two passes, their merge with the advantages, moments (up to
+    # 18,944 rows a step in one call forms them in the merge), loss;
     # then per row chunk recompute (or the launch that finds nothing to recompute), dH and dW.  Data parallel: advantages,
     # totals, rectification and the sequence counts are launches of their own.
     launches = (6 if w.block == 0 else 3 if w.block < 0 else 2 if args.w_dv else 1) + 5 + (3 if args.with_dw else 2) * chunks
     if world > 1 or args.with_dw:
         launches += 4 if world > 1 else 3
+    elif T <= 18944:
+        launches -= 1
     return dict(ms_per_step=total_ms / args.steps, e2e_ms=e2e_ms, n_valid=n_valid, T=T, seg=seg, clocks=clocks, diag=diag,
                 h2d=h2d, d2h=d2h, streaming=streaming, zero_rows=int(T - live.sum() - (batch.mask.cpu().numpy() == 0).sum()),
                 rows_recompute=rows_recompute, rows_recompute_one_call=rows_recompute_one_call, rows_dh=rows_dh, bwd_row_chunks=chunks, launches_per_step=launches,
