@@ -10,6 +10,11 @@
 // warpgroup (warps 12..15) that moves each stage's block scales from shared to tensor memory, where the
 // block-scaled MMA reads them; their scale columns leave room for one accumulator only.  The rollout pass with
 // fp32 per-block scales has a kernel of its own (lmhead_fp8.cu).
+//
+// The producer and the MMA issuer are one elected thread each (elect.sync; a branch on lane == 0 issues copies and MMAs 10% to 20%
+// slower).  Where a stage takes four copies for 512 clocks of MMAs that was the bound: 9,216 rows, d = 4096, 65,536 columns,
+// microscaling FP8 2.14 -> 1.91 ms, FP4 1.08 -> 0.91; trainer pass of 613 rows 605 -> 596 us.  What is left there is the MMAs and the
+// operand copies together (FP8 1.79 ms; 1.34 without the copies, 1.42 with half the MMAs).
 #include <type_traits>
 
 #include "lmhead_common.cuh"
