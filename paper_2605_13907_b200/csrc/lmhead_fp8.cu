@@ -61,7 +61,10 @@ static_assert(Fp8Cfg<4>::kSmem <= 232448 && Fp8Cfg<1>::kSmem <= 232448, "shared 
 // half pair of a longer batch stays with the others: behind whole pairs the launch ends with those, and giving it fewer, longer
 // ranges cost more than it saved (613 rows 525 -> 545 us, 1,100 rows 885 -> 926), because pairs that do not walk the vocabulary
 // together do not share its codes through L2.
-template <int SG, int TILES>
+// RUN: blocks that a run of the promotion loop takes, the buffers alternating from buffer 0 on: SG, or with one block per stage 2 where
+// a tile has an even number of stages (d a multiple of 256), else 1.  Block 128 with RUN = 2 against 1 (sustained, under the power cap):
+// 9,216 rows, d = 4096, 65,536 columns 3.25 -> 3.17 ms, 2,000 rows and 151,936 columns 1,670 -> 1,652 us, 640 rows 614 -> 601 us.
+template <int SG, int TILES, int RUN>
 __global__ void __launch_bounds__(kThreads, 1)
 lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmSA, const __grid_constant__ CUtensorMap tmSB,
@@ -241,11 +244,13 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 F2 acc[TILES][kHalfCols / 2];                  // columns 2 n, 2 n + 1 of this thread's half, rows of both tiles
 #pragma unroll
                 for (int n = 0; n < kHalfCols / 2; ++n) acc[0][n] = acc[TILES - 1][n] = F2{0.f, 0.f};
-                for (int ks = 0; ks < a.ksteps && ok; ++ks) {
+                for (int ks = 0; ks < a.ksteps && ok; ks += RUN / SG) {
                     const float* sS = reinterpret_cast<const float*>(scale_base + sc.idx * C::kSlotBytes);
-#pragma unroll(SG > 1 ? 2 : 1)
-                    for (int g = 0; g < SG; ++g) {
-                        if (SG > 1) tb.idx = g & 1;       // a stage starts with buffer 0: known when the loop is unrolled by two
+#pragma unroll(RUN > 1 ? 2 : 1)
+                    for (int n = 0; n < RUN; ++n) {
+                        const int g = SG > 1 ? n : 0;     // block of its stage
+                        if (RUN > 1) tb.idx = n & 1;      // a run starts with buffer 0: known when the loop is unrolled by two
+                        if (SG == 1 && n > 0) sS = reinterpret_cast<const float*>(scale_base + sc.idx * C::kSlotBytes);
                         if (!ready && !mbar_wait_warp_spin(&tfull[tb.idx], tb.phase, abort_flag, a.wait_cycles)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t buf = tb.idx;
@@ -287,9 +292,9 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&tempty[buf]);
-                        if (SG > 1) {
-                            tb.idx = (g + 1) & 1;
-                            tb.phase ^= g & 1;
+                        if (RUN > 1) {
+                            tb.idx = (n + 1) & 1;
+                            tb.phase ^= n & 1;
                         } else {
                             tb.advance();
                         }
@@ -297,11 +302,17 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         const bool seen = mbar_test_wait(&tfull[tb.idx], tb.phase);
                         promote(I3{}, vb);
                         ready = __all_sync(0xffffffffu, seen);
+                        if (SG == 1) {                    // the stage's scales have been used (and the warp has just met)
+                            if (lane == 0) mbar_arrive(&sempty[sc.idx]);
+                            sc.advance();
+                        }
                     }
                     if (!ok) break;
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sempty[sc.idx]);
-                    sc.advance();
+                    if (SG > 1) {                             // (inside the loop it costs block 32 3%)
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&sempty[sc.idx]);
+                        sc.advance();
+                    }
                 }
                 if (!ok) break;
                 // streaming log-sum-exp over this thread's columns of its two rows
@@ -368,19 +379,20 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 
 }  // namespace
 
-template <int SG>
-static cudaError_t launch_sg(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA, const CUtensorMap& tmSB, const LmheadArgs& args,
-                             int num_ctas, cudaStream_t stream) {
-    return launch_pdl(args.rows <= kBM ? lmhead_fp8_block_kernel<SG, 1> : lmhead_fp8_block_kernel<SG, 2>, num_ctas, kThreads, Fp8Cfg<SG>::kSmem, stream, tmA,
-                      tmB, tmSA, tmSB, args);
+template <int SG, int RUN>
+static cudaError_t launch_run(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA, const CUtensorMap& tmSB, const LmheadArgs& args,
+                              int num_ctas, cudaStream_t stream) {
+    return launch_pdl(args.rows <= kBM ? lmhead_fp8_block_kernel<SG, 1, RUN> : lmhead_fp8_block_kernel<SG, 2, RUN>, num_ctas, kThreads, Fp8Cfg<SG>::kSmem,
+                      stream, tmA, tmB, tmSA, tmSB, args);
 }
 
 cudaError_t launch_lmhead_fp8_block(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,
                                     const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream) {
     switch (args.sgroups) {
-        case 1: return launch_sg<1>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
-        case 2: return launch_sg<2>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
-        case 4: return launch_sg<4>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
+        case 1: return args.ksteps % 2 == 0 ? launch_run<1, 2>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream)
+                                            : launch_run<1, 1>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
+        case 2: return launch_run<2, 2>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
+        case 4: return launch_run<4, 4>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -390,12 +402,14 @@ cudaError_t lmhead_fp8_block_prepare() {
     auto allow = [&](auto kernel, int bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
-    allow(lmhead_fp8_block_kernel<1, 1>, Fp8Cfg<1>::kSmem);
-    allow(lmhead_fp8_block_kernel<1, 2>, Fp8Cfg<1>::kSmem);
-    allow(lmhead_fp8_block_kernel<2, 1>, Fp8Cfg<2>::kSmem);
-    allow(lmhead_fp8_block_kernel<2, 2>, Fp8Cfg<2>::kSmem);
-    allow(lmhead_fp8_block_kernel<4, 1>, Fp8Cfg<4>::kSmem);
-    allow(lmhead_fp8_block_kernel<4, 2>, Fp8Cfg<4>::kSmem);
+    allow(lmhead_fp8_block_kernel<1, 1, 1>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<1, 2, 1>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<1, 1, 2>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<1, 2, 2>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<2, 1, 2>, Fp8Cfg<2>::kSmem);
+    allow(lmhead_fp8_block_kernel<2, 2, 2>, Fp8Cfg<2>::kSmem);
+    allow(lmhead_fp8_block_kernel<4, 1, 4>, Fp8Cfg<4>::kSmem);
+    allow(lmhead_fp8_block_kernel<4, 2, 4>, Fp8Cfg<4>::kSmem);
     return e;
 }
 
