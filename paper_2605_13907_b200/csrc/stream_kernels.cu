@@ -145,9 +145,14 @@ __device__ __forceinline__ void run_advantage(const AdvJob& j, int s) {
     j.adv[s] = static_cast<float>(a);
 }
 
-// FlagsJob by blocks of kQThreads threads: one warp per 128-row tile.
+// FlagsJob by blocks of kQThreads threads: one warp per 128-row tile, and a thread for each sequence whose advantage is formed on the
+// way: with the threads of the tiles alone (a quarter of T) each had several to form, one after the other, ahead of both passes (step
+// of 1,024 rows in 4 x 256 sequences 57.8 -> 44.2 us, in 16 x 64 45.3 -> 40.5, of 18,944 rows in 74 x 256 105.6 -> 89.3).
 constexpr int kFlagTiles = kQThreads / 32;
-inline unsigned flag_blocks(const FlagsJob& f) { return static_cast<unsigned>(((f.T + 127) / 128 + kFlagTiles - 1) / kFlagTiles); }
+inline unsigned flag_blocks(const FlagsJob& f) {
+    const int64_t tiles = ((f.T + 127) / 128 + kFlagTiles - 1) / kFlagTiles, seqs = (static_cast<int64_t>(f.adv.S) + kQThreads - 1) / kQThreads;
+    return static_cast<unsigned>(tiles > seqs ? tiles : seqs);
+}
 __device__ __forceinline__ void run_flags(const FlagsJob& f, unsigned block, unsigned nblocks) {
     const int64_t tile = static_cast<int64_t>(block) * kFlagTiles + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
