@@ -55,6 +55,12 @@ struct Fp8Cfg {
     static constexpr int kSmem = 1024 + kStages * kStageBytes + kSlots * kSlotBytes + kBarriers * 8 + 64;
 };
 static_assert(Fp8Cfg<4>::kSmem <= 232448 && Fp8Cfg<1>::kSmem <= 232448, "shared memory of the FP8 pass");
+// With one block per stage a slot's scales are given back without a barrier of the warp between the other lanes' reads and lane 0's
+// arrival (a vote orders no memory accesses).  What orders them is the way of the operands: fill m waits for the MMAs of fill
+// m - kStages, those waited for the buffer of the block two before theirs, and every warp gave that buffer back behind a
+// __syncwarp that follows all its reads of the block before.  So when fill m is requested the scales of fills up to
+// m - kStages - 3 have been read, and a slot may be written again that many fills later or more.
+static_assert(Fp8Cfg<1>::kSlots >= kStages + 3, "a scale slot is rewritten only after all lanes have read it");
 
 // TILES: row tiles that are promoted, 2, or 1 for a batch of no more than one (kBM rows): half the tensor-memory loads and
 // arithmetic, the same scale loads.  100 rows at d = 4096, V = 151936 190 -> 159 us, block 32 (65,536 columns) 264 -> 172.  The last,
@@ -302,7 +308,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                         const bool seen = mbar_test_wait(&tfull[tb.idx], tb.phase);
                         promote(I3{}, vb);
                         ready = __all_sync(0xffffffffu, seen);
-                        if (SG == 1) {                    // the stage's scales have been used (and the warp has just met)
+                        if (SG == 1) {                    // the stage's scales have been used (what orders the reads: see kSlots)
                             if (lane == 0) mbar_arrive(&sempty[sc.idx]);
                             sc.advance();
                         }
