@@ -20,6 +20,7 @@ the mixing coefficient.
 from __future__ import annotations
 
 import argparse
+import ctypes
 import importlib
 import json
 import os
@@ -240,6 +241,27 @@ def rank_workload(args, rank: int):
     return w
 
 
+# ------------------------------------------------------------------------------------------ launches
+def kernels_of(call) -> int:
+    """Kernels that `call` enqueues on the current stream, counted in a capture of it (nothing of it runs)."""
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        call()
+    cuda = ctypes.CDLL("libcuda.so.1")
+    raw, n, kind = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(), ctypes.c_int()
+    if cuda.cuGraphGetNodes(raw, None, ctypes.byref(n)) != 0:
+        raise RuntimeError("cuGraphGetNodes")
+    nodes = (ctypes.c_void_p * n.value)()
+    if cuda.cuGraphGetNodes(raw, nodes, ctypes.byref(n)) != 0:
+        raise RuntimeError("cuGraphGetNodes")
+    kernels = 0
+    for node in nodes:
+        if cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) != 0:
+            raise RuntimeError("cuGraphNodeGetType")
+        kernels += kind.value == 0                          # CU_GRAPH_NODE_TYPE_KERNEL
+    return kernels
+
+
 # ------------------------------------------------------------------------------------------ one rank's measurement
 def measure_rank(args, rank: int, world: int, local: int) -> dict:
     """Everything one rank measures on its GPU: the timed steps, the end-to-end steps, clocks, and (rank 0, one GPU) the
@@ -440,15 +462,15 @@ def measure_rank(args, rank: int, world: int, local: int) -> dict:
     blk_rows = max(128, min(blk_rows, (T + 127) // 128 * 128))
     chunks = -(-T // blk_rows)
     rows_recompute_one_call = int(rows_in_tile[live_tiles & (128 * np.arange(len(live_tiles)) >= blk_rows)].sum())
-    # kernels per step: quantisers with the opening of the log-probs, two passes, their merge with the advantages, moments (up to
-    # 18,944 rows a step in one call forms them in the merge), loss;
-    # then per row chunk recompute (or the launch that finds nothing to recompute), dH and dW.  Data parallel: advantages,
-    # totals, rectification and the sequence counts are launches of their own.
-    launches = (6 if w.block == 0 else 3 if w.block < 0 else 2 if args.w_dv else 1) + 5 + (3 if args.with_dw else 2) * chunks
-    if world > 1 or args.with_dw:
-        launches += 4 if world > 1 else 3
-    elif T <= 18944:
-        launches -= 1
+    if world == 1:
+        launches = kernels_of(one_step)
+    else:                                                   # the stages around the all-reduce, whose own kernels do not count
+        launches = (kernels_of(lambda: step.forward(batch.H, batch.W, batch.tokens, batch.mask)) +
+                    kernels_of(lambda: ais.diag_moments(step.shape, step.params, step.lp_train, step.lp_roll, batch.mask, offs, rew, step.adv,
+                                                        step.n_valid_seq, step.moments, step.workspace, seq_logw=step.seq_logw)) +
+                    kernels_of(lambda: ais.diag_finalize(step.shape, step.params, step.moments, step.lp_train, step.lp_roll, batch.mask,
+                                                         step.rho, step.w_tilde, step.diag, seq_offsets=offs, seq_logw=step.seq_logw)) +
+                    kernels_of(lambda: step.backward(batch.H, batch.W, batch.tokens, batch.mask, offs, dW=dW_buf)))
     return dict(ms_per_step=total_ms / args.steps, e2e_ms=e2e_ms, n_valid=n_valid, T=T, seg=seg, clocks=clocks, diag=diag,
                 h2d=h2d, d2h=d2h, streaming=streaming, zero_rows=int(T - live.sum() - (batch.mask.cpu().numpy() == 0).sum()),
                 rows_recompute=rows_recompute, rows_recompute_one_call=rows_recompute_one_call, rows_dh=rows_dh, bwd_row_chunks=chunks, launches_per_step=launches,
