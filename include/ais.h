@@ -327,7 +327,9 @@ int ais_loss_bwd(const ais_shape* shape, const ais_params* params,
  * follows from them and dH then have the same precision, but not the same bits, as the stages called one by one: the
  * exponentials are summed about 0 instead of their maximum, and dH's scratch is rounded to bf16 before its row factor
  * instead of after it.  (The loss is a sum that cancels to a small part of its terms; two such results agree to about
- * 1e-7 of the sum of the terms' absolute values, not of the loss.)  Quantises by shape->fp8_block; the codes' row strides
+ * 1e-7 of the sum of the terms' absolute values, not of the loss.)  With AIS_STAGE_LOGPROB and AIS_STAGE_DIAGNOSE the batch
+ * moments of a short batch are summed in fp64 row by row where the log-probs are formed: the diagnostics, and rho and w_tilde
+ * through alpha, may differ from ais_diagnostics' in their last bits.  Quantises by shape->fp8_block; the codes' row strides
  * are those ais_logprob_fwd expects.  Stops at the first stage that returns an error; the stages before it have run.
  */
 #define AIS_STAGE_QUANTIZE_H 1u
