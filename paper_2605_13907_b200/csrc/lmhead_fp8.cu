@@ -67,9 +67,10 @@ static_assert(Fp8Cfg<1>::kSlots >= kStages + 3, "a scale slot is rewritten only 
 // half pair of a longer batch stays with the others: behind whole pairs the launch ends with those, and giving it fewer, longer
 // ranges cost more than it saved (613 rows 525 -> 545 us, 1,100 rows 885 -> 926), because pairs that do not walk the vocabulary
 // together do not share its codes through L2.
-// RUN: blocks that a run of the promotion loop takes, the buffers alternating from buffer 0 on: SG, or with one block per stage 2 where
-// a tile has an even number of stages (d a multiple of 256), else 1.  Block 128 with RUN = 2 against 1 (sustained, under the power cap):
-// 9,216 rows, d = 4096, 65,536 columns 3.25 -> 3.17 ms, 2,000 rows and 151,936 columns 1,670 -> 1,652 us, 640 rows 614 -> 601 us.
+// RUN: blocks that a run of the promotion loop takes, the buffers alternating from buffer 0 on: SG, or with one block per stage and one row
+// tile 2 where a tile has an even number of stages (d a multiple of 256: 20 rows x 2048, 32,000 columns 41.9 -> 40.8 us, 100 x 4096,
+// 4,096 columns 20.6 -> 20.3), else 1.  With two row tiles runs of two are no faster at d = 4096 (12,000 rows, 65,536 columns 4,389 and
+// 4,384 us) and slower where a tile has few stages (d = 256, 20,000 rows, 16,384 columns 198 -> 213, 8,000 and 8,192 56.5 -> 60.9).
 template <int SG, int TILES, int RUN>
 __global__ void __launch_bounds__(kThreads, 1)
 lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -385,20 +386,21 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 
 }  // namespace
 
-template <int SG, int RUN>
-static cudaError_t launch_run(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA, const CUtensorMap& tmSB, const LmheadArgs& args,
-                              int num_ctas, cudaStream_t stream) {
-    return launch_pdl(args.rows <= kBM ? lmhead_fp8_block_kernel<SG, 1, RUN> : lmhead_fp8_block_kernel<SG, 2, RUN>, num_ctas, kThreads, Fp8Cfg<SG>::kSmem,
-                      stream, tmA, tmB, tmSA, tmSB, args);
+template <int SG>
+static cudaError_t launch_blocks(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA, const CUtensorMap& tmSB, const LmheadArgs& args,
+                                 int num_ctas, cudaStream_t stream) {
+    constexpr int kRun1 = SG == 1 ? 2 : SG;                                // of one row tile
+    auto kernel = lmhead_fp8_block_kernel<SG, 2, SG>;
+    if (args.rows <= kBM) kernel = SG > 1 || args.ksteps % 2 == 0 ? lmhead_fp8_block_kernel<SG, 1, kRun1> : lmhead_fp8_block_kernel<SG, 1, SG>;
+    return launch_pdl(kernel, num_ctas, kThreads, Fp8Cfg<SG>::kSmem, stream, tmA, tmB, tmSA, tmSB, args);
 }
 
 cudaError_t launch_lmhead_fp8_block(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA,
                                     const CUtensorMap& tmSB, const LmheadArgs& args, int num_ctas, cudaStream_t stream) {
     switch (args.sgroups) {
-        case 1: return args.ksteps % 2 == 0 ? launch_run<1, 2>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream)
-                                            : launch_run<1, 1>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
-        case 2: return launch_run<2, 2>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
-        case 4: return launch_run<4, 4>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
+        case 1: return launch_blocks<1>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
+        case 2: return launch_blocks<2>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
+        case 4: return launch_blocks<4>(tmA, tmB, tmSA, tmSB, args, num_ctas, stream);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -411,7 +413,6 @@ cudaError_t lmhead_fp8_block_prepare() {
     allow(lmhead_fp8_block_kernel<1, 1, 1>, Fp8Cfg<1>::kSmem);
     allow(lmhead_fp8_block_kernel<1, 2, 1>, Fp8Cfg<1>::kSmem);
     allow(lmhead_fp8_block_kernel<1, 1, 2>, Fp8Cfg<1>::kSmem);
-    allow(lmhead_fp8_block_kernel<1, 2, 2>, Fp8Cfg<1>::kSmem);
     allow(lmhead_fp8_block_kernel<2, 1, 2>, Fp8Cfg<2>::kSmem);
     allow(lmhead_fp8_block_kernel<2, 2, 2>, Fp8Cfg<2>::kSmem);
     allow(lmhead_fp8_block_kernel<4, 1, 4>, Fp8Cfg<4>::kSmem);
