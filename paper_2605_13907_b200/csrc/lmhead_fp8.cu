@@ -28,12 +28,20 @@
 // 7.80 ms, 9,216 rows, d = 4096, 65,536 columns), block 64 4.53 -> 4.35 ms; unrolled by four 1,038 (instruction fetch).
 // What the promotion contends for is the path out of shared memory: a broadcast 16-byte load returns 512 bytes, four clocks of
 // it, and the MMAs take all of it while they run (8 KB of operands per 64 clocks).  In a copy of the loop with real MMAs and
-// without the rest of the kernel a block takes 753 clocks with no MMA, 840 with the two of block 32 and 1,187 with the eight of
+// without the rest of the kernel a block takes 753 clocks with no MMA, 831 to 840 with the two of block 32 and 1,187 with the eight of
 // block 128, against 687, 720 and 791 with the column scales taken as constants; operand copies add nothing to that.  Loads of
 // scales by shuffle (1,232), 16x256b tensor-memory loads (eight rows x 16 columns per thread, a third of the scale traffic, but
 // half the tensor-memory rate: 1,137) and 128 x 256 tiles of them (1,141) do not get below it.
-// The roles with one thread are entered through elect.sync: with `lane == 0` a stage's copies and a block's MMAs took 10% to 20%
-// longer to issue (hand-overs alone, no promotion: 928 -> 847 clocks per block, block 32 414 -> 343).
+// How the roles with one thread are entered.  Through elect.sync a stage's copies and a block's MMAs take 10% to 20% less to issue
+// than behind `lane == 0` (hand-overs alone, no promotion: 928 -> 847 clocks per block, block 32 414 -> 343).  That shortens what a
+// short launch waits for, but in a long one the MMAs then meet the promotion of the block before on the path out of shared memory.
+// Pass alone, block 128, in turn on one box, both behind `lane == 0` / issuers elected / both elected (us; rows x d, columns):
+//   600 x 4096, 4,096 30.2 / 29.0 / 29.1;  1,100 x 4096, 16,384 125.4 / 121.4 / 122.8;  3,000 x 2048, 16,384 147.4 / 145.7 / 147.7;
+//   12,000 x 512, 65,536 690 / 689 / 688;  6,000 x 1024, 32,000 301.1 / 303.9 / 304.5;  12,000 x 4096, 65,536 4,260 / 4,316 / 4,389;
+//   20,000 x 2048, 16,384 928 / 944 / 953
+// block 64, 9,216 x 4096, 65,536 4,582 / 4,637 / 4,643;  block 32 7,740 / 7,780 / 7,816.  One row tile: 100 x 4096, 4,096 25.3 / 25.9 /
+// 20.6.  So ELECT holds up to kElectRows rows and below kElectSteps stages per tile, and with it the producer is elected too, but for
+// pairs of row tiles of block 128.
 #include <type_traits>
 
 #include "lmhead_common.cuh"
@@ -69,9 +77,9 @@ static_assert(Fp8Cfg<1>::kSlots >= kStages + 3, "a scale slot is rewritten only 
 // together do not share its codes through L2.
 // RUN: blocks that a run of the promotion loop takes, the buffers alternating from buffer 0 on: SG, or with one block per stage and one row
 // tile 2 where a tile has an even number of stages (d a multiple of 256: 20 rows x 2048, 32,000 columns 41.9 -> 40.8 us, 100 x 4096,
-// 4,096 columns 20.6 -> 20.3), else 1.  With two row tiles runs of two are no faster at d = 4096 (12,000 rows, 65,536 columns 4,389 and
-// 4,384 us) and slower where a tile has few stages (d = 256, 20,000 rows, 16,384 columns 198 -> 213, 8,000 and 8,192 56.5 -> 60.9).
-template <int SG, int TILES, int RUN>
+// 4,096 columns 20.6 -> 20.3), else 1.  With two row tiles runs of two are no faster at d = 4096 (12,000 rows, 65,536 columns 4,260 and
+// 4,256 us) and slower where a tile has few stages (d = 256, 20,000 rows, 16,384 columns 199 -> 217, 8,000 and 8,192 57.4 -> 62.1).
+template <int SG, int TILES, int RUN, bool ELECT>
 __global__ void __launch_bounds__(kThreads, 1)
 lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         const __grid_constant__ CUtensorMap tmSA, const __grid_constant__ CUtensorMap tmSB,
@@ -126,7 +134,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         reg_dealloc<40>();
         if (warp == 0) {
             // ------------------------------------------------------------------ TMA producer
-            if (elect_one()) {
+            if (ELECT && (TILES == 1 || SG > 1) ? elect_one() : lane == 0) {
                 Pipe st(kStages), sc(C::kSlots);
                 uint32_t issued = 0;
                 bool ok = true;
@@ -169,7 +177,7 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             // block (block n of the CTA goes to buffer n % 2).  One thread cannot keep up: it shares its scheduler with
             // two promotion warps, and wait + four MMAs + two commits took it about 1,300 clocks per block against the
             // 542 the tensor core needs.  The two threads are independent: different buffers, different barriers.
-            if (elect_one()) {
+            if (ELECT ? elect_one() : lane == 0) {
                 const uint32_t me = warp - 1;
                 constexpr uint32_t idesc = make_idesc(kFmtE4M3, kFmtE4M3, kBM, kPairCols, 0, 0);
                 const uint64_t desc0 = smem_desc_sw128(0, 16, 1024);           // descriptor of address 0: add (address >> 4)
@@ -386,12 +394,18 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 
 }  // namespace
 
+// ELECT: up to twelve row pairs, or few stages per tile.  Around the first line, d = 5120, V = 262144, issuers behind `lane == 0` and
+// elected: 1,152 rows 2,225 and 2,159 us, 2,304 4,005 and 4,041, 3,200 5,708 and 5,742; d = 4096, V = 151936: 2,176 rows 1,874 and 1,827,
+// 3,200 2,698 and 2,694, 6,272 5,313 and 5,355.
+constexpr int64_t kElectRows = 12 * kPairRows;
+constexpr int kElectSteps = 8;
+
 template <int SG>
 static cudaError_t launch_blocks(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA, const CUtensorMap& tmSB, const LmheadArgs& args,
                                  int num_ctas, cudaStream_t stream) {
     constexpr int kRun1 = SG == 1 ? 2 : SG;                                // of one row tile
-    auto kernel = lmhead_fp8_block_kernel<SG, 2, SG>;
-    if (args.rows <= kBM) kernel = SG > 1 || args.ksteps % 2 == 0 ? lmhead_fp8_block_kernel<SG, 1, kRun1> : lmhead_fp8_block_kernel<SG, 1, SG>;
+    auto kernel = args.rows <= kElectRows || args.ksteps < kElectSteps ? lmhead_fp8_block_kernel<SG, 2, SG, true> : lmhead_fp8_block_kernel<SG, 2, SG, false>;
+    if (args.rows <= kBM) kernel = SG > 1 || args.ksteps % 2 == 0 ? lmhead_fp8_block_kernel<SG, 1, kRun1, true> : lmhead_fp8_block_kernel<SG, 1, SG, true>;
     return launch_pdl(kernel, num_ctas, kThreads, Fp8Cfg<SG>::kSmem, stream, tmA, tmB, tmSA, tmSB, args);
 }
 
@@ -410,13 +424,16 @@ cudaError_t lmhead_fp8_block_prepare() {
     auto allow = [&](auto kernel, int bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
-    allow(lmhead_fp8_block_kernel<1, 1, 1>, Fp8Cfg<1>::kSmem);
-    allow(lmhead_fp8_block_kernel<1, 2, 1>, Fp8Cfg<1>::kSmem);
-    allow(lmhead_fp8_block_kernel<1, 1, 2>, Fp8Cfg<1>::kSmem);
-    allow(lmhead_fp8_block_kernel<2, 1, 2>, Fp8Cfg<2>::kSmem);
-    allow(lmhead_fp8_block_kernel<2, 2, 2>, Fp8Cfg<2>::kSmem);
-    allow(lmhead_fp8_block_kernel<4, 1, 4>, Fp8Cfg<4>::kSmem);
-    allow(lmhead_fp8_block_kernel<4, 2, 4>, Fp8Cfg<4>::kSmem);
+    allow(lmhead_fp8_block_kernel<1, 1, 1, true>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<1, 1, 2, true>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<1, 2, 1, true>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<1, 2, 1, false>, Fp8Cfg<1>::kSmem);
+    allow(lmhead_fp8_block_kernel<2, 1, 2, true>, Fp8Cfg<2>::kSmem);
+    allow(lmhead_fp8_block_kernel<2, 2, 2, true>, Fp8Cfg<2>::kSmem);
+    allow(lmhead_fp8_block_kernel<2, 2, 2, false>, Fp8Cfg<2>::kSmem);
+    allow(lmhead_fp8_block_kernel<4, 1, 4, true>, Fp8Cfg<4>::kSmem);
+    allow(lmhead_fp8_block_kernel<4, 2, 4, true>, Fp8Cfg<4>::kSmem);
+    allow(lmhead_fp8_block_kernel<4, 2, 4, false>, Fp8Cfg<4>::kSmem);
     return e;
 }
 
