@@ -851,9 +851,10 @@ __device__ __forceinline__ void add_run(double* acc, int n, float p, float sv, f
 // The merge of both passes and the batch moments in one kernel, for batches of up to kMergeMomentRows rows: the sixteen warps
 // merge 32 rows as combine_kernel does (eight warps per pass, the same order), then one warp forms the terms of its 32 rows
 // and their sums in fp64, one row of partial sums per block.  A small batch is a chain of launches, and the moments kernel (start,
-// walk, fp64 sums) is one of them, while every row's log-probs are in a register here: a step of 512 rows 46.4 -> 42.5 us, of
-// 3,001 rows (d = 512, V = 4096) 90.5 -> 86.7.  The limit is the number of partial sums that the totals behind it are formed from,
-// no more than the moments kernel leaves.
+// walk, fp64 sums) is one of them, while every row's log-probs are in a register here.  Steps of d = 256, V = 1024 with the moments
+// kernel and without: 512 rows 42.1 -> 39.6 us, 4,096 61.2 -> 58.2, 9,217 68.8 -> 66.2, 12,288 79.7 -> 77.6, 18,944 87.7 -> 86.4; log-probs
+// and diagnostics alone 4,096 31.1 -> 28.7, 18,944 51.7 -> 51.1.  The limit is what the buffer of partial sums holds (kDiagBlocks rows of
+// them, of which the moments kernel leaves one per 2,048 rows); the gain shrinks towards it because every block behind adds them up.
 __global__ void __launch_bounds__(2 * 32 * kCombWarps) merge_moments_kernel(const CombineJob j0, const CombineJob j1, int64_t part_ld,
                                                                             const uint8_t* __restrict__ mask, int64_t T, uint32_t* status,
                                                                             const MomentsJob mj) {
@@ -1552,7 +1553,7 @@ __global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const __grid_co
         r.range = seqs_of_rows_warp(a.seq_offsets, a.S, tile * 128, tile * 128 + 127 < a.T ? tile * 128 + 127 : a.T - 1);
     };
     // The first rows and their sequences are asked for ahead of the sums that alpha waits for: a small batch is one chain of
-    // loads (step of 512 rows 42.5 -> 39.6 us, with the single block's sums taken from shared memory below).
+    // loads (step of 512 rows 42.4 -> 41.4 us, of 3,001 rows, d = 512, V = 4096, 85.8 -> 85.0).
     Rows in;
     if (tile0 < tiles) load_rows(tile0, in);
     float alpha = 0.f;
@@ -1649,6 +1650,7 @@ __global__ void __launch_bounds__(kDiagThreads) loss_coef_kernel(const __grid_co
         for (int i = blockIdx.x * kDiagThreads + threadIdx.x; i < a.nclear; i += gridDim.x * kDiagThreads) a.clear[i] = make_uint4(0, 0, 0, 0);
     double sums[2] = {J, KL};
     block_sums(sums, scratch, totals);
+    // A single block has its sums at hand and needs no counter of finished blocks (512 rows 41.4 -> 39.2 us).
     double Jall = totals[0], KLall = totals[1];
     if (gridDim.x > 1) {
         if (threadIdx.x < 2) a.partials[2 * blockIdx.x + threadIdx.x] = totals[threadIdx.x];
