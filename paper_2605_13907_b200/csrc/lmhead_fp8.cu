@@ -35,13 +35,16 @@
 // How the roles with one thread are entered.  Through elect.sync a stage's copies and a block's MMAs take 10% to 20% less to issue
 // than behind `lane == 0` (hand-overs alone, no promotion: 928 -> 847 clocks per block, block 32 414 -> 343).  That shortens what a
 // short launch waits for, but in a long one the MMAs then meet the promotion of the block before on the path out of shared memory.
-// Pass alone, block 128, in turn on one box, both behind `lane == 0` / issuers elected / both elected (us; rows x d, columns):
-//   600 x 4096, 4,096 30.2 / 29.0 / 29.1;  1,100 x 4096, 16,384 125.4 / 121.4 / 122.8;  3,000 x 2048, 16,384 147.4 / 145.7 / 147.7;
-//   12,000 x 512, 65,536 690 / 689 / 688;  6,000 x 1024, 32,000 301.1 / 303.9 / 304.5;  12,000 x 4096, 65,536 4,260 / 4,316 / 4,389;
-//   20,000 x 2048, 16,384 928 / 944 / 953
-// block 64, 9,216 x 4096, 65,536 4,582 / 4,637 / 4,643;  block 32 7,740 / 7,780 / 7,816.  One row tile: 100 x 4096, 4,096 25.3 / 25.9 /
-// 20.6.  So ELECT holds up to kElectRows rows and below kElectSteps stages per tile, and with it the producer is elected too, but for
-// pairs of row tiles of block 128.
+// Block 128, both behind `lane == 0` / issuers elected / both elected (us, in turn on one box; rows x d, columns):
+//   pass alone: 600 x 4096, 4,096 30.2 / 29.0 / 29.1;  1,100 x 4096, 16,384 125.4 / 121.4 / 122.8;  3,000 x 2048, 16,384 147.4 / 145.7 /
+//   147.7;  6,000 x 1024, 32,000 301 / 304 / 305;  12,000 x 4096, 65,536 4,260 / 4,316 / 4,389;  one row tile, 100 x 4096, 4,096 25.3 /
+//   25.9 / 20.6
+//   whole step, 9,217 x 4096, 151,936 25,080 / 24,900 / 24,920 (issues that keep pace cost a long pass time and the passes behind it gain
+//   more: the step runs at the power cap); log-probs alone 15,840 / 15,830 / 15,980
+// Blocks of 64 and 32, behind `lane == 0` and elected: pass alone 12,000 x 4096, 65,536 5,917 and 6,022, 10,407 and 10,506; whole step,
+// 9,217 x 4096, 151,936 28,930 and 29,210, 36,890 and 37,360.  Here it is the stages of a tile that decide.
+// So the issuers of block 128 are elected, its producer for one row tile only; both roles of smaller blocks are below kElectSteps stages
+// per tile (ELECT).
 #include <type_traits>
 
 #include "lmhead_common.cuh"
@@ -77,8 +80,8 @@ static_assert(Fp8Cfg<1>::kSlots >= kStages + 3, "a scale slot is rewritten only 
 // together do not share its codes through L2.
 // RUN: blocks that a run of the promotion loop takes, the buffers alternating from buffer 0 on: SG, or with one block per stage and one row
 // tile 2 where a tile has an even number of stages (d a multiple of 256: 20 rows x 2048, 32,000 columns 41.9 -> 40.8 us, 100 x 4096,
-// 4,096 columns 20.6 -> 20.3), else 1.  With two row tiles runs of two are no faster at d = 4096 (12,000 rows, 65,536 columns 4,260 and
-// 4,256 us) and slower where a tile has few stages (d = 256, 20,000 rows, 16,384 columns 199 -> 217, 8,000 and 8,192 57.4 -> 62.1).
+// 4,096 columns 20.6 -> 20.3), else 1.  With two row tiles runs of two are no faster at d = 4096 (12,000 rows, 65,536 columns 4,316 and
+// 4,350 us) and slower where a tile has few stages (d = 256, 20,000 rows, 16,384 columns 196 -> 212, 8,000 and 8,192 56.7 -> 61.0).
 template <int SG, int TILES, int RUN, bool ELECT>
 __global__ void __launch_bounds__(kThreads, 1)
 lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -394,17 +397,17 @@ lmhead_fp8_block_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
 
 }  // namespace
 
-// ELECT: up to twelve row pairs, or few stages per tile.  Around the first line, d = 5120, V = 262144, issuers behind `lane == 0` and
-// elected: 1,152 rows 2,225 and 2,159 us, 2,304 4,005 and 4,041, 3,200 5,708 and 5,742; d = 4096, V = 151936: 2,176 rows 1,874 and 1,827,
-// 3,200 2,698 and 2,694, 6,272 5,313 and 5,355.
-constexpr int64_t kElectRows = 12 * kPairRows;
+// ELECT with several blocks per stage: below eight stages per tile.  Block 64, behind `lane == 0` and elected, 1,100 and 3,000 rows, 16,384
+// columns: d = 256 27.4 and 27.1, 49.0 and 48.5 us; 512 37.3 and 37.2, 70.6 and 70.5; 1024 56.5 and 56.6, 112.6 and 113.0 (600 rows, 4,096
+// columns 18.9 and 18.8); 4096 173.3 and 174.6, 387.0 and 390.4.
 constexpr int kElectSteps = 8;
 
 template <int SG>
 static cudaError_t launch_blocks(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmSA, const CUtensorMap& tmSB, const LmheadArgs& args,
                                  int num_ctas, cudaStream_t stream) {
     constexpr int kRun1 = SG == 1 ? 2 : SG;                                // of one row tile
-    auto kernel = args.rows <= kElectRows || args.ksteps < kElectSteps ? lmhead_fp8_block_kernel<SG, 2, SG, true> : lmhead_fp8_block_kernel<SG, 2, SG, false>;
+    auto kernel = lmhead_fp8_block_kernel<SG, 2, SG, true>;
+    if (SG > 1 && args.ksteps >= kElectSteps) kernel = lmhead_fp8_block_kernel<SG, 2, SG, SG == 1>;
     if (args.rows <= kBM) kernel = SG > 1 || args.ksteps % 2 == 0 ? lmhead_fp8_block_kernel<SG, 1, kRun1, true> : lmhead_fp8_block_kernel<SG, 1, SG, true>;
     return launch_pdl(kernel, num_ctas, kThreads, Fp8Cfg<SG>::kSmem, stream, tmA, tmB, tmSA, tmSB, args);
 }
@@ -427,7 +430,6 @@ cudaError_t lmhead_fp8_block_prepare() {
     allow(lmhead_fp8_block_kernel<1, 1, 1, true>, Fp8Cfg<1>::kSmem);
     allow(lmhead_fp8_block_kernel<1, 1, 2, true>, Fp8Cfg<1>::kSmem);
     allow(lmhead_fp8_block_kernel<1, 2, 1, true>, Fp8Cfg<1>::kSmem);
-    allow(lmhead_fp8_block_kernel<1, 2, 1, false>, Fp8Cfg<1>::kSmem);
     allow(lmhead_fp8_block_kernel<2, 1, 2, true>, Fp8Cfg<2>::kSmem);
     allow(lmhead_fp8_block_kernel<2, 2, 2, true>, Fp8Cfg<2>::kSmem);
     allow(lmhead_fp8_block_kernel<2, 2, 2, false>, Fp8Cfg<2>::kSmem);

@@ -60,10 +60,9 @@ def _log_probs_from_codes(s, tokens, T, V, d, block):
     (300, 384, 40008, 0),        # pairs of row tiles, an odd number of stages
     (900, 640, 20000, 64),       # four pairs x 64 ranges: two units on most CTAs
     (900, 512, 20000, 64),
-    (3072, 1024, 5000, 64),      # the most and the fewest rows and stages of the two ways in which the MMA issuers are entered
-    (3073, 1024, 5000, 64),
-    (3073, 896, 5000, 64),
-    (3073, 1152, 5000, 64),
+    (700, 896, 5000, 64),        # seven, eight and nine stages per tile: the two ways in which copies and MMAs of smaller blocks are issued
+    (700, 1024, 5000, 64),
+    (700, 1152, 5000, 64),
 ])
 def test_rollout_log_probs_over_several_column_tiles(T, d, V, ranges, block):
     """Several column tiles and units per CTA: operand stages, scale slots and accumulator buffers go round more than once, the
